@@ -52,6 +52,44 @@ def test_pack_weights_gptq_bit_exact(resq, N, K, r, fp16, dead_col):
         assert not host(W.w4_i8 if dead_col >= r else W.w8)[:, dead_col - r if dead_col >= r else dead_col].any()
 
 
+@pytest.mark.parametrize("N,K,r,kind", [
+    (1200, 288, 32, "dense"),    # several rows per CTA, a last CTA with fewer, a last block of one 32-column group
+    (600, 544, 512, "dense"),    # segment boundary on a block boundary
+    (8, 32, 0, "dense"),         # one group
+    (2400, 256, 64, "dense"),    # eight rows per CTA
+    (8, 14336, 1792, "sparse"),  # rows too wide for two CTAs per SM
+    (16, 512, 64, "ties"),       # quotients on half-integers, no feedback
+    (16, 512, 64, "tiny"),       # diagonal below the normal float range, zero rows
+])
+def test_pack_weights_gptq_edges(resq, N, K, r, kind):
+    """Bit for bit against the fp64 sweep where the kernel's tiling and its two division routes have edges."""
+    rng = np.random.default_rng(N + K)
+    Wp = synth.projected_weights_direct(N, K, seed=900 + N)
+    U = np.diag(rng.uniform(0.3, 3.0, K))
+    if kind == "dense":
+        U += np.triu(rng.standard_normal((K, K)) * 0.2, 1)
+    elif kind == "sparse":
+        j = rng.integers(0, K - 1, 256)
+        U[j, j + 1 + (rng.random(256) * (K - 1 - j)).astype(int)] = 0.3
+    elif kind == "ties":
+        Wp = (rng.integers(-14, 15, (N, K)) * 0.5 / 64).astype(np.float32)
+        Wp[:, :r] = rng.integers(-254, 255, (N, r)) * 0.5 / 64
+        Wp[:, 0], Wp[:, r] = 127 / 64, 7 / 64  # scales exactly 1/64
+    else:
+        U *= 1e-39
+        U[:, 5] += 1e-41 * (np.arange(K) < 5)
+        Wp[3] = 0.0
+        Wp[4, 1:] = 0.0
+    U = np.ascontiguousarray(U.astype(np.float32))
+    pw = gptq.pack_weights_gptq(Wp, r, U)
+    W = resq.resq_pack_weights_gptq(resq.layer_desc(K, N, r), dev(Wp), dev(U))
+    assert (host(W.w8) == pw.q8).all()
+    assert (host(W.w4_i8) == pw.q4).all()
+    assert (host(W.w4) == pw.w4_packed).all()
+    assert (host(W.s_w8).view(np.uint32) == pw.s8.view(np.uint32)).all()
+    assert (host(W.s_w4).view(np.uint32) == pw.s4.view(np.uint32)).all()
+
+
 def test_layer_on_gptq_weights(resq):
     """resq_linear consumes the GPTQ-rounded weights like any packed weights: output exact against the oracle's layer."""
     T, K, N, r = 48, 1024, 264, 128
