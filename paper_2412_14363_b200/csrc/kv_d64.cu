@@ -1,9 +1,8 @@
 // Attention-block path for d_head = 64 (Section 4.3, Eq. 8; Section 5.1): the same arithmetic and cache format as the
 // d_head = 128 kernels -- 8-bit U_C projection of query and key, per-head asymmetric cache codes with the first
 // d/8 = 8 coefficients in 8 bits and the other 56 in 4 -- written plainly: one warp per head vector, lane l owning
-// coefficients l and l + 32, every division a true IEEE division.  Attention runs one warp per (query row, query
-// head) with one cache position per lane and everything in fp32.  These kernels cover the small model geometry;
-// the tuned paths (mma.sync single-query kernel, tcgen05 tile kernel) are those of d_head = 128.
+// coefficients l and l + 32, every division a true IEEE division.  Attention runs on mma.sync tiles with fp32-accurate
+// weights (below).
 //
 // Block layout for d_head = 64 (the d = 128 layout with every code array halved): per half (key, then value)
 //   c8 [32][8] | c4 [32][28] | meta [32][4] fp32      = 256 + 896 + 512 = 1664 bytes, 3328 per block.
@@ -11,6 +10,7 @@
 #include <cuda_fp16.h>
 
 #include "internal.h"
+#include "ptx.cuh"
 
 namespace resq {
 namespace {
@@ -27,11 +27,6 @@ __device__ __forceinline__ float warp_max(float v) {
 __device__ __forceinline__ float warp_min(float v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v = fminf(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
-}
-__device__ __forceinline__ float warp_sum(float v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
 
@@ -154,92 +149,455 @@ __global__ void __launch_bounds__(kWarps * 32) project_append64_kernel(const Pro
     }
 }
 
+// ---- attention -------------------------------------------------------------------------------------------------
+// Rows (a query row's head vectors that share a KV head) meet STEP cache positions at a time on mma.sync m16n8k16 /
+// m16n8k8, 16 rows per warp, fp32 accumulators.  Two forms of one kernel:
+//   TEAM = 4  four warps share a tile of 64 rows -- 64 / g consecutive tokens of one sequence times the g heads -- and
+//             walk the sequence together (a causal run of new tokens);
+//   TEAM = 1  the g <= 8 rows of one (query row, KV head) are alone: the 12 warps of the CTA take every 12th step
+//             each, with a tile of their own, and their sums are merged at the end (single-query and many-query forms).
+// With few CTAs a cluster splits the steps further and rank 0 merges the sums through distributed shared memory, so
+// no global scratch is needed.
+//
+// A step: the raw blocks arrive by cp.async two steps ahead; the codes are expanded, centred (code - 128, code - 8), to
+// exact halves in two tiles [position][64 coefficients]; K fragments come from ldmatrix, V fragments from
+// ldmatrix.trans, P straight from the score accumulators.  Scales and zero-points act in fp32 on the accumulators:
+//   score = s8 S8 + s4 S4 + (z8 + 128 s8) sum(q8) + (z4 + 8 s4) sum(q4)         (q half, codes exact: products exact)
+//   out   = sum_j p_j s_j (c_j - c0) + sum_j p_j (z_j + c0 s_j)
+// The weights p_j s_j keep fp32's precision as the second product's operand: scaled by 2^(12 - E), E the exponent of the
+// largest value scale so far, they are split into two halves hi + lo (22 bits), two products per fragment.
+// The eight coefficients of a 32-bit word of nibbles are stored in the order 0 4 1 5 2 6 3 7 (one shift and mask per
+// pair); the query fragments are gathered in that order and the outputs put back.
+//
+// What bounds it: the softmax arithmetic and the operand conversions on the CUDA cores (about 20 instructions per score
+// of which two thirds per pair) and, for few rows, the latency of a step; not HBM, not the tensor pipe (26 % busy).
+// 32 query / 8 KV heads, project-and-append included: 1000 new tokens 1355 -> 83 us, a step of 16 sequences of
+// 1024-2048 positions 507 -> 24.6 us, against one warp per (row, query head) that dequantized each position per head.
 struct Attn64Params {
     const uint8_t* cache;
     const __half* q;   // [rows][Hq][64]
     float* out;
-    int rows, Hq, Hkv, n_seqs, capacity;
+    int rows, Hq, Hkv, g, n_seqs, capacity, splits;  // splits: CTAs of a cluster
     const int32_t* seq_of_row;  // null: seq_const if >= 0, else the row index
     const int32_t* len_of_row;  // null: len0 + row + 1
     int seq_const, len0;
     int* status;
 };
 
-// One warp per (row, query head): 32 cache positions at a time, one per lane for the scores, then coefficient-owning
-// lanes (l and l + 32) for the weighted sum of the dequantized values.  Softmax is the running-maximum form in fp32.
-__global__ void __launch_bounds__(kWarps * 32) attention64_kernel(const Attn64Params p) {
-    __shared__ float qs[kWarps][D];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const long long item = static_cast<long long>(blockIdx.x) * kWarps + warp;
-    if (item >= static_cast<long long>(p.rows) * p.Hq) return;
-    const int row = static_cast<int>(item / p.Hq), hq = static_cast<int>(item % p.Hq);
-    const int kvh = hq / (p.Hq / p.Hkv);
-    float* dst = p.out + item * D;
-    int b = p.seq_of_row ? p.seq_of_row[row] : (p.seq_const >= 0 ? p.seq_const : row);
-    int len = p.len_of_row ? p.len_of_row[row] : p.len0 + row + 1;
-    if (b < 0 || b >= p.n_seqs) {
-        if (lane == 0) atomicOr(p.status, kStatusBitIndex);
-        b = 0;
-        len = 0;
+constexpr int kPitch = 144;        // bytes per position of an expanded tile: 64 halves + 16 (ldmatrix without conflicts)
+constexpr int kRecPitch = 68;      // floats per row of a record: 64 sums, maximum, sum of weights
+constexpr int kSplitWarps = 12;    // TEAM = 1: what fits 227 KB
+
+template <int TEAM>
+struct A64 {
+    static constexpr int kStep = TEAM == 1 ? 32 : 64;
+    static constexpr int kNWarps = TEAM == 1 ? kSplitWarps : TEAM;
+    static constexpr int kRaw = kStep / 32 * kBlock;
+    static constexpr int kTeamBytes = 2 * kRaw + 2 * kStep * kPitch + 2 * kStep * 16;
+    static constexpr int kSmem = kTeamBytes * (kNWarps / TEAM);
+    static constexpr int kRows = TEAM == 1 ? 8 : 16;  // rows of a warp in use
+};
+static_assert(A64<1>::kSmem >= kSplitWarps * 8 * kRecPitch * 4 && A64<4>::kSmem >= 4 * 16 * kRecPitch * 4, "records fit");
+
+__device__ __forceinline__ void mma16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void mma8(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t b0) {
+    asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%0,%1,%2,%3};"
+                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a0), "r"(a1), "r"(b0));
+}
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], uint32_t addr) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], uint32_t addr) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ float exp2_approx(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ uint32_t h2_bits(__half2 v) { return *reinterpret_cast<const uint32_t*>(&v); }
+// a, b as two pairs of halves, hi + lo.
+__device__ __forceinline__ void split_h2(float a, float b, uint32_t& hi, uint32_t& lo) {
+    const __half2 h = __floats2half2_rn(a, b);
+    const float2 f = __half22float2(h);
+    hi = h2_bits(h);
+    lo = h2_bits(__floats2half2_rn(a - f.x, b - f.y));
+}
+// Eight codes as halves minus their centre: `word` of nibbles (order 0 4 1 5 2 6 3 7), or eight bytes.
+__device__ __forceinline__ uint4 nibbles_centred(uint32_t word) {
+    const __half2 bias = __half2half2(__ushort_as_half(0x6408));  // 1024 + 8
+    uint32_t v[4];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+        const uint32_t b = ((word >> (4 * m)) & 0x000F000Fu) | 0x64006400u;
+        v[m] = h2_bits(__hsub2(*reinterpret_cast<const __half2*>(&b), bias));
     }
-    if (len < 0 || len > p.capacity) {
-        if (lane == 0) atomicOr(p.status, kStatusBitIndex);
-        len = len < 0 ? 0 : p.capacity;
+    return make_uint4(v[0], v[1], v[2], v[3]);
+}
+__device__ __forceinline__ uint4 bytes_centred(uint2 w) {
+    const __half2 bias = __half2half2(__ushort_as_half(0x6480));  // 1024 + 128
+    uint32_t v[4] = {__byte_perm(w.x, 0x64646464u, 0x4140), __byte_perm(w.x, 0x64646464u, 0x4342),
+                     __byte_perm(w.y, 0x64646464u, 0x4140), __byte_perm(w.y, 0x64646464u, 0x4342)};
+#pragma unroll
+    for (int m = 0; m < 4; ++m) v[m] = h2_bits(__hsub2(*reinterpret_cast<const __half2*>(&v[m]), bias));
+    return make_uint4(v[0], v[1], v[2], v[3]);
+}
+// Coefficient at element e (0..7) of chunk j (0: the 8-bit segment, 1..7: words of nibbles).
+__device__ __forceinline__ int coef64(int j, int e) { return j == 0 ? e : 8 * j + (e >> 1) + ((e & 1) << 2); }
+
+template <int TEAM>
+__global__ void __launch_bounds__(A64<TEAM>::kNWarps * 32, TEAM == 1 ? 1 : 3) attention64_kernel(const Attn64Params p) {
+    using C = A64<TEAM>;
+    constexpr int STEP = C::kStep, NT = STEP / 8;
+    constexpr bool TWO = TEAM != 1;  // rows lane / 4 + 8 are in use
+    constexpr int RH = TWO ? 2 : 1;
+    extern __shared__ __align__(128) uint8_t smem64[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gr = lane >> 2, c = lane & 3;
+    const int team = warp / TEAM, tt = threadIdx.x - team * TEAM * 32;  // thread of the team
+    uint8_t* raw = smem64 + static_cast<size_t>(team) * C::kTeamBytes;
+    uint8_t* Kt = raw + 2 * C::kRaw;
+    uint8_t* Vt = Kt + STEP * kPitch;
+    float4* colK = reinterpret_cast<float4*>(Vt + STEP * kPitch);
+    float4* colV = colK + STEP;
+    const int rank = static_cast<int>(blockIdx.x % p.splits), item = static_cast<int>(blockIdx.x / p.splits);
+    const int kvh = item % p.Hkv, n_tiles = static_cast<int>(gridDim.x) / p.splits / p.Hkv;
+    const int tile = TEAM == 1 ? item / p.Hkv : n_tiles - 1 - item / p.Hkv;  // long tiles of all heads first
+    auto team_sync = [&] {
+        if (TEAM == 1) __syncwarp();
+        else __syncthreads();
+    };
+
+    // ---- rows of this lane, positions they see, the sequence
+    int tok[RH], head[RH], pos_i[RH];
+    int b, limit, pos_min;  // positions any row of the tile sees; the smallest of the rows' own positions
+    if (TEAM == 1) {
+        const int row = tile;
+        b = p.seq_of_row ? p.seq_of_row[row] : (p.seq_const >= 0 ? p.seq_const : row);
+        int len = p.len_of_row ? p.len_of_row[row] : p.len0 + row + 1;
+        const bool report = kvh == 0 && rank == 0 && threadIdx.x == 0;
+        if (b < 0 || b >= p.n_seqs) {
+            if (report) atomicOr(p.status, kStatusBitIndex);
+            b = 0;
+            len = 0;
+        }
+        if (len < 0 || len > p.capacity) {
+            if (report) atomicOr(p.status, kStatusBitIndex);
+            len = len < 0 ? 0 : p.capacity;
+        }
+        limit = len;
+        pos_min = len - 1;
+        tok[0] = gr < p.g ? row : -1;
+        head[0] = kvh * p.g + gr;
+        pos_i[0] = len - 1;
+    } else {
+        b = p.seq_const;
+        const int R0 = tile * 64, n_rows = p.rows * p.g;
+        pos_min = p.len0 + R0 / p.g;
+        limit = p.len0 + min(p.rows - 1, (R0 + 63) / p.g) + 1;
+#pragma unroll
+        for (int h = 0; h < RH; ++h) {
+            const int R = R0 + warp * 16 + gr + 8 * h;
+            tok[h] = R < n_rows ? R / p.g : -1;
+            head[h] = kvh * p.g + R % p.g;
+            pos_i[h] = tok[h] >= 0 ? p.len0 + tok[h] : -1;
+        }
     }
-    qs[warp][lane] = __half2float(p.q[item * D + lane]);
-    qs[warp][lane + 32] = __half2float(p.q[item * D + lane + 32]);
-    __syncwarp();
-    const float* qv = qs[warp];
     const uint8_t* blocks = p.cache + (static_cast<size_t>(b) * p.Hkv + kvh) * (p.capacity / RESQ_KV_BLOCK) * kBlock;
-    float m = -INFINITY, l = 0.f, acc0 = 0.f, acc1 = 0.f;
-    for (int j0 = 0; j0 < len; j0 += 32) {
-        const uint8_t* blk = blocks + static_cast<size_t>(j0 / 32) * kBlock;
-        // score of position j0 + lane
-        float sc = -INFINITY;
-        if (j0 + lane < len) {
-            const float4 km = *reinterpret_cast<const float4*>(blk + kC8 + kC4 + lane * 16);
-            const uint8_t* c8 = blk + lane * R8;
-            const uint8_t* c4 = blk + kC8 + lane * (N4 / 2);
-            float dot = 0.f;
-#pragma unroll
-            for (int i = 0; i < R8; ++i) dot = fmaf(qv[i], fmaf(static_cast<float>(c8[i]), km.x, km.y), dot);
-#pragma unroll
-            for (int i = 0; i < N4 / 2; ++i) {
-                const uint32_t by = c4[i];
-                dot = fmaf(qv[R8 + 2 * i], fmaf(static_cast<float>(by & 15u), km.z, km.w), dot);
-                dot = fmaf(qv[R8 + 2 * i + 1], fmaf(static_cast<float>(by >> 4), km.z, km.w), dot);
-            }
-            sc = dot * 0.125f;  // 1 / sqrt(64)
+    const int n_blocks = (limit + 31) >> 5, n_steps = (limit + STEP - 1) / STEP;
+    // this team's steps: first, first + stride, .. < end
+    const int first = TEAM == 1 ? rank * kSplitWarps + team : static_cast<int>(static_cast<long long>(n_steps) * rank / p.splits);
+    const int end = TEAM == 1 ? n_steps : static_cast<int>(static_cast<long long>(n_steps) * (rank + 1) / p.splits);
+    const int stride = TEAM == 1 ? kSplitWarps * p.splits : 1;
+
+    auto issue = [&](int s, int buf) {  // copies of step s (if it exists) into a raw buffer; always one group
+        if (s < end) {
+            const int nb = min(STEP / 32, n_blocks - s * (STEP / 32));
+            const uint8_t* src = blocks + static_cast<size_t>(s) * C::kRaw;
+            for (int i = tt; i < nb * (kBlock / 16); i += TEAM * 32)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(raw + buf * C::kRaw + i * 16)), "l"(src + i * 16)
+                             : "memory");
         }
-        const float m_new = fmaxf(m, warp_max(sc));
-        const float corr = __expf(m - m_new);  // 0 on the first block (m = -inf)
-        const float pj = j0 + lane < len ? __expf(sc - m_new) : 0.f;
-        l = l * corr + warp_sum(pj);
-        acc0 *= corr;
-        acc1 *= corr;
-        m = m_new;
-        // values: lane owns coefficients lane and lane + 32
-        const uint8_t* vb = blk + kHalf;
-        const int n = min(32, len - j0);
-        for (int j = 0; j < n; ++j) {
-            const float pw = __shfl_sync(0xffffffffu, pj, j);
-            const float4 vm = *reinterpret_cast<const float4*>(vb + kC8 + kC4 + j * 16);
-            float v0;
-            if (lane < R8) {
-                v0 = fmaf(static_cast<float>(vb[j * R8 + lane]), vm.x, vm.y);
-            } else {
-                const uint32_t by = vb[kC8 + j * (N4 / 2) + ((lane - R8) >> 1)];
-                v0 = fmaf(static_cast<float>((lane & 1) ? by >> 4 : by & 15u), vm.z, vm.w);
-            }
-            const uint32_t by1 = vb[kC8 + j * (N4 / 2) + ((lane + 32 - R8) >> 1)];
-            const float v1 = fmaf(static_cast<float>((lane & 1) ? by1 >> 4 : by1 & 15u), vm.z, vm.w);
-            acc0 = fmaf(pw, v0, acc0);
-            acc1 = fmaf(pw, v1, acc1);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    issue(first, 0);
+    issue(first + stride, 1);
+
+    // ---- query fragments: chunk 0 (m16n8k8), chunks 1-6 as three k16 pairs, chunk 7 (m16n8k8); sums per segment
+    uint32_t qa[8][2];
+    float qs8[2] = {0.f, 0.f}, qs4[2] = {0.f, 0.f};
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const bool ok = h < RH && tok[h < RH ? h : 0] >= 0;
+        const __half* qrow = p.q + (static_cast<size_t>(ok ? tok[h < RH ? h : 0] : 0) * p.Hq + (ok ? head[h < RH ? h : 0] : 0)) * D;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            __half2 v = __floats2half2_rn(0.f, 0.f);
+            if (ok) v = __halves2half2(qrow[coef64(j, 2 * c)], qrow[coef64(j, 2 * c + 1)]);
+            qa[j][h] = h2_bits(v);
+            const float2 f = __half22float2(v);
+            if (j == 0) qs8[h] += f.x + f.y;
+            else qs4[h] += f.x + f.y;
+        }
+#pragma unroll
+        for (int o = 1; o < 4; o <<= 1) {
+            qs8[h] += __shfl_xor_sync(0xffffffffu, qs8[h], o);
+            qs4[h] += __shfl_xor_sync(0xffffffffu, qs4[h], o);
         }
     }
-    const float inv = l > 0.f ? 1.f / l : 0.f;
-    dst[lane] = acc0 * inv;
-    dst[lane + 32] = acc1 * inv;
+
+    float O[8][4], m_run[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f}, zs8[2] = {0.f, 0.f}, zs4[2] = {0.f, 0.f};
+#pragma unroll
+    for (int j = 0; j < 8; ++j) O[j][0] = O[j][1] = O[j][2] = O[j][3] = 0.f;
+    constexpr int kExpMin = -114;  // 2^(12 - E) stays a normal float for E in [-114, 127]
+    int E = kExpMin;
+    const float kScore = 1.4426950408889634f * 0.125f;  // log2(e) / sqrt(64)
+    const uint32_t k_addr = smem_u32(Kt) + (lane & 7) * kPitch + (lane >> 3) * 16;
+    const uint32_t v_addr = smem_u32(Vt) + ((lane & 7) + ((lane >> 3) & 1) * 8) * kPitch + (lane >> 4) * 16;
+
+    int buf = 0;
+    for (int s = first; s < end; s += stride, buf ^= 1) {
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        team_sync();  // the step's bytes are in place and nobody reads the previous tiles
+        const uint8_t* rb = raw + buf * C::kRaw;
+        const int j0 = s * STEP;
+        // ---- expand: items of eight coefficients, chunks 0-7 of the keys then of the values
+#pragma unroll
+        for (int i = 0; i < STEP * 16 / (TEAM * 32); ++i) {
+            const int item = i * TEAM * 32 + tt, pos = item % STEP, ch = item / STEP;  // ch is uniform over a warp
+            const uint8_t* half_base = rb + (pos >> 5) * kBlock + (ch >= 8 ? kHalf : 0);
+            const int j = ch & 7, pp = pos & 31;
+            uint4 v;
+            if (j == 0) v = bytes_centred(*reinterpret_cast<const uint2*>(half_base + pp * R8));
+            else v = nibbles_centred(*reinterpret_cast<const uint32_t*>(half_base + kC8 + pp * (N4 / 2) + 4 * (j - 1)));
+            *reinterpret_cast<uint4*>((ch >= 8 ? Vt : Kt) + pos * kPitch + j * 16) = v;
+        }
+        // ---- per-position constants; positions past the tile's limit hold anything and are zeroed by selection
+        int e_new;
+        {
+            float vm = 0.f;
+#pragma unroll
+            for (int i = 0; i < STEP / 32; ++i) {
+                const float4 m = *reinterpret_cast<const float4*>(rb + i * kBlock + kHalf + kC8 + kC4 + lane * 16);
+                if (j0 + 32 * i + lane < limit) vm = fmaxf(vm, fmaxf(m.x, m.z));
+            }
+            const uint32_t eb = __reduce_max_sync(0xffffffffu, __float_as_uint(vm)) >> 23;
+            e_new = max(E, max(static_cast<int>(eb) - 127, kExpMin));
+        }
+        const float f = __uint_as_float(static_cast<uint32_t>(127 + 12 - e_new) << 23);
+#pragma unroll
+        for (int i = 0; i < (2 * STEP) / (TEAM * 32); ++i) {
+            const int item = i * TEAM * 32 + tt, pos = item % STEP;
+            const bool is_v = item >= STEP;
+            float4 m = *reinterpret_cast<const float4*>(rb + (pos >> 5) * kBlock + (is_v ? kHalf : 0) + kC8 + kC4 + (pos & 31) * 16);
+            if (j0 + pos >= limit) m = make_float4(0.f, 0.f, 0.f, 0.f);
+            m.y = fmaf(128.f, m.x, m.y);
+            m.w = fmaf(8.f, m.z, m.w);
+            if (is_v) colV[pos] = make_float4(m.x * f, m.y, m.z * f, m.w);
+            else colK[pos] = make_float4(m.x * kScore, m.y * kScore, m.z * kScore, m.w * kScore);
+        }
+        team_sync();
+        issue(s + 2 * stride, buf);  // everybody is done with this raw buffer
+
+        // ---- scores
+        float sc[NT][2 * RH];
+        float mx[2] = {-INFINITY, -INFINITY};
+        const bool masked = j0 + STEP - 1 > pos_min;
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt) {
+            uint32_t k0[4], k1[4];
+            ldsm4(k0, k_addr + nt * 8 * kPitch);
+            ldsm4(k1, k_addr + nt * 8 * kPitch + 64);
+            float s8[4] = {0.f, 0.f, 0.f, 0.f}, s4[4] = {0.f, 0.f, 0.f, 0.f};
+            mma8(s8, qa[0][0], qa[0][1], k0[0]);
+            mma16(s4, qa[1][0], qa[1][1], qa[2][0], qa[2][1], k0[1], k0[2]);
+            mma16(s4, qa[3][0], qa[3][1], qa[4][0], qa[4][1], k0[3], k1[0]);
+            mma16(s4, qa[5][0], qa[5][1], qa[6][0], qa[6][1], k1[1], k1[2]);
+            mma8(s4, qa[7][0], qa[7][1], k1[3]);
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int pos = 8 * nt + 2 * c + e;
+                const float4 k = colK[pos];
+#pragma unroll
+                for (int h = 0; h < RH; ++h) {
+                    float x = fmaf(k.x, s8[2 * h + e], fmaf(k.z, s4[2 * h + e], fmaf(k.y, qs8[h], k.w * qs4[h])));
+                    if (masked && j0 + pos > pos_i[h]) x = -INFINITY;
+                    sc[nt][2 * h + e] = x;
+                    mx[h] = fmaxf(mx[h], x);
+                }
+            }
+        }
+        // ---- running maximum and the scale of the sums
+        float m_use[RH], corr[RH];
+        bool moved = e_new != E;
+#pragma unroll
+        for (int h = 0; h < RH; ++h) {
+            mx[h] = fmaxf(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], 1));
+            mx[h] = fmaxf(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], 2));
+            const float m_new = fmaxf(m_run[h], mx[h]);
+            m_use[h] = m_new == -INFINITY ? 0.f : m_new;
+            corr[h] = exp2_approx(m_run[h] - m_use[h]);
+            moved |= m_new != m_run[h];
+            m_run[h] = m_new;
+        }
+        if (__any_sync(0xffffffffu, moved)) {
+            const float de = static_cast<float>(E - e_new);
+#pragma unroll
+            for (int h = 0; h < RH; ++h) {
+                l[h] *= corr[h];
+                zs8[h] *= corr[h];
+                zs4[h] *= corr[h];
+                const float co = corr[h] * exp2_approx(de);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    O[j][2 * h] *= co;
+                    O[j][2 * h + 1] *= co;
+                }
+            }
+            E = e_new;
+        }
+        // ---- weights and the second product, 32 positions at a time: the tensor core's fp32 sums are truncated, so a
+        // chain of products runs over 32 positions only and is then added to the running sums with rounding
+#pragma unroll
+        for (int kp = 0; kp < STEP / 32; ++kp) {
+            uint32_t p8h[2][4], p8l[2][4], p4h[2][4], p4l[2][4];
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                const int nt = 4 * kp + t, pos = 8 * nt + 2 * c;
+                const float4 va = colV[pos], vb = colV[pos + 1];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int i = 2 * (t & 1) + h;
+                    if (h >= RH) {
+                        p8h[t >> 1][i] = p8l[t >> 1][i] = p4h[t >> 1][i] = p4l[t >> 1][i] = 0u;
+                        continue;
+                    }
+                    const float pa = exp2_approx(sc[nt][2 * (h % RH)] - m_use[h % RH]);
+                    const float pb = exp2_approx(sc[nt][2 * (h % RH) + 1] - m_use[h % RH]);
+                    l[h] += pa + pb;
+                    zs8[h] = fmaf(pa, va.y, fmaf(pb, vb.y, zs8[h]));
+                    zs4[h] = fmaf(pa, va.w, fmaf(pb, vb.w, zs4[h]));
+                    split_h2(pa * va.x, pb * vb.x, p8h[t >> 1][i], p8l[t >> 1][i]);
+                    split_h2(pa * va.z, pb * vb.z, p4h[t >> 1][i], p4l[t >> 1][i]);
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < 8; j += 2) {
+                float d0[4] = {0.f, 0.f, 0.f, 0.f}, d1[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                for (int ks = 0; ks < 2; ++ks) {
+                    uint32_t v[4];
+                    ldsm4t(v, v_addr + (2 * kp + ks) * 16 * kPitch + j * 16);
+                    if (j == 0) {
+                        mma16(d0, p8l[ks][0], p8l[ks][1], p8l[ks][2], p8l[ks][3], v[0], v[1]);
+                        mma16(d0, p8h[ks][0], p8h[ks][1], p8h[ks][2], p8h[ks][3], v[0], v[1]);
+                    } else {
+                        mma16(d0, p4l[ks][0], p4l[ks][1], p4l[ks][2], p4l[ks][3], v[0], v[1]);
+                        mma16(d0, p4h[ks][0], p4h[ks][1], p4h[ks][2], p4h[ks][3], v[0], v[1]);
+                    }
+                    mma16(d1, p4l[ks][0], p4l[ks][1], p4l[ks][2], p4l[ks][3], v[2], v[3]);
+                    mma16(d1, p4h[ks][0], p4h[ks][1], p4h[ks][2], p4h[ks][3], v[2], v[3]);
+                }
+#pragma unroll
+                for (int e = 0; e < 2 * RH; ++e) {
+                    O[j][e] += d0[e];
+                    O[j + 1][e] += d1[e];
+                }
+            }
+        }
+    }
+
+    // ---- records of the warps (unnormalised sums with the zero-points, maximum, sum of weights), then the merge
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+    float* rec = reinterpret_cast<float*>(smem64);  // [warp][row][kRecPitch], over the tiles
+    const float unscale = __uint_as_float(static_cast<uint32_t>(127 - 12 + E) << 23);
+#pragma unroll
+    for (int h = 0; h < RH; ++h) {
+#pragma unroll
+        for (int o = 1; o < 4; o <<= 1) {
+            l[h] += __shfl_xor_sync(0xffffffffu, l[h], o);
+            zs8[h] += __shfl_xor_sync(0xffffffffu, zs8[h], o);
+            zs4[h] += __shfl_xor_sync(0xffffffffu, zs4[h], o);
+        }
+        float* r = rec + (warp * C::kRows + gr + 8 * h) * kRecPitch;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const float z = j == 0 ? zs8[h] : zs4[h];
+            r[coef64(j, 2 * c)] = fmaf(O[j][2 * h], unscale, z);
+            r[coef64(j, 2 * c + 1)] = fmaf(O[j][2 * h + 1], unscale, z);
+        }
+        if (c == 0) {
+            r[D] = m_run[h];
+            r[D + 1] = l[h];
+        }
+    }
+    __syncwarp();
+    if (p.splits > 1) cluster_sync_all();
+    else __syncthreads();
+    if (rank == 0) {
+        constexpr int kParts = TEAM == 1 ? kSplitWarps : 1;  // records of a row in one CTA
+        const int n_rows = TEAM == 1 ? p.g : 64;
+        for (int i = threadIdx.x; i < n_rows * (D / 4); i += blockDim.x) {
+            const int row = i / (D / 4), c4 = i % (D / 4);
+            const int R = tile * 64 + row;
+            if (TEAM != 1 && R >= p.rows * p.g) continue;
+            const uint32_t local = smem_u32(rec + row * kRecPitch);  // TEAM = 4: warps' rows follow one another
+            float M = -INFINITY, L = 0.f;
+            float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int rk = 0; rk < p.splits; ++rk) {
+                const uint32_t base = cluster_map_addr(local, rk);
+#pragma unroll 4
+                for (int w = 0; w < kParts; ++w) {
+                    const uint32_t a = base + w * C::kRows * kRecPitch * 4;
+                    const float2 ml = ld_cluster_f2(a + D * 4);
+                    const float4 o = ld_cluster_f4(a + c4 * 16);
+                    const float m_new = fmaxf(M, ml.x);
+                    const float ref = m_new == -INFINITY ? 0.f : m_new;
+                    const float f0 = exp2_approx(M - ref), f1 = exp2_approx(ml.x - ref);
+                    L = L * f0 + ml.y * f1;
+                    acc = make_float4(acc.x * f0 + o.x * f1, acc.y * f0 + o.y * f1, acc.z * f0 + o.z * f1, acc.w * f0 + o.w * f1);
+                    M = m_new;
+                }
+            }
+            const float inv = L > 0.f ? 1.f / L : 0.f;
+            const int t = TEAM == 1 ? tile : R / p.g, hq = kvh * p.g + (TEAM == 1 ? row : R % p.g);
+            *reinterpret_cast<float4*>(p.out + (static_cast<size_t>(t) * p.Hq + hq) * D + 4 * c4) =
+                make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv);
+        }
+    }
+    __syncwarp();
+    if (p.splits > 1) cluster_sync_all();  // the records stay until rank 0 has read them
+}
+
+template <int TEAM>
+cudaError_t launch_attention64_form(const Attn64Params& p, unsigned tiles, cudaStream_t st) {
+    static bool attr_set[64] = {};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev >= 64 || !attr_set[dev]) {
+        e = cudaFuncSetAttribute(attention64_kernel<TEAM>, cudaFuncAttributeMaxDynamicSharedMemorySize, A64<TEAM>::kSmem);
+        if (e != cudaSuccess) return e;
+        if (dev < 64) attr_set[dev] = true;
+    }
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(tiles * static_cast<unsigned>(p.Hkv * p.splits));
+    cfg.blockDim = dim3(A64<TEAM>::kNWarps * 32);
+    cfg.dynamicSmemBytes = A64<TEAM>::kSmem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = static_cast<unsigned>(p.splits);
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    count_launch();
+    return cudaLaunchKernelEx(&cfg, attention64_kernel<TEAM>, p);
 }
 
 }  // namespace
@@ -291,6 +649,7 @@ cudaError_t launch_attention64(const resq_kv_cache_t& cache, const void* q16, in
     p.rows = rows;
     p.Hq = n_q_heads;
     p.Hkv = cache.n_kv_heads;
+    p.g = n_q_heads / cache.n_kv_heads;
     p.n_seqs = cache.n_seqs;
     p.capacity = cache.capacity;
     p.seq_of_row = seq_of_row;
@@ -298,10 +657,19 @@ cudaError_t launch_attention64(const resq_kv_cache_t& cache, const void* q16, in
     p.seq_const = seq_const;
     p.len0 = len0;
     p.status = device_status_ptr();
-    const long long items = static_cast<long long>(rows) * n_q_heads;
-    count_launch();
-    attention64_kernel<<<static_cast<unsigned>((items + kWarps - 1) / kWarps), kWarps * 32, 0, st>>>(p);
-    return cudaGetLastError();
+    p.splits = 1;
+    if (seq_const >= 0 && !seq_of_row && !len_of_row) {  // a causal run of one sequence
+        const long long tiles = (static_cast<long long>(rows) * p.g + 63) / 64;
+        const int steps = (len0 + rows + 63) / 64;
+        // three CTAs per SM are in flight; at least four steps per CTA of a cluster
+        while (p.splits < 8 && tiles * p.Hkv * p.splits * 2 <= 3 * 148 && steps >= 8 * p.splits) p.splits *= 2;
+        return launch_attention64_form<4>(p, static_cast<unsigned>(tiles), st);
+    }
+    // one CTA per SM is in flight; at least two steps per warp (the lengths are on the device: the capacity stands in)
+    while (p.splits < 8 && static_cast<long long>(rows) * p.Hkv * p.splits * 2 <= 148 &&
+           cache.capacity / 32 >= 4 * kSplitWarps * p.splits)
+        p.splits *= 2;
+    return launch_attention64_form<1>(p, static_cast<unsigned>(rows), st);
 }
 
 }  // namespace resq

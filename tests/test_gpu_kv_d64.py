@@ -138,3 +138,50 @@ def test_attention_three_forms_against_the_oracle(resq, kv, uc):
     ref = okv.attention_decode(hq16[:2], K_hat, V_hat, [S0, S1], Hq, Hkv)
     assert np.abs(host(one) - ref).max() <= 1e-4 * vmax
     assert resq.resq_device_status() == resq.OK
+
+
+@pytest.mark.parametrize("Hq,Hkv,lens,T", [
+    (8, 8, [1, 33, 1029, 2050], 1),     # one head per group; few CTAs: the positions are split over a cluster
+    (16, 2, [705, 64, 31], 43),         # eight heads per group, a tile of 64 rows ends inside a token's group
+    (12, 4, [130], 130),                # three heads per group: rows of a token on both sides of a tile edge
+    (64, 8, [385] * 5, 9),              # no split: 40 (sequence, head) pairs
+])
+def test_attention_tile_edges(resq, kv, uc, Hq, Hkv, lens, T):
+    """Single-query over all sequences, the causal run of the last T positions of the first, and the same rows as many
+    queries, on caches whose unwritten bytes are 0xFF.  |out - oracle| <= 2e-5 max|v|: everything is fp32 (a weight is two
+    halves, 2^-22), a score of at most 40 in log2 units carries 2^-22 of itself."""
+    W_C, wq, s_u = uc
+    B, cap = len(lens), (max(lens) + 31) // 32 * 32 + 32
+    cache = kv.KvCache(B, Hkv, cap, d_head=D)
+    cache.data.fill_(0xFF)
+    K_hat, V_hat = [], []
+    for b, n in enumerate(lens):
+        k = synth.head_vectors(n, Hkv, D, stream=1100 + b, lead=1.0, scale=1.5)
+        v = synth.head_vectors(n, Hkv, D, stream=1200 + b, lead=4.0, shift=0.3, scale=10.0 ** (2 * b - 2))
+        kv.resq_kv_append(cache, bf16_to_dev(synth.f32_to_bf16_bits(k)), bf16_to_dev(synth.f32_to_bf16_bits(v)),
+                          dev(np.full(n, b, np.int32)), dev(np.arange(n, dtype=np.int32)), wq, s_u)
+        hk, hv = _oracle_records(k, v, W_C)
+        dk, dv = okv.kv_dequantize(hk).reshape(n, Hkv, D), okv.kv_dequantize(hv).reshape(n, Hkv, D)
+        K_hat.append([dk[:, h] for h in range(Hkv)])
+        V_hat.append([dv[:, h] for h in range(Hkv)])
+    vmax = [max(np.abs(x).max() for x in V) for V in V_hat]
+    n_q = max(T, B)
+    q16 = torch.empty((n_q, Hq, D), dtype=torch.float16, device="cuda")
+    kv.resq_query_project(bf16_to_dev(synth.f32_to_bf16_bits(synth.head_vectors(n_q, Hq, D, stream=1300, lead=1.0, scale=1.5))),
+                          wq, s_u, q16)
+    hq16 = host(q16)
+    one = torch.full((B, Hq, D), float("nan"), dtype=torch.float32, device="cuda")
+    kv.resq_attention_decode(cache, q16[:B].contiguous(), dev(np.array(lens, np.int32)), one, kv.attention_workspace(cache, Hq))
+    ref = okv.attention_decode(hq16[:B], K_hat, V_hat, lens, Hq, Hkv)
+    for b in range(B):
+        assert np.abs(host(one)[b] - ref[b]).max() <= 2e-5 * vmax[b], b
+    pos0 = lens[0] - T
+    q = q16[:T].contiguous()
+    ref = okv.attention_queries(hq16[:T], K_hat, V_hat, np.zeros(T, np.int32), np.arange(pos0 + 1, pos0 + T + 1), Hq, Hkv)
+    run = torch.full((T, Hq, D), float("nan"), dtype=torch.float32, device="cuda")
+    kv.resq_attention_prefill(cache, q, 0, pos0, run)
+    assert np.abs(host(run) - ref).max() <= 2e-5 * vmax[0]
+    many = torch.full((T, Hq, D), float("nan"), dtype=torch.float32, device="cuda")
+    kv.resq_attention_queries(cache, q, dev(np.zeros(T, np.int32)), dev(np.arange(pos0 + 1, pos0 + T + 1, dtype=np.int32)), many)
+    assert np.abs(host(many) - ref).max() <= 2e-5 * vmax[0]
+    assert resq.resq_device_status() == resq.OK
