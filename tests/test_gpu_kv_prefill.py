@@ -57,6 +57,9 @@ def _fill(kv, uc, cache, b, n, Hkv, stream, v_scale=1.0, v_shift=0.3):
     (5, 90, 8, 8, 1e-4),       # value scales far below / above 1: the power-of-two normalisation
     (5, 90, 8, 8, 3e3),
     (260, 1, 8, 2, 1.0),       # a single new token (a generation step written as a prefill)
+    (2000, 40, 8, 2, 1.0),     # few CTAs, many steps: the steps are split over a cluster of eight
+    (600, 100, 12, 4, 30.0),   # a cluster of four whose first tile of rows sees fewer steps than the last
+    (1, 600, 32, 8, 1.0),      # two tiles per CTA, the last CTA's second tile empty
 ])
 def test_attention_prefill_against_the_oracle(resq, kv, uc, prefix, T, Hq, Hkv, v_scale):
     S = prefix + T
@@ -82,6 +85,34 @@ def test_attention_prefill_against_the_oracle(resq, kv, uc, prefix, T, Hq, Hkv, 
         vmax = np.abs(V_hat[h // g]).max()
         err = np.abs(got[:, h] - ref[:, h]).max()
         assert err <= 1e-3 * vmax, (h, err, vmax)
+
+
+@pytest.mark.parametrize("prefix,T,Hq,Hkv", [(0, 400, 8, 2), (900, 60, 4, 4), (0, 300, 32, 16)])
+def test_attention_prefill_with_scores_that_keep_growing(resq, kv, uc, prefix, T, Hq, Hkv):
+    """Keys that grow with the position: a row's maximum rises by far more than 2^8 over
+    its steps, so the output accumulator is rescaled along the way, in one-tile, two-tile and split forms."""
+    S = prefix + T
+    W_C, wq, s_u = uc
+    cache = kv.KvCache(1, Hkv, (S + 31) // 32 * 32)
+    cache.data.fill_(0xFF)
+    ramp = (0.2 + 6.0 * np.arange(S) / S)[:, None, None].astype(np.float32)
+    k = synth.to_bf16_values(synth.head_vectors(S, Hkv, D, stream=760, lead=1.0, scale=1.0) * ramp)
+    v = synth.head_vectors(S, Hkv, D, stream=761, lead=4.0, shift=0.3)
+    kv.resq_kv_append(cache, bf16_to_dev(synth.f32_to_bf16_bits(k)), bf16_to_dev(synth.f32_to_bf16_bits(v)),
+                      dev(np.zeros(S, np.int32)), dev(np.arange(S, dtype=np.int32)), wq, s_u)
+    Yk, _, _ = okv.project_int8(k.reshape(-1, D), *okv.quantize_uc(W_C))
+    dk = okv.kv_dequantize(okv.kv_quantize(Yk)).reshape(S, Hkv, D)
+    dv = okv.kv_dequantize(okv.kv_quantize(v.reshape(-1, D))).reshape(S, Hkv, D)
+    K_hat, V_hat = [dk[:, h] for h in range(Hkv)], [dv[:, h] for h in range(Hkv)]
+    q = synth.head_vectors(T, Hq, D, stream=762, lead=1.0, scale=2.0)
+    q16 = torch.empty((T, Hq, D), dtype=torch.float16, device="cuda")
+    kv.resq_query_project(bf16_to_dev(synth.f32_to_bf16_bits(q)), wq, s_u, q16)
+    out = torch.full((T, Hq, D), float("nan"), dtype=torch.float32, device="cuda")
+    kv.resq_attention_prefill(cache, q16, 0, prefix, out)
+    assert resq.resq_device_status() == resq.OK
+    ref = okv.attention_queries(host(q16), [K_hat], [V_hat], np.zeros(T, np.int32), np.arange(prefix + 1, S + 1), Hq, Hkv)
+    for h in range(Hq):
+        assert np.abs(host(out)[:, h] - ref[:, h]).max() <= 1e-3 * np.abs(V_hat[h // (Hq // Hkv)]).max(), h
 
 
 def test_attention_prefill_agrees_with_the_many_query_call(resq, kv, uc):
