@@ -589,8 +589,7 @@ int resq_uc_quantize(const float* W_C, int d_head, int8_t* wq, float* s_u, void*
     if (!W_C || !wq || !s_u) return RESQ_ERR_NULL;
     if (!aligned16(W_C) || !aligned16(wq) || !aligned16(s_u)) return RESQ_ERR_ALIGN;
     if (int e = check_arch()) return e;
-    if (d_head == 64) return cuda_status(launch_uc_quantize64(W_C, wq, s_u, static_cast<cudaStream_t>(stream)));
-    return cuda_status(launch_uc_quantize(W_C, wq, s_u, static_cast<cudaStream_t>(stream)));
+    return cuda_status(launch_uc_quantize(W_C, d_head, wq, s_u, static_cast<cudaStream_t>(stream)));
 }
 
 int resq_query_project(const void* q, int64_t rows, int d_head, const int8_t* wq, const float* s_u, void* q_out,
@@ -599,7 +598,7 @@ int resq_query_project(const void* q, int64_t rows, int d_head, const int8_t* wq
     if (!q || !wq || !s_u || !q_out) return RESQ_ERR_NULL;
     if (!aligned16(q) || !aligned16(wq) || !aligned16(s_u) || !aligned16(q_out)) return RESQ_ERR_ALIGN;
     if (int e = check_arch()) return e;
-    return cuda_status((d_head == 64 ? launch_qkv_project_append64 : launch_qkv_project_append)(nullptr, q, rows, q_out, nullptr, nullptr, 0, nullptr, nullptr, wq, s_u,
+    return cuda_status(launch_qkv_project_append(nullptr, d_head, q, rows, q_out, nullptr, nullptr, 0, nullptr, nullptr, wq, s_u,
                                                  static_cast<cudaStream_t>(stream)));
 }
 
@@ -610,7 +609,7 @@ int resq_kv_append(const resq_kv_cache_t* cache, const void* k, const void* v, i
     if (!k || !v || !seq_ids || !positions || !wq || !s_u) return RESQ_ERR_NULL;
     if (!aligned16(k) || !aligned16(v) || !aligned16(wq) || !aligned16(s_u)) return RESQ_ERR_ALIGN;
     if (int e = check_arch()) return e;
-    return cuda_status((cache->d_head == 64 ? launch_qkv_project_append64 : launch_qkv_project_append)(cache, nullptr, 0, nullptr, k, v, T, seq_ids, positions, wq, s_u,
+    return cuda_status(launch_qkv_project_append(cache, cache->d_head, nullptr, 0, nullptr, k, v, T, seq_ids, positions, wq, s_u,
                                                  static_cast<cudaStream_t>(stream)));
 }
 
@@ -623,7 +622,7 @@ int resq_qkv_project_append(const resq_kv_cache_t* cache, const void* q, int n_q
     if (!aligned16(q) || !aligned16(q_out) || !aligned16(k) || !aligned16(v) || !aligned16(wq) || !aligned16(s_u))
         return RESQ_ERR_ALIGN;
     if (int e = check_arch()) return e;
-    return cuda_status((cache->d_head == 64 ? launch_qkv_project_append64 : launch_qkv_project_append)(cache, q, T * n_q_heads, q_out, k, v, T, seq_ids, positions, wq, s_u,
+    return cuda_status(launch_qkv_project_append(cache, cache->d_head, q, T * n_q_heads, q_out, k, v, T, seq_ids, positions, wq, s_u,
                                                  static_cast<cudaStream_t>(stream)));
 }
 

@@ -139,6 +139,37 @@ def test_fused_project_append_matches_the_two_calls(resq, kv, uc):
         assert (host(ca.data) != 7).any()
 
 
+@pytest.mark.parametrize("d", [128, 64])
+def test_many_vectors_write_what_few_at_a_time_write(resq, kv, d):
+    """One call with more than 12288 head vectors (16-vector warp tiles, the last ones ragged) and the same tokens in calls
+    of 100 (one warp per vector, checked against the oracle above and in test_gpu_kv_d64.py): the same bytes."""
+    T, Hq, Hkv = 309, 24, 8
+    wq, s_u = kv.resq_uc_quantize(dev(np.ascontiguousarray(synth.haar_orthogonal(d).T.astype(np.float32))))
+    heads = {n: synth.head_vectors(T, h, d, stream=800 + i, lead=4.0, scale=0.7)
+             for i, (n, h) in enumerate((("q", Hq), ("k", Hkv), ("v", Hkv)))}
+    for x in heads.values():
+        x[5, 1] = 0.0                    # a zero vector
+        x[6, 0, : d // 8] = x[6, 0, 0]   # a constant 8-bit segment
+        x[7, 2, d // 8:] = -1.5          # a constant 4-bit segment
+        x[8, 3] *= 1e30
+        x[9, 3] = synth.to_bf16_values(x[9, 3] * np.float32(1e-30))
+        x[10, 0] = np.tile(np.arange(8, dtype=np.float32) - 3.5, d // 8)  # quotients on half-integers
+        x[10, 0, :2] = 127.0, 0.0
+    q, k, v = (bf16_to_dev(synth.f32_to_bf16_bits(heads[n])) for n in "qkv")
+    seq_ids, positions = dev((np.arange(T) % 3).astype(np.int32)), dev((np.arange(T) // 3).astype(np.int32))
+    ca, cb = kv.KvCache(3, Hkv, 128, d), kv.KvCache(3, Hkv, 128, d)
+    ca.data.fill_(7)
+    cb.data.fill_(7)
+    qa, qb = (torch.zeros((T, Hq, d), dtype=torch.float16, device="cuda") for _ in range(2))
+    kv.resq_qkv_project_append(ca, q, qa, k, v, seq_ids, positions, wq, s_u)
+    for t in range(0, T, 100):
+        part = slice(t, min(T, t + 100))
+        kv.resq_qkv_project_append(cb, q[part], qb[part], k[part], v[part], seq_ids[part].clone(), positions[part].clone(), wq, s_u)
+    assert resq.resq_device_status() == resq.OK
+    assert (host(qa).view(np.uint16) == host(qb).view(np.uint16)).all()
+    assert (host(ca.data) == host(cb.data)).all()
+
+
 def _attention_case(kv, seq_lens, Hq, Hkv, capacity, seed, v_scale=1.0, v_shift=0.3, fill=0xFF, device_consumer=False):
     """Cache image built on the CPU from the oracle's codes (no GPU kernel upstream), attention on both sides."""
     B = len(seq_lens)
