@@ -229,7 +229,7 @@ int resq_project_quantize(const void* X, const void* P, int T, int K, int r, int
                                                   x4 ? x4 + static_cast<size_t>(t0) * K4 / 2 : nullptr, s_x8 + t0,
                                                   s_x4 + t0, false,
                                                   x4_i8 ? x4_i8 + static_cast<size_t>(t0) * K4 : nullptr,
-                                                  static_cast<size_t>(K) * 4, st, true);
+                                                  static_cast<size_t>(K) * 4, st);
             e != cudaSuccess)
             return cuda_status(e);
     }
@@ -264,12 +264,13 @@ int resq_project(const void* X, const void* P, int T, int K, float* C, void* wor
 static int mixed_gemm_impl(const resq_layer_desc_t* d, int T, const int8_t* x8, const uint8_t* x4,
                            const int8_t* x4e_ready, const float* s_x8, const float* s_x4, const resq_weights_t* W,
                            void* Y, int y_dtype, int32_t* dbg8, int32_t* dbg4, char* ws, const Workspace& map,
-                           cudaStream_t st) {
+                           cudaStream_t st, bool after_quantizer) {
     const bool fp16 = d->w_scale_dtype == RESQ_SCALE_FP16;
     const size_t K4 = static_cast<size_t>(d->K - d->r);
     if (T <= kDecodeMaxT) {
         const cudaError_t e = launch_mixed_gemm_stream(T, d->n_out, d->K, d->r, x8, x4, s_x8, s_x4, W->w8, W->w4,
-                                                       W->s_w8, W->s_w4, fp16, Y, y_dtype, dbg8, dbg4, st);
+                                                       W->s_w8, W->s_w4, fp16, Y, y_dtype, dbg8, dbg4, st,
+                                                       after_quantizer);
         if (e != cudaErrorNotSupported) return cuda_status(e);
         // Rows too wide to stage 9-16 tokens of activation codes beside the weight rings run as two launches of at
         // most 8 tokens (the weights are streamed twice; only reduction lengths beyond ~24k reach this).
@@ -282,7 +283,7 @@ static int mixed_gemm_impl(const resq_layer_desc_t* d, int T, const int8_t* x8, 
                 x4 + static_cast<size_t>(t0) * (K4 / 2), s_x8 + t0, s_x4 + t0, W->w8, W->w4, W->s_w8, W->s_w4, fp16,
                 static_cast<char*>(Y) + static_cast<size_t>(t0) * d->n_out * ysz, y_dtype,
                 dbg8 ? dbg8 + static_cast<size_t>(t0) * d->n_out : nullptr,
-                dbg4 ? dbg4 + static_cast<size_t>(t0) * d->n_out : nullptr, st);
+                dbg4 ? dbg4 + static_cast<size_t>(t0) * d->n_out : nullptr, st, after_quantizer && t0 == 0);
             if (e2 == cudaErrorNotSupported) return RESQ_ERR_SHAPE;
             if (e2 != cudaSuccess) return cuda_status(e2);
         }
@@ -328,7 +329,7 @@ int resq_mixed_gemm(const resq_layer_desc_t* d, int T, const int8_t* x8, const u
     if (!workspace || workspace_bytes < map.total) return RESQ_ERR_WORKSPACE;
     if (int e = check_arch()) return e;
     return mixed_gemm_impl(d, T, x8, x4, x4_i8, s_x8, s_x4, W, Y, y_dtype, dbg_acc8, dbg_acc4,
-                           static_cast<char*>(workspace), map, static_cast<cudaStream_t>(stream));
+                           static_cast<char*>(workspace), map, static_cast<cudaStream_t>(stream), false);
 }
 
 int resq_linear(const resq_layer_desc_t* d, int T, const void* X, const void* P, const resq_weights_t* W, void* Y,
@@ -353,7 +354,7 @@ int resq_linear(const resq_layer_desc_t* d, int T, const void* X, const void* P,
                                       workspace_bytes - map.panel, stream))
         return e;
     return mixed_gemm_impl(d, T, x8, x4, x4e, s_x8, s_x4, W, Y, y_dtype, nullptr, nullptr, ws, map,
-                           static_cast<cudaStream_t>(stream));
+                           static_cast<cudaStream_t>(stream), true);
 }
 
 // ---------------------------------------------------------------- asymmetric activations (Section 5.1)
@@ -411,14 +412,14 @@ static int mixed_gemm_asym_impl(const resq_layer_desc_t* d, int T, const uint8_t
                                 const uint8_t* u4e_ready, const float* s_x8, const float* s_x4, const float* z_x8,
                                 const float* z_x4, const resq_weights_t* W, const int32_t* wsum8, const int32_t* wsum4,
                                 void* Y, int y_dtype, int32_t* dbg8, int32_t* dbg4, char* ws, const Workspace& map,
-                                cudaStream_t st) {
+                                cudaStream_t st, bool after_quantizer) {
     const size_t K4 = static_cast<size_t>(d->K - d->r);
     if (T <= kDecodeMaxT && u4) {
         // Few tokens and packed codes at hand: the weight-streaming kernel (falls through if it cannot stage them).
         const cudaError_t e = launch_mixed_gemm_stream(T, d->n_out, d->K, d->r, reinterpret_cast<const int8_t*>(u8), u4,
                                                        s_x8, s_x4, W->w8, W->w4, W->s_w8, W->s_w4,
                                                        d->w_scale_dtype == RESQ_SCALE_FP16, Y, y_dtype, dbg8, dbg4, st,
-                                                       z_x8, z_x4, wsum8, wsum4);
+                                                       after_quantizer, z_x8, z_x4, wsum8, wsum4);
         if (e != cudaErrorNotSupported) return cuda_status(e);
         if (T > 8) {
             // Rows too wide to stage 9-16 tokens beside the weight rings: two launches of at most 8 tokens, as in the
@@ -432,7 +433,8 @@ static int mixed_gemm_asym_impl(const resq_layer_desc_t* d, int T, const uint8_t
                     u4 + static_cast<size_t>(t0) * (K4 / 2), s_x8 + t0, s_x4 + t0, W->w8, W->w4, W->s_w8, W->s_w4,
                     d->w_scale_dtype == RESQ_SCALE_FP16, static_cast<char*>(Y) + static_cast<size_t>(t0) * d->n_out * ysz,
                     y_dtype, dbg8 ? dbg8 + static_cast<size_t>(t0) * d->n_out : nullptr,
-                    dbg4 ? dbg4 + static_cast<size_t>(t0) * d->n_out : nullptr, st, z_x8 + t0, z_x4 + t0, wsum8, wsum4);
+                    dbg4 ? dbg4 + static_cast<size_t>(t0) * d->n_out : nullptr, st, after_quantizer && t0 == 0, z_x8 + t0,
+                    z_x4 + t0, wsum8, wsum4);
                 if (e2 == cudaErrorNotSupported) {
                     if (t0 > 0) return RESQ_ERR_SHAPE;  // cannot happen: the plan does not depend on the row offset
                     done = false;
@@ -483,7 +485,7 @@ int resq_mixed_gemm_asym(const resq_layer_desc_t* d, int T, const uint8_t* u8, c
     if (!workspace || workspace_bytes < map.total) return RESQ_ERR_WORKSPACE;
     if (int e = check_arch()) return e;
     return mixed_gemm_asym_impl(d, T, u8, u4, u4_u8, s_x8, s_x4, z_x8, z_x4, W, wsum8, wsum4, Y, y_dtype, dbg_acc8,
-                                dbg_acc4, static_cast<char*>(workspace), map, static_cast<cudaStream_t>(stream));
+                                dbg_acc4, static_cast<char*>(workspace), map, static_cast<cudaStream_t>(stream), false);
 }
 
 int resq_linear_asym(const resq_layer_desc_t* d, int T, const void* X, const void* P, const resq_weights_t* W,
@@ -512,7 +514,7 @@ int resq_linear_asym(const resq_layer_desc_t* d, int T, const void* X, const voi
                                            workspace_bytes - map.panel, stream))
         return e;
     return mixed_gemm_asym_impl(d, T, u8, u4, u4e, s_x8, s_x4, z_x8, z_x4, W, wsum8, wsum4, Y, y_dtype, nullptr,
-                                nullptr, ws, map, static_cast<cudaStream_t>(stream));
+                                nullptr, ws, map, static_cast<cudaStream_t>(stream), true);
 }
 
 size_t resq_workspace_bytes_asym(const resq_layer_desc_t* d, int T, int has_P, int has_w4_i8) {

@@ -684,18 +684,9 @@ cudaError_t launch_variant(const CUtensorMap (&tm)[4], const Params& p, int grid
         if (e != cudaSuccess) return e;
         attr_set[dev] = true;
     }
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid, 1, 1);
-    cfg.blockDim = dim3(kThreads, 1, 1);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = p.early_weights ? 1 : 0;
+    // the kernel waits for the preceding grid itself, before or after its first weights (early_weights)
     count_launch();
-    return cudaLaunchKernelEx(&cfg, kern, tm[0], tm[1], tm[2], tm[3], p);
+    return launch_programmatic(kern, grid, kThreads, smem, st, tm[0], tm[1], tm[2], tm[3], p);
 }
 
 // How a launch cuts its work and its shared memory: chunk width, staging form, ring depth, grid.
@@ -753,6 +744,9 @@ void fill_split(const Plan& pl, int& uq, int& urem, int (&tab)[2][kWarps + 1]) {
 
 }  // namespace
 
+// Behind a row quantizer the whole ring is requested before the wait for it: the quantizer of at most 16 rows needs neither
+// the SMs nor the bandwidth.
+static constexpr int kAfterQuantizer = 2;
 static int g_early_weights = 0;
 void set_decode_early_weights(int on) { g_early_weights = on < 0 ? 0 : (on > 2 ? 2 : on); }
 
@@ -760,8 +754,8 @@ void set_decode_early_weights(int on) { g_early_weights = on < 0 ? 0 : (on > 2 ?
 cudaError_t launch_mixed_gemm_stream(int T, int N, int K, int r, const int8_t* x8, const uint8_t* x4,
                                      const float* s_x8, const float* s_x4, const int8_t* w8, const uint8_t* w4,
                                      const void* s_w8, const void* s_w4, bool w_scale_fp16, void* Y, int y_dtype,
-                                     int32_t* dbg8, int32_t* dbg4, cudaStream_t st, const float* z_x8,
-                                     const float* z_x4, const int32_t* wsum8, const int32_t* wsum4) {
+                                     int32_t* dbg8, int32_t* dbg4, cudaStream_t st, bool after_quantizer,
+                                     const float* z_x8, const float* z_x4, const int32_t* wsum8, const int32_t* wsum4) {
     const bool asym = z_x8 != nullptr;  // then x8 / x4 hold unsigned codes
     int dev = 0, sms = 148;
     cudaError_t e = cudaGetDevice(&dev);
@@ -776,7 +770,7 @@ cudaError_t launch_mixed_gemm_stream(int T, int N, int K, int r, const int8_t* x
     p.c8 = pl.c8; p.c4 = pl.c4; p.pitch8 = pl.pitch8; p.pitch4 = pl.pitch4;
     p.nstages = pl.nstages;
     p.ring_ofs = static_cast<int>(pl.fixed);
-    p.early_weights = g_early_weights;
+    p.early_weights = g_early_weights ? g_early_weights : after_quantizer ? kAfterQuantizer : 0;
     p.x8 = x8; p.x4 = x4; p.s_x8 = s_x8; p.s_x4 = s_x4; p.s_w8 = s_w8; p.s_w4 = s_w4;
     p.w_fp16 = w_scale_fp16 ? 1 : 0;
     p.z_x8 = z_x8; p.z_x4 = z_x4; p.wsum8 = wsum8; p.wsum4 = wsum4;

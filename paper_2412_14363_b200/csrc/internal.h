@@ -18,15 +18,30 @@ void count_launch(int n = 1);
 constexpr int kStatusBitTimeout = 1;  // a bounded wait ran out
 constexpr int kStatusBitIndex = 2;    // an index read on the device was out of range
 
+// Launch with programmatic stream serialization: the kernel's CTAs may be scheduled while the preceding grid drains, so the
+// kernel executes griddepcontrol.wait before it touches anything of it -- and before it lets its own dependents start.
+template <class... P, class... A>
+cudaError_t launch_programmatic(void (*kern)(P...), size_t grid, int threads, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(grid), 1, 1);
+    cfg.blockDim = dim3(static_cast<unsigned>(threads), 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+
 // ---- kernels (launch wrappers; return cudaGetLastError()) ----------------------------------
 // Split quantization of the rows of a [rows][K] matrix (Eq. 2 for activations, Eq. 3 for weights).
 //   in_is_f32: rows are fp32 (weights, projected coefficients) instead of bf16.
 //   scale_fp16: scales are rounded to and stored as fp16 (weights only).
-//   programmatic: enqueue with programmatic stream serialization (the kernel waits for the preceding grid itself,
-//                 so its CTAs can be scheduled while that grid drains); only the whole-row kernel honours it.
 cudaError_t launch_split_quantize(const void* in, bool in_is_f32, size_t rows, int K, int r, int8_t* q8,
                                   uint8_t* q4, void* s8, void* s4, bool scale_fp16, int8_t* q4_i8,
-                                  size_t in_row_stride, cudaStream_t st, bool programmatic = false);
+                                  size_t in_row_stride, cudaStream_t st);
 
 // GPTQ rounding of the rows of W [N][K] fp32 with the upper Cholesky factor U [K][K] fp32 of the inverse Hessian
 // (Section 5.1); dead: optional [K] bytes, non-zero = the column's weights are zeroed.  Returns cudaErrorNotSupported
@@ -68,9 +83,12 @@ cudaError_t launch_weight_row_sums(const int8_t* w8, const uint8_t* w4, int N, i
 cudaError_t launch_mixed_gemm_stream(int T, int N, int K, int r, const int8_t* x8, const uint8_t* x4,
                                      const float* s_x8, const float* s_x4, const int8_t* w8, const uint8_t* w4,
                                      const void* s_w8, const void* s_w4, bool w_scale_fp16, void* Y, int y_dtype,
-                                     int32_t* dbg8, int32_t* dbg4, cudaStream_t st, const float* z_x8 = nullptr,
-                                     const float* z_x4 = nullptr, const int32_t* wsum8 = nullptr,
-                                     const int32_t* wsum4 = nullptr);  // z_x8 != NULL: asymmetric, unsigned codes
+                                     int32_t* dbg8, int32_t* dbg4, cudaStream_t st, bool after_quantizer = false,
+                                     const float* z_x8 = nullptr, const float* z_x4 = nullptr,
+                                     const int32_t* wsum8 = nullptr, const int32_t* wsum4 = nullptr);
+// z_x8 != NULL: asymmetric, unsigned codes.  after_quantizer: the kernel enqueued just before is one of the row
+// quantizers above, which lets a dependent start only once everything before IT is complete: the weights may be streamed
+// while it runs.
 void set_decode_early_weights(int on);
 
 // Online projection C = X·P (bf16 x bf16 -> fp32) on tcgen05 kind::f16, CTA pairs; writes fp32 C [T][K].

@@ -129,6 +129,9 @@ mixed_gemm_kernel(const __grid_constant__ CUtensorMap tmA8, const __grid_constan
     cluster_sync_all();  // the peer's barriers exist before anything is signalled across
     tc_fence_after();
     const uint32_t tmem_base = sh->tmem_base;
+    // Launched with programmatic stream serialization: the set-up above ran under the tail of the preceding grid.
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer
@@ -377,9 +380,8 @@ cudaError_t launch_mixed_gemm_tiles(int T, int N, int K, int r, const int8_t* x8
     const int tiles = p.m_tiles * p.n_tiles;
     const int pairs = tiles < sms / 2 ? tiles : sms / 2;
     count_launch();
-    if (asym) mixed_gemm_kernel<true><<<2 * pairs, kThreads, kSmemBytes, st>>>(tA8, tA4, tB8, tB4, p);
-    else mixed_gemm_kernel<false><<<2 * pairs, kThreads, kSmemBytes, st>>>(tA8, tA4, tB8, tB4, p);
-    return cudaGetLastError();
+    return launch_programmatic(asym ? mixed_gemm_kernel<true> : mixed_gemm_kernel<false>, 2 * pairs, kThreads, kSmemBytes, st,
+                               tA8, tA4, tB8, tB4, p);
 }
 
 }  // namespace resq

@@ -180,6 +180,7 @@ project_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_c
     cluster_sync_all();  // the peer's barriers exist before anything is signalled across
     tc_fence_after();
     const uint32_t tmem_base = sh->tmem_base;
+    griddep_wait();  // the set-up above ran under the tail of the preceding grid
     griddep_launch_dependents();  // a kernel enqueued with programmatic serialization is scheduled as SMs free up
 
     if (warp == 0) {
@@ -354,6 +355,7 @@ project_gemm_few_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_co
     cluster_sync_all();
     tc_fence_after();
     const uint32_t tmem_base = sh->tmem_base;
+    griddep_wait();  // the set-up above ran under the tail of the preceding grid
     griddep_launch_dependents();  // a kernel enqueued with programmatic serialization is scheduled as SMs free up
 
     if (warp == 0) {
@@ -543,8 +545,9 @@ cudaError_t launch_project_few(const void* X, const void* P, int T, int K, float
     const int items = p.full_items + p.split_tiles * p.splits;
     const int pairs = items < all_pairs ? items : all_pairs;
     count_launch();
-    project_gemm_few_kernel<<<2 * pairs, kThreads, kFewSmemBytes, st>>>(tX, tP, p, ntok);
-    if (cudaError_t le = cudaGetLastError(); le != cudaSuccess) return le;
+    if (cudaError_t e = launch_programmatic(project_gemm_few_kernel, 2 * pairs, kThreads, kFewSmemBytes, st, tX, tP, p, ntok);
+        e != cudaSuccess)
+        return e;
     if (p.split_tiles > 0) {
         return launch_reduce(p, st);
     }
@@ -611,8 +614,8 @@ cudaError_t launch_project_gemm(const void* X, const void* P, int T, int K, floa
         }
     }
     count_launch();
-    project_gemm_pair_kernel<<<2 * pairs, kThreads, kSmemBytes, st>>>(tX, tP, p);
-    if (cudaError_t le = cudaGetLastError(); le != cudaSuccess) return le;
+    e = launch_programmatic(project_gemm_pair_kernel, 2 * pairs, kThreads, kSmemBytes, st, tX, tP, p);
+    if (e != cudaSuccess) return e;
     if (p.split_tiles > 0) return launch_reduce(p, st);
     return cudaSuccess;
 }

@@ -222,27 +222,49 @@ __device__ __forceinline__ void fast_codes(const Chunk<F32>& ch, float s, float 
     }
 }
 
+// The asymmetric form (Eq. 1, second form): code = round-half-even(fl(fl(x - z) / s)) clamped to [0, qmax].  The same
+// bracket around 1 / s on d = fl(x - z): quotients reach 255, where a bracketed product still rounds to an integer in one
+// fma and the argument above is about relative errors only.
+template <bool F32>
+__device__ __forceinline__ void fast_codes_asym(const Chunk<F32>& ch, float z, float s, float inv, bool exact_only, float qmax,
+                                                uint32_t (&t)[8]) {
+    const float v_lo = fmaf(inv, -kBracket, inv), v_hi = fmaf(inv, kBracket, inv);
+    uint32_t differ = 0;
+    float d[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        d[i] = __fsub_rn(ch.get(i), z);
+        t[i] = __float_as_uint(fmaf(d[i], v_lo, kMagic));
+        differ |= t[i] ^ __float_as_uint(fmaf(d[i], v_hi, kMagic));
+    }
+    if (exact_only || differ != 0) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) t[i] = __float_as_uint(fminf(fmaxf(rintf(__fdiv_rn(d[i], s)), 0.f), qmax) + kMagic);
+    }
+}
+
 // Low bytes of four words -> one word.
 __device__ __forceinline__ uint32_t pack_low_bytes(uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
     return __byte_perm(__byte_perm(a, b, 0x0040), __byte_perm(c, d, 0x0040), 0x5410);
 }
 
-template <bool F32>
+// ASYM: asymmetric codes (unsigned), with the zero-points z8_out / z4_out; else symmetric ones.
+template <bool F32, bool ASYM>
 __global__ void __launch_bounds__(kThreads)
 split_quantize_fast_kernel(const void* __restrict__ in, size_t in_row_bytes, size_t rows, int K, int r,
                            int rows_per_cta, int nstages, int8_t* __restrict__ q8, uint8_t* __restrict__ q4,
-                           float* __restrict__ s8_out, float* __restrict__ s4_out, int8_t* __restrict__ q4e,
-                           int* __restrict__ status) {
+                           float* __restrict__ s8_out, float* __restrict__ s4_out, float* __restrict__ z8_out,
+                           float* __restrict__ z4_out, int8_t* __restrict__ q4e, int* __restrict__ status) {
     extern __shared__ __align__(128) uint8_t stage[];
     __shared__ uint64_t bar[2];
     __shared__ int abort_flag;
-    __shared__ float red[2][kThreads / 32];
-    // A kernel enqueued behind this one with programmatic stream serialization may start its own
-    // input-independent prologue now; it still waits for this grid to finish before reading the codes.
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    // Enqueued with programmatic stream serialization itself (behind the projection GEMM), this grid may have been
-    // scheduled before its input was complete: wait for the preceding grid (returns at once otherwise).
+    __shared__ float red[ASYM ? 4 : 2][kThreads / 32];
+    // Enqueued with programmatic stream serialization, this grid may have been scheduled before its input was complete:
+    // wait for the preceding grid.  Only then may the kernel enqueued behind this one start its own prologue, so that a
+    // dependent that is running finds everything enqueued before this grid complete (the product that follows in
+    // resq_linear streams its weights at once; it still waits for this grid before it reads the codes).
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const uint32_t row_bytes = static_cast<uint32_t>(K) * (F32 ? 4u : 2u);
     const size_t group_bytes = static_cast<size_t>(row_bytes) * rows_per_cta;
     const size_t groups = (rows + rows_per_cta - 1) / rows_per_cta;
@@ -296,62 +318,111 @@ split_quantize_fast_kernel(const void* __restrict__ in, size_t in_row_bytes, siz
         const bool live = grp < nrows;
         const uint8_t* srow = stage + buf * group_bytes + static_cast<size_t>(live ? grp : 0) * row_bytes;
 
-        float a8 = 0.f, a4 = 0.f;
-        if (live) {
-            if constexpr (F32) {
-                for (int c = j; c < rchunks; c += tpr) a8 = fmaxf(a8, chunk_absmax(lds_chunk<F32>(srow, c)));
-                float m0 = 0.f, m1 = 0.f;  // two chains: the INT4 segment is 7/8 of the row
-                int c = rchunks + j;
-                for (; c + tpr < nchunks; c += 2 * tpr) {
-                    m0 = fmaxf(m0, chunk_absmax(lds_chunk<F32>(srow, c)));
-                    m1 = fmaxf(m1, chunk_absmax(lds_chunk<F32>(srow, c + tpr)));
-                }
-                if (c < nchunks) m0 = fmaxf(m0, chunk_absmax(lds_chunk<F32>(srow, c)));
-                a4 = fmaxf(m0, m1);
-            } else {
-                // bf16 rows: sign bits cleared, maxima kept as packed pairs until the end (two operations per pair)
-                const uint4* v = reinterpret_cast<const uint4*>(srow);
-                uint32_t m8 = 0, m4a = 0, m4b = 0;
-                auto acc = [](uint32_t& m, const uint4 u) {
-                    const uint32_t w[4] = {u.x & 0x7FFF7FFFu, u.y & 0x7FFF7FFFu, u.z & 0x7FFF7FFFu, u.w & 0x7FFF7FFFu};
-                    __nv_bfloat162 mm = *reinterpret_cast<const __nv_bfloat162*>(&m);
+        // ---- pass 1: the largest magnitude of the two segments (a8, a4), or their ranges ([lo8, a8], [lo4, a4])
+        constexpr float kBig = 3.402823466e38f;
+        float a8 = ASYM ? -kBig : 0.f, a4 = a8, lo8 = kBig, lo4 = kBig;
+        if constexpr (ASYM) {
+            if (live) {
+                if constexpr (F32) {
+                    auto acc = [](const Chunk<F32>& ch, float& lo, float& hi) {
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) mm = __hmax2(mm, *reinterpret_cast<const __nv_bfloat162*>(&w[i]));
-                    m = *reinterpret_cast<const uint32_t*>(&mm);
-                };
-                for (int c = j; c < rchunks; c += tpr) acc(m8, v[c]);
-                int c = rchunks + j;
+                        for (int i = 0; i < 8; ++i) { lo = fminf(lo, ch.get(i)); hi = fmaxf(hi, ch.get(i)); }
+                    };
+                    for (int c = j; c < rchunks; c += tpr) acc(lds_chunk<F32>(srow, c), lo8, a8);
+                    for (int c = rchunks + j; c < nchunks; c += tpr) acc(lds_chunk<F32>(srow, c), lo4, a4);
+                } else {
+                    // bf16 rows: extrema kept as packed pairs until the end (two operations per pair)
+                    const uint4* v = reinterpret_cast<const uint4*>(srow);
+                    auto acc = [](const uint4 u, __nv_bfloat162& lo, __nv_bfloat162& hi) {
+                        const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            const __nv_bfloat162 x = *reinterpret_cast<const __nv_bfloat162*>(&w[i]);
+                            lo = __hmin2(lo, x);
+                            hi = __hmax2(hi, x);
+                        }
+                    };
+                    const uint32_t big = 0x7F7F7F7Fu, small = 0xFF7FFF7Fu;  // the largest finite bf16, and its negative
+                    __nv_bfloat162 l8 = *reinterpret_cast<const __nv_bfloat162*>(&big), h8 = *reinterpret_cast<const __nv_bfloat162*>(&small);
+                    __nv_bfloat162 l4 = l8, h4 = h8;
+                    for (int c = j; c < rchunks; c += tpr) acc(v[c], l8, h8);
 #pragma unroll 2
-                for (; c + tpr < nchunks; c += 2 * tpr) {
-                    acc(m4a, v[c]);
-                    acc(m4b, v[c + tpr]);
+                    for (int c = rchunks + j; c < nchunks; c += tpr) acc(v[c], l4, h4);
+                    lo8 = fminf(__low2float(l8), __high2float(l8)); a8 = fmaxf(__low2float(h8), __high2float(h8));
+                    lo4 = fminf(__low2float(l4), __high2float(l4)); a4 = fmaxf(__low2float(h4), __high2float(h4));
                 }
-                if (c < nchunks) acc(m4a, v[c]);
-                auto unpack = [](uint32_t m) { return fmaxf(__uint_as_float(m << 16), __uint_as_float(m & 0xFFFF0000u)); };
-                a8 = unpack(m8);
-                a4 = fmaxf(unpack(m4a), unpack(m4b));
+            }
+        } else {
+            if (live) {
+                if constexpr (F32) {
+                    for (int c = j; c < rchunks; c += tpr) a8 = fmaxf(a8, chunk_absmax(lds_chunk<F32>(srow, c)));
+                    float m0 = 0.f, m1 = 0.f;  // two chains: the INT4 segment is 7/8 of the row
+                    int c = rchunks + j;
+                    for (; c + tpr < nchunks; c += 2 * tpr) {
+                        m0 = fmaxf(m0, chunk_absmax(lds_chunk<F32>(srow, c)));
+                        m1 = fmaxf(m1, chunk_absmax(lds_chunk<F32>(srow, c + tpr)));
+                    }
+                    if (c < nchunks) m0 = fmaxf(m0, chunk_absmax(lds_chunk<F32>(srow, c)));
+                    a4 = fmaxf(m0, m1);
+                } else {
+                    // bf16 rows: sign bits cleared, maxima kept as packed pairs until the end (two operations per pair)
+                    const uint4* v = reinterpret_cast<const uint4*>(srow);
+                    uint32_t m8 = 0, m4a = 0, m4b = 0;
+                    auto acc = [](uint32_t& m, const uint4 u) {
+                        const uint32_t w[4] = {u.x & 0x7FFF7FFFu, u.y & 0x7FFF7FFFu, u.z & 0x7FFF7FFFu, u.w & 0x7FFF7FFFu};
+                        __nv_bfloat162 mm = *reinterpret_cast<const __nv_bfloat162*>(&m);
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) mm = __hmax2(mm, *reinterpret_cast<const __nv_bfloat162*>(&w[i]));
+                        m = *reinterpret_cast<const uint32_t*>(&mm);
+                    };
+                    for (int c = j; c < rchunks; c += tpr) acc(m8, v[c]);
+                    int c = rchunks + j;
+#pragma unroll 2
+                    for (; c + tpr < nchunks; c += 2 * tpr) {
+                        acc(m4a, v[c]);
+                        acc(m4b, v[c + tpr]);
+                    }
+                    if (c < nchunks) acc(m4a, v[c]);
+                    auto unpack = [](uint32_t m) { return fmaxf(__uint_as_float(m << 16), __uint_as_float(m & 0xFFFF0000u)); };
+                    a8 = unpack(m8);
+                    a4 = fmaxf(unpack(m4a), unpack(m4b));
+                }
             }
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             a8 = fmaxf(a8, __shfl_xor_sync(0xffffffffu, a8, o));
             a4 = fmaxf(a4, __shfl_xor_sync(0xffffffffu, a4, o));
+            if constexpr (ASYM) {
+                lo8 = fminf(lo8, __shfl_xor_sync(0xffffffffu, lo8, o));
+                lo4 = fminf(lo4, __shfl_xor_sync(0xffffffffu, lo4, o));
+            }
         }
         if (tpr > 32) {
             const int warp = threadIdx.x >> 5, wpr = tpr >> 5;
             if ((threadIdx.x & 31) == 0) {
                 red[0][warp] = a8;
                 red[1][warp] = a4;
+                if constexpr (ASYM) {
+                    red[2][warp] = lo8;
+                    red[3][warp] = lo4;
+                }
             }
             __syncthreads();
             for (int w = 0; w < wpr; ++w) {
                 a8 = fmaxf(a8, red[0][grp * wpr + w]);
                 a4 = fmaxf(a4, red[1][grp * wpr + w]);
+                if constexpr (ASYM) {
+                    lo8 = fminf(lo8, red[2][grp * wpr + w]);
+                    lo4 = fminf(lo4, red[3][grp * wpr + w]);
+                }
             }
         }
         if (live) {
             const size_t row = row0 + grp;
-            const float s8 = __fdiv_rn(a8, 127.f), s4 = __fdiv_rn(a4, 7.f);
+            if (ASYM && rchunks == 0) lo8 = a8 = 0.f;  // uniform 4-bit layer: the empty INT8 segment has s = 0, z = 0
+            const float s8 = ASYM ? __fdiv_rn(__fsub_rn(a8, lo8), 255.f) : __fdiv_rn(a8, 127.f);
+            const float s4 = ASYM ? __fdiv_rn(__fsub_rn(a4, lo4), 15.f) : __fdiv_rn(a4, 7.f);
             const float inv8 = s8 > 0.f ? __frcp_rn(s8) : 0.f, inv4 = s4 > 0.f ? __frcp_rn(s4) : 0.f;
             // The product form needs a finite, normal reciprocal; otherwise every chunk takes the division.
             const bool exact8 = s8 > 0.f && !(inv8 >= 1.1754944e-38f && inv8 <= 3.0e38f);
@@ -359,14 +430,22 @@ split_quantize_fast_kernel(const void* __restrict__ in, size_t in_row_bytes, siz
             if (j == 0) {
                 s8_out[row] = s8;
                 s4_out[row] = s4;
+                if constexpr (ASYM) {
+                    z8_out[row] = lo8;
+                    z4_out[row] = lo4;
+                }
             }
+            auto codes = [&](const Chunk<F32>& ch, float z, float s, float inv, bool exact, float qmax, uint32_t (&t)[8]) {
+                if constexpr (ASYM) fast_codes_asym(ch, z, s, inv, exact, qmax, t);
+                else fast_codes(ch, s, inv, exact, t);
+            };
             int8_t* q8row = q8 + row * static_cast<size_t>(r);
             uint8_t* q4row = q4 ? q4 + row * static_cast<size_t>(K4 >> 1) : nullptr;
             int8_t* q4e_row = q4e ? q4e + row * static_cast<size_t>(K4) : nullptr;
 
             for (int c = j; c < rchunks; c += tpr) {
                 uint32_t t[8];
-                if (s8 > 0.f) fast_codes(lds_chunk<F32>(srow, c), s8, inv8, exact8, t);
+                if (s8 > 0.f) codes(lds_chunk<F32>(srow, c), lo8, s8, inv8, exact8, 255.f, t);
                 else {
 #pragma unroll
                     for (int k = 0; k < 8; ++k) t[k] = 0;
@@ -377,7 +456,7 @@ split_quantize_fast_kernel(const void* __restrict__ in, size_t in_row_bytes, siz
 #pragma unroll 2
             for (int c = rchunks + j; c < nchunks; c += tpr) {
                 uint32_t t[8];
-                if (s4 > 0.f) fast_codes(lds_chunk<F32>(srow, c), s4, inv4, exact4, t);
+                if (s4 > 0.f) codes(lds_chunk<F32>(srow, c), lo4, s4, inv4, exact4, 15.f, t);
                 else {
 #pragma unroll
                     for (int k = 0; k < 8; ++k) t[k] = 0;
@@ -503,6 +582,8 @@ hadamard_quantize_kernel(const __nv_bfloat16* __restrict__ X, size_t rows, int K
     const int nchunks = K >> 3, rchunks = r >> 3;
     const int K4 = K - r;
     const uint8_t* srow = reinterpret_cast<const uint8_t*>(hrow);
+    asm volatile("griddepcontrol.wait;" ::: "memory");  // launched with programmatic stream serialization
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     for (size_t row = blockIdx.x; row < rows; row += gridDim.x) {
         // 1. widen the bf16 row (M = 1; otherwise the small factor below reads its groups straight from global memory)
         const uint4* xp = reinterpret_cast<const uint4*>(X + row * static_cast<size_t>(K));
@@ -654,57 +735,69 @@ hadamard_quantize_kernel(const __nv_bfloat16* __restrict__ X, size_t rows, int K
 
 }  // namespace
 
+namespace {
+
+// The fast kernel on `rows` rows that fit its staging (launch_split_quantize, launch_split_quantize_asym).
+template <bool F32, bool ASYM>
+cudaError_t launch_fast(const void* in, size_t rows, int K, int r, int8_t* q8, uint8_t* q4, float* s8, float* s4, float* z8,
+                        float* z4, int8_t* q4_i8, size_t in_row_stride_bytes, cudaStream_t st) {
+    const size_t row_bytes = static_cast<size_t>(K) * (F32 ? 4 : 2);
+    int rpc = 1;  // rows per CTA and step: 1, 2, 4 or 8, about half of kFastGroupBytes of staging
+    while (rpc < 8 && row_bytes * rpc * 2 <= static_cast<size_t>(kFastGroupBytes)) rpc *= 2;
+    while (rpc > 1 && rows / rpc < 148) rpc /= 2;  // few rows (a generation step): all threads of a CTA on one row
+    const size_t groups = (rows + rpc - 1) / rpc;
+    const size_t group_bytes = row_bytes * rpc;
+    auto kern = split_quantize_fast_kernel<F32, ASYM>;
+    static bool attr_set[64] = {};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev >= 64 || !attr_set[dev]) {
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kFastMaxRowBytes);
+        if (e != cudaSuccess) return e;
+        if (dev < 64) attr_set[dev] = true;
+    }
+    auto ctas_per_sm = [](size_t smem) {  // shared memory and the 2048-thread limit; registers allow 8 CTAs of 256
+        const size_t by_smem = (227u * 1024u) / (smem + 1024u);
+        return by_smem < 1 ? size_t(1) : (by_smem > 8 ? size_t(8) : by_smem);
+    };
+    // Two stages when they are cheap (several CTAs per SM still fit) and a CTA has more than one group to do.
+    int nstages = 1;
+    size_t grid = 148 * ctas_per_sm(group_bytes);
+    if (groups > grid && 2 * group_bytes <= 64u * 1024u) {
+        nstages = 2;
+        grid = 148 * ctas_per_sm(2 * group_bytes);
+    }
+    if (grid > groups) grid = groups;
+    // The kernel waits for the preceding grid itself (griddepcontrol.wait on entry), so it may always be scheduled
+    // while that grid drains; for the few rows of a generation step this hides most of its launch.
+    count_launch();
+    return launch_programmatic(kern, grid, kThreads, group_bytes * nstages, st, in, in_row_stride_bytes, rows, K, r, rpc, nstages, q8,
+                               q4, s8, s4, z8, z4, q4_i8, device_status_ptr());
+}
+
+}  // namespace
+
+cudaError_t launch_split_quantize_asym(const void* in, bool in_is_f32, size_t rows, int K, int r, uint8_t* u8,
+                                       uint8_t* u4, float* s8, float* s4, float* z8, float* z4, uint8_t* u4_u8,
+                                       size_t in_row_stride_bytes, cudaStream_t st) {
+    if (rows == 0) return cudaSuccess;
+    const size_t row_bytes = static_cast<size_t>(K) * (in_is_f32 ? 4 : 2);
+    if (row_bytes > static_cast<size_t>(kFastMaxRowBytes) || in_row_stride_bytes % 16 != 0) return cudaErrorNotSupported;
+    auto launch = in_is_f32 ? launch_fast<true, true> : launch_fast<false, true>;
+    return launch(in, rows, K, r, reinterpret_cast<int8_t*>(u8), u4, s8, s4, z8, z4, reinterpret_cast<int8_t*>(u4_u8),
+                  in_row_stride_bytes, st);
+}
+
 cudaError_t launch_split_quantize(const void* in, bool in_is_f32, size_t rows, int K, int r, int8_t* q8,
                                   uint8_t* q4, void* s8, void* s4, bool scale_fp16, int8_t* q4_i8,
-                                  size_t in_row_stride_bytes, cudaStream_t st, bool programmatic) {
+                                  size_t in_row_stride_bytes, cudaStream_t st) {
     if (rows == 0) return cudaSuccess;
     const size_t row_bytes = static_cast<size_t>(K) * (in_is_f32 ? 4 : 2);
     if (!scale_fp16 && row_bytes <= static_cast<size_t>(kFastMaxRowBytes) && in_row_stride_bytes % 16 == 0) {
-        int rpc = 1;  // rows per CTA and step: 1, 2, 4 or 8, about half of kFastGroupBytes of staging
-        while (rpc < 8 && row_bytes * rpc * 2 <= static_cast<size_t>(kFastGroupBytes)) rpc *= 2;
-        while (rpc > 1 && rows / rpc < 148) rpc /= 2;  // few rows (a generation step): all threads of a CTA on one row
-        const size_t groups = (rows + rpc - 1) / rpc;
-        const size_t group_bytes = row_bytes * rpc;
-        // Two stages when they are cheap (several CTAs per SM still fit) and a CTA has more than one group to do.
-        auto kern = in_is_f32 ? split_quantize_fast_kernel<true> : split_quantize_fast_kernel<false>;
-        static bool attr_set[2][64] = {};
-        int dev = 0;
-        cudaError_t e = cudaGetDevice(&dev);
-        if (e != cudaSuccess) return e;
-        if (dev < 64 && !attr_set[in_is_f32][dev]) {
-            e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kFastMaxRowBytes);
-            if (e != cudaSuccess) return e;
-            attr_set[in_is_f32][dev] = true;
-        }
-        auto ctas_per_sm = [](size_t smem) {  // shared memory and the 2048-thread limit; registers allow 8 CTAs of 256
-            const size_t by_smem = (227u * 1024u) / (smem + 1024u);
-            return by_smem < 1 ? size_t(1) : (by_smem > 8 ? size_t(8) : by_smem);
-        };
-        int nstages = 1;
-        size_t grid = 148 * ctas_per_sm(group_bytes);
-        if (groups > grid && 2 * group_bytes <= 64u * 1024u) {
-            nstages = 2;
-            grid = 148 * ctas_per_sm(2 * group_bytes);
-        }
-        if (grid > groups) grid = groups;
-        {
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3(static_cast<unsigned>(grid), 1, 1);
-            cfg.blockDim = dim3(kThreads, 1, 1);
-            cfg.dynamicSmemBytes = group_bytes * nstages;
-            cfg.stream = st;
-            cudaLaunchAttribute attr[1];
-            attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-            attr[0].val.programmaticStreamSerializationAllowed = 1;
-            cfg.attrs = attr;
-            // The kernel waits for the preceding grid itself (griddepcontrol.wait on entry), so it may always be
-            // scheduled while that grid drains; for the few rows of a generation step this hides most of its launch.
-            (void)programmatic;
-            cfg.numAttrs = 1;
-            count_launch();
-            return cudaLaunchKernelEx(&cfg, kern, in, in_row_stride_bytes, rows, K, r, rpc, nstages, q8, q4,
-                                      static_cast<float*>(s8), static_cast<float*>(s4), q4_i8, device_status_ptr());
-        }
+        auto launch = in_is_f32 ? launch_fast<true, false> : launch_fast<false, false>;
+        return launch(in, rows, K, r, q8, q4, static_cast<float*>(s8), static_cast<float*>(s4), nullptr, nullptr, q4_i8,
+                      in_row_stride_bytes, st);
     }
     const unsigned grid = static_cast<unsigned>(rows < 148u * 64u ? rows : 148u * 64u);
     count_launch();
@@ -770,17 +863,16 @@ cudaError_t launch_hadamard_quantize(const void* X, size_t rows, int K, int r, i
     const __nv_bfloat16* x = static_cast<const __nv_bfloat16*>(X);
     // 1024 threads per row only when rows do not outnumber the SMs: at 28672-wide rows (two 256-thread CTAs per SM)
     // the wide form measured slower for many rows (0.89 against 0.72 ms at 8192 rows).
+    const bool wide = rows <= kWideMaxRows;
+    auto kern = wide ? (m == 1    ? hadamard_quantize_kernel<1, kWideThreads>
+                        : m == 12 ? hadamard_quantize_kernel<12, kWideThreads>
+                                  : hadamard_quantize_kernel<28, kWideThreads>)
+                     : (m == 1    ? hadamard_quantize_kernel<1, kThreads>
+                        : m == 12 ? hadamard_quantize_kernel<12, kThreads>
+                                  : hadamard_quantize_kernel<28, kThreads>);
     count_launch();
-    if (rows <= kWideMaxRows) {
-        if (m == 1) hadamard_quantize_kernel<1, kWideThreads><<<grid, kWideThreads, smem, st>>>(x, rows, K, kbits, r, inv_sqrt_k, q8, q4, s8, s4, q4_i8);
-        else if (m == 12) hadamard_quantize_kernel<12, kWideThreads><<<grid, kWideThreads, smem, st>>>(x, rows, K, kbits, r, inv_sqrt_k, q8, q4, s8, s4, q4_i8);
-        else hadamard_quantize_kernel<28, kWideThreads><<<grid, kWideThreads, smem, st>>>(x, rows, K, kbits, r, inv_sqrt_k, q8, q4, s8, s4, q4_i8);
-        return cudaGetLastError();
-    }
-    if (m == 1) hadamard_quantize_kernel<1, kThreads><<<grid, kThreads, smem, st>>>(x, rows, K, kbits, r, inv_sqrt_k, q8, q4, s8, s4, q4_i8);
-    else if (m == 12) hadamard_quantize_kernel<12, kThreads><<<grid, kThreads, smem, st>>>(x, rows, K, kbits, r, inv_sqrt_k, q8, q4, s8, s4, q4_i8);
-    else hadamard_quantize_kernel<28, kThreads><<<grid, kThreads, smem, st>>>(x, rows, K, kbits, r, inv_sqrt_k, q8, q4, s8, s4, q4_i8);
-    return cudaGetLastError();
+    return launch_programmatic(kern, grid, wide ? kWideThreads : kThreads, smem, st, x, rows, K, kbits, r, inv_sqrt_k, q8, q4,
+                               s8, s4, q4_i8);
 }
 
 }  // namespace resq
