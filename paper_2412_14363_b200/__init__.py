@@ -100,9 +100,17 @@ def _ptr(t) -> Optional[int]:
     return None if t is None else t.data_ptr()
 
 
+def _nbytes(t) -> int:
+    return 0 if t is None else t.nbytes
+
+
 def _stream() -> int:
+    """The current stream's handle.  torch.cuda.current_stream() builds a Stream object through four layers of device
+    checks, 3.2 us of a call whose kernels take 6.6 (one token, 2048 x 3072); the raw getters take 0.2."""
     import torch
-    return torch.cuda.current_stream().cuda_stream
+    if not torch.cuda.is_initialized():
+        torch.cuda.init()
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _check(status: int, where: str):
@@ -245,13 +253,9 @@ def resq_mixed_gemm(W: Weights, x8, x4, s_x8, s_x4, Y, workspace, dbg_acc8=None,
 
 def resq_linear(W: Weights, X, P, Y, workspace):
     import torch
-    T = X.shape[0]
-    y_dtype = Y_BF16 if Y.dtype == torch.bfloat16 else Y_FP32
-    ws = W.struct()
-    _check(lib.resq_linear(ctypes.byref(W.desc), T, _ptr(X), _ptr(P), ctypes.byref(ws), _ptr(Y), y_dtype,
-                           _ptr(workspace),
-                           0 if workspace is None else workspace.numel() * workspace.element_size(), _stream()),
-           "resq_linear")
+    y_dtype = Y_BF16 if Y.dtype is torch.bfloat16 else Y_FP32
+    _check(lib.resq_linear(W.desc, X.shape[0], X.data_ptr(), _ptr(P), W.struct(), Y.data_ptr(), y_dtype,
+                           _ptr(workspace), _nbytes(workspace), _stream()), "resq_linear")
 
 
 def resq_unpack_int4(packed, out):
@@ -284,8 +288,6 @@ def alloc_workspace(desc: LayerDesc, T: int, has_P: bool, has_w4_i8: bool, devic
 
 
 # --------------------------------------------------------------------------- asymmetric activations
-def _nbytes(t) -> int:
-    return 0 if t is None else t.numel() * t.element_size()
 
 
 def resq_weight_row_sums(W: Weights):
