@@ -65,6 +65,13 @@ cudaError_t launch_mixed_gemm_tiles(int T, int N, int K, int r, const int8_t* x8
                                     int32_t* dbg8, int32_t* dbg4, cudaStream_t st, const float* z_x8 = nullptr,
                                     const float* z_x4 = nullptr, const int32_t* wsum8 = nullptr,
                                     const int32_t* wsum4 = nullptr);
+// The same for token counts where few tiles of that kernel exist (mixed_gemm_mid.cu); cudaErrorNotSupported, with nothing
+// launched, where its rule leaves the shape to the tile kernel.
+cudaError_t launch_mixed_gemm_mid(int T, int N, int K, int r, const int8_t* x8, const int8_t* x4e, const float* s_x8,
+                                  const float* s_x4, const int8_t* w8, const int8_t* w4e, const void* s_w8,
+                                  const void* s_w4, bool w_scale_fp16, void* Y, int y_dtype, int32_t* dbg8, int32_t* dbg4,
+                                  cudaStream_t st, const float* z_x8, const float* z_x4, const int32_t* wsum8,
+                                  const int32_t* wsum4);
 // z_x8 != NULL selects asymmetric activations: x8 / x4e then hold UNSIGNED codes (0..255, 0..15) and the
 // epilogue adds z_x8[t] * s_w8[n] * wsum8[n] + z_x4[t] * s_w4[n] * wsum4[n].
 

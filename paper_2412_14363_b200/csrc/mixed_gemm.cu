@@ -165,37 +165,40 @@ mixed_gemm_kernel(const __grid_constant__ CUtensorMap tmA8, const __grid_constan
             }
         }
     } else if (warp == 1) {
-        // ------------------------------------------------------------ MMA issuer (even CTA only)
-        if (lane == 0 && rank == 0) {
+        // ------------------------------------------------------------ MMA issuer (even CTA only): the whole warp, converged,
+        // one lane issues (descriptors stay in uniform registers; a thread alone in a branch needs about as long to issue
+        // a k-block's four products as the tensor core to run them)
+        if (rank == 0) {
+            const bool leader = elect_one();
             const uint32_t idesc = ASYM ? make_idesc_u8s8(2 * BM, p.bn) : make_idesc_i8(2 * BM, p.bn);
             int stage = 0;
             uint32_t phase = 0, acc_phase = 0;
+            auto wait = [&](uint64_t* bar, uint32_t parity) {
+                const bool ok = !__any_sync(0xffffffffu, !mbar_wait(bar, parity, abort_flag, p.status));
+                tc_fence_after();
+                return ok;
+            };
             bool ok = true;
             for (int tile = pair; tile < num_tiles && ok; tile += npairs) {
                 // INT4 columns are free once the previous tile's epilogue has copied them out.
-                if (!mbar_wait(&sh->acc4_empty, acc_phase ^ 1, abort_flag, p.status)) { ok = false; break; }
-                tc_fence_after();
+                if (!(ok = wait(&sh->acc4_empty, acc_phase ^ 1))) break;
                 for (int kb = 0; kb < kb_total; ++kb) {
                     const bool seg4 = kb < p.kb4;
-                    if (kb == p.kb4) {
-                        // ... the INT8 columns once it has finished with the tile.
-                        if (!mbar_wait(&sh->acc8_empty, acc_phase ^ 1, abort_flag, p.status)) { ok = false; break; }
-                        tc_fence_after();
-                    }
-                    if (!mbar_wait(&sh->full[stage], phase, abort_flag, p.status)) { ok = false; break; }
-                    tc_fence_after();
+                    // ... the INT8 columns once it has finished with the tile.
+                    if (kb == p.kb4 && !(ok = wait(&sh->acc8_empty, acc_phase ^ 1))) break;
+                    if (!(ok = wait(&sh->full[stage], phase))) break;
                     const uint64_t a_desc = make_smem_desc_k128(smem_u32(sA + stage * A_BYTES));
                     const uint64_t b_desc = make_smem_desc_k128(smem_u32(sB + stage * B_BYTES));
                     const uint32_t d = tmem_base + (seg4 ? static_cast<uint32_t>(BN) : 0u);
                     const bool first = kb == 0 || kb == p.kb4;
 #pragma unroll
                     for (int k = 0; k < BK / 32; ++k)
-                        mma_i8_ss_pair(d, a_desc + 2 * k, b_desc + 2 * k, idesc, (first && k == 0) ? 0u : 1u);
-                    tc_commit_pair(&sh->empty[stage], 3);  // frees the ring slot in both CTAs once these MMAs have read it
+                        mma_i8_ss_pair_if(leader, d, a_desc + 2 * k, b_desc + 2 * k, idesc, (first && k == 0) ? 0u : 1u);
+                    tc_commit_pair_if(leader, &sh->empty[stage], 3);  // frees the ring slot in both CTAs once these MMAs have read it
                     if (++stage == STAGES) { stage = 0; phase ^= 1; }
                 }
                 if (!ok) break;
-                tc_commit_pair(&sh->acc_full, 3);
+                tc_commit_pair_if(leader, &sh->acc_full, 3);
                 acc_phase ^= 1;
             }
         }
@@ -304,6 +307,7 @@ mixed_gemm_kernel(const __grid_constant__ CUtensorMap tmA8, const __grid_constan
     }
 
     // ---------------------------------------------------------------- teardown
+    __syncwarp();
     tc_fence_before();
     __syncthreads();
     cluster_sync_all();  // neither CTA leaves while the other may still read its shared memory or signal it
@@ -338,6 +342,10 @@ cudaError_t launch_mixed_gemm_tiles(int T, int N, int K, int r, const int8_t* x8
                                     const void* s_w8, const void* s_w4, bool w_scale_fp16, void* Y, int y_dtype,
                                     int32_t* dbg8, int32_t* dbg4, cudaStream_t st, const float* z_x8,
                                     const float* z_x4, const int32_t* wsum8, const int32_t* wsum4) {
+    if (const cudaError_t em = launch_mixed_gemm_mid(T, N, K, r, x8, x4e, s_x8, s_x4, w8, w4e, s_w8, s_w4, w_scale_fp16, Y, y_dtype,
+                                                     dbg8, dbg4, st, z_x8, z_x4, wsum8, wsum4);
+        em != cudaErrorNotSupported)
+        return em;
     const bool asym = z_x8 != nullptr;  // then x8 / x4e hold unsigned codes
     static bool attr_set[64] = {};
     int dev = 0;

@@ -1,0 +1,401 @@
+// Mixed-precision GEMM (Eq. 4 + dequantizing epilogue) for token counts between the weight-streaming kernel and the
+// large-tile kernel: ragged batches, chunked prefill beside generation, a few hundred tokens at most.
+//
+// The large-tile kernel (mixed_gemm.cu) gives a CTA pair 256 tokens x 256 channels.  With few tokens that leaves most SMs
+// idle (a 4096-channel layer is 16 tiles), computes rows of padding, and walks the whole reduction serially.  Here
+//   * the operands change places: 256 channels are the M rows of the pair's product (cta_group::2), the tokens are its N
+//     columns, N a multiple of 32 up to 256, so the padding is at most 31 tokens per tile;
+//   * the reduction is cut over the S = 1, 2 or 3 pairs of a cluster: each pair streams its share of the k-blocks (INT4
+//     blocks first, then INT8 ones) and accumulates exact int32 sums in its own TMEM; the pairs then exchange partial sums
+//     through distributed shared memory (over the drained ring), each finishing the 16-token groups g with g % S = its
+//     index.  Integer sums: the result does not depend on S, and no global scratch is needed.
+//   * a lane is a channel, so the stores of one token are contiguous across the warp.
+// Roles per CTA as in mixed_gemm.cu: TMA producer, MMA issuer (even CTA of a pair), 8 epilogue warps; one tile per cluster,
+// no persistence.  The rule that picks this kernel, N and S is mid_plan below.  All waits are bounded.
+//
+// What bounds it: the latency of the TMA ring up to N = 128 (0.21 us per k-block of 24 KB, 8 stages), operand delivery beyond,
+// and about 7 us of launch, first copies, epilogue and drain.  us, tile kernel -> this one: 4096 x 6144 at 17 / 128 / 300 /
+// 700 tokens 17.5 -> 8.7, 24 -> 12.3, 24.7 -> 14.3, 24.9 -> 19.6; 14336 x 4096 at 17 / 300 / 1537 tokens 41 -> 15.3, 47 -> 23,
+// 89 -> 68.5.  Products issued by a thread alone in a branch: 0.27 us per k-block whatever N.
+#include <cuda.h>
+#include <cuda_bf16.h>
+#include <cuda_fp16.h>
+
+#include "internal.h"
+#include "ptx.cuh"
+
+namespace resq {
+namespace {
+
+constexpr int BM = 128, BK = 128;  // channel rows per CTA; bytes (= codes) per k-block
+constexpr int kMaxStages = 10;
+constexpr int A_BYTES = BM * BK;
+constexpr int kRingBytes = 6 * (A_BYTES + 128 * BK);  // a stage holds 128 channel rows and ntok / 2 token rows (at most 128)
+constexpr int kThreads = 320;
+constexpr int kEpiThreads = 256;
+constexpr uint32_t kTmemCols = 512, kColAcc4 = 256;
+constexpr int kGroupBytes = 16 * BM * 4;  // partial sums of 16 tokens x 128 channels
+
+struct Params {
+    int T, N, kb4, kb8;
+    int ntok, tok_tiles, splits, stages;
+    const float* s_x8;
+    const float* s_x4;
+    const void* s_w8;
+    const void* s_w4;
+    int w_fp16;
+    const float* z_x8;  // asymmetric activations only
+    const float* z_x4;
+    const int32_t* wsum8;
+    const int32_t* wsum4;
+    void* Y;
+    int y_dtype;
+    int32_t* dbg8;
+    int32_t* dbg4;
+    int* status;
+};
+
+struct __align__(8) Shared {
+    uint64_t full[kMaxStages];
+    uint64_t empty[kMaxStages];
+    uint64_t acc_full;
+    uint32_t tmem_base;
+    int abort_flag;
+    float sx8[256], sx4[256], zx8[256], zx4[256];
+};
+
+constexpr size_t kSmemBytes = 1024 + kRingBytes + sizeof(Shared);
+
+__device__ __forceinline__ float load_scale(const void* p, int i, int fp16) {
+    return fp16 ? __half2float(reinterpret_cast<const __half*>(p)[i]) : reinterpret_cast<const float*>(p)[i];
+}
+
+// Slot of 16-token group g among the groups that pair `owner` of `splits` does not finish itself.
+__device__ __forceinline__ int slot_of(int g, int owner, int splits) { return g - (g + splits - 1 - owner) / splits; }
+
+template <bool ASYM>
+__global__ void __launch_bounds__(kThreads, 1)
+mixed_gemm_mid_kernel(const __grid_constant__ CUtensorMap tmW8, const __grid_constant__ CUtensorMap tmW4,
+                      const __grid_constant__ CUtensorMap tmX8, const __grid_constant__ CUtensorMap tmX4, const Params p) {
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    Shared* sh = reinterpret_cast<Shared*>(smem + kRingBytes);
+    const uint32_t stage_bytes = A_BYTES + static_cast<uint32_t>(p.ntok / 2) * BK;
+    volatile int* abort_flag = &sh->abort_flag;
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int rank = static_cast<int>(cluster_ctarank()), pair = rank >> 1, h = rank & 1;
+    const int tile = static_cast<int>(blockIdx.x) / (2 * p.splits);
+    const int t0 = (tile % p.tok_tiles) * p.ntok;                    // the tile's first token
+    const int n0 = (tile / p.tok_tiles) * (2 * BM) + h * BM;         // this CTA's first channel
+    const int kbt = p.kb4 + p.kb8;
+    const int kb0 = kbt * pair / p.splits, kb1 = kbt * (pair + 1) / p.splits;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < p.stages; ++s) {
+            mbar_init(&sh->full[s], 1);
+            mbar_init(&sh->empty[s], 1);
+        }
+        mbar_init(&sh->acc_full, 1);
+        sh->abort_flag = 0;
+        fence_mbar_init();
+        tma_prefetch_desc(&tmW8);
+        tma_prefetch_desc(&tmW4);
+        tma_prefetch_desc(&tmX8);
+        tma_prefetch_desc(&tmX4);
+    }
+    if (warp == 1) {
+        tmem_alloc_pair(&sh->tmem_base, kTmemCols);
+        tmem_relinquish_pair();
+    }
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync_all();  // the other CTAs' barriers exist before anything is signalled across
+    tc_fence_after();
+    const uint32_t tmem_base = sh->tmem_base;
+    asm volatile("griddepcontrol.wait;" ::: "memory");  // the set-up above ran under the tail of the preceding grid
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+
+    const int quad = warp & 3, part = (warp - 2) >> 2;  // epilogue warps: TMEM lane quadrant, which half of the groups
+    const int groups = p.ntok / 16;
+    const uint32_t lane_addr = tmem_base + (static_cast<uint32_t>(quad * 32) << 16);
+    const int row = quad * 32 + lane;
+    // Slice i of the reduction holds INT4 blocks / INT8 blocks.
+    auto has4 = [&](int i) { return kbt * i / p.splits < p.kb4; };
+    auto has8 = [&](int i) { return kbt * (i + 1) / p.splits > p.kb4; };
+    const uint32_t part8 = static_cast<uint32_t>(groups - groups / p.splits) * kGroupBytes;  // INT8 sums behind the INT4 ones
+    bool ok = true;
+
+    if (warp == 0) {
+        // ------------------------------------------------------------ TMA producer
+        if (lane == 0) {
+            int stage = 0;
+            uint32_t phase = 0;
+            for (int kb = kb0; kb < kb1; ++kb) {
+                if (!mbar_wait(&sh->empty[stage], phase ^ 1, abort_flag, p.status)) { ok = false; break; }
+                // The even CTA arms its barrier for the bytes of both CTAs; the odd one only sends its bytes there (if
+                // they land first, the pending arrival keeps the phase open).
+                const uint32_t full_addr = cluster_map(&sh->full[stage], rank & ~1);
+                if (h == 0) mbar_arrive_expect_tx(&sh->full[stage], 2 * stage_bytes);
+                const bool seg4 = kb < p.kb4;
+                const int x = (seg4 ? kb : kb - p.kb4) * BK;
+                tma_load_2d_pair(smem + stage * stage_bytes, seg4 ? &tmW4 : &tmW8, full_addr, x, n0);
+                tma_load_2d_pair(smem + stage * stage_bytes + A_BYTES, seg4 ? &tmX4 : &tmX8, full_addr, x, t0 + h * (p.ntok / 2));
+                if (++stage == p.stages) { stage = 0; phase ^= 1; }
+            }
+            if (!ok) {  // give the copies already in flight time to land before the CTA gives up its shared memory
+                const uint64_t since = global_timer_ns();
+                while (global_timer_ns() - since < 1000000ull) {}
+            }
+        }
+    } else if (warp == 1) {
+        // ------------------------------------------------------------ MMA issuer (even CTA of the pair): the whole warp,
+        // converged, one lane issues.  A thread alone in a branch takes about 100 cycles per instruction to move the
+        // descriptors, more than a product of 32 to 128 tokens lasts.
+        if (h == 0) {
+            const bool leader = elect_one();
+            // signed weights times signed or unsigned activations
+            const uint32_t idesc = (2u << 4) | (1u << 7) | (ASYM ? 0u : 1u << 10) | (static_cast<uint32_t>(p.ntok >> 3) << 17) |
+                                   (static_cast<uint32_t>(2 * BM >> 4) << 24);
+            const uint16_t both = static_cast<uint16_t>(3u << (rank & ~1));
+            int stage = 0;
+            uint32_t phase = 0;
+            for (int kb = kb0; kb < kb1; ++kb) {
+                ok = !__any_sync(0xffffffffu, !mbar_wait(&sh->full[stage], phase, abort_flag, p.status));
+                if (!ok) break;
+                tc_fence_after();
+                const uint32_t base = smem_u32(smem) + stage * stage_bytes;
+                const uint64_t a_desc = make_smem_desc_k128(base);
+                const uint64_t b_desc = make_smem_desc_k128(base + A_BYTES);
+                const uint32_t d = tmem_base + (kb < p.kb4 ? kColAcc4 : 0u);
+                const bool first = kb == kb0 || kb == p.kb4;
+#pragma unroll
+                for (int k = 0; k < BK / 32; ++k)
+                    mma_i8_ss_pair_if(leader, d, a_desc + 2 * k, b_desc + 2 * k, idesc, (first && k == 0) ? 0u : 1u);
+                tc_commit_pair_if(leader, &sh->empty[stage], both);
+                if (++stage == p.stages) { stage = 0; phase ^= 1; }
+            }
+            if (ok) tc_commit_pair_if(leader, &sh->acc_full, both);
+        }
+    } else {
+        // ------------------------------------------------------------ epilogue, first half: token scales, partial sums out
+        const int et = threadIdx.x - 64;
+        const int t = t0 + et;
+        const bool live = et < p.ntok && t < p.T;
+        sh->sx8[et] = live ? __ldg(p.s_x8 + t) : 0.f;
+        sh->sx4[et] = live ? __ldg(p.s_x4 + t) : 0.f;
+        if (ASYM) {
+            sh->zx8[et] = live ? __ldg(p.z_x8 + t) : 0.f;
+            sh->zx4[et] = live ? __ldg(p.z_x4 + t) : 0.f;
+        }
+        ok = mbar_wait(&sh->acc_full, 0, abort_flag, p.status);
+        ok = !__any_sync(0xffffffffu, !ok);
+        tc_fence_after();
+        if (p.splits > 1 && ok) {
+            const bool w4 = has4(pair), w8 = has8(pair);
+            for (int g = part; g < groups; g += 2) {
+                if (g % p.splits == pair) continue;
+                uint8_t* dst = smem + slot_of(g, pair, p.splits) * kGroupBytes + row * 16;
+                uint32_t a[16];
+                if (w4) {
+                    tmem_ld16(lane_addr + kColAcc4 + 16 * g, a);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        *reinterpret_cast<uint4*>(dst + q * (BM * 16)) = make_uint4(a[4 * q], a[4 * q + 1], a[4 * q + 2], a[4 * q + 3]);
+                }
+                if (w8) {
+                    tmem_ld16(lane_addr + 16 * g, a);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        *reinterpret_cast<uint4*>(dst + part8 + q * (BM * 16)) =
+                            make_uint4(a[4 * q], a[4 * q + 1], a[4 * q + 2], a[4 * q + 3]);
+                }
+            }
+        }
+    }
+    __syncwarp();
+    if (p.splits > 1) cluster_sync_all();
+    else __syncthreads();  // the token scales
+
+    if (warp >= 2) {
+        // ------------------------------------------------------------ epilogue, second half: sums, scales, stores
+        const int n = n0 + row;
+        const bool n_ok = n < p.N && ok;
+        const float sw8 = n_ok ? load_scale(p.s_w8, n, p.w_fp16) : 0.f;
+        const float sw4 = n_ok ? load_scale(p.s_w4, n, p.w_fp16) : 0.f;
+        const float zc8 = ASYM && n_ok ? static_cast<float>(p.wsum8[n]) * sw8 : 0.f;
+        const float zc4 = ASYM && n_ok ? static_cast<float>(p.wsum4[n]) * sw4 : 0.f;
+        const bool w4 = has4(pair), w8 = has8(pair);
+        for (int k = part; pair + k * p.splits < groups; k += 2) {
+            const int g = pair + k * p.splits;  // g % splits == pair
+            uint32_t a4[16], a8[16];
+            tmem_ld16(lane_addr + kColAcc4 + 16 * g, a4);
+            tmem_ld16(lane_addr + 16 * g, a8);
+            tmem_ld_wait();
+            if (!w4)
+#pragma unroll
+                for (int j = 0; j < 16; ++j) a4[j] = 0;
+            if (!w8)
+#pragma unroll
+                for (int j = 0; j < 16; ++j) a8[j] = 0;
+            for (int i = 0; i < p.splits; ++i) {
+                if (i == pair) continue;
+                const uint32_t src = cluster_map(smem + slot_of(g, i, p.splits) * kGroupBytes + row * 16, 2 * i + h);
+                const bool r4 = has4(i), r8 = has8(i);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    if (r4) {
+                        const uint4 v = ld_cluster_u4(src + q * (BM * 16));
+                        a4[4 * q] += v.x; a4[4 * q + 1] += v.y; a4[4 * q + 2] += v.z; a4[4 * q + 3] += v.w;
+                    }
+                    if (r8) {
+                        const uint4 v = ld_cluster_u4(src + part8 + q * (BM * 16));
+                        a8[4 * q] += v.x; a8[4 * q + 1] += v.y; a8[4 * q + 2] += v.z; a8[4 * q + 3] += v.w;
+                    }
+                }
+            }
+            if (!n_ok) continue;
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+                const int tt = 16 * g + j, t = t0 + tt;
+                if (t >= p.T) break;
+                const size_t off = static_cast<size_t>(t) * p.N + n;
+                const float t8 = static_cast<float>(static_cast<int>(a8[j])) * (sh->sx8[tt] * sw8);
+                const float t4 = static_cast<float>(static_cast<int>(a4[j])) * (sh->sx4[tt] * sw4);
+                float y = t8 + t4;
+                if (ASYM) y += sh->zx8[tt] * zc8 + sh->zx4[tt] * zc4;
+                if (p.y_dtype == RESQ_Y_BF16) reinterpret_cast<__nv_bfloat16*>(p.Y)[off] = __float2bfloat16_rn(y);
+                else reinterpret_cast<float*>(p.Y)[off] = y;
+                if (p.dbg8) {
+                    p.dbg8[off] = static_cast<int>(a8[j]);
+                    p.dbg4[off] = static_cast<int>(a4[j]);
+                }
+            }
+        }
+    }
+
+    // ---------------------------------------------------------------- teardown
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync_all();  // no CTA leaves while another may still read its shared memory or signal it
+    if (threadIdx.x == 0 && sh->abort_flag) atomicOr(p.status, kStatusBitTimeout);
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_dealloc_pair(tmem_base, kTmemCols);
+    }
+}
+
+typedef CUresult (*EncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
+                             const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
+                             CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+
+// [rows][kbytes] uint8 matrix, box = 128 bytes x box_rows, 128-byte swizzle, zero fill out of range.
+bool make_map_u8(CUtensorMap* m, const void* base, uint64_t rows, uint64_t kbytes, uint32_t box_rows) {
+    EncodeFn enc = reinterpret_cast<EncodeFn>(tensor_map_encode_fn());
+    if (!enc) return false;
+    cuuint64_t dims[2] = {kbytes, rows};
+    cuuint64_t strides[1] = {kbytes};
+    cuuint32_t box[2] = {128, box_rows};
+    cuuint32_t estr[2] = {1, 1};
+    return enc(m, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<void*>(base), dims, strides, box, estr,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+struct Plan {
+    int ntok, tok_tiles, splits;
+    bool use;
+};
+
+// Which (token tile, split) and whether at all.  Modelled times in ns, fitted to measurements over six layer shapes
+// (2048 x 3072 to 14336 x 4096 and 4096 x 28672) and 17 to 2048 tokens, weights in L2:
+//   this kernel  waves * (k-blocks per pair * c(N) + 3200 + 27 N - 1500) + 1500, c = 214 up to N = 128, 297 at 256 (fewer
+//                stages fit), plus the exchange: 1200 + 5 N (S = 2), 2200 + 6 N (S = 3); one wave is 74 pairs; clusters of
+//                four fit one wave up to 128 CTAs, clusters of six up to 96 (144 took two), eight never paid;
+//   tile kernel  rounds * (k-blocks * 294 + 5000) + 10600, a round being 74 tiles of 256 x 256.
+// Layers wider than L2 holds (64 MB of codes) pay a DRAM latency per wave here, which the persistent kernel hides.
+Plan mid_plan(int T, int N, int kbt) {
+    const long ch = (N + 2 * BM - 1) / (2 * BM);
+    const long tile_rounds = (ch * ((T + 255) / 256) + 73) / 74;
+    long best = tile_rounds * (kbt * 294L + 5000) + 10600;
+    const long wave_extra = static_cast<long>(N) * kbt * BK > (64L << 20) ? 4000 : 0;
+    Plan pl = {0, 0, 0, false};
+    for (int ntok = 256; ntok >= 32; ntok -= 32) {
+        const int nt = (T + ntok - 1) / ntok;
+        if (ntok > 32 && (T + ntok - 33) / (ntok - 32) == nt) continue;  // a narrower tile covers T with as many
+        const long c = ntok <= 128 ? 214 : ntok == 160 ? 222 : ntok == 192 ? 231 : ntok == 224 ? 250 : 297;
+        for (int s = 1; s <= 3; ++s) {
+            const long ctas = ch * nt * 2 * s;
+            if (s > 1 && (ctas > (s == 2 ? 128 : 96) || kbt < 4 * s)) break;
+            const long waves = s > 1 ? 1 : (ch * nt + 73) / 74;
+            const long one = (kbt + s - 1) / s * c + 3200 + 27L * ntok + (s == 2 ? 1200 + 5L * ntok : s == 3 ? 2200 + 6L * ntok : 0);
+            long t = waves * (one - 1500 + wave_extra) + 1500;
+            if (waves > 1) t += t / 20;  // a tie goes to the persistent kernel
+            if (t < best) {
+                best = t;
+                pl = {ntok, nt, s, true};
+            }
+        }
+    }
+    return pl;
+}
+
+}  // namespace
+
+cudaError_t launch_mixed_gemm_mid(int T, int N, int K, int r, const int8_t* x8, const int8_t* x4e, const float* s_x8,
+                                  const float* s_x4, const int8_t* w8, const int8_t* w4e, const void* s_w8,
+                                  const void* s_w4, bool w_scale_fp16, void* Y, int y_dtype, int32_t* dbg8, int32_t* dbg4,
+                                  cudaStream_t st, const float* z_x8, const float* z_x4, const int32_t* wsum8,
+                                  const int32_t* wsum4) {
+    const int K4 = K - r, kb8 = (r + BK - 1) / BK, kb4 = (K4 + BK - 1) / BK;
+    const Plan pl = mid_plan(T, N, kb4 + kb8);
+    if (!pl.use) return cudaErrorNotSupported;
+    const bool asym = z_x8 != nullptr;  // then x8 / x4e hold unsigned codes
+    static bool attr_set[64] = {};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev >= 64 || !attr_set[dev]) {
+        for (auto k : {mixed_gemm_mid_kernel<false>, mixed_gemm_mid_kernel<true>})
+            if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSmemBytes))) != cudaSuccess)
+                return e;
+        if (dev < 64) attr_set[dev] = true;
+    }
+    CUtensorMap tW8, tW4, tX8, tX4;
+    if (!make_map_u8(&tW4, w4e, N, K4, BM) || !make_map_u8(&tX4, x4e, T, K4, pl.ntok / 2)) return cudaErrorInvalidValue;
+    if (r > 0) {
+        if (!make_map_u8(&tW8, w8, N, r, BM) || !make_map_u8(&tX8, x8, T, r, pl.ntok / 2)) return cudaErrorInvalidValue;
+    } else {  // uniform INT4: no INT8 blocks, these maps are never used
+        tW8 = tW4;
+        tX8 = tX4;
+    }
+    Params p;
+    p.T = T; p.N = N; p.kb4 = kb4; p.kb8 = kb8;
+    p.ntok = pl.ntok; p.tok_tiles = pl.tok_tiles; p.splits = pl.splits;
+    p.stages = kRingBytes / (A_BYTES + pl.ntok / 2 * BK);
+    if (p.stages > kMaxStages) p.stages = kMaxStages;
+    p.s_x8 = s_x8; p.s_x4 = s_x4; p.s_w8 = s_w8; p.s_w4 = s_w4;
+    p.w_fp16 = w_scale_fp16 ? 1 : 0;
+    p.z_x8 = z_x8; p.z_x4 = z_x4; p.wsum8 = wsum8; p.wsum4 = wsum4;
+    p.Y = Y; p.y_dtype = y_dtype; p.dbg8 = dbg8; p.dbg4 = dbg8 ? dbg4 : nullptr;
+    p.status = device_status_ptr();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>((N + 2 * BM - 1) / (2 * BM) * pl.tok_tiles * 2 * pl.splits));
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = kSmemBytes;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = static_cast<unsigned>(2 * pl.splits);
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    count_launch();
+    return cudaLaunchKernelEx(&cfg, asym ? mixed_gemm_mid_kernel<true> : mixed_gemm_mid_kernel<false>, tW8, tW4, tX8, tX4, p);
+}
+
+}  // namespace resq

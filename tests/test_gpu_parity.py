@@ -209,6 +209,25 @@ def test_mixed_gemm_bit_exact(resq, T, K, N, r, fp16, w4i8):
     check_output(res, pw, y32, ybf)
 
 
+@pytest.mark.parametrize("T,K,N,r", [
+    (33, 6144, 264, 768),     # one token tile of 64, the reduction over three pairs, a channel tile of 8
+    (70, 5792, 1032, 736),    # partial k-blocks at the end of both segments, token groups of 16 unevenly over the pairs
+    (150, 2048, 4096, 0),     # no INT8 blocks
+    (224, 8192, 2056, 4096),  # INT4 and INT8 blocks in both halves of the reduction
+    (300, 1024, 6144, 128),   # no split: many narrow token tiles
+    (700, 544, 3080, 32),     # five k-blocks
+    (1100, 2080, 3072, 288),  # more tiles than fit the GPU at once
+])
+def test_mixed_gemm_token_counts_between(resq, T, K, N, r):
+    """Token counts between the weight-streaming and the large-tile kernel: accumulators bit for bit at the edges of the
+    token tiles, channel tiles, k-blocks and splits of the reduction."""
+    _, _, pw, res = oracle_case(T, K, N, r, seed_shift=T)
+    a8, a4, y32, ybf = run_mixed_gemm(resq, pw, res)
+    assert (a8 == res.acc8).all()
+    assert (a4 == res.acc4).all()
+    check_output(res, pw, y32, ybf)
+
+
 def test_mixed_gemm_extreme_codes(resq):
     """All codes at the clip limits (-128 / -8): the accumulators reach their largest magnitudes."""
     T, K, N, r = 130, 1024, 256, 128
