@@ -72,6 +72,12 @@ constexpr size_t kSmemBytes = 1024 + STAGES * (A_BYTES + B_BYTES) + sizeof(Share
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void griddep_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// A converged warp's wait before tensor-core instructions.
+__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag, const int* status) {
+    const bool ok = !__any_sync(0xffffffffu, !mbar_wait(bar, parity, abort_flag, status));
+    tc_fence_after();
+    return ok;
+}
 __device__ __forceinline__ void epi_barrier() { asm volatile("bar.sync 1, %0;" ::"n"(kEpiThreads) : "memory"); }
 
 // Tile order: row panels of `panel_tiles` pair tiles; inside a panel the m index runs fastest.
@@ -212,8 +218,10 @@ project_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_c
             }
         }
     } else if (warp == 1) {
-        // ------------------------------------------------------------ MMA issuer (even CTA only)
-        if (lane == 0 && rank == 0) {
+        // ------------------------------------------------------------ MMA issuer (even CTA only): the whole warp,
+        // converged, one lane issues (see mma_f16_ss_if)
+        if (rank == 0) {
+            const bool leader = elect_one();
             constexpr uint32_t idesc = make_idesc_bf16(2 * BM, BN) | (1u << 16);  // B is N-major
             int stage = 0;
             uint32_t phase = 0;
@@ -222,22 +230,20 @@ project_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_c
             bool ok = true;
             for (int item = pair; item < num_items && ok; item += npairs) {
                 const int nkb = item_info(p, item).nkb;
-                if (!mbar_wait(&sh->acc_empty[buf], acc_phase[buf] ^ 1, abort_flag, p.status)) { ok = false; break; }
-                tc_fence_after();
+                if (!(ok = warp_wait(&sh->acc_empty[buf], acc_phase[buf] ^ 1, abort_flag, p.status))) break;
                 const uint32_t d = tmem_base + static_cast<uint32_t>(buf * BN);
                 for (int kb = 0; kb < nkb; ++kb) {
-                    if (!mbar_wait(&sh->full[stage], phase, abort_flag, p.status)) { ok = false; break; }
-                    tc_fence_after();
+                    if (!(ok = warp_wait(&sh->full[stage], phase, abort_flag, p.status))) break;
                     const uint64_t a_desc = make_smem_desc_k128(smem_u32(sA + stage * A_BYTES));
                     const uint64_t b_desc = make_smem_desc_mn128(smem_u32(sB + stage * B_BYTES), B_BOX_BYTES);
 #pragma unroll
                     for (int k = 0; k < BK / 16; ++k)  // 16 k per instruction: 32 B of an A row, 2 KB of a B box
-                        mma_f16_ss_pair(d, a_desc + 2 * k, b_desc + (2048 >> 4) * k, idesc, (kb == 0 && k == 0) ? 0u : 1u);
-                    tc_commit_pair(&sh->empty[stage], 3);  // frees the stage in both CTAs
+                        mma_f16_ss_pair_if(leader, d, a_desc + 2 * k, b_desc + (2048 >> 4) * k, idesc, (kb == 0 && k == 0) ? 0u : 1u);
+                    tc_commit_pair_if(leader, &sh->empty[stage], 3);  // frees the stage in both CTAs
                     if (++stage == STAGES) { stage = 0; phase ^= 1; }
                 }
                 if (!ok) break;
-                tc_commit_pair(&sh->acc_full[buf], 3);
+                tc_commit_pair_if(leader, &sh->acc_full[buf], 3);
                 acc_phase[buf] ^= 1;
                 buf ^= 1;
             }
@@ -280,6 +286,7 @@ project_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_c
     }
 
     // ---------------------------------------------------------------- teardown
+    __syncwarp();
     tc_fence_before();
     __syncthreads();
     cluster_sync_all();  // neither CTA leaves while the other may still read its shared memory or signal it
@@ -384,8 +391,10 @@ project_gemm_few_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_co
             }
         }
     } else if (warp == 1) {
-        // ------------------------------------------------------------ MMA issuer (even CTA only)
-        if (lane == 0 && rank == 0) {
+        // ------------------------------------------------------------ MMA issuer (even CTA only): the whole warp,
+        // converged, one lane issues (see mma_f16_ss_if)
+        if (rank == 0) {
+            const bool leader = elect_one();
             const uint32_t idesc = make_idesc_bf16(2 * BM, ntok) | (1u << 15);  // A (the P tile) is M-major
             int stage = 0;
             uint32_t phase = 0;
@@ -394,22 +403,20 @@ project_gemm_few_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_co
             bool ok = true;
             for (int item = pair; item < num_items && ok; item += npairs) {
                 const int nkb = item_info(p, item).nkb;
-                if (!mbar_wait(&sh->acc_empty[buf], acc_phase[buf] ^ 1, abort_flag, p.status)) { ok = false; break; }
-                tc_fence_after();
+                if (!(ok = warp_wait(&sh->acc_empty[buf], acc_phase[buf] ^ 1, abort_flag, p.status))) break;
                 const uint32_t d = tmem_base + static_cast<uint32_t>(buf * kFewMaxT);
                 for (int kb = 0; kb < nkb; ++kb) {
-                    if (!mbar_wait(&sh->full[stage], phase, abort_flag, p.status)) { ok = false; break; }
-                    tc_fence_after();
+                    if (!(ok = warp_wait(&sh->full[stage], phase, abort_flag, p.status))) break;
                     const uint64_t a_desc = make_smem_desc_mn128(smem_u32(sP + stage * B_BYTES), B_BOX_BYTES);
                     const uint64_t b_desc = make_smem_desc_k128(smem_u32(sX + stage * FX_BYTES));
 #pragma unroll
                     for (int k = 0; k < BK / 16; ++k)  // 16 i per instruction: 2 KB of a P box, 32 B of a token row
-                        mma_f16_ss_pair(d, a_desc + (2048 >> 4) * k, b_desc + 2 * k, idesc, (kb == 0 && k == 0) ? 0u : 1u);
-                    tc_commit_pair(&sh->empty[stage], 3);
+                        mma_f16_ss_pair_if(leader, d, a_desc + (2048 >> 4) * k, b_desc + 2 * k, idesc, (kb == 0 && k == 0) ? 0u : 1u);
+                    tc_commit_pair_if(leader, &sh->empty[stage], 3);
                     if (++stage == FSTAGES) { stage = 0; phase ^= 1; }
                 }
                 if (!ok) break;
-                tc_commit_pair(&sh->acc_full[buf], 3);
+                tc_commit_pair_if(leader, &sh->acc_full[buf], 3);
                 acc_phase[buf] ^= 1;
                 buf ^= 1;
             }
@@ -450,6 +457,7 @@ project_gemm_few_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_co
     }
 
     // ---------------------------------------------------------------- teardown
+    __syncwarp();
     tc_fence_before();
     __syncthreads();
     cluster_sync_all();
@@ -496,8 +504,11 @@ cudaError_t launch_reduce(const Params& p, cudaStream_t st) {
 }
 
 // T <= kFewMaxT.  Chooses the K split: every tile becomes `s` slices; the cost of a choice is the number of k-blocks
-// the busiest pair streams, rounds x slice length.  A finer split is taken only when it is at least 2 % better, and
-// only while the partial tiles stay within the scratch and within 1/16 of the bytes of P.
+// the busiest pair streams, rounds x (slice length + 3): a work item costs about three k-blocks beside its stream (accumulator
+// hand-over, partial tile out and back in).  A finer split is taken only when it is at least 2 % better, and only while
+// the partial tiles stay within the scratch and within 1/16 of the bytes of P.  Measured at T = 3, K = 14336: 3 / 5 / 9 / 13 / 25
+// slices 74.3 / 67.7 / 69.6 / 70.3 / 79.4 us (25 is what the count without the 3 takes); K = 8192, T = 2: 2 / 9 / 16 slices
+// 25.9 / 28.2 / 30.8 us.
 cudaError_t launch_project_few(const void* X, const void* P, int T, int K, float* C, cudaStream_t st, void* scratch,
                                size_t scratch_bytes, int dev) {
     static bool attr_set[64] = {};
@@ -524,7 +535,8 @@ cudaError_t launch_project_few(const void* X, const void* P, int T, int K, float
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int tiles = p.n_tiles, all_pairs = sms / 2;
     int best_s = 1, best_slice = p.kb_total;
-    long best_cost = static_cast<long>((tiles + all_pairs - 1) / all_pairs) * p.kb_total;
+    constexpr long kItemBlocks = 3;
+    long best_cost = static_cast<long>((tiles + all_pairs - 1) / all_pairs) * (p.kb_total + kItemBlocks);
     if (scratch) {
         const size_t p_bytes = static_cast<size_t>(K) * K * 2;
         const size_t limit = scratch_bytes < p_bytes / 16 ? scratch_bytes : p_bytes / 16;
@@ -533,7 +545,7 @@ cudaError_t launch_project_few(const void* X, const void* P, int T, int K, float
             if ((p.kb_total + kb_slice - 1) / kb_slice != s) continue;  // same slices as a smaller s
             if (static_cast<size_t>(tiles) * s * T * BN * sizeof(float) > limit) break;
             const long rounds = (static_cast<long>(tiles) * s + all_pairs - 1) / all_pairs;
-            const long cost = rounds * kb_slice;
+            const long cost = rounds * (kb_slice + kItemBlocks);
             if (cost * 50 < best_cost * 49) { best_cost = cost; best_s = s; best_slice = kb_slice; }
         }
     }

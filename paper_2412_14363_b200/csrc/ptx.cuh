@@ -345,6 +345,16 @@ __device__ __forceinline__ void mma_i8_ss_pair_if(bool issue, uint32_t d_tmem, u
         ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(static_cast<uint32_t>(issue))
         : "memory");
 }
+__device__ __forceinline__ void mma_f16_ss_pair_if(bool issue, uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
+                                                   uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "setp.ne.b32 q, %5, 0;\n\t"
+        "@q tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(static_cast<uint32_t>(issue))
+        : "memory");
+}
 __device__ __forceinline__ void tc_commit_pair_if(bool issue, uint64_t* bar, uint16_t cta_mask) {
     asm volatile(
         "{\n\t.reg .pred q;\n\t"
