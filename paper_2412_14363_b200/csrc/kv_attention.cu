@@ -193,6 +193,7 @@ __global__ void __launch_bounds__(kWarps * 32, 1) attention_decode_kernel(const 
     }
     if (threadIdx.x == 0) abort_flag = 0;
     __syncthreads();
+    griddep_wait();               // launched with programmatic stream serialization itself
     griddep_launch_dependents();  // the merge kernel may be scheduled as SMs free up; it waits for this grid itself
 
     // ---- this warp's run of the global block list
@@ -475,7 +476,8 @@ __global__ void __launch_bounds__(kWarps * 32, 1) attention_decode_kernel(const 
 // t, the block agrees on the maximum), then group g adds the weighted records g, g + G, ... eight at a time, one
 // output coefficient per thread, and the G partial sums are added in group order.  G = 4 when few (sequence, head)
 // pairs share the grid's warps (long contexts: hundreds of records each), else 1.  Launched so that it may start
-// while the attention kernel drains: everything before griddepcontrol.wait reads only the sequence lengths.
+// while the attention kernel drains: everything before griddepcontrol.wait reads only the sequence lengths, which are
+// complete (the attention kernel lets its dependents start after its own wait).
 constexpr int kMaxGroups = 4;
 __global__ void __launch_bounds__(kD * kMaxGroups) attention_combine_kernel(const AttnParams p) {
     __shared__ long long red[2][kD * kMaxGroups / 32];
@@ -609,8 +611,7 @@ cudaError_t launch_attention_decode(const resq_kv_cache_t& cache, const void* q1
     p.group = n_q_heads / cache.n_kv_heads;
     p.capacity = cache.capacity;
     count_launch(2);
-    attention_decode_kernel<<<148, kWarps * 32, kSmem, st>>>(p);
-    if (cudaError_t e = cudaGetLastError(); e != cudaSuccess) return e;
+    if (cudaError_t e = launch_programmatic(attention_decode_kernel, 148, kWarps * 32, kSmem, st, p); e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(n_rows * n_q_heads, 1, 1);
     // few (sequence, head) pairs share the grid's warps: each has many records, so four groups of threads add them

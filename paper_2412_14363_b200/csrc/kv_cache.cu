@@ -212,6 +212,8 @@ __global__ void __launch_bounds__(kWarps * 32) kv_project_kernel(const ProjectPa
     __shared__ float su_s[D];
     __shared__ __align__(16) uint8_t rec_s[kWarps][16 * H::kRec];
     __shared__ long long slot_s[kWarps][16];
+    asm volatile("griddepcontrol.wait;" ::: "memory");  // launched with programmatic stream serialization
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     stage_uc<D>(p.wq, p.s_u, w_s, su_s);
     __syncthreads();
 
@@ -356,6 +358,8 @@ __global__ void __launch_bounds__(kWarps * 32) head_vector_kernel(const ProjectP
         kind = it < p.q_rows ? 0 : it < p.q_rows + p.kv_rows ? 1 : 2;  // query, key, value
         row = kind == 0 ? it : kind == 1 ? it - p.q_rows : it - p.q_rows - p.kv_rows;
     };
+    asm volatile("griddepcontrol.wait;" ::: "memory");  // launched with programmatic stream serialization
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     int kind = 0;
     long long row = 0;
     float x[N];
@@ -465,10 +469,8 @@ cudaError_t launch_project(const ProjectParams& p, cudaStream_t st) {
         return static_cast<unsigned>(ctas < 148 * 8 ? ctas : 148 * 8);
     };
     if (vectors <= kFewVectors)
-        head_vector_kernel<D><<<grid(vectors), kWarps * 32, 0, st>>>(p);
-    else
-        kv_project_kernel<D><<<grid((p.q_rows + 15) / 16 + 2 * ((p.kv_rows + 15) / 16)), kWarps * 32, 0, st>>>(p);
-    return cudaGetLastError();
+        return launch_programmatic(head_vector_kernel<D>, grid(vectors), kWarps * 32, 0, st, p);
+    return launch_programmatic(kv_project_kernel<D>, grid((p.q_rows + 15) / 16 + 2 * ((p.kv_rows + 15) / 16)), kWarps * 32, 0, st, p);
 }
 
 }  // namespace

@@ -138,6 +138,8 @@ __global__ void __launch_bounds__(A64<TEAM>::kNWarps * 32, TEAM == 1 ? 1 : 3) at
         else __syncthreads();
     };
 
+    asm volatile("griddepcontrol.wait;" ::: "memory");  // launched with programmatic stream serialization
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     // ---- rows of this lane, positions they see, the sequence
     int tok[RH], head[RH], pos_i[RH];
     int b, limit, pos_min;  // positions any row of the tile sees; the smallest of the rows' own positions
@@ -456,12 +458,15 @@ cudaError_t launch_attention64_form(const Attn64Params& p, unsigned tiles, cudaS
     cfg.blockDim = dim3(A64<TEAM>::kNWarps * 32);
     cfg.dynamicSmemBytes = A64<TEAM>::kSmem;
     cfg.stream = st;
-    cudaLaunchAttribute attr{};
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = static_cast<unsigned>(p.splits);
-    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
+    cudaLaunchAttribute attr[2] = {};
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = static_cast<unsigned>(p.splits);
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    // The causal form's CTAs (three per SM, long tiles first) would crowd the SMs that drain first: 58 -> 68 us.
+    cfg.numAttrs = TEAM == 1 ? 2 : 1;
     count_launch();
     return cudaLaunchKernelEx(&cfg, attention64_kernel<TEAM>, p);
 }

@@ -277,6 +277,8 @@ __global__ void __launch_bounds__(Geometry<NT>::kThreads, 1) attention_prefill_k
         tmem_relinquish();
     }
 
+    asm volatile("griddepcontrol.wait;" ::: "memory");  // the set-up above ran under the tail of the preceding grid
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     // ---- the largest value scale of the positions visited
     {
         float vmax = 0.f;
@@ -585,12 +587,15 @@ cudaError_t launch_prefill(const PrefillParams& p, long long tiles, cudaStream_t
     cfg.blockDim = dim3(Geometry<NT>::kThreads);
     cfg.dynamicSmemBytes = Geometry<NT>::kSmem;
     cfg.stream = st;
-    cudaLaunchAttribute attr{};
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = static_cast<unsigned>(p.splits);
-    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
+    cudaLaunchAttribute attr[2] = {};
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = static_cast<unsigned>(p.splits);
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    // More CTAs than SMs start in order of length only behind a drained grid.
+    cfg.numAttrs = tiles * p.Hkv * p.splits <= 148 ? 2 : 1;
     count_launch();
     return cudaLaunchKernelEx(&cfg, attention_prefill_kernel<NT>, p);
 }
