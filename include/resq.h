@@ -111,8 +111,8 @@ int resq_pack_weights(const resq_layer_desc_t* desc, const float* W_proj, int8_t
  * rows as given; columns are visited in order, column j is rounded to code_j = clamp(round-half-even(w_j / s)), and
  * (w_j - code_j s) / U_inv[j][j] times U_inv[j][j+1:] is subtracted from the columns not yet visited.  All of it in
  * fp64, one rounding per operation in this order, so the codes are reproducible bit for bit.  An offline step: the
- * sweep is a chain of K dependent steps per row.  K * 9 bytes (a row in shared memory) must not exceed 200 KB, else
- * RESQ_ERR_SHAPE.  Outputs as resq_pack_weights.
+ * sweep is a chain of K dependent steps per row.  K * 9 bytes must not exceed 200 KB (a row's state stays in shared
+ * memory), else RESQ_ERR_SHAPE.  Outputs as resq_pack_weights.
  */
 int resq_pack_weights_gptq(const resq_layer_desc_t* desc, const float* W_proj, const float* U_inv,
                            const uint8_t* dead_cols, int8_t* w8, uint8_t* w4, void* s_w8, void* s_w4, int8_t* w4_i8,
@@ -273,7 +273,8 @@ int resq_project_quantize_static(const void* X, const void* P, int T, int K, int
  *  RESQ_OPT_DECODE_EARLY_WEIGHTS (default 0): when 1, the few-token kernel (T <= 16) is launched so
  *    that it may begin while the preceding kernel of the stream is still running; it then streams its
  *    packed weights into shared memory at once and only waits for that kernel before it reads the
- *    activation codes and scales.  Generation is memory-bound (paper, Introduction), and this hides
+ *    activation codes and scales.  (Inside resq_linear / resq_linear_asym that kernel is the library's quantizer,
+ *    which starts its dependents only once everything before it is complete, so there it is always done.)  Generation is memory-bound (paper, Introduction), and this hides
  *    the ramp of each short kernel behind the tail of the previous one.  The caller promises that the
  *    packed weights and their scales were complete before the preceding kernel was enqueued (true
  *    for weights packed at load time; false if resq_pack_weights is the preceding kernel).
