@@ -154,12 +154,6 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {  
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-// Arrives once on `bar` when every tcgen05.mma issued so far by this thread has completed.
-__device__ __forceinline__ void tc_commit(uint64_t* bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-                 : "memory");
-}
-
 // Shared-memory matrix descriptor for a K-major operand tile whose rows are 128 bytes long and
 // stored with the 128-byte swizzle (the layout TMA writes with SWIZZLE_128B): 8-row groups are
 // 1024 bytes apart.  The tile base must be 1024-byte aligned; advancing along K inside the 128-byte
@@ -188,26 +182,6 @@ __host__ __device__ constexpr uint32_t make_idesc_bf16(int M, int N) {  // bf16 
            (static_cast<uint32_t>(M >> 4) << 24);
 }
 
-// D[tmem] (+)= A[smem] · B[smem]^T, one instruction (K = 32 bytes of each operand row).
-__device__ __forceinline__ void mma_i8_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                          uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-__device__ __forceinline__ void mma_f16_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                           uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-
 // Forms for a warp that walks its loop converged, with one lane's `issue` set: no branch around the instruction, so the
 // descriptors stay in uniform registers (a thread alone in a branch moves them there for every instruction).
 __device__ __forceinline__ void mma_f16_ss_if(bool issue, uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
@@ -231,6 +205,7 @@ __device__ __forceinline__ void mma_f16_ts_if(bool issue, uint32_t d_tmem, uint3
         ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(static_cast<uint32_t>(issue))
         : "memory");
 }
+// Arrives once on `bar` when every tcgen05.mma issued so far by the issuing lane has completed.
 __device__ __forceinline__ void tc_commit_if(bool issue, uint64_t* bar) {
     asm volatile(
         "{\n\t.reg .pred q;\n\t"
@@ -315,26 +290,9 @@ __device__ __forceinline__ void tmem_relinquish_pair() {
 __device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols) {
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
-// D (+)= A·B^T over the pair: 256 rows (128 from each CTA's shared memory), N columns (N/2 from each).
-__device__ __forceinline__ void mma_f16_ss_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                                uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-__device__ __forceinline__ void mma_i8_ss_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                               uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::2.kind::i8 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-// Converged-warp forms (see mma_f16_ss_if).
+// D (+)= A·B^T over the pair: 256 rows (128 from each CTA's shared memory), N columns (N/2 from each).  Converged-warp forms
+// (see mma_f16_ss_if).  The commit arrives once, on the mbarrier at this shared-memory offset in every CTA of `cta_mask`,
+// when all pair MMAs issued so far have completed.
 __device__ __forceinline__ void mma_i8_ss_pair_if(bool issue, uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
                                                   uint32_t accumulate) {
     asm volatile(
@@ -362,14 +320,6 @@ __device__ __forceinline__ void tc_commit_pair_if(bool issue, uint64_t* bar, uin
         "@q tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n\t}" ::"r"(
             smem_u32(bar)),
         "h"(cta_mask), "r"(static_cast<uint32_t>(issue))
-        : "memory");
-}
-// Arrives once, on the mbarrier at this shared-memory offset in every CTA of `cta_mask`, when all
-// pair MMAs issued so far by this thread have completed.
-__device__ __forceinline__ void tc_commit_pair(uint64_t* bar, uint16_t cta_mask) {
-    asm volatile(
-        "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
-        ::"r"(smem_u32(bar)), "h"(cta_mask)
         : "memory");
 }
 

@@ -96,3 +96,34 @@ def test_asymmetric_product_rounding_agrees_outside_guard_band():
                 else:
                     fallbacks += 1
     assert checked > 10000 and fallbacks > 500
+
+
+def test_asymmetric_bracketing_products_agree_only_on_the_defined_code():
+    """The row quantizer's form for asymmetric codes: d = fl(x - z) times the two factors that bracket 1 / s."""
+    rng = np.random.default_rng(5)
+    checked = fallbacks = 0
+    for bits, qmax in ((8, 255), (4, 15)):
+        for _ in range(40):
+            lo = np.float32(rng.uniform(-10, 10))
+            hi = np.float32(lo + np.float32(np.exp(rng.uniform(-12, 12))))
+            s = np.float32(np.float32(hi - lo) / np.float32(qmax))
+            inv = np.float32(np.float32(1.0) / s)
+            v_lo = _f32(Fraction(float(inv)) * (1 - Fraction(1, 2 ** 20)))
+            v_hi = _f32(Fraction(float(inv)) * (1 + Fraction(1, 2 ** 20)))
+            k = rng.integers(0, qmax, 200).astype(np.float32) + np.float32(0.5)
+            near = (np.float32(lo) + (k * s).astype(np.float32)).astype(np.float32)
+            near = (near.view(np.int32) + rng.integers(-4, 5, 200).astype(np.int32)).view(np.float32)
+            x = np.concatenate([near, rng.uniform(lo, hi, 200).astype(np.float32)])
+            x = x[(x >= lo) & (x <= hi)]
+            row = np.concatenate([[lo, hi], x]).astype(np.float32)
+            out = oracle.split_quantize_asym(np.tile(row, 2)[None, :], row.size)  # both segments hold the same data
+            codes = out[0 if bits == 8 else 1][0]
+            for xv, code in zip(row, codes):
+                d = Fraction(float(np.float32(xv - lo)))
+                n_lo = _rint_half_even(d * Fraction(float(v_lo)))
+                if n_lo == _rint_half_even(d * Fraction(float(v_hi))):
+                    assert n_lo == int(code), (float(xv), float(s), n_lo, int(code))
+                    checked += 1
+                else:
+                    fallbacks += 1
+    assert checked > 10000 and fallbacks > 500
