@@ -12,8 +12,8 @@
 //   softmax  4 warps per tile, one row per thread: score = s8 S8 + s4 S4 + (z8 + 128 s8) sum(q8) + (z4 + 8 s4) sum(q4) in
 //            fp32 minus the row's reference, p = 2^score, sums of p and of p (z + c0 s) in fp32, and the operands
 //            P8 = half(p s8_v 2^-E), P4 = half(p s4_v 2^-E) written over the S8 columns it has just read.
-// 2^E is the largest value scale of the positions the CTA visits (read ahead of the walk), so the products stay in half's
-// normal range.  The reference of a row is the maximum of its first step and is raised only when a score exceeds
+// 2^E is the largest finite value scale of the positions the CTA visits (read ahead of the walk), so the products stay in
+// half's normal range.  The reference of a row is the maximum of its first step and is raised only when a score exceeds
 // it by 2^8; that rare step rescales the row's output accumulator in TMEM.  So there is one pass over the cache, weights
 // are at most 2^8 (half holds 2^16) and no smaller against the row's maximum than with an exact one.
 // While one tile's softmax runs, the other tile's products do; the stages let the expansion run a step ahead.  With few
@@ -21,9 +21,10 @@
 //
 // The coefficients of a 32-bit word of nibbles are kept in the order 0 4 1 5 2 6 3 7 (one shift and mask per pair of
 // tile elements); the query tile is written in the same order and the output un-permuted on the way out.
-// Positions beyond a row's own are masked by selection and the constants of positions past the tile's last are zeroed
-// by selection, so unwritten cache positions of a loaded block may hold anything.  All waits are bounded; after a
-// failed wait every role leaves its loop, copies and products in flight are waited for, and TMEM is freed.
+// Positions beyond a row's own are masked by selection, in the scores and in the constants of the weights, and the
+// constants of positions past the tile's last are zeroed by selection, so unwritten cache positions of a loaded block
+// may hold anything.  All waits are bounded; after a failed wait every role leaves its loop, copies and products in
+// flight are waited for, and TMEM is freed.
 //
 // What bounds it: shared-memory traffic (the softmax constants come as broadcasts, two wavefronts per 16 bytes, beside the
 // tensor core's reads of Q, K and V) and the latency of a row's chain S -> weights -> O -> next S, about 4300 cycles per
@@ -198,10 +199,16 @@ struct RowState {
     f2 l, z8, z4;  // sums of p and of p times the zero-points (with the centre)
 };
 
-// Scores of one step minus the row's reference, as 32 pairs; returns their maximum.
+// The pair with what is not seen replaced by 0.
+__device__ __forceinline__ f2 seen(f2 v, bool lo, bool hi) {
+    const float2 f = unpack2(v);
+    return pack2(lo ? f.x : 0.f, hi ? f.y : 0.f);
+}
+
+// Scores of one step minus the row's reference, as 32 pairs; returns their maximum.  Positions of the step beyond `last` are
+// hidden from the row.
 template <bool MASKED>
-__device__ __forceinline__ float step_scores(f2 (&sc)[32], uint32_t tmem_s, const float4* col_k, int j0, int pos_i, f2 q8, f2 q4,
-                                             float neg_m) {
+__device__ __forceinline__ float step_scores(f2 (&sc)[32], uint32_t tmem_s, const float4* col_k, int last, f2 q8, f2 q4, float neg_m) {
     const f2 nm = pack2(neg_m, neg_m);
     float mx = -INFINITY;
     uint32_t a8[2][8], a4[2][8];
@@ -226,14 +233,45 @@ __device__ __forceinline__ float step_scores(f2 (&sc)[32], uint32_t tmem_s, cons
             sc[pr] = fma2(s.x, v8, fma2(s.y, v4, fma2(z.x, q8, fma2(z.y, q4, nm))));
             float2 f = unpack2(sc[pr]);
             if (MASKED) {
-                if (j0 + 2 * pr > pos_i) f.x = -INFINITY;
-                if (j0 + 2 * pr + 1 > pos_i) f.y = -INFINITY;
+                if (2 * pr > last) f.x = -INFINITY;
+                if (2 * pr + 1 > last) f.y = -INFINITY;
                 sc[pr] = pack2(f.x, f.y);
             }
             mx = fmaxf(mx, fmaxf(f.x, f.y));
         }
     }
     return mx;
+}
+
+// Weights of one step: their sums into the row's state, the operands of the output product over the scores in TMEM.
+// A hidden position's weight is 0 already, but its scales and zero-points belong to a token the row must not see and may
+// be infinite or NaN: they are zeroed by selection too, so that the products are 0.
+template <bool MASKED>
+__device__ __forceinline__ void step_weights(RowState& st, const f2 (&sc)[32], uint32_t tmem_row, const float4* col_v, int last) {
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        uint32_t w8[8], w4[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int pr = 8 * c + i;
+            f2x2 s = lds_pairs(col_v + 2 * pr);
+            f2x2 z = lds_pairs(col_v + 2 * pr + 1);
+            if (MASKED) {
+                const bool lo = 2 * pr <= last, hi = 2 * pr + 1 <= last;
+                s = {seen(s.x, lo, hi), seen(s.y, lo, hi)};
+                z = {seen(z.x, lo, hi), seen(z.y, lo, hi)};
+            }
+            const float2 f = unpack2(sc[pr]);
+            const f2 e = pack2(ex2(f.x), ex2(f.y));
+            st.l = add2(st.l, e);
+            st.z8 = fma2(e, z.x, st.z8);
+            st.z4 = fma2(e, z.y, st.z4);
+            w8[i] = half_pair(mul2(e, s.x));
+            w4[i] = half_pair(mul2(e, s.y));
+        }
+        tmem_st8(tmem_row + kColP8 + 8 * c, w8);
+        tmem_st8(tmem_row + kColP4 + 8 * c, w4);
+    }
 }
 
 template <int NT>
@@ -285,7 +323,8 @@ __global__ void __launch_bounds__(Geometry<NT>::kThreads, 1) attention_prefill_k
         const int end = min(limit, (first + n_steps) * kStep);
         for (int j = first * kStep + tid; j < end; j += G::kThreads) {
             const float4 m = __ldg(reinterpret_cast<const float4*>(blocks + static_cast<size_t>(j >> 5) * kBlockBytes + kOffVm) + (j & 31));
-            vmax = fmaxf(vmax, fmaxf(m.x, m.z));
+            // a scale that is not finite makes the rows that see it infinite or NaN whatever E is
+            vmax = fmaxf(vmax, fmaxf(m.x <= 3.402823466e38f ? m.x : 0.f, m.z <= 3.402823466e38f ? m.z : 0.f));
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) vmax = fmaxf(vmax, __shfl_xor_sync(0xffffffffu, vmax, o));
@@ -354,8 +393,10 @@ __global__ void __launch_bounds__(Geometry<NT>::kThreads, 1) attention_prefill_k
             const float4 *col_k = sh->col_k[n & 1], *col_v = sh->col_v[n & 1];
             f2 sc[32];
             float m_use = st.m == -INFINITY ? 0.f : st.m, mx;
-            if (j0 + kStep - 1 > pos_first) mx = step_scores<true>(sc, tmem_row, col_k, j0, pos_i, q8, q4, -m_use);
-            else mx = step_scores<false>(sc, tmem_row, col_k, j0, pos_i, q8, q4, -m_use);
+            const bool masked = j0 + kStep - 1 > pos_first;
+            const int last = pos_i - j0;  // the step's last position that this row sees
+            if (masked) mx = step_scores<true>(sc, tmem_row, col_k, last, q8, q4, -m_use);
+            else mx = step_scores<false>(sc, tmem_row, col_k, last, q8, q4, -m_use);
             // ---- raise the reference where a score leaves it too far behind (and set it at the first position seen)
             const bool raise = mx > (st.m == -INFINITY ? -INFINITY : kSlack);
             if (__any_sync(0xffffffffu, raise)) {
@@ -381,25 +422,8 @@ __global__ void __launch_bounds__(Geometry<NT>::kThreads, 1) attention_prefill_k
                 }
             }
             // ---- weights, their sums, the operands of the output product
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                uint32_t w8[8], w4[8];
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const int pr = 8 * c + i;
-                    const f2x2 s = lds_pairs(col_v + 2 * pr);
-                    const f2x2 z = lds_pairs(col_v + 2 * pr + 1);
-                    const float2 f = unpack2(sc[pr]);
-                    const f2 e = pack2(ex2(f.x), ex2(f.y));
-                    st.l = add2(st.l, e);
-                    st.z8 = fma2(e, z.x, st.z8);
-                    st.z4 = fma2(e, z.y, st.z4);
-                    w8[i] = half_pair(mul2(e, s.x));
-                    w4[i] = half_pair(mul2(e, s.y));
-                }
-                tmem_st8(tmem_row + kColP8 + 8 * c, w8);
-                tmem_st8(tmem_row + kColP4 + 8 * c, w4);
-            }
+            if (masked) step_weights<true>(st, sc, tmem_row, col_v, last);
+            else step_weights<false>(st, sc, tmem_row, col_v, last);
             tmem_st_wait();
             tc_fence_before();
             mbar_arrive(&sh->p_full[tile]);
