@@ -4,6 +4,7 @@
 //
 // Block layout for d_head = 64 (the d = 128 layout with every code array halved): per half (key, then value)
 //   c8 [32][8] | c4 [32][28] | meta [32][4] fp32      = 256 + 896 + 512 = 1664 bytes, 3328 per block.
+#include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
 #include "internal.h"
@@ -25,20 +26,23 @@ constexpr int kC8 = 32 * R8, kC4 = 32 * (N4 / 2), kHalf = kC8 + kC4 + 512, kBloc
 // With few CTAs a cluster splits the steps further and rank 0 merges the sums through distributed shared memory, so
 // no global scratch is needed.
 //
-// A step: the raw blocks arrive by cp.async two steps ahead; the codes are expanded, centred (code - 128, code - 8), to
-// exact halves in two tiles [position][64 coefficients]; K fragments come from ldmatrix, V fragments from
-// ldmatrix.trans, P straight from the score accumulators.  Scales and zero-points act in fp32 on the accumulators:
+// A step: the raw blocks arrive by cp.async two steps ahead; the codes are expanded, centred (code - 128, code - 8), in two
+// tiles [position][64 coefficients], keys as exact halves, values as exact bf16; K fragments come from ldmatrix, V
+// fragments from ldmatrix.trans, P straight from the score accumulators.  Scales and zero-points act in fp32 on the
+// accumulators:
 //   score = s8 S8 + s4 S4 + (z8 + 128 s8) sum(q8) + (z4 + 8 s4) sum(q4)         (q half, codes exact: products exact)
 //   out   = sum_j p_j s_j (c_j - c0) + sum_j p_j (z_j + c0 s_j)
-// The weights p_j s_j keep fp32's precision as the second product's operand: scaled by 2^(12 - E), E the exponent of the
-// largest value scale so far, they are split into two halves hi + lo (22 bits), two products per fragment.
+// The weights p_j s_j enter the second product as they are in fp32: as three bf16 values of 8 bits each, which add up to
+// all 24, three products per fragment.  (Two halves under a common power of two hold 22 bits of the largest weight only:
+// a value scale 2^20 above the others, on a position with next to no weight, left 2e-5 of the rest.)
 // The eight coefficients of a 32-bit word of nibbles are stored in the order 0 4 1 5 2 6 3 7 (one shift and mask per
 // pair); the query fragments are gathered in that order and the outputs put back.
 //
 // What bounds it: the softmax arithmetic and the operand conversions on the CUDA cores (about 20 instructions per score
 // of which two thirds per pair) and, for few rows, the latency of a step; not HBM, not the tensor pipe (26 % busy).
-// 32 query / 8 KV heads, project-and-append included: 1000 new tokens 1355 -> 83 us, a step of 16 sequences of
-// 1024-2048 positions 507 -> 24.6 us, against one warp per (row, query head) that dequantized each position per head.
+// 32 query / 8 KV heads, project-and-append included: 1000 new tokens 1355 -> 72 us (two halves per weight: 68), a step of
+// 16 sequences of 1024-2048 positions 507 -> 22.9 us (20.6), against one warp per (row, query head) that dequantized each
+// position per head.
 struct Attn64Params {
     const uint8_t* cache;
     const __half* q;   // [rows][Hq][64]
@@ -69,6 +73,10 @@ __device__ __forceinline__ void mma16(float (&d)[4], uint32_t a0, uint32_t a1, u
     asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
                  : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
+__device__ __forceinline__ void mma16_bf16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
 __device__ __forceinline__ void mma8(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t b0) {
     asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%0,%1,%2,%3};"
                  : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a0), "r"(a1), "r"(b0));
@@ -87,12 +95,16 @@ __device__ __forceinline__ float exp2_approx(float x) {
     return y;
 }
 __device__ __forceinline__ uint32_t h2_bits(__half2 v) { return *reinterpret_cast<const uint32_t*>(&v); }
-// a, b as two pairs of halves, hi + lo.
-__device__ __forceinline__ void split_h2(float a, float b, uint32_t& hi, uint32_t& lo) {
-    const __half2 h = __floats2half2_rn(a, b);
-    const float2 f = __half22float2(h);
-    hi = h2_bits(h);
-    lo = h2_bits(__floats2half2_rn(a - f.x, b - f.y));
+// The bits of a float that bf16 keeps.
+__device__ __forceinline__ float bf16_part(float x) { return __uint_as_float(__float_as_uint(x) & 0xFFFF0000u); }
+// a, b as three pairs of bf16 that add up to them exactly: 8 bits each, cut off, of what the ones before leave.
+__device__ __forceinline__ void split_bf16(float a, float b, uint32_t (&part)[3]) {
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        part[i] = __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632);
+        a -= bf16_part(a);
+        b -= bf16_part(b);
+    }
 }
 // Eight codes as halves minus their centre: `word` of nibbles (order 0 4 1 5 2 6 3 7), or eight bytes.
 __device__ __forceinline__ uint4 nibbles_centred(uint32_t word) {
@@ -111,6 +123,24 @@ __device__ __forceinline__ uint4 bytes_centred(uint2 w) {
                      __byte_perm(w.y, 0x64646464u, 0x4140), __byte_perm(w.y, 0x64646464u, 0x4342)};
 #pragma unroll
     for (int m = 0; m < 4; ++m) v[m] = h2_bits(__hsub2(*reinterpret_cast<const __half2*>(&v[m]), bias));
+    return make_uint4(v[0], v[1], v[2], v[3]);
+}
+// The same as bf16, which holds 128 + (0..127) exactly: the bytes' upper bits move the centre.
+__device__ __forceinline__ uint32_t minus_bf16(uint32_t v, uint32_t centre) {
+    const __nv_bfloat162 d = __hsub2(*reinterpret_cast<const __nv_bfloat162*>(&v), *reinterpret_cast<const __nv_bfloat162*>(&centre));
+    return *reinterpret_cast<const uint32_t*>(&d);
+}
+__device__ __forceinline__ uint4 nibbles_centred_bf16(uint32_t word) {
+    uint32_t v[4];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) v[m] = minus_bf16(((word >> (4 * m)) & 0x000F000Fu) | 0x43004300u, 0x43084308u);  // 128 + 8
+    return make_uint4(v[0], v[1], v[2], v[3]);
+}
+__device__ __forceinline__ uint4 bytes_centred_bf16(uint2 w) {
+    uint32_t v[4] = {__byte_perm(w.x, 0u, 0x4140), __byte_perm(w.x, 0u, 0x4342), __byte_perm(w.y, 0u, 0x4140), __byte_perm(w.y, 0u, 0x4342)};
+#pragma unroll
+    for (int m = 0; m < 4; ++m)  // code < 128: (128 + code) - 256, else (128 + code - 128) - 128
+        v[m] = minus_bf16((v[m] & 0x007F007Fu) | 0x43004300u, (~v[m] & 0x00800080u) | 0x43004300u);
     return make_uint4(v[0], v[1], v[2], v[3]);
 }
 // Coefficient at element e (0..7) of chunk j (0: the 8-bit segment, 1..7: words of nibbles).
@@ -221,8 +251,6 @@ __global__ void __launch_bounds__(A64<TEAM>::kNWarps * 32, TEAM == 1 ? 1 : 3) at
     float O[8][4], m_run[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f}, zs8[2] = {0.f, 0.f}, zs4[2] = {0.f, 0.f};
 #pragma unroll
     for (int j = 0; j < 8; ++j) O[j][0] = O[j][1] = O[j][2] = O[j][3] = 0.f;
-    constexpr int kExpMin = -114;  // 2^(12 - E) stays a normal float for E in [-114, 127]
-    int E = kExpMin;
     const float kScore = 1.4426950408889634f * 0.125f;  // log2(e) / sqrt(64)
     const uint32_t k_addr = smem_u32(Kt) + (lane & 7) * kPitch + (lane >> 3) * 16;
     const uint32_t v_addr = smem_u32(Vt) + ((lane & 7) + ((lane >> 3) & 1) * 8) * kPitch + (lane >> 4) * 16;
@@ -240,23 +268,16 @@ __global__ void __launch_bounds__(A64<TEAM>::kNWarps * 32, TEAM == 1 ? 1 : 3) at
             const uint8_t* half_base = rb + (pos >> 5) * kBlock + (ch >= 8 ? kHalf : 0);
             const int j = ch & 7, pp = pos & 31;
             uint4 v;
-            if (j == 0) v = bytes_centred(*reinterpret_cast<const uint2*>(half_base + pp * R8));
-            else v = nibbles_centred(*reinterpret_cast<const uint32_t*>(half_base + kC8 + pp * (N4 / 2) + 4 * (j - 1)));
+            if (j == 0) {
+                const uint2 w = *reinterpret_cast<const uint2*>(half_base + pp * R8);
+                v = ch >= 8 ? bytes_centred_bf16(w) : bytes_centred(w);
+            } else {
+                const uint32_t w = *reinterpret_cast<const uint32_t*>(half_base + kC8 + pp * (N4 / 2) + 4 * (j - 1));
+                v = ch >= 8 ? nibbles_centred_bf16(w) : nibbles_centred(w);
+            }
             *reinterpret_cast<uint4*>((ch >= 8 ? Vt : Kt) + pos * kPitch + j * 16) = v;
         }
         // ---- per-position constants; positions past the tile's limit hold anything and are zeroed by selection
-        int e_new;
-        {
-            float vm = 0.f;
-#pragma unroll
-            for (int i = 0; i < STEP / 32; ++i) {
-                const float4 m = *reinterpret_cast<const float4*>(rb + i * kBlock + kHalf + kC8 + kC4 + lane * 16);
-                if (j0 + 32 * i + lane < limit) vm = fmaxf(vm, fmaxf(m.x, m.z));
-            }
-            const uint32_t eb = __reduce_max_sync(0xffffffffu, __float_as_uint(vm)) >> 23;
-            e_new = max(E, max(static_cast<int>(eb) - 127, kExpMin));
-        }
-        const float f = __uint_as_float(static_cast<uint32_t>(127 + 12 - e_new) << 23);
 #pragma unroll
         for (int i = 0; i < (2 * STEP) / (TEAM * 32); ++i) {
             const int item = i * TEAM * 32 + tt, pos = item % STEP;
@@ -265,7 +286,7 @@ __global__ void __launch_bounds__(A64<TEAM>::kNWarps * 32, TEAM == 1 ? 1 : 3) at
             if (j0 + pos >= limit) m = make_float4(0.f, 0.f, 0.f, 0.f);
             m.y = fmaf(128.f, m.x, m.y);
             m.w = fmaf(8.f, m.z, m.w);
-            if (is_v) colV[pos] = make_float4(m.x * f, m.y, m.z * f, m.w);
+            if (is_v) colV[pos] = m;
             else colK[pos] = make_float4(m.x * kScore, m.y * kScore, m.z * kScore, m.w * kScore);
         }
         team_sync();
@@ -299,9 +320,9 @@ __global__ void __launch_bounds__(A64<TEAM>::kNWarps * 32, TEAM == 1 ? 1 : 3) at
                 }
             }
         }
-        // ---- running maximum and the scale of the sums
+        // ---- running maximum
         float m_use[RH], corr[RH];
-        bool moved = e_new != E;
+        bool moved = false;
 #pragma unroll
         for (int h = 0; h < RH; ++h) {
             mx[h] = fmaxf(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], 1));
@@ -313,26 +334,23 @@ __global__ void __launch_bounds__(A64<TEAM>::kNWarps * 32, TEAM == 1 ? 1 : 3) at
             m_run[h] = m_new;
         }
         if (__any_sync(0xffffffffu, moved)) {
-            const float de = static_cast<float>(E - e_new);
 #pragma unroll
             for (int h = 0; h < RH; ++h) {
                 l[h] *= corr[h];
                 zs8[h] *= corr[h];
                 zs4[h] *= corr[h];
-                const float co = corr[h] * exp2_approx(de);
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
-                    O[j][2 * h] *= co;
-                    O[j][2 * h + 1] *= co;
+                    O[j][2 * h] *= corr[h];
+                    O[j][2 * h + 1] *= corr[h];
                 }
             }
-            E = e_new;
         }
         // ---- weights and the second product, 32 positions at a time: the tensor core's fp32 sums are truncated, so a
         // chain of products runs over 32 positions only and is then added to the running sums with rounding
 #pragma unroll
         for (int kp = 0; kp < STEP / 32; ++kp) {
-            uint32_t p8h[2][4], p8l[2][4], p4h[2][4], p4l[2][4];
+            uint32_t p8[2][3][4], p4[2][3][4];
 #pragma unroll
             for (int t = 0; t < 4; ++t) {
                 const int nt = 4 * kp + t, pos = 8 * nt + 2 * c;
@@ -340,36 +358,36 @@ __global__ void __launch_bounds__(A64<TEAM>::kNWarps * 32, TEAM == 1 ? 1 : 3) at
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     const int i = 2 * (t & 1) + h;
-                    if (h >= RH) {
-                        p8h[t >> 1][i] = p8l[t >> 1][i] = p4h[t >> 1][i] = p4l[t >> 1][i] = 0u;
-                        continue;
+                    uint32_t w8[3] = {0u, 0u, 0u}, w4[3] = {0u, 0u, 0u};
+                    if (h < RH) {
+                        const float pa = exp2_approx(sc[nt][2 * (h % RH)] - m_use[h % RH]);
+                        const float pb = exp2_approx(sc[nt][2 * (h % RH) + 1] - m_use[h % RH]);
+                        l[h] += pa + pb;
+                        zs8[h] = fmaf(pa, va.y, fmaf(pb, vb.y, zs8[h]));
+                        zs4[h] = fmaf(pa, va.w, fmaf(pb, vb.w, zs4[h]));
+                        split_bf16(pa * va.x, pb * vb.x, w8);
+                        split_bf16(pa * va.z, pb * vb.z, w4);
                     }
-                    const float pa = exp2_approx(sc[nt][2 * (h % RH)] - m_use[h % RH]);
-                    const float pb = exp2_approx(sc[nt][2 * (h % RH) + 1] - m_use[h % RH]);
-                    l[h] += pa + pb;
-                    zs8[h] = fmaf(pa, va.y, fmaf(pb, vb.y, zs8[h]));
-                    zs4[h] = fmaf(pa, va.w, fmaf(pb, vb.w, zs4[h]));
-                    split_h2(pa * va.x, pb * vb.x, p8h[t >> 1][i], p8l[t >> 1][i]);
-                    split_h2(pa * va.z, pb * vb.z, p4h[t >> 1][i], p4l[t >> 1][i]);
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) {
+                        p8[t >> 1][k][i] = w8[k];
+                        p4[t >> 1][k][i] = w4[k];
+                    }
                 }
             }
 #pragma unroll
             for (int j = 0; j < 8; j += 2) {
                 float d0[4] = {0.f, 0.f, 0.f, 0.f}, d1[4] = {0.f, 0.f, 0.f, 0.f};
+                uint32_t v[2][4];
+                ldsm4t(v[0], v_addr + 2 * kp * 16 * kPitch + j * 16);
+                ldsm4t(v[1], v_addr + (2 * kp + 1) * 16 * kPitch + j * 16);
 #pragma unroll
-                for (int ks = 0; ks < 2; ++ks) {
-                    uint32_t v[4];
-                    ldsm4t(v, v_addr + (2 * kp + ks) * 16 * kPitch + j * 16);
-                    if (j == 0) {
-                        mma16(d0, p8l[ks][0], p8l[ks][1], p8l[ks][2], p8l[ks][3], v[0], v[1]);
-                        mma16(d0, p8h[ks][0], p8h[ks][1], p8h[ks][2], p8h[ks][3], v[0], v[1]);
-                    } else {
-                        mma16(d0, p4l[ks][0], p4l[ks][1], p4l[ks][2], p4l[ks][3], v[0], v[1]);
-                        mma16(d0, p4h[ks][0], p4h[ks][1], p4h[ks][2], p4h[ks][3], v[0], v[1]);
+                for (int k = 2; k >= 0; --k)  // the small parts first
+#pragma unroll
+                    for (int ks = 0; ks < 2; ++ks) {
+                        mma16_bf16(d0, j == 0 ? p8[ks][k] : p4[ks][k], v[ks][0], v[ks][1]);
+                        mma16_bf16(d1, p4[ks][k], v[ks][2], v[ks][3]);
                     }
-                    mma16(d1, p4l[ks][0], p4l[ks][1], p4l[ks][2], p4l[ks][3], v[2], v[3]);
-                    mma16(d1, p4h[ks][0], p4h[ks][1], p4h[ks][2], p4h[ks][3], v[2], v[3]);
-                }
 #pragma unroll
                 for (int e = 0; e < 2 * RH; ++e) {
                     O[j][e] += d0[e];
@@ -383,7 +401,6 @@ __global__ void __launch_bounds__(A64<TEAM>::kNWarps * 32, TEAM == 1 ? 1 : 3) at
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();
     float* rec = reinterpret_cast<float*>(smem64);  // [warp][row][kRecPitch], over the tiles
-    const float unscale = __uint_as_float(static_cast<uint32_t>(127 - 12 + E) << 23);
 #pragma unroll
     for (int h = 0; h < RH; ++h) {
 #pragma unroll
@@ -396,8 +413,8 @@ __global__ void __launch_bounds__(A64<TEAM>::kNWarps * 32, TEAM == 1 ? 1 : 3) at
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
             const float z = j == 0 ? zs8[h] : zs4[h];
-            r[coef64(j, 2 * c)] = fmaf(O[j][2 * h], unscale, z);
-            r[coef64(j, 2 * c + 1)] = fmaf(O[j][2 * h + 1], unscale, z);
+            r[coef64(j, 2 * c)] = O[j][2 * h] + z;
+            r[coef64(j, 2 * c + 1)] = O[j][2 * h + 1] + z;
         }
         if (c == 0) {
             r[D] = m_run[h];

@@ -148,8 +148,7 @@ def test_attention_three_forms_against_the_oracle(resq, kv, uc):
 ])
 def test_attention_tile_edges(resq, kv, uc, Hq, Hkv, lens, T):
     """Single-query over all sequences, the causal run of the last T positions of the first, and the same rows as many
-    queries, on caches whose unwritten bytes are 0xFF.  |out - oracle| <= 2e-5 max|v|: everything is fp32 (a weight is two
-    halves, 2^-22), a score of at most 40 in log2 units carries 2^-22 of itself."""
+    queries, on caches whose unwritten bytes are 0xFF.  |out - oracle| <= 2e-5 max|v|: everything is fp32, a score of at most 40 in log2 units carries 2^-22 of itself."""
     W_C, wq, s_u = uc
     B, cap = len(lens), (max(lens) + 31) // 32 * 32 + 32
     cache = kv.KvCache(B, Hkv, cap, d_head=D)
@@ -184,4 +183,41 @@ def test_attention_tile_edges(resq, kv, uc, Hq, Hkv, lens, T):
     many = torch.full((T, Hq, D), float("nan"), dtype=torch.float32, device="cuda")
     kv.resq_attention_queries(cache, q, dev(np.zeros(T, np.int32)), dev(np.arange(pos0 + 1, pos0 + T + 1, dtype=np.int32)), many)
     assert np.abs(host(many) - ref).max() <= 2e-5 * vmax[0]
+    assert resq.resq_device_status() == resq.OK
+
+
+@pytest.mark.parametrize("outlier", [5, -1])
+@pytest.mark.parametrize("k", [20, 28])
+def test_attention_beside_a_far_larger_value_scale(resq, kv, uc, outlier, k):
+    """One position's values are 2^k times the others' and its key is so far from every query that its weight is below 2^-100
+    (outlier = 5), or it is the run's last token, which only the last row attends: the outputs keep the accuracy of a cache
+    without it, 2e-5 of the largest other value (the bound of test_attention_tile_edges)."""
+    W_C, wq, s_u = uc
+    Hq, Hkv, S, T = 8, 2, 140, 40
+    K = synth.head_vectors(S, Hkv, D, stream=1400, lead=1.0, scale=1.5)
+    v = synth.head_vectors(S, Hkv, D, stream=1401, lead=4.0, shift=0.3)
+    q = synth.head_vectors(T, Hq, D, stream=1402, lead=1.0, scale=0.5)
+    common = np.where(np.arange(D) % 2, 4.0, -4.0).astype(np.float32)
+    q = synth.to_bf16_values(q + common)
+    K[outlier] = synth.to_bf16_values(-2.0 * common)      # score about -2 * 16 * 64 / 8 = -256
+    v[outlier] = v[outlier] * np.float32(2.0 ** k)
+    cache = kv.KvCache(1, Hkv, 160, d_head=D)
+    cache.data.fill_(0xFF)
+    kv.resq_kv_append(cache, bf16_to_dev(synth.f32_to_bf16_bits(K)), bf16_to_dev(synth.f32_to_bf16_bits(v)),
+                      dev(np.zeros(S, np.int32)), dev(np.arange(S, dtype=np.int32)), wq, s_u)
+    hk, hv = _oracle_records(K, v, W_C)
+    dk, dv = okv.kv_dequantize(hk).reshape(S, Hkv, D), okv.kv_dequantize(hv).reshape(S, Hkv, D)
+    K_hat, V_hat = [dk[:, h] for h in range(Hkv)], [dv[:, h] for h in range(Hkv)]
+    others = np.arange(S) != outlier % S
+    vmax = max(np.abs(x[others]).max() for x in V_hat)
+    q16 = torch.empty((T, Hq, D), dtype=torch.float16, device="cuda")
+    kv.resq_query_project(bf16_to_dev(synth.f32_to_bf16_bits(q)), wq, s_u, q16)
+    lens = np.arange(S - T + 1, S + 1)
+    ref = okv.attention_queries(host(q16), [K_hat], [V_hat], np.zeros(T, np.int32), lens, Hq, Hkv)
+    run = torch.full((T, Hq, D), float("nan"), dtype=torch.float32, device="cuda")
+    kv.resq_attention_prefill(cache, q16, 0, S - T, run)
+    assert np.abs(host(run) - ref).max() <= 2e-5 * vmax
+    many = torch.full((T, Hq, D), float("nan"), dtype=torch.float32, device="cuda")
+    kv.resq_attention_queries(cache, q16, dev(np.zeros(T, np.int32)), dev(lens.astype(np.int32)), many)
+    assert np.abs(host(many) - ref).max() <= 2e-5 * vmax
     assert resq.resq_device_status() == resq.OK
