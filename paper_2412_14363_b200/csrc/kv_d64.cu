@@ -7,6 +7,8 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include <type_traits>
+
 #include "internal.h"
 #include "ptx.cuh"
 
@@ -347,54 +349,63 @@ __global__ void __launch_bounds__(A64<TEAM>::kNWarps * 32, TEAM == 1 ? 1 : 3) at
             }
         }
         // ---- weights and the second product, 32 positions at a time: the tensor core's fp32 sums are truncated, so a
-        // chain of products runs over 32 positions only and is then added to the running sums with rounding
+        // chain of products runs over 32 positions only and is then added to the running sums with rounding.  HIDE: some
+        // positions are hidden from some rows; their weights are 0 already, but their scales and zero-points belong to a
+        // later token and may be infinite or NaN, so those are zeroed by selection too.
+        auto second_product = [&](auto hide) {
+            constexpr bool HIDE = decltype(hide)::value;
 #pragma unroll
-        for (int kp = 0; kp < STEP / 32; ++kp) {
-            uint32_t p8[2][3][4], p4[2][3][4];
+            for (int kp = 0; kp < STEP / 32; ++kp) {
+                uint32_t p8[2][3][4], p4[2][3][4];
 #pragma unroll
-            for (int t = 0; t < 4; ++t) {
-                const int nt = 4 * kp + t, pos = 8 * nt + 2 * c;
-                const float4 va = colV[pos], vb = colV[pos + 1];
+                for (int t = 0; t < 4; ++t) {
+                    const int nt = 4 * kp + t, pos = 8 * nt + 2 * c;
+                    const float4 va = colV[pos], vb = colV[pos + 1];
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int i = 2 * (t & 1) + h;
-                    uint32_t w8[3] = {0u, 0u, 0u}, w4[3] = {0u, 0u, 0u};
-                    if (h < RH) {
-                        const float pa = exp2_approx(sc[nt][2 * (h % RH)] - m_use[h % RH]);
-                        const float pb = exp2_approx(sc[nt][2 * (h % RH) + 1] - m_use[h % RH]);
-                        l[h] += pa + pb;
-                        zs8[h] = fmaf(pa, va.y, fmaf(pb, vb.y, zs8[h]));
-                        zs4[h] = fmaf(pa, va.w, fmaf(pb, vb.w, zs4[h]));
-                        split_bf16(pa * va.x, pb * vb.x, w8);
-                        split_bf16(pa * va.z, pb * vb.z, w4);
+                    for (int h = 0; h < 2; ++h) {
+                        const int i = 2 * (t & 1) + h;
+                        uint32_t w8[3] = {0u, 0u, 0u}, w4[3] = {0u, 0u, 0u};
+                        if (h < RH) {
+                            const float pa = exp2_approx(sc[nt][2 * (h % RH)] - m_use[h % RH]);
+                            const float pb = exp2_approx(sc[nt][2 * (h % RH) + 1] - m_use[h % RH]);
+                            const float4 a = HIDE && j0 + pos > pos_i[h % RH] ? make_float4(0.f, 0.f, 0.f, 0.f) : va;
+                            const float4 b = HIDE && j0 + pos + 1 > pos_i[h % RH] ? make_float4(0.f, 0.f, 0.f, 0.f) : vb;
+                            l[h] += pa + pb;
+                            zs8[h] = fmaf(pa, a.y, fmaf(pb, b.y, zs8[h]));
+                            zs4[h] = fmaf(pa, a.w, fmaf(pb, b.w, zs4[h]));
+                            split_bf16(pa * a.x, pb * b.x, w8);
+                            split_bf16(pa * a.z, pb * b.z, w4);
+                        }
+#pragma unroll
+                        for (int k = 0; k < 3; ++k) {
+                            p8[t >> 1][k][i] = w8[k];
+                            p4[t >> 1][k][i] = w4[k];
+                        }
                     }
+                }
 #pragma unroll
-                    for (int k = 0; k < 3; ++k) {
-                        p8[t >> 1][k][i] = w8[k];
-                        p4[t >> 1][k][i] = w4[k];
+                for (int j = 0; j < 8; j += 2) {
+                    float d0[4] = {0.f, 0.f, 0.f, 0.f}, d1[4] = {0.f, 0.f, 0.f, 0.f};
+                    uint32_t v[2][4];
+                    ldsm4t(v[0], v_addr + 2 * kp * 16 * kPitch + j * 16);
+                    ldsm4t(v[1], v_addr + (2 * kp + 1) * 16 * kPitch + j * 16);
+#pragma unroll
+                    for (int k = 2; k >= 0; --k)  // the small parts first
+#pragma unroll
+                        for (int ks = 0; ks < 2; ++ks) {
+                            mma16_bf16(d0, j == 0 ? p8[ks][k] : p4[ks][k], v[ks][0], v[ks][1]);
+                            mma16_bf16(d1, p4[ks][k], v[ks][2], v[ks][3]);
+                        }
+#pragma unroll
+                    for (int e = 0; e < 2 * RH; ++e) {
+                        O[j][e] += d0[e];
+                        O[j + 1][e] += d1[e];
                     }
                 }
             }
-#pragma unroll
-            for (int j = 0; j < 8; j += 2) {
-                float d0[4] = {0.f, 0.f, 0.f, 0.f}, d1[4] = {0.f, 0.f, 0.f, 0.f};
-                uint32_t v[2][4];
-                ldsm4t(v[0], v_addr + 2 * kp * 16 * kPitch + j * 16);
-                ldsm4t(v[1], v_addr + (2 * kp + 1) * 16 * kPitch + j * 16);
-#pragma unroll
-                for (int k = 2; k >= 0; --k)  // the small parts first
-#pragma unroll
-                    for (int ks = 0; ks < 2; ++ks) {
-                        mma16_bf16(d0, j == 0 ? p8[ks][k] : p4[ks][k], v[ks][0], v[ks][1]);
-                        mma16_bf16(d1, p4[ks][k], v[ks][2], v[ks][3]);
-                    }
-#pragma unroll
-                for (int e = 0; e < 2 * RH; ++e) {
-                    O[j][e] += d0[e];
-                    O[j + 1][e] += d1[e];
-                }
-            }
-        }
+        };
+        if (TWO && masked) second_product(std::true_type{});
+        else second_product(std::false_type{});
     }
 
     // ---- records of the warps (unnormalised sums with the zero-points, maximum, sum of weights), then the merge

@@ -39,6 +39,9 @@ def _run(resq, kv, d, prefix, T, Hq, Hkv, last):
     (128, 0, 37, 8, 2),      # one tile of rows per CTA
     (128, 1, 600, 32, 8),    # two
     (128, 2000, 40, 8, 2),   # the steps split over a cluster
+    (64, 0, 37, 8, 2),
+    (64, 100, 300, 12, 2),   # rows of a token on both sides of a tile edge
+    (64, 2000, 40, 8, 2),    # the steps split over a cluster
 ])
 def test_rows_do_not_see_a_later_token(d, prefix, T, Hq, Hkv, last):
     import paper_2412_14363_b200 as resq
