@@ -276,8 +276,9 @@ int resq_project_quantize_static(const void* X, const void* P, int T, int K, int
  *    activation codes and scales.  (Inside resq_linear / resq_linear_asym that kernel is the library's quantizer,
  *    which starts its dependents only once everything before it is complete, so there it is always done.)  Generation is memory-bound (paper, Introduction), and this hides
  *    the ramp of each short kernel behind the tail of the previous one.  The caller promises that the
- *    packed weights and their scales were complete before the preceding kernel was enqueued (true
- *    for weights packed at load time; false if resq_pack_weights is the preceding kernel).
+ *    kernel enqueued just before writes none of the packed weights and scales (true for weights packed at load
+ *    time; false if resq_pack_weights is that kernel): what was enqueued before the call that enqueued that one is
+ *    complete when the few-token kernel starts.
  *  RESQ_OPT_WAIT_LIMIT_US (default 2 000 000): wall-clock limit, in microseconds, of a single wait inside a
  *    kernel (for a copy to land, for a pipeline stage to be released).  Stored on the CURRENT device with a
  *    blocking copy; kernels enqueued afterwards on that device use it.  value >= 1; the kernels look at the

@@ -116,8 +116,6 @@ __device__ __forceinline__ void mma_s8(int (&d)[4], uint32_t a0, uint32_t a1, ui
             : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-__device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void griddep_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // One per-channel scale: the raw bits now, the value when it is needed (an item's scales are requested when its
 // first chunk is, and used after its last: converting at once would make the warp wait for a DRAM round trip
@@ -205,7 +203,6 @@ mixed_gemm_stream_kernel(const __grid_constant__ CUtensorMap tmW8, const __grid_
         for (int s = 0; s < p.nstages; ++s) mbar_init(&full[s], 1);
         fence_mbar_init();
     }
-    griddep_launch_dependents();
 
     // Every weight byte is read once: mark the lines evict-first so that the activations, the scales
     // and whatever the neighbouring kernels keep in L2 stay there.
@@ -252,6 +249,7 @@ mixed_gemm_stream_kernel(const __grid_constant__ CUtensorMap tmW8, const __grid_
     if (threadIdx.x < kWarps) ctl->arrived[threadIdx.x] = 0;
     if (threadIdx.x == 0) ctl->abort_flag = 0;
     if (p.early_weights) griddep_wait();
+    griddep_launch_dependents();
 
     // The tokens are the 8 columns of the product (one group of 8 per TT): this thread feeds the codes of token g
     // (and g + 8) and holds the sums of tokens 2 tig, 2 tig + 1 (and + 8).  Their scales and zero-points:

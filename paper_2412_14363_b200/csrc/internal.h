@@ -19,7 +19,7 @@ constexpr int kStatusBitTimeout = 1;  // a bounded wait ran out
 constexpr int kStatusBitIndex = 2;    // an index read on the device was out of range
 
 // Launch with programmatic stream serialization: the kernel's CTAs may be scheduled while the preceding grid drains, so the
-// kernel executes griddepcontrol.wait before it touches anything of it -- and before it lets its own dependents start.
+// kernel calls griddep_wait before it touches anything of it; when it lets its own dependents start: ptx.cuh.
 template <class... P, class... A>
 cudaError_t launch_programmatic(void (*kern)(P...), size_t grid, int threads, size_t smem, cudaStream_t st, A... args) {
     cudaLaunchConfig_t cfg = {};

@@ -48,8 +48,6 @@ struct AttnParams {
     int n_cache_seqs;
 };
 
-__device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void griddep_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 __device__ __forceinline__ int clamped_len(const int32_t* seq_lens, int b, int capacity) {
     const int len = seq_lens[b];

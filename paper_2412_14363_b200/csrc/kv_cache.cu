@@ -17,6 +17,7 @@
 #include <type_traits>
 
 #include "internal.h"
+#include "ptx.cuh"
 #include "../../include/resq_kv.h"
 
 namespace resq {
@@ -212,8 +213,8 @@ __global__ void __launch_bounds__(kWarps * 32) kv_project_kernel(const ProjectPa
     __shared__ float su_s[D];
     __shared__ __align__(16) uint8_t rec_s[kWarps][16 * H::kRec];
     __shared__ long long slot_s[kWarps][16];
-    asm volatile("griddepcontrol.wait;" ::: "memory");  // launched with programmatic stream serialization
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    griddep_wait();  // launched with programmatic stream serialization
+    griddep_launch_dependents();
     stage_uc<D>(p.wq, p.s_u, w_s, su_s);
     __syncthreads();
 
@@ -358,8 +359,8 @@ __global__ void __launch_bounds__(kWarps * 32) head_vector_kernel(const ProjectP
         kind = it < p.q_rows ? 0 : it < p.q_rows + p.kv_rows ? 1 : 2;  // query, key, value
         row = kind == 0 ? it : kind == 1 ? it - p.q_rows : it - p.q_rows - p.kv_rows;
     };
-    asm volatile("griddepcontrol.wait;" ::: "memory");  // launched with programmatic stream serialization
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    griddep_wait();  // launched with programmatic stream serialization
+    griddep_launch_dependents();
     int kind = 0;
     long long row = 0;
     float x[N];

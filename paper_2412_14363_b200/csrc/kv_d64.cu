@@ -170,8 +170,8 @@ __global__ void __launch_bounds__(A64<TEAM>::kNWarps * 32, TEAM == 1 ? 1 : 3) at
         else __syncthreads();
     };
 
-    asm volatile("griddepcontrol.wait;" ::: "memory");  // launched with programmatic stream serialization
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    griddep_wait();  // launched with programmatic stream serialization
+    griddep_launch_dependents();
     // ---- rows of this lane, positions they see, the sequence
     int tok[RH], head[RH], pos_i[RH];
     int b, limit, pos_min;  // positions any row of the tile sees; the smallest of the rows' own positions

@@ -315,8 +315,8 @@ __global__ void __launch_bounds__(Geometry<NT>::kThreads, 1) attention_prefill_k
         tmem_relinquish();
     }
 
-    asm volatile("griddepcontrol.wait;" ::: "memory");  // the set-up above ran under the tail of the preceding grid
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    griddep_wait();  // the set-up above ran under the tail of the preceding grid
+    griddep_launch_dependents();
     // ---- the largest value scale of the positions visited
     {
         float vmax = 0.f;

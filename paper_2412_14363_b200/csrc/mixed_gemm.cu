@@ -130,8 +130,8 @@ mixed_gemm_kernel(const __grid_constant__ CUtensorMap tmA8, const __grid_constan
     tc_fence_after();
     const uint32_t tmem_base = sh->tmem_base;
     // Launched with programmatic stream serialization: the set-up above ran under the tail of the preceding grid.
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    griddep_wait();
+    griddep_launch_dependents();
 
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer

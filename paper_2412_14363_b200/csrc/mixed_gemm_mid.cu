@@ -113,8 +113,8 @@ mixed_gemm_mid_kernel(const __grid_constant__ CUtensorMap tmW8, const __grid_con
     cluster_sync_all();  // the other CTAs' barriers exist before anything is signalled across
     tc_fence_after();
     const uint32_t tmem_base = sh->tmem_base;
-    asm volatile("griddepcontrol.wait;" ::: "memory");  // the set-up above ran under the tail of the preceding grid
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    griddep_wait();  // the set-up above ran under the tail of the preceding grid
+    griddep_launch_dependents();
 
     const int quad = warp & 3, part = (warp - 2) >> 2;  // epilogue warps: TMEM lane quadrant, which half of the groups
     const int groups = p.ntok / 16;

@@ -69,8 +69,6 @@ struct __align__(8) Shared {
 
 constexpr size_t kSmemBytes = 1024 + STAGES * (A_BYTES + B_BYTES) + sizeof(Shared);
 
-__device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void griddep_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // A converged warp's wait before tensor-core instructions.
 __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag, const int* status) {
@@ -118,7 +116,9 @@ __device__ __forceinline__ Item item_info(const Params& p, int item) {
 
 // C tile = sum of its partial tiles, slices in index order (deterministic).  One thread per four columns of one
 // row; the slices' loads are issued eight at a time and added in order.  Launched with programmatic stream
-// serialization behind the GEMM: its CTAs are scheduled as the GEMM's retire and wait here for the whole grid.
+// serialization behind the GEMM: its CTAs are scheduled as the GEMM's retire and wait here for the whole grid.  It lets its
+// own dependents start before that wait (ptx.cuh): the GEMM of the same call had waited before this kernel was started.
+// Behind the wait: 2048 x 2048 at one token, calls back to back in a graph, 5.2 -> 5.6 us.
 __global__ void __launch_bounds__(256) project_reduce_kernel(const Params p) {
     griddep_launch_dependents();
     const int t = blockIdx.y;

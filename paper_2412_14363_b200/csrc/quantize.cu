@@ -263,8 +263,8 @@ split_quantize_fast_kernel(const void* __restrict__ in, size_t in_row_bytes, siz
     // wait for the preceding grid.  Only then may the kernel enqueued behind this one start its own prologue, so that a
     // dependent that is running finds everything enqueued before this grid complete (the product that follows in
     // resq_linear streams its weights at once; it still waits for this grid before it reads the codes).
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    griddep_wait();
+    griddep_launch_dependents();
     const uint32_t row_bytes = static_cast<uint32_t>(K) * (F32 ? 4u : 2u);
     const size_t group_bytes = static_cast<size_t>(row_bytes) * rows_per_cta;
     const size_t groups = (rows + rows_per_cta - 1) / rows_per_cta;
@@ -582,8 +582,8 @@ hadamard_quantize_kernel(const __nv_bfloat16* __restrict__ X, size_t rows, int K
     const int nchunks = K >> 3, rchunks = r >> 3;
     const int K4 = K - r;
     const uint8_t* srow = reinterpret_cast<const uint8_t*>(hrow);
-    asm volatile("griddepcontrol.wait;" ::: "memory");  // launched with programmatic stream serialization
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    griddep_wait();  // launched with programmatic stream serialization
+    griddep_launch_dependents();
     for (size_t row = blockIdx.x; row < rows; row += gridDim.x) {
         // 1. widen the bf16 row (M = 1; otherwise the small factor below reads its groups straight from global memory)
         const uint4* xp = reinterpret_cast<const uint4*>(X + row * static_cast<size_t>(K));

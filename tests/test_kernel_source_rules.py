@@ -1,0 +1,47 @@
+"""Rules that the CUDA sources keep because breaking them shows on a GPU only by chance."""
+import os
+import re
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2412_14363_b200", "csrc")
+SOURCES = sorted(f for f in os.listdir(CSRC) if f.endswith((".cu", ".cuh")))
+
+
+def _code(name):
+    text = open(os.path.join(CSRC, name)).read()
+    return re.sub(r"//[^\n]*", "", re.sub(r"/\*.*?\*/", "", text, flags=re.S))
+
+
+def _block(text, start):
+    """text from the first brace at or after `start` to the one that closes it."""
+    i = text.index("{", start)
+    depth = 0
+    for j in range(i, len(text)):
+        depth += {"{": 1, "}": -1}.get(text[j], 0)
+        if depth == 0:
+            return text[i:j + 1]
+    raise AssertionError("unbalanced braces")
+
+
+def _kernels(text):
+    """(head, body) of every kernel: its signature and its definition."""
+    for m in re.finditer(r"__global__", text):
+        body = _block(text, text.index(")", m.start()))
+        yield text[m.start():text.index(body, m.start())], body
+
+
+# Kernels whose predecessor is always a kernel of the same call that lets its dependents start after its own wait.
+BEHIND_A_WAIT = {"project_reduce_kernel"}
+
+
+@pytest.mark.parametrize("name", SOURCES)
+def test_a_kernel_waits_before_it_lets_dependents_start(name):
+    """Else a kernel that reads something before its own wait (weights, sequence lengths) could run beside one that was
+    enqueued two calls before it and still writes that."""
+    for head, body in _kernels(_code(name)):
+        if "griddep_launch_dependents" in body:
+            assert "griddep_wait" in body, head
+            if any(k in head for k in BEHIND_A_WAIT):
+                continue
+            assert body.rindex("griddep_wait") < body.index("griddep_launch_dependents"), head
