@@ -121,8 +121,8 @@ __device__ __forceinline__ void mma_s8(int (&d)[4], uint32_t a0, uint32_t a1, ui
 // first chunk is, and used after its last: converting at once would make the warp wait for a DRAM round trip
 // before it touches the weights that are already in its ring).
 __device__ __forceinline__ uint32_t load_scale_raw(const void* p, int n, int fp16) {
-    if (fp16) return __ldg(reinterpret_cast<const unsigned short*>(p) + n);
-    return __ldg(reinterpret_cast<const uint32_t*>(p) + n);
+    if (fp16) return reinterpret_cast<const unsigned short*>(p)[n];
+    return reinterpret_cast<const uint32_t*>(p)[n];
 }
 __device__ __forceinline__ float scale_value(uint32_t raw, int fp16) {
     return fp16 ? __half2float(__ushort_as_half(static_cast<unsigned short>(raw))) : __uint_as_float(raw);
@@ -282,7 +282,7 @@ mixed_gemm_stream_kernel(const __grid_constant__ CUtensorMap tmW8, const __grid_
                 const int i = base + b * kThreads + threadIdx.x;
                 const int t = i / v8, o = i - t * v8;
                 v[b] = make_uint4(0, 0, 0, 0);
-                if (i < n8 && t < p.T && o < r8) v[b] = __ldg(reinterpret_cast<const uint4*>(p.x8 + static_cast<size_t>(t) * p.r) + o);
+                if (i < n8 && t < p.T && o < r8) v[b] = reinterpret_cast<const uint4*>(p.x8 + static_cast<size_t>(t) * p.r)[o];
             }
         };
         auto store8 = [&](int base, const uint4 (&v)[kBatch]) {
@@ -300,7 +300,7 @@ mixed_gemm_stream_kernel(const __grid_constant__ CUtensorMap tmW8, const __grid_
                 const int i = base + b * kThreads + threadIdx.x;
                 const int t = i / v4, o = i - t * v4;
                 v[b] = make_uint4(0, 0, 0, 0);
-                if (i < n4 && t < p.T && o < r4) v[b] = __ldg(reinterpret_cast<const uint4*>(p.x4 + static_cast<size_t>(t) * p.row4) + o);
+                if (i < n4 && t < p.T && o < r4) v[b] = reinterpret_cast<const uint4*>(p.x4 + static_cast<size_t>(t) * p.row4)[o];
             }
         };
         auto store4 = [&](int base, const uint4 (&v)[kBatch]) {
@@ -383,7 +383,7 @@ mixed_gemm_stream_kernel(const __grid_constant__ CUtensorMap tmW8, const __grid_
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
                         const int i = i0 + 32 * k + lane;
-                        v[k] = i < r4 ? __ldg(row + i) : make_uint4(0, 0, 0, 0);
+                        v[k] = i < r4 ? row[i] : make_uint4(0, 0, 0, 0);
                     }
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
@@ -464,8 +464,8 @@ mixed_gemm_stream_kernel(const __grid_constant__ CUtensorMap tmW8, const __grid_
             rw8[h] = load_scale_raw(p.s_w8, n, p.w_fp16);
             rw4[h] = load_scale_raw(p.s_w4, n, p.w_fp16);
             if (ASYM) {
-                ws8[h] = __ldg(p.wsum8 + n);
-                ws4[h] = __ldg(p.wsum4 + n);
+                ws8[h] = p.wsum8[n];
+                ws4[h] = p.wsum4[n];
             }
         }
         // Sums of this warp's part of the item: element i of group tt is unit i >> 1 (channel n0 + 8 (i >> 1)),

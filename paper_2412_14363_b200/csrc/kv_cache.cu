@@ -66,7 +66,7 @@ __device__ __forceinline__ void load_row(const __nv_bfloat16* row, int c, bool l
 #pragma unroll
         for (int hf = 0; hf < 2; ++hf) {
             uint2 u = make_uint2(0u, 0u);
-            if (live) u = __ldg(reinterpret_cast<const uint2*>(row + 32 * ks + 16 * hf + 4 * c));
+            if (live) u = *reinterpret_cast<const uint2*>(row + 32 * ks + 16 * hf + 4 * c);
             float* o = v + 8 * ks + 4 * hf;
             o[0] = __uint_as_float(u.x << 16); o[1] = __uint_as_float(u.x & 0xFFFF0000u);
             o[2] = __uint_as_float(u.y << 16); o[3] = __uint_as_float(u.y & 0xFFFF0000u);
@@ -198,7 +198,7 @@ template <int D>
 __device__ __forceinline__ void stage_uc(const int8_t* wq, const float* s_u, uint8_t* w_s, float* su_s) {
     for (int i = threadIdx.x; i < D * (D / 16); i += blockDim.x) {  // 16-byte pieces
         const int n = i / (D / 16), pc = i % (D / 16);
-        *reinterpret_cast<uint4*>(w_s + n * Head<D>::kWStride + pc * 16) = __ldg(reinterpret_cast<const uint4*>(wq + n * D) + pc);
+        *reinterpret_cast<uint4*>(w_s + n * Head<D>::kWStride + pc * 16) = reinterpret_cast<const uint4*>(wq + n * D)[pc];
     }
     for (int i = threadIdx.x; i < D; i += blockDim.x) su_s[i] = s_u[i];
 }

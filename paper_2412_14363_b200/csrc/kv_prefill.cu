@@ -322,7 +322,7 @@ __global__ void __launch_bounds__(Geometry<NT>::kThreads, 1) attention_prefill_k
         float vmax = 0.f;
         const int end = min(limit, (first + n_steps) * kStep);
         for (int j = first * kStep + tid; j < end; j += G::kThreads) {
-            const float4 m = __ldg(reinterpret_cast<const float4*>(blocks + static_cast<size_t>(j >> 5) * kBlockBytes + kOffVm) + (j & 31));
+            const float4 m = reinterpret_cast<const float4*>(blocks + static_cast<size_t>(j >> 5) * kBlockBytes + kOffVm)[j & 31];
             // a scale that is not finite makes the rows that see it infinite or NaN whatever E is
             vmax = fmaxf(vmax, fmaxf(m.x <= 3.402823466e38f ? m.x : 0.f, m.z <= 3.402823466e38f ? m.z : 0.f));
         }
@@ -342,9 +342,12 @@ __global__ void __launch_bounds__(Geometry<NT>::kThreads, 1) attention_prefill_k
         const uint4* src = reinterpret_cast<const uint4*>(p.q + (static_cast<size_t>(tq) * p.Hq + hq) * 128);
         uint8_t* dst = Qs + tile * kQBytes + row * 128;
         const int sw = row & 7;
+        uint4 qv[16];  // the whole row on its way before anything is stored
+#pragma unroll
+        for (int c = 0; c < 16; ++c) qv[c] = row_ok ? src[c] : make_uint4(0, 0, 0, 0);
 #pragma unroll
         for (int c = 0; c < 16; ++c) {
-            uint4 v = row_ok ? __ldg(src + c) : make_uint4(0, 0, 0, 0);
+            uint4 v = qv[c];
             const __half2* h = reinterpret_cast<const __half2*>(&v);
             float s = 0.f;
 #pragma unroll

@@ -230,10 +230,10 @@ mixed_gemm_kernel(const __grid_constant__ CUtensorMap tmA8, const __grid_constan
             if (sh->epi_stop) break;
             const int row = m0 + quad * 32 + lane;
             const bool row_ok = row < p.T;
-            const float sx8 = row_ok ? __ldg(p.s_x8 + row) : 0.f;
-            const float sx4 = row_ok ? __ldg(p.s_x4 + row) : 0.f;
-            const float zx8 = ASYM && row_ok ? __ldg(p.z_x8 + row) : 0.f;
-            const float zx4 = ASYM && row_ok ? __ldg(p.z_x4 + row) : 0.f;
+            const float sx8 = row_ok ? p.s_x8[row] : 0.f;
+            const float sx4 = row_ok ? p.s_x4[row] : 0.f;
+            const float zx8 = ASYM && row_ok ? p.z_x8[row] : 0.f;
+            const float zx4 = ASYM && row_ok ? p.z_x4[row] : 0.f;
             if (!mbar_wait(&sh->acc_full, acc_phase, abort_flag, p.status)) continue;  // flag is set; leave at the next sample
             acc_phase ^= 1;
             tc_fence_after();

@@ -182,11 +182,13 @@ mixed_gemm_mid_kernel(const __grid_constant__ CUtensorMap tmW8, const __grid_con
         const int et = threadIdx.x - 64;
         const int t = t0 + et;
         const bool live = et < p.ntok && t < p.T;
-        sh->sx8[et] = live ? __ldg(p.s_x8 + t) : 0.f;
-        sh->sx4[et] = live ? __ldg(p.s_x4 + t) : 0.f;
+        const float sx8 = live ? p.s_x8[t] : 0.f, sx4 = live ? p.s_x4[t] : 0.f;
+        const float zx8 = ASYM && live ? p.z_x8[t] : 0.f, zx4 = ASYM && live ? p.z_x4[t] : 0.f;
+        sh->sx8[et] = sx8;
+        sh->sx4[et] = sx4;
         if (ASYM) {
-            sh->zx8[et] = live ? __ldg(p.z_x8 + t) : 0.f;
-            sh->zx4[et] = live ? __ldg(p.z_x4 + t) : 0.f;
+            sh->zx8[et] = zx8;
+            sh->zx4[et] = zx4;
         }
         ok = mbar_wait(&sh->acc_full, 0, abort_flag, p.status);
         ok = !__any_sync(0xffffffffu, !ok);

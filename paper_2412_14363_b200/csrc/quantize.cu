@@ -32,11 +32,11 @@ __device__ __forceinline__ Chunk<F32> load_chunk(const void* row, int c) {
     Chunk<F32> o;
     if constexpr (F32) {
         const uint4* p = reinterpret_cast<const uint4*>(row) + 2 * c;
-        uint4 a = __ldg(p), b = __ldg(p + 1);
+        uint4 a = p[0], b = p[1];
         o.w[0] = a.x; o.w[1] = a.y; o.w[2] = a.z; o.w[3] = a.w;
         o.w[4] = b.x; o.w[5] = b.y; o.w[6] = b.z; o.w[7] = b.w;
     } else {
-        uint4 u = __ldg(reinterpret_cast<const uint4*>(row) + c);
+        uint4 u = reinterpret_cast<const uint4*>(row)[c];
         o.w[0] = u.x; o.w[1] = u.y; o.w[2] = u.z; o.w[3] = u.w;
     }
     return o;
@@ -251,7 +251,7 @@ __device__ __forceinline__ uint32_t pack_low_bytes(uint32_t a, uint32_t b, uint3
 // ASYM: asymmetric codes (unsigned), with the zero-points z8_out / z4_out; else symmetric ones.
 template <bool F32, bool ASYM>
 __global__ void __launch_bounds__(kThreads)
-split_quantize_fast_kernel(const void* __restrict__ in, size_t in_row_bytes, size_t rows, int K, int r,
+split_quantize_fast_kernel(const void* in, size_t in_row_bytes, size_t rows, int K, int r,
                            int rows_per_cta, int nstages, int8_t* __restrict__ q8, uint8_t* __restrict__ q4,
                            float* __restrict__ s8_out, float* __restrict__ s4_out, float* __restrict__ z8_out,
                            float* __restrict__ z4_out, int8_t* __restrict__ q4e, int* __restrict__ status) {
@@ -482,7 +482,7 @@ __global__ void unpack_int4_kernel(const uint8_t* __restrict__ packed, int8_t* _
     // one 32-bit packed word (8 codes) per thread -> 8 bytes
     for (size_t i = blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x; i < nwords;
          i += static_cast<size_t>(gridDim.x) * blockDim.x) {
-        const uint32_t w = __ldg(reinterpret_cast<const uint32_t*>(packed) + i);
+        const uint32_t w = reinterpret_cast<const uint32_t*>(packed)[i];
         uint32_t o[2] = {0, 0};
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
@@ -573,7 +573,7 @@ __device__ __forceinline__ void butterfly_pass(float* hrow, int K, int s, int ti
 // generation step, where one row's chain of passes is all there is to wait for.
 template <int M, int NT>
 __global__ void __launch_bounds__(NT)
-hadamard_quantize_kernel(const __nv_bfloat16* __restrict__ X, size_t rows, int K, int kbits, int r, float inv_sqrt_k,
+hadamard_quantize_kernel(const __nv_bfloat16* X, size_t rows, int K, int kbits, int r, float inv_sqrt_k,
                          int8_t* __restrict__ q8, uint8_t* __restrict__ q4, float* __restrict__ s8_out,
                          float* __restrict__ s4_out, int8_t* __restrict__ q4e) {
     extern __shared__ __align__(16) float hrow[];  // [K]
@@ -588,7 +588,7 @@ hadamard_quantize_kernel(const __nv_bfloat16* __restrict__ X, size_t rows, int K
         // 1. widen the bf16 row (M = 1; otherwise the small factor below reads its groups straight from global memory)
         const uint4* xp = reinterpret_cast<const uint4*>(X + row * static_cast<size_t>(K));
         for (int c = tid; M == 1 && c < nchunks; c += NT) {
-            const uint4 u = __ldg(xp + c);
+            const uint4 u = xp[c];
             const uint32_t w[4] = {u.x, u.y, u.z, u.w};
             float4 a, b;
             a.x = __uint_as_float(w[0] << 16); a.y = __uint_as_float(w[0] & 0xFFFF0000u);
@@ -611,7 +611,7 @@ hadamard_quantize_kernel(const __nv_bfloat16* __restrict__ X, size_t rows, int K
                 float x[M], y[M], ps[H2], ms[H2];
 #pragma unroll
                 for (int i = 0; i < M / 4; ++i) {
-                    const uint2 u = __ldg(xg + i);
+                    const uint2 u = xg[i];
                     x[4 * i] = __uint_as_float(u.x << 16); x[4 * i + 1] = __uint_as_float(u.x & 0xFFFF0000u);
                     x[4 * i + 2] = __uint_as_float(u.y << 16); x[4 * i + 3] = __uint_as_float(u.y & 0xFFFF0000u);
                 }

@@ -45,3 +45,15 @@ def test_a_kernel_waits_before_it_lets_dependents_start(name):
             if any(k in head for k in BEHIND_A_WAIT):
                 continue
             assert body.rindex("griddep_wait") < body.index("griddep_launch_dependents"), head
+
+
+@pytest.mark.parametrize("name", SOURCES)
+def test_what_another_grid_may_still_write_is_not_read_as_read_only(name):
+    """A kernel that may start beside its producer reads with plain or .cg loads: the read-only path (__ldg, or what the compiler
+    makes of a const __restrict__ pointer) is for data nobody writes during the whole life of the kernel, and the wait does
+    not order it."""
+    text = _code(name)
+    assert "__ldg(" not in text
+    for head, body in _kernels(text):
+        if "griddep_wait" in body:
+            assert not re.search(r"const\s+\w+\s*\*\s*__restrict__", head), head
