@@ -528,9 +528,9 @@ __global__ void __launch_bounds__(Geometry<NT>::kThreads, 1) attention_prefill_k
 #pragma unroll 1
         for (int c = 0; c < 4; ++c) {
             uint32_t o[32];
+            __syncwarp();
             tmem_ld32(tmem_row + kColO4 + 32 * c, o);
             tmem_ld_wait();
-            if (!dst) continue;
 #pragma unroll
             for (int grp = 0; grp < 4; ++grp) {  // eight columns = eight coefficients
                 const int n0 = 32 * c + 8 * grp;
@@ -540,6 +540,7 @@ __global__ void __launch_bounds__(Geometry<NT>::kThreads, 1) attention_prefill_k
 #pragma unroll
                 for (int i = 0; i < 8; ++i)
                     f[i] = (n_steps > 0 ? fmaf(__uint_as_float(o[8 * grp + i]), out_scale, z) : 0.f) * inv;
+                if (!dst) continue;
                 float* d = dst + (seg8 ? n0 - 112 : 16 + n0);
                 *reinterpret_cast<float4*>(d) = seg8 ? make_float4(f[0], f[1], f[2], f[3]) : make_float4(f[0], f[2], f[4], f[6]);
                 *reinterpret_cast<float4*>(d + 4) = seg8 ? make_float4(f[4], f[5], f[6], f[7]) : make_float4(f[1], f[3], f[5], f[7]);

@@ -234,12 +234,14 @@ mixed_gemm_kernel(const __grid_constant__ CUtensorMap tmA8, const __grid_constan
             const float sx4 = row_ok ? p.s_x4[row] : 0.f;
             const float zx8 = ASYM && row_ok ? p.z_x8[row] : 0.f;
             const float zx4 = ASYM && row_ok ? p.z_x4[row] : 0.f;
-            if (!mbar_wait(&sh->acc_full, acc_phase, abort_flag, p.status)) continue;  // flag is set; leave at the next sample
+            // whole warps go on together; if a wait ran out, the flag is set: leave at the next sample
+            if (__any_sync(0xffffffffu, !mbar_wait(&sh->acc_full, acc_phase, abort_flag, p.status))) continue;
             acc_phase ^= 1;
             tc_fence_after();
             const uint32_t lane_addr = tmem_base + (static_cast<uint32_t>(quad * 32) << 16) + ch * (BN / 2);
             // Phase 1: the INT4 accumulator values of this thread's 128 columns, raw, into registers.
             uint32_t a4[4][32];
+            __syncwarp();
 #pragma unroll
             for (int c = 0; c < 4; ++c) tmem_ld32(lane_addr + BN + c * 32, a4[c]);
             tmem_ld_wait();
@@ -249,6 +251,7 @@ mixed_gemm_kernel(const __grid_constant__ CUtensorMap tmA8, const __grid_constan
 #pragma unroll
             for (int c = 0; c < 8; ++c) {
                 uint32_t a8[16];
+                __syncwarp();
                 tmem_ld16(lane_addr + c * 16, a8);
                 tmem_ld_wait();
                 if (p.kb8 == 0) {  // uniform INT4: the INT8 accumulator was never written

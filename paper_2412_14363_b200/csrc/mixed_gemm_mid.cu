@@ -233,6 +233,7 @@ mixed_gemm_mid_kernel(const __grid_constant__ CUtensorMap tmW8, const __grid_con
         for (int k = part; pair + k * p.splits < groups; k += 2) {
             const int g = pair + k * p.splits;  // g % splits == pair
             uint32_t a4[16], a8[16];
+            __syncwarp();  // TMEM loads are for the whole, converged warp; lanes beyond the channels only skip their stores
             tmem_ld16(lane_addr + kColAcc4 + 16 * g, a4);
             tmem_ld16(lane_addr + 16 * g, a8);
             tmem_ld_wait();
@@ -258,21 +259,22 @@ mixed_gemm_mid_kernel(const __grid_constant__ CUtensorMap tmW8, const __grid_con
                     }
                 }
             }
-            if (!n_ok) continue;
+            if (n_ok) {
 #pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                const int tt = 16 * g + j, t = t0 + tt;
-                if (t >= p.T) break;
-                const size_t off = static_cast<size_t>(t) * p.N + n;
-                const float t8 = static_cast<float>(static_cast<int>(a8[j])) * (sh->sx8[tt] * sw8);
-                const float t4 = static_cast<float>(static_cast<int>(a4[j])) * (sh->sx4[tt] * sw4);
-                float y = t8 + t4;
-                if (ASYM) y += sh->zx8[tt] * zc8 + sh->zx4[tt] * zc4;
-                if (p.y_dtype == RESQ_Y_BF16) reinterpret_cast<__nv_bfloat16*>(p.Y)[off] = __float2bfloat16_rn(y);
-                else reinterpret_cast<float*>(p.Y)[off] = y;
-                if (p.dbg8) {
-                    p.dbg8[off] = static_cast<int>(a8[j]);
-                    p.dbg4[off] = static_cast<int>(a4[j]);
+                for (int j = 0; j < 16; ++j) {
+                    const int tt = 16 * g + j, t = t0 + tt;
+                    if (t >= p.T) break;
+                    const size_t off = static_cast<size_t>(t) * p.N + n;
+                    const float t8 = static_cast<float>(static_cast<int>(a8[j])) * (sh->sx8[tt] * sw8);
+                    const float t4 = static_cast<float>(static_cast<int>(a4[j])) * (sh->sx4[tt] * sw4);
+                    float y = t8 + t4;
+                    if (ASYM) y += sh->zx8[tt] * zc8 + sh->zx4[tt] * zc4;
+                    if (p.y_dtype == RESQ_Y_BF16) reinterpret_cast<__nv_bfloat16*>(p.Y)[off] = __float2bfloat16_rn(y);
+                    else reinterpret_cast<float*>(p.Y)[off] = y;
+                    if (p.dbg8) {
+                        p.dbg8[off] = static_cast<int>(a8[j]);
+                        p.dbg4[off] = static_cast<int>(a4[j]);
+                    }
                 }
             }
         }

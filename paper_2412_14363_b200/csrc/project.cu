@@ -260,7 +260,7 @@ project_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_c
             if (et == 0) sh->epi_stop = *abort_flag;
             epi_barrier();
             if (sh->epi_stop) break;
-            if (!mbar_wait(&sh->acc_full[buf], acc_phase[buf], abort_flag, p.status)) continue;
+            if (__any_sync(0xffffffffu, !mbar_wait(&sh->acc_full[buf], acc_phase[buf], abort_flag, p.status))) continue;  // whole warps
             acc_phase[buf] ^= 1;
             tc_fence_after();
             const int lrow = rank * BM + quad * 32 + lane;  // row inside the pair's tile
@@ -268,6 +268,7 @@ project_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_c
 #pragma unroll 1
             for (int c = 0; c < BN / 32; ++c) {
                 uint32_t v[32];
+                __syncwarp();
                 tmem_ld32(lane_addr + c * 32, v);
                 tmem_ld_wait();
                 const int nb = it.n0 + c * 32;
@@ -433,7 +434,7 @@ project_gemm_few_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_co
             if (et == 0) sh->epi_stop = *abort_flag;
             epi_barrier();
             if (sh->epi_stop) break;
-            if (!mbar_wait(&sh->acc_full[buf], acc_phase[buf], abort_flag, p.status)) continue;
+            if (__any_sync(0xffffffffu, !mbar_wait(&sh->acc_full[buf], acc_phase[buf], abort_flag, p.status))) continue;  // whole warps
             acc_phase[buf] ^= 1;
             tc_fence_after();
             const int jj = rank * BM + quad * 32 + lane;  // column inside the tile
@@ -442,6 +443,7 @@ project_gemm_few_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_co
 #pragma unroll 1
             for (int c = 0; c < ntok / 16; ++c) {
                 uint32_t v[16];
+                __syncwarp();
                 tmem_ld16(lane_addr + c * 16, v);
                 tmem_ld_wait();
                 if (col_ok) {

@@ -57,3 +57,30 @@ def test_what_another_grid_may_still_write_is_not_read_as_read_only(name):
     for head, body in _kernels(text):
         if "griddep_wait" in body:
             assert not re.search(r"const\s+\w+\s*\*\s*__restrict__", head), head
+
+
+@pytest.mark.parametrize("name", SOURCES)
+def test_tensor_memory_is_reached_by_whole_warps(name):
+    """A TMEM load or store is for all 32 lanes at once.  A loop in which lanes may part ways (rows, columns or outputs that some
+    lanes do not have) brings them together again before the next iteration's access, and no lane goes on past a wait that
+    ran out for another."""
+    text = _code(name)
+    for m in re.finditer(r"tmem_(?:ld|st)\d+\(", text):
+        loops = [f for f in re.finditer(r"\bfor \(", text[:m.start()])]
+        enclosing = None
+        for f in loops:
+            close, depth = f.end(), 1
+            while depth:
+                depth += {"(": 1, ")": -1}.get(text[close], 0)
+                close += 1
+            if text[close:].lstrip().startswith("{"):
+                body = _block(text, close)
+                if text.index(body, close) + len(body) > m.start():
+                    enclosing = (text.index(body, close), body)
+        if enclosing is None:
+            continue
+        at, body = enclosing
+        if re.search(r"\bcontinue;|\b\w+_ok\b", body[m.start() - at:]):
+            assert "__syncwarp();" in body[:m.start() - at], (name, text[m.start():m.start() + 60])
+    for m in re.finditer(r"if \(!mbar_wait\(&sh->acc_full", text):
+        raise AssertionError((name, text[m.start():m.start() + 80]))
