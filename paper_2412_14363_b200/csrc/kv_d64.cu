@@ -7,7 +7,8 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
-#include <type_traits>
+#include <cfloat>
+#include <climits>
 
 #include "internal.h"
 #include "ptx.cuh"
@@ -65,7 +66,7 @@ struct A64 {
     static constexpr int kStep = TEAM == 1 ? 32 : 64;
     static constexpr int kNWarps = TEAM == 1 ? kSplitWarps : TEAM;
     static constexpr int kRaw = kStep / 32 * kBlock;
-    static constexpr int kTeamBytes = 2 * kRaw + 2 * kStep * kPitch + 2 * kStep * 16;
+    static constexpr int kTeamBytes = 2 * kRaw + 2 * kStep * kPitch + 2 * kStep * 16 + 16;
     static constexpr int kSmem = kTeamBytes * (kNWarps / TEAM);
     static constexpr int kRows = TEAM == 1 ? 8 : 16;  // rows of a warp in use
 };
@@ -162,6 +163,7 @@ __global__ void __launch_bounds__(A64<TEAM>::kNWarps * 32, TEAM == 1 ? 1 : 3) at
     uint8_t* Vt = Kt + STEP * kPitch;
     float4* colK = reinterpret_cast<float4*>(Vt + STEP * kPitch);
     float4* colV = colK + STEP;
+    int* bad = reinterpret_cast<int*>(colV + STEP);  // the first position whose value's 8-bit / 4-bit constants are not finite
     const int rank = static_cast<int>(blockIdx.x % p.splits), item = static_cast<int>(blockIdx.x / p.splits);
     const int kvh = item % p.Hkv, n_tiles = static_cast<int>(gridDim.x) / p.splits / p.Hkv;
     const int tile = TEAM == 1 ? item / p.Hkv : n_tiles - 1 - item / p.Hkv;  // long tiles of all heads first
@@ -224,6 +226,7 @@ __global__ void __launch_bounds__(A64<TEAM>::kNWarps * 32, TEAM == 1 ? 1 : 3) at
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
+    if (tt == 0) bad[0] = bad[1] = INT_MAX;
     issue(first, 0);
     issue(first + stride, 1);
 
@@ -288,8 +291,19 @@ __global__ void __launch_bounds__(A64<TEAM>::kNWarps * 32, TEAM == 1 ? 1 : 3) at
             if (j0 + pos >= limit) m = make_float4(0.f, 0.f, 0.f, 0.f);
             m.y = fmaf(128.f, m.x, m.y);
             m.w = fmaf(8.f, m.z, m.w);
-            if (is_v) colV[pos] = m;
-            else colK[pos] = make_float4(m.x * kScore, m.y * kScore, m.z * kScore, m.w * kScore);
+            if (is_v) {
+                // a value's constants that are not finite become 0 (they would turn a hidden position's weight of 0 into NaN);
+                // the first such position is noted for the rows that see it
+                if (!(fabsf(m.x) <= FLT_MAX && fabsf(m.y) <= FLT_MAX)) {
+                    m.x = m.y = 0.f;
+                    atomicMin(bad, j0 + pos);
+                }
+                if (!(fabsf(m.z) <= FLT_MAX && fabsf(m.w) <= FLT_MAX)) {
+                    m.z = m.w = 0.f;
+                    atomicMin(bad + 1, j0 + pos);
+                }
+                colV[pos] = m;
+            } else colK[pos] = make_float4(m.x * kScore, m.y * kScore, m.z * kScore, m.w * kScore);
         }
         team_sync();
         issue(s + 2 * stride, buf);  // everybody is done with this raw buffer
@@ -349,67 +363,60 @@ __global__ void __launch_bounds__(A64<TEAM>::kNWarps * 32, TEAM == 1 ? 1 : 3) at
             }
         }
         // ---- weights and the second product, 32 positions at a time: the tensor core's fp32 sums are truncated, so a
-        // chain of products runs over 32 positions only and is then added to the running sums with rounding.  HIDE: some
-        // positions are hidden from some rows; their weights are 0 already, but their scales and zero-points belong to a
-        // later token and may be infinite or NaN, so those are zeroed by selection too.
-        auto second_product = [&](auto hide) {
-            constexpr bool HIDE = decltype(hide)::value;
+        // chain of products runs over 32 positions only and is then added to the running sums with rounding
 #pragma unroll
-            for (int kp = 0; kp < STEP / 32; ++kp) {
-                uint32_t p8[2][3][4], p4[2][3][4];
+        for (int kp = 0; kp < STEP / 32; ++kp) {
+            uint32_t p8[2][3][4], p4[2][3][4];
 #pragma unroll
-                for (int t = 0; t < 4; ++t) {
-                    const int nt = 4 * kp + t, pos = 8 * nt + 2 * c;
-                    const float4 va = colV[pos], vb = colV[pos + 1];
+            for (int t = 0; t < 4; ++t) {
+                const int nt = 4 * kp + t, pos = 8 * nt + 2 * c;
+                const float4 va = colV[pos], vb = colV[pos + 1];
 #pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const int i = 2 * (t & 1) + h;
-                        uint32_t w8[3] = {0u, 0u, 0u}, w4[3] = {0u, 0u, 0u};
-                        if (h < RH) {
-                            const float pa = exp2_approx(sc[nt][2 * (h % RH)] - m_use[h % RH]);
-                            const float pb = exp2_approx(sc[nt][2 * (h % RH) + 1] - m_use[h % RH]);
-                            const float4 a = HIDE && j0 + pos > pos_i[h % RH] ? make_float4(0.f, 0.f, 0.f, 0.f) : va;
-                            const float4 b = HIDE && j0 + pos + 1 > pos_i[h % RH] ? make_float4(0.f, 0.f, 0.f, 0.f) : vb;
-                            l[h] += pa + pb;
-                            zs8[h] = fmaf(pa, a.y, fmaf(pb, b.y, zs8[h]));
-                            zs4[h] = fmaf(pa, a.w, fmaf(pb, b.w, zs4[h]));
-                            split_bf16(pa * a.x, pb * b.x, w8);
-                            split_bf16(pa * a.z, pb * b.z, w4);
-                        }
-#pragma unroll
-                        for (int k = 0; k < 3; ++k) {
-                            p8[t >> 1][k][i] = w8[k];
-                            p4[t >> 1][k][i] = w4[k];
-                        }
+                for (int h = 0; h < 2; ++h) {
+                    const int i = 2 * (t & 1) + h;
+                    uint32_t w8[3] = {0u, 0u, 0u}, w4[3] = {0u, 0u, 0u};
+                    if (h < RH) {
+                        const float pa = exp2_approx(sc[nt][2 * (h % RH)] - m_use[h % RH]);
+                        const float pb = exp2_approx(sc[nt][2 * (h % RH) + 1] - m_use[h % RH]);
+                        l[h] += pa + pb;
+                        zs8[h] = fmaf(pa, va.y, fmaf(pb, vb.y, zs8[h]));
+                        zs4[h] = fmaf(pa, va.w, fmaf(pb, vb.w, zs4[h]));
+                        split_bf16(pa * va.x, pb * vb.x, w8);
+                        split_bf16(pa * va.z, pb * vb.z, w4);
                     }
-                }
 #pragma unroll
-                for (int j = 0; j < 8; j += 2) {
-                    float d0[4] = {0.f, 0.f, 0.f, 0.f}, d1[4] = {0.f, 0.f, 0.f, 0.f};
-                    uint32_t v[2][4];
-                    ldsm4t(v[0], v_addr + 2 * kp * 16 * kPitch + j * 16);
-                    ldsm4t(v[1], v_addr + (2 * kp + 1) * 16 * kPitch + j * 16);
-#pragma unroll
-                    for (int k = 2; k >= 0; --k)  // the small parts first
-#pragma unroll
-                        for (int ks = 0; ks < 2; ++ks) {
-                            mma16_bf16(d0, j == 0 ? p8[ks][k] : p4[ks][k], v[ks][0], v[ks][1]);
-                            mma16_bf16(d1, p4[ks][k], v[ks][2], v[ks][3]);
-                        }
-#pragma unroll
-                    for (int e = 0; e < 2 * RH; ++e) {
-                        O[j][e] += d0[e];
-                        O[j + 1][e] += d1[e];
+                    for (int k = 0; k < 3; ++k) {
+                        p8[t >> 1][k][i] = w8[k];
+                        p4[t >> 1][k][i] = w4[k];
                     }
                 }
             }
-        };
-        if (TWO && masked) second_product(std::true_type{});
-        else second_product(std::false_type{});
+#pragma unroll
+            for (int j = 0; j < 8; j += 2) {
+                float d0[4] = {0.f, 0.f, 0.f, 0.f}, d1[4] = {0.f, 0.f, 0.f, 0.f};
+                uint32_t v[2][4];
+                ldsm4t(v[0], v_addr + 2 * kp * 16 * kPitch + j * 16);
+                ldsm4t(v[1], v_addr + (2 * kp + 1) * 16 * kPitch + j * 16);
+#pragma unroll
+                for (int k = 2; k >= 0; --k)  // the small parts first
+#pragma unroll
+                    for (int ks = 0; ks < 2; ++ks) {
+                        mma16_bf16(d0, j == 0 ? p8[ks][k] : p4[ks][k], v[ks][0], v[ks][1]);
+                        mma16_bf16(d1, p4[ks][k], v[ks][2], v[ks][3]);
+                    }
+#pragma unroll
+                for (int e = 0; e < 2 * RH; ++e) {
+                    O[j][e] += d0[e];
+                    O[j + 1][e] += d1[e];
+                }
+            }
+        }
     }
 
     // ---- records of the warps (unnormalised sums with the zero-points, maximum, sum of weights), then the merge
     asm volatile("cp.async.wait_group 0;" ::: "memory");
+    team_sync();
+    const int bad8 = bad[0], bad4 = bad[1];
     __syncthreads();
     float* rec = reinterpret_cast<float*>(smem64);  // [warp][row][kRecPitch], over the tiles
 #pragma unroll
@@ -423,7 +430,7 @@ __global__ void __launch_bounds__(A64<TEAM>::kNWarps * 32, TEAM == 1 ? 1 : 3) at
         float* r = rec + (warp * C::kRows + gr + 8 * h) * kRecPitch;
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-            const float z = j == 0 ? zs8[h] : zs4[h];
+            const float z = pos_i[h] >= (j == 0 ? bad8 : bad4) ? NAN : j == 0 ? zs8[h] : zs4[h];
             r[coef64(j, 2 * c)] = O[j][2 * h] + z;
             r[coef64(j, 2 * c + 1)] = O[j][2 * h + 1] + z;
         }

@@ -21,9 +21,10 @@
 //
 // The coefficients of a 32-bit word of nibbles are kept in the order 0 4 1 5 2 6 3 7 (one shift and mask per pair of
 // tile elements); the query tile is written in the same order and the output un-permuted on the way out.
-// Positions beyond a row's own are masked by selection, in the scores and in the constants of the weights, and the
-// constants of positions past the tile's last are zeroed by selection, so unwritten cache positions of a loaded block
-// may hold anything.  All waits are bounded; after a failed wait every role leaves its loop, copies and products in
+// Positions beyond a row's own are masked by selection in the scores; the constants of positions past the tile's last are
+// zeroed by selection, and so are a value's constants that are not finite (they would turn a hidden position's weight of 0 into
+// NaN); the first such position is noted for the rows that do see it.  So unwritten cache positions of a loaded block, and later
+// tokens, may hold anything.  All waits are bounded; after a failed wait every role leaves its loop, copies and products in
 // flight are waited for, and TMEM is freed.
 //
 // What bounds it: shared-memory traffic (the softmax constants come as broadcasts, two wavefronts per 16 bytes, beside the
@@ -35,6 +36,9 @@
 #include "ptx.cuh"
 
 #include <cuda_fp16.h>
+
+#include <cfloat>
+#include <climits>
 
 namespace resq {
 namespace {
@@ -60,6 +64,7 @@ struct Shared {
     // centre; values (s8 s8 s4 s4) times 2^-E, (z8 z8 z4 z4) with the centre
     float4 col_k[2][kStep], col_v[2][kStep];
     float warp_max[16];
+    int bad8, bad4;  // the first position visited whose value constants of the 8-bit / 4-bit segment are infinite or NaN
     uint64_t raw_full[2], kv_full[2], kv_empty[2], s_full[2], p_full[2], pv_done[2], drain;
     uint32_t tmem_base;
     int abort_flag;
@@ -159,9 +164,10 @@ __device__ __forceinline__ uint4 bytes_centred(uint2 w) {
                       centred(__byte_perm(w.y, 0x64646464u, 0x4140), b), centred(__byte_perm(w.y, 0x64646464u, 0x4342), b));
 }
 
-// One step of the expanding warps: thread = (position tid % 64, chunk parity tid / 64).
+// One step of the expanding warps: thread = (position tid % 64, chunk parity tid / 64).  The constants of
+// positions from n_valid on, and a value's that are not finite, become 0; bad8 / bad4 note the latter (j0: the first position).
 __device__ __forceinline__ void expand_step(const uint8_t* raw, uint8_t* stage, float4* col_k, float4* col_v, int tid,
-                                            int n_valid, float p_scale) {
+                                            int n_valid, float p_scale, int j0, int* bad8, int* bad4) {
     const int j = tid & 63, jp = j & 31, par = tid >> 6, sw = j & 7;
     const uint8_t* blk = raw + (j >> 5) * kBlockBytes;
     uint8_t* krow = stage + j * 128;
@@ -184,6 +190,14 @@ __device__ __forceinline__ void expand_step(const uint8_t* raw, uint8_t* stage, 
     if (j >= n_valid) m = make_float4(0.f, 0.f, 0.f, 0.f);
     m.y = fmaf(128.f, m.x, m.y);
     m.w = fmaf(8.f, m.z, m.w);
+    if (is_v && !(fabsf(m.x) <= FLT_MAX && fabsf(m.y) <= FLT_MAX)) {
+        m.x = m.y = 0.f;
+        atomicMin(bad8, j0 + j);
+    }
+    if (is_v && !(fabsf(m.z) <= FLT_MAX && fabsf(m.w) <= FLT_MAX)) {
+        m.z = m.w = 0.f;
+        atomicMin(bad4, j0 + j);
+    }
     const float kScore = 1.4426950408889634f * 0.08838834764831845f;  // log2(e) / sqrt(128)
     const float fs = is_v ? p_scale : kScore, fz = is_v ? 1.f : kScore;
     float* dst = reinterpret_cast<float*>(is_v ? col_v : col_k) + (j >> 1) * 8 + (j & 1);
@@ -198,12 +212,6 @@ struct RowState {
     float m;       // reference, log2 units; -inf: no position seen yet
     f2 l, z8, z4;  // sums of p and of p times the zero-points (with the centre)
 };
-
-// The pair with what is not seen replaced by 0.
-__device__ __forceinline__ f2 seen(f2 v, bool lo, bool hi) {
-    const float2 f = unpack2(v);
-    return pack2(lo ? f.x : 0.f, hi ? f.y : 0.f);
-}
 
 // Scores of one step minus the row's reference, as 32 pairs; returns their maximum.  Positions of the step beyond `last` are
 // hidden from the row.
@@ -244,23 +252,15 @@ __device__ __forceinline__ float step_scores(f2 (&sc)[32], uint32_t tmem_s, cons
 }
 
 // Weights of one step: their sums into the row's state, the operands of the output product over the scores in TMEM.
-// A hidden position's weight is 0 already, but its scales and zero-points belong to a token the row must not see and may
-// be infinite or NaN: they are zeroed by selection too, so that the products are 0.
-template <bool MASKED>
-__device__ __forceinline__ void step_weights(RowState& st, const f2 (&sc)[32], uint32_t tmem_row, const float4* col_v, int last) {
+__device__ __forceinline__ void step_weights(RowState& st, const f2 (&sc)[32], uint32_t tmem_row, const float4* col_v) {
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
         uint32_t w8[8], w4[8];
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             const int pr = 8 * c + i;
-            f2x2 s = lds_pairs(col_v + 2 * pr);
-            f2x2 z = lds_pairs(col_v + 2 * pr + 1);
-            if (MASKED) {
-                const bool lo = 2 * pr <= last, hi = 2 * pr + 1 <= last;
-                s = {seen(s.x, lo, hi), seen(s.y, lo, hi)};
-                z = {seen(z.x, lo, hi), seen(z.y, lo, hi)};
-            }
+            const f2x2 s = lds_pairs(col_v + 2 * pr);
+            const f2x2 z = lds_pairs(col_v + 2 * pr + 1);
             const float2 f = unpack2(sc[pr]);
             const f2 e = pack2(ex2(f.x), ex2(f.y));
             st.l = add2(st.l, e);
@@ -307,6 +307,7 @@ __global__ void __launch_bounds__(Geometry<NT>::kThreads, 1) attention_prefill_k
         }
         mbar_init(&sh->drain, 1);
         sh->abort_flag = 0;
+        sh->bad8 = sh->bad4 = INT_MAX;
         fence_mbar_init();
     }
     if (warp == G::kMmaWarp) {
@@ -324,7 +325,7 @@ __global__ void __launch_bounds__(Geometry<NT>::kThreads, 1) attention_prefill_k
         for (int j = first * kStep + tid; j < end; j += G::kThreads) {
             const float4 m = reinterpret_cast<const float4*>(blocks + static_cast<size_t>(j >> 5) * kBlockBytes + kOffVm)[j & 31];
             // a scale that is not finite makes the rows that see it infinite or NaN whatever E is
-            vmax = fmaxf(vmax, fmaxf(m.x <= 3.402823466e38f ? m.x : 0.f, m.z <= 3.402823466e38f ? m.z : 0.f));
+            vmax = fmaxf(vmax, fmaxf(m.x <= FLT_MAX ? m.x : 0.f, m.z <= FLT_MAX ? m.z : 0.f));
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) vmax = fmaxf(vmax, __shfl_xor_sync(0xffffffffu, vmax, o));
@@ -425,8 +426,7 @@ __global__ void __launch_bounds__(Geometry<NT>::kThreads, 1) attention_prefill_k
                 }
             }
             // ---- weights, their sums, the operands of the output product
-            if (masked) step_weights<true>(st, sc, tmem_row, col_v, last);
-            else step_weights<false>(st, sc, tmem_row, col_v, last);
+            step_weights(st, sc, tmem_row, col_v);
             tmem_st_wait();
             tc_fence_before();
             mbar_arrive(&sh->p_full[tile]);
@@ -434,6 +434,9 @@ __global__ void __launch_bounds__(Geometry<NT>::kThreads, 1) attention_prefill_k
         if (!__any_sync(0xffffffffu, !ok) && n_steps > 0)
             ok = mbar_wait(&sh->pv_done[tile], (n_steps - 1) & 1, &sh->abort_flag, p.status);
         tc_fence_after();
+        // a row that sees a value whose constants are not finite gets NaN in that segment
+        if (pos_i >= sh->bad8) st.z8 = pack2(NAN, NAN);
+        if (pos_i >= sh->bad4) st.z4 = pack2(NAN, NAN);
     } else if (warp < G::kMmaWarp) {
         const int et = tid - 32 * G::kSoftmaxWarps;
         int issued = 0;
@@ -454,7 +457,7 @@ __global__ void __launch_bounds__(Geometry<NT>::kThreads, 1) attention_prefill_k
                          "selp.b32 %0, 1, 0, q;\n\t}" : "=r"(all_ok) : "r"(ok ? 1 : 0) : "memory");
             if (!all_ok) { ok = false; break; }
             expand_step(raw + (n & 1) * kRawBytes, stages + (n & 1) * kStageBytes, sh->col_k[n & 1], sh->col_v[n & 1], et,
-                        limit - (first + n) * kStep, p_scale);
+                        limit - (first + n) * kStep, p_scale, (first + n) * kStep, &sh->bad8, &sh->bad4);
             fence_proxy_async_smem();
             mbar_arrive(&sh->kv_full[n & 1]);
             asm volatile("bar.sync 1, 128;" ::: "memory");  // everybody has read the raw buffer

@@ -50,3 +50,4 @@ def test_rows_do_not_see_a_later_token(d, prefix, T, Hq, Hkv, last):
     got = _run(resq, kv, d, prefix, T, Hq, Hkv, last)
     assert np.isfinite(ref).all()
     assert (got[:-1].view(np.uint32) == ref[:-1].view(np.uint32)).all()
+    assert not np.isfinite(got[-1]).any()  # the row that does see it
