@@ -22,6 +22,7 @@
 #include <cuda_fp16.h>
 
 #include "internal.h"
+#include "plans.h"
 
 namespace resq {
 namespace {
@@ -29,9 +30,8 @@ namespace {
 constexpr int kThreads = 256;  // = columns of a block
 constexpr int kWarps = kThreads / 32;
 constexpr int kAhead = 32;        // columns of U a thread requests ahead of their use (L2 latency)
-constexpr int kMaxRows = kWarps;  // one warp per row rounds
+static_assert(kGptqMaxRows <= kWarps, "one warp per row rounds");
 constexpr size_t kRowLimit = 200 * 1024;   // accepted rows: 9 bytes per weight within this (the documented bound)
-constexpr size_t kSmemPerCta = 225 * 1024;  // dynamic shared memory of a CTA (one per SM)
 
 struct Params {
     const float* W;       // [N][K]
@@ -297,7 +297,7 @@ cudaError_t launch_rows(const Params& p, cudaStream_t st) {
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev >= 64 || !attr_set[dev]) {
-        e = cudaFuncSetAttribute(gptq_rows_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSmemPerCta));
+        e = cudaFuncSetAttribute(gptq_rows_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kGptqSmemPerCta));
         if (e != cudaSuccess) return e;
         if (dev < 64) attr_set[dev] = true;
     }
@@ -312,14 +312,9 @@ cudaError_t launch_rows(const Params& p, cudaStream_t st) {
 cudaError_t launch_pack_gptq(const float* W, const float* U, const uint8_t* dead, int N, int K, int r, int8_t* w8,
                              uint8_t* w4, void* s8, void* s4, bool scale_fp16, int8_t* w4e, cudaStream_t st) {
     if (static_cast<size_t>(K) * 9 > kRowLimit) return cudaErrorNotSupported;
-    // Rows per CTA (one CTA per SM): as many as fit, then no more than spread the rows evenly over the rounds this takes.
-    int R = static_cast<int>(kSmemPerCta / (static_cast<size_t>(K) * 8));
-    if (R > kMaxRows) R = kMaxRows;
-    const int rounds = (N + 148 * R - 1) / (148 * R);
-    R = (N + 148 * rounds - 1) / (148 * rounds);
     Params p{W, U, dead, N, K, r, w8, w4, s8, s4, scale_fp16 ? 1 : 0, w4e};
     count_launch();
-    switch (R) {
+    switch (gptq_rows_per_cta(N, K)) {
         case 1: return launch_rows<1>(p, st);
         case 2: return launch_rows<2>(p, st);
         case 3: return launch_rows<3>(p, st);

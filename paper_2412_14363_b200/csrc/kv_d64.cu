@@ -11,6 +11,7 @@
 #include <climits>
 
 #include "internal.h"
+#include "plans.h"
 #include "ptx.cuh"
 
 namespace resq {
@@ -24,8 +25,14 @@ constexpr int kC8 = 32 * R8, kC4 = 32 * (N4 / 2), kHalf = kC8 + kC4 + 512, kBloc
 // m16n8k8, 16 rows per warp, fp32 accumulators.  Two forms of one kernel:
 //   TEAM = 4  four warps share a tile of 64 rows -- 64 / g consecutive tokens of one sequence times the g heads -- and
 //             walk the sequence together (a causal run of new tokens);
-//   TEAM = 1  the g <= 8 rows of one (query row, KV head) are alone: the 12 warps of the CTA take every 12th step
-//             each, with a tile of their own, and their sums are merged at the end (single-query and many-query forms).
+//   TEAM = 1  the g <= 8 rows of one (query row, KV head) -- an item -- are alone: the warps of the CTA take every NW-th
+//             step each, with a tile of their own, and their sums are merged at the end (single-query and many-query forms).
+//             NW = 12, one CTA per SM, for few items.  From 888 of them (two rounds of 3 x 148 CTAs) NW = 4, three CTAs
+//             per SM, which overlap each other's start and merge.  With more items than SMs, NW neighbouring ones whose
+//             lengths are short (the lengths are on the device) are taken by one CTA, a warp each; with NW = 4 all are
+//             once they fill four rounds that way.  us for rows of 32 positions, 8 KV heads, one / four heads per group, before and
+//             after: 110 rows 21 / 22 -> 11 / 12, 1000 rows 177 / 187 -> 21 / 24, 4096 rows 713 / 754 -> 74 / 82 (one warp per query head:
+//             13 / 15, 31 / 89, 92 / 333).
 // With few CTAs a cluster splits the steps further and rank 0 merges the sums through distributed shared memory, so
 // no global scratch is needed.
 //
@@ -36,21 +43,23 @@ constexpr int kC8 = 32 * R8, kC4 = 32 * (N4 / 2), kHalf = kC8 + kC4 + 512, kBloc
 //   score = s8 S8 + s4 S4 + (z8 + 128 s8) sum(q8) + (z4 + 8 s4) sum(q4)         (q half, codes exact: products exact)
 //   out   = sum_j p_j s_j (c_j - c0) + sum_j p_j (z_j + c0 s_j)
 // The weights p_j s_j enter the second product as they are in fp32: as three bf16 values of 8 bits each, which add up to
-// all 24, three products per fragment.  (Two halves under a common power of two hold 22 bits of the largest weight only:
-// a value scale 2^20 above the others, on a position with next to no weight, left 2e-5 of the rest.)
+// all 24, three products per fragment (TEAM = 1: two, its rows fill half a fragment).  (Two halves under a common power of
+// two hold 22 bits of the largest weight only: a value scale 2^20 above the others, on a position with next to no
+// weight, left 2e-5 of the rest.)
 // The eight coefficients of a 32-bit word of nibbles are stored in the order 0 4 1 5 2 6 3 7 (one shift and mask per
 // pair); the query fragments are gathered in that order and the outputs put back.
 //
 // What bounds it: the softmax arithmetic and the operand conversions on the CUDA cores (about 20 instructions per score
 // of which two thirds per pair) and, for few rows, the latency of a step; not HBM, not the tensor pipe (26 % busy).
-// 32 query / 8 KV heads, project-and-append included: 1000 new tokens 1355 -> 72 us (two halves per weight: 68), a step of
-// 16 sequences of 1024-2048 positions 507 -> 22.9 us (20.6), against one warp per (row, query head) that dequantized each
+// 32 query / 8 KV heads, project-and-append included: 1000 new tokens 1355 -> 71 us (two halves per weight: 68), a step of
+// 16 sequences of 1024-2048 positions 507 -> 21.1 us (20.6), against one warp per (row, query head) that dequantized each
 // position per head.
 struct Attn64Params {
     const uint8_t* cache;
     const __half* q;   // [rows][Hq][64]
     float* out;
     int rows, Hq, Hkv, g, n_seqs, capacity, splits;  // splits: CTAs of a cluster
+    int pack, short_steps;      // TEAM = 1: whether a CTA takes NW neighbouring items, a warp each (Pack); up to how many steps
     const int32_t* seq_of_row;  // null: seq_const if >= 0, else the row index
     const int32_t* len_of_row;  // null: len0 + row + 1
     int seq_const, len0;
@@ -59,18 +68,17 @@ struct Attn64Params {
 
 constexpr int kPitch = 144;        // bytes per position of an expanded tile: 64 halves + 16 (ldmatrix without conflicts)
 constexpr int kRecPitch = 68;      // floats per row of a record: 64 sums, maximum, sum of weights
-constexpr int kSplitWarps = 12;    // TEAM = 1: what fits 227 KB
 
-template <int TEAM>
+template <int TEAM, int NW>  // NW: warps of a CTA
 struct A64 {
     static constexpr int kStep = TEAM == 1 ? 32 : 64;
-    static constexpr int kNWarps = TEAM == 1 ? kSplitWarps : TEAM;
+    static constexpr int kNWarps = NW;
     static constexpr int kRaw = kStep / 32 * kBlock;
     static constexpr int kTeamBytes = 2 * kRaw + 2 * kStep * kPitch + 2 * kStep * 16 + 16;
     static constexpr int kSmem = kTeamBytes * (kNWarps / TEAM);
     static constexpr int kRows = TEAM == 1 ? 8 : 16;  // rows of a warp in use
 };
-static_assert(A64<1>::kSmem >= kSplitWarps * 8 * kRecPitch * 4 && A64<4>::kSmem >= 4 * 16 * kRecPitch * 4, "records fit");
+static_assert(A64<1, 4>::kTeamBytes >= 8 * kRecPitch * 4 && A64<4, 4>::kSmem >= 4 * 16 * kRecPitch * 4, "records fit");
 
 __device__ __forceinline__ void mma16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
     asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
@@ -149,12 +157,29 @@ __device__ __forceinline__ uint4 bytes_centred_bf16(uint2 w) {
 // Coefficient at element e (0..7) of chunk j (0: the 8-bit segment, 1..7: words of nibbles).
 __device__ __forceinline__ int coef64(int j, int e) { return j == 0 ? e : 8 * j + (e >> 1) + ((e & 1) << 2); }
 
-template <int TEAM>
-__global__ void __launch_bounds__(A64<TEAM>::kNWarps * 32, TEAM == 1 ? 1 : 3) attention64_kernel(const Attn64Params p) {
-    using C = A64<TEAM>;
+// Sequence and attended positions of query row `row` (TEAM = 1); out-of-range entries are clamped and, if asked, reported.
+__device__ __forceinline__ int row_length(const Attn64Params& p, int row, bool report, int& b) {
+    b = p.seq_of_row ? p.seq_of_row[row] : (p.seq_const >= 0 ? p.seq_const : row);
+    int len = p.len_of_row ? p.len_of_row[row] : p.len0 + row + 1;
+    if (b < 0 || b >= p.n_seqs) {
+        if (report) atomicOr(p.status, kStatusBitIndex);
+        b = 0;
+        len = 0;
+    }
+    if (len < 0 || len > p.capacity) {
+        if (report) atomicOr(p.status, kStatusBitIndex);
+        len = len < 0 ? 0 : p.capacity;
+    }
+    return len;
+}
+
+template <int TEAM, int NW>
+__global__ void __launch_bounds__(NW * 32, NW == 4 ? 3 : 1) attention64_kernel(const Attn64Params p) {
+    using C = A64<TEAM, NW>;
     constexpr int STEP = C::kStep, NT = STEP / 8;
     constexpr bool TWO = TEAM != 1;  // rows lane / 4 + 8 are in use
     constexpr int RH = TWO ? 2 : 1;
+    constexpr int PARTS = TWO ? 3 : 2;  // products per fragment for a weight's three parts
     extern __shared__ __align__(128) uint8_t smem64[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gr = lane >> 2, c = lane & 3;
     const int team = warp / TEAM, tt = threadIdx.x - team * TEAM * 32;  // thread of the team
@@ -164,7 +189,31 @@ __global__ void __launch_bounds__(A64<TEAM>::kNWarps * 32, TEAM == 1 ? 1 : 3) at
     float4* colK = reinterpret_cast<float4*>(Vt + STEP * kPitch);
     float4* colV = colK + STEP;
     int* bad = reinterpret_cast<int*>(colV + STEP);  // the first position whose value's 8-bit / 4-bit constants are not finite
-    const int rank = static_cast<int>(blockIdx.x % p.splits), item = static_cast<int>(blockIdx.x / p.splits);
+    const int rank = static_cast<int>(blockIdx.x % p.splits);
+    int item = static_cast<int>(blockIdx.x / p.splits);
+    int part = 0, parts = 1;  // TEAM = 1: this warp's place among the warps that share an item
+    griddep_wait();  // launched with programmatic stream serialization
+    griddep_launch_dependents();
+    if (TEAM == 1) {
+        part = warp;
+        parts = NW;
+        if (p.pack) {
+            const int n_items = p.rows * p.Hkv, base = p.pack == kPackAlways ? item * NW : item / NW * NW;
+            bool together = p.pack == kPackAlways;
+            if (!together) {
+                const int last = min(base + NW, n_items) - 1, row = min(base / p.Hkv + lane, last / p.Hkv);  // at most NW rows
+                int seq;
+                together = __reduce_max_sync(0xffffffffu, row_length(p, row, false, seq)) <= p.short_steps * C::kStep;
+                if (together && item != base) return;  // the block's first CTA takes them all
+            }
+            if (together) {
+                item = base + warp;
+                part = 0;
+                parts = 1;
+            }
+            if (item >= n_items) return;
+        }
+    }
     const int kvh = item % p.Hkv, n_tiles = static_cast<int>(gridDim.x) / p.splits / p.Hkv;
     const int tile = TEAM == 1 ? item / p.Hkv : n_tiles - 1 - item / p.Hkv;  // long tiles of all heads first
     auto team_sync = [&] {
@@ -172,25 +221,12 @@ __global__ void __launch_bounds__(A64<TEAM>::kNWarps * 32, TEAM == 1 ? 1 : 3) at
         else __syncthreads();
     };
 
-    griddep_wait();  // launched with programmatic stream serialization
-    griddep_launch_dependents();
     // ---- rows of this lane, positions they see, the sequence
     int tok[RH], head[RH], pos_i[RH];
     int b, limit, pos_min;  // positions any row of the tile sees; the smallest of the rows' own positions
     if (TEAM == 1) {
         const int row = tile;
-        b = p.seq_of_row ? p.seq_of_row[row] : (p.seq_const >= 0 ? p.seq_const : row);
-        int len = p.len_of_row ? p.len_of_row[row] : p.len0 + row + 1;
-        const bool report = kvh == 0 && rank == 0 && threadIdx.x == 0;
-        if (b < 0 || b >= p.n_seqs) {
-            if (report) atomicOr(p.status, kStatusBitIndex);
-            b = 0;
-            len = 0;
-        }
-        if (len < 0 || len > p.capacity) {
-            if (report) atomicOr(p.status, kStatusBitIndex);
-            len = len < 0 ? 0 : p.capacity;
-        }
+        const int len = row_length(p, row, kvh == 0 && rank == 0 && part == 0 && lane == 0, b);
         limit = len;
         pos_min = len - 1;
         tok[0] = gr < p.g ? row : -1;
@@ -212,9 +248,9 @@ __global__ void __launch_bounds__(A64<TEAM>::kNWarps * 32, TEAM == 1 ? 1 : 3) at
     const uint8_t* blocks = p.cache + (static_cast<size_t>(b) * p.Hkv + kvh) * (p.capacity / RESQ_KV_BLOCK) * kBlock;
     const int n_blocks = (limit + 31) >> 5, n_steps = (limit + STEP - 1) / STEP;
     // this team's steps: first, first + stride, .. < end
-    const int first = TEAM == 1 ? rank * kSplitWarps + team : static_cast<int>(static_cast<long long>(n_steps) * rank / p.splits);
+    const int first = TEAM == 1 ? rank * parts + part : static_cast<int>(static_cast<long long>(n_steps) * rank / p.splits);
     const int end = TEAM == 1 ? n_steps : static_cast<int>(static_cast<long long>(n_steps) * (rank + 1) / p.splits);
-    const int stride = TEAM == 1 ? kSplitWarps * p.splits : 1;
+    const int stride = TEAM == 1 ? parts * p.splits : 1;
 
     auto issue = [&](int s, int buf) {  // copies of step s (if it exists) into a raw buffer; always one group
         if (s < end) {
@@ -366,7 +402,7 @@ __global__ void __launch_bounds__(A64<TEAM>::kNWarps * 32, TEAM == 1 ? 1 : 3) at
         // chain of products runs over 32 positions only and is then added to the running sums with rounding
 #pragma unroll
         for (int kp = 0; kp < STEP / 32; ++kp) {
-            uint32_t p8[2][3][4], p4[2][3][4];
+            uint32_t p8[2][PARTS][4], p4[2][PARTS][4];
 #pragma unroll
             for (int t = 0; t < 4; ++t) {
                 const int nt = 4 * kp + t, pos = 8 * nt + 2 * c;
@@ -374,7 +410,7 @@ __global__ void __launch_bounds__(A64<TEAM>::kNWarps * 32, TEAM == 1 ? 1 : 3) at
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     const int i = 2 * (t & 1) + h;
-                    uint32_t w8[3] = {0u, 0u, 0u}, w4[3] = {0u, 0u, 0u};
+                    uint32_t w8[3], w4[3];
                     if (h < RH) {
                         const float pa = exp2_approx(sc[nt][2 * (h % RH)] - m_use[h % RH]);
                         const float pb = exp2_approx(sc[nt][2 * (h % RH) + 1] - m_use[h % RH]);
@@ -386,8 +422,15 @@ __global__ void __launch_bounds__(A64<TEAM>::kNWarps * 32, TEAM == 1 ? 1 : 3) at
                     }
 #pragma unroll
                     for (int k = 0; k < 3; ++k) {
-                        p8[t >> 1][k][i] = w8[k];
-                        p4[t >> 1][k][i] = w4[k];
+                        if (TWO) {
+                            p8[t >> 1][k][i] = w8[k];
+                            p4[t >> 1][k][i] = w4[k];
+                        } else if (h == 0) {  // the middle part takes the unused rows of the first one's product
+                            p8[t >> 1][k == 2][i + (k == 1)] = w8[k];
+                            p4[t >> 1][k == 2][i + (k == 1)] = w4[k];
+                        } else if (k == 0) {
+                            p8[t >> 1][1][i] = p4[t >> 1][1][i] = 0u;
+                        }
                     }
                 }
             }
@@ -398,7 +441,7 @@ __global__ void __launch_bounds__(A64<TEAM>::kNWarps * 32, TEAM == 1 ? 1 : 3) at
                 ldsm4t(v[0], v_addr + 2 * kp * 16 * kPitch + j * 16);
                 ldsm4t(v[1], v_addr + (2 * kp + 1) * 16 * kPitch + j * 16);
 #pragma unroll
-                for (int k = 2; k >= 0; --k)  // the small parts first
+                for (int k = PARTS - 1; k >= 0; --k)  // the small parts first
 #pragma unroll
                     for (int ks = 0; ks < 2; ++ks) {
                         mma16_bf16(d0, j == 0 ? p8[ks][k] : p4[ks][k], v[ks][0], v[ks][1]);
@@ -406,8 +449,8 @@ __global__ void __launch_bounds__(A64<TEAM>::kNWarps * 32, TEAM == 1 ? 1 : 3) at
                     }
 #pragma unroll
                 for (int e = 0; e < 2 * RH; ++e) {
-                    O[j][e] += d0[e];
-                    O[j + 1][e] += d1[e];
+                    O[j][e] += TWO ? d0[e] : d0[e] + d0[2 + e];
+                    O[j + 1][e] += TWO ? d1[e] : d1[e] + d1[2 + e];
                 }
             }
         }
@@ -417,8 +460,8 @@ __global__ void __launch_bounds__(A64<TEAM>::kNWarps * 32, TEAM == 1 ? 1 : 3) at
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     team_sync();
     const int bad8 = bad[0], bad4 = bad[1];
-    __syncthreads();
-    float* rec = reinterpret_cast<float*>(smem64);  // [warp][row][kRecPitch], over the tiles
+    // over the warp's own tiles, or (TEAM = 4) over the CTA's: [row][kRecPitch]
+    float* rec = reinterpret_cast<float*>(TEAM == 1 ? raw : smem64 + warp * C::kRows * kRecPitch * 4);
 #pragma unroll
     for (int h = 0; h < RH; ++h) {
 #pragma unroll
@@ -427,7 +470,7 @@ __global__ void __launch_bounds__(A64<TEAM>::kNWarps * 32, TEAM == 1 ? 1 : 3) at
             zs8[h] += __shfl_xor_sync(0xffffffffu, zs8[h], o);
             zs4[h] += __shfl_xor_sync(0xffffffffu, zs4[h], o);
         }
-        float* r = rec + (warp * C::kRows + gr + 8 * h) * kRecPitch;
+        float* r = rec + (gr + 8 * h) * kRecPitch;
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
             const float z = pos_i[h] >= (j == 0 ? bad8 : bad4) ? NAN : j == 0 ? zs8[h] : zs4[h];
@@ -441,22 +484,23 @@ __global__ void __launch_bounds__(A64<TEAM>::kNWarps * 32, TEAM == 1 ? 1 : 3) at
     }
     __syncwarp();
     if (p.splits > 1) cluster_sync_all();
-    else __syncthreads();
+    else if (TEAM != 1 || parts > 1) __syncthreads();
     if (rank == 0) {
-        constexpr int kParts = TEAM == 1 ? kSplitWarps : 1;  // records of a row in one CTA
         const int n_rows = TEAM == 1 ? p.g : 64;
-        for (int i = threadIdx.x; i < n_rows * (D / 4); i += blockDim.x) {
+        const int sharers = TEAM == 1 ? parts * 32 : NW * 32, me = TEAM == 1 ? part * 32 + lane : static_cast<int>(threadIdx.x);
+        uint8_t* rec0 = TEAM == 1 ? raw - part * C::kTeamBytes : smem64;  // the item's first record
+        for (int i = me; i < n_rows * (D / 4); i += sharers) {
             const int row = i / (D / 4), c4 = i % (D / 4);
             const int R = tile * 64 + row;
             if (TEAM != 1 && R >= p.rows * p.g) continue;
-            const uint32_t local = smem_u32(rec + row * kRecPitch);  // TEAM = 4: warps' rows follow one another
+            const uint32_t local = smem_u32(rec0) + row * kRecPitch * 4;  // TEAM = 4: warps' rows follow one another
             float M = -INFINITY, L = 0.f;
             float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
             for (int rk = 0; rk < p.splits; ++rk) {
                 const uint32_t base = cluster_map_addr(local, rk);
 #pragma unroll 4
-                for (int w = 0; w < kParts; ++w) {
-                    const uint32_t a = base + w * C::kRows * kRecPitch * 4;
+                for (int w = 0; w < parts; ++w) {
+                    const uint32_t a = base + w * C::kTeamBytes;
                     const float2 ml = ld_cluster_f2(a + D * 4);
                     const float4 o = ld_cluster_f4(a + c4 * 16);
                     const float m_new = fmaxf(M, ml.x);
@@ -477,21 +521,23 @@ __global__ void __launch_bounds__(A64<TEAM>::kNWarps * 32, TEAM == 1 ? 1 : 3) at
     if (p.splits > 1) cluster_sync_all();  // the records stay until rank 0 has read them
 }
 
-template <int TEAM>
-cudaError_t launch_attention64_form(const Attn64Params& p, unsigned tiles, cudaStream_t st) {
+template <int TEAM, int NW>
+cudaError_t launch_attention64_form(const Attn64Params& p, long long ctas, cudaStream_t st) {
+    using C = A64<TEAM, NW>;
+    const auto kern = attention64_kernel<TEAM, NW>;
     static bool attr_set[64] = {};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev >= 64 || !attr_set[dev]) {
-        e = cudaFuncSetAttribute(attention64_kernel<TEAM>, cudaFuncAttributeMaxDynamicSharedMemorySize, A64<TEAM>::kSmem);
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmem);
         if (e != cudaSuccess) return e;
         if (dev < 64) attr_set[dev] = true;
     }
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(tiles * static_cast<unsigned>(p.Hkv * p.splits));
-    cfg.blockDim = dim3(A64<TEAM>::kNWarps * 32);
-    cfg.dynamicSmemBytes = A64<TEAM>::kSmem;
+    cfg.gridDim = dim3(static_cast<unsigned>(ctas));
+    cfg.blockDim = dim3(NW * 32);
+    cfg.dynamicSmemBytes = C::kSmem;
     cfg.stream = st;
     cudaLaunchAttribute attr[2] = {};
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -501,9 +547,9 @@ cudaError_t launch_attention64_form(const Attn64Params& p, unsigned tiles, cudaS
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     // The causal form's CTAs (three per SM, long tiles first) would crowd the SMs that drain first: 58 -> 68 us.
-    cfg.numAttrs = TEAM == 1 ? 2 : 1;
+    cfg.numAttrs = TEAM == 1 || cfg.gridDim.x <= 148 ? 2 : 1;
     count_launch();
-    return cudaLaunchKernelEx(&cfg, attention64_kernel<TEAM>, p);
+    return cudaLaunchKernelEx(&cfg, kern, p);
 }
 
 }  // namespace
@@ -528,19 +574,13 @@ cudaError_t launch_attention64(const resq_kv_cache_t& cache, const void* q16, in
     p.seq_const = seq_const;
     p.len0 = len0;
     p.status = device_status_ptr();
-    p.splits = 1;
-    if (seq_const >= 0 && !seq_of_row && !len_of_row) {  // a causal run of one sequence
-        const long long tiles = (static_cast<long long>(rows) * p.g + 63) / 64;
-        const int steps = (len0 + rows + 63) / 64;
-        // three CTAs per SM are in flight; at least four steps per CTA of a cluster
-        while (p.splits < 8 && tiles * p.Hkv * p.splits * 2 <= 3 * 148 && steps >= 8 * p.splits) p.splits *= 2;
-        return launch_attention64_form<4>(p, static_cast<unsigned>(tiles), st);
-    }
-    // one CTA per SM is in flight; at least two steps per warp (the lengths are on the device: the capacity stands in)
-    while (p.splits < 8 && static_cast<long long>(rows) * p.Hkv * p.splits * 2 <= 148 &&
-           cache.capacity / 32 >= 4 * kSplitWarps * p.splits)
-        p.splits *= 2;
-    return launch_attention64_form<1>(p, static_cast<unsigned>(rows), st);
+    const bool run = seq_const >= 0 && !seq_of_row && !len_of_row;  // a causal run of one sequence
+    const Attn64Plan pl = run ? attention64_run_plan(len0, rows, p.g, p.Hkv) : attention64_rows_plan(rows, p.Hkv, cache.capacity);
+    p.splits = pl.splits;
+    p.pack = pl.pack;
+    p.short_steps = pl.short_steps;
+    if (run) return launch_attention64_form<4, 4>(p, pl.ctas, st);
+    return pl.warps == 4 ? launch_attention64_form<1, 4>(p, pl.ctas, st) : launch_attention64_form<1, 12>(p, pl.ctas, st);
 }
 
 }  // namespace resq

@@ -33,6 +33,7 @@
 // one 128-row tile per CTA whose phases follow one another in two passes, 404 us as it stands (431 with the products
 // issued by a thread alone in a branch).
 #include "internal.h"
+#include "plans.h"
 #include "ptx.cuh"
 
 #include <cuda_fp16.h>
@@ -647,15 +648,9 @@ cudaError_t launch_attention_prefill(const resq_kv_cache_t& cache, const void* q
     p.g = n_q_heads / cache.n_kv_heads;
     p.pos0 = pos0;
     p.status = device_status_ptr();
-    // Two tiles per CTA share the expanded codes and fill each other's waits; one where single tiles do not fill the SMs.
-    const long long rows = static_cast<long long>(T) * p.g, single = (rows + kRows - 1) / kRows;
-    const int nt = single * p.Hkv <= 148 ? 1 : 2;
-    const long long tiles = (single + nt - 1) / nt;
-    const int steps = (pos0 + T + kStep - 1) / kStep;
-    // one CTA per SM is in flight; at least four steps per CTA of a cluster pay for the merge
-    p.splits = 1;
-    while (p.splits < 8 && tiles * p.Hkv * p.splits * 2 <= 148 && steps >= 8 * p.splits) p.splits *= 2;
-    return nt == 1 ? launch_prefill<1>(p, tiles, st) : launch_prefill<2>(p, tiles, st);
+    const PrefillPlan pl = prefill_plan(pos0, T, p.g, p.Hkv);
+    p.splits = pl.splits;
+    return pl.tiles_per_cta == 1 ? launch_prefill<1>(p, pl.row_groups, st) : launch_prefill<2>(p, pl.row_groups, st);
 }
 
 }  // namespace resq

@@ -11,7 +11,7 @@
 //     index.  Integer sums: the result does not depend on S, and no global scratch is needed.
 //   * a lane is a channel, so the stores of one token are contiguous across the warp.
 // Roles per CTA as in mixed_gemm.cu: TMA producer, MMA issuer (even CTA of a pair), 8 epilogue warps; one tile per cluster,
-// no persistence.  The rule that picks this kernel, N and S is mid_plan below.  All waits are bounded.
+// no persistence.  The rule that picks this kernel, N and S is mid_plan (plans.h).  All waits are bounded.
 //
 // What bounds it: the latency of the TMA ring up to N = 128 (0.21 us per k-block of 24 KB, 8 stages), operand delivery beyond,
 // and about 7 us of launch, first copies, epilogue and drain.  us, tile kernel -> this one: 4096 x 6144 at 17 / 128 / 300 /
@@ -22,6 +22,7 @@
 #include <cuda_fp16.h>
 
 #include "internal.h"
+#include "plans.h"
 #include "ptx.cuh"
 
 namespace resq {
@@ -308,44 +309,6 @@ bool make_map_u8(CUtensorMap* m, const void* base, uint64_t rows, uint64_t kbyte
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-struct Plan {
-    int ntok, tok_tiles, splits;
-    bool use;
-};
-
-// Which (token tile, split) and whether at all.  Modelled times in ns, fitted to measurements over six layer shapes
-// (2048 x 3072 to 14336 x 4096 and 4096 x 28672) and 17 to 2048 tokens, weights in L2:
-//   this kernel  waves * (k-blocks per pair * c(N) + 3200 + 27 N - 1500) + 1500, c = 214 up to N = 128, 297 at 256 (fewer
-//                stages fit), plus the exchange: 1200 + 5 N (S = 2), 2200 + 6 N (S = 3); one wave is 74 pairs; clusters of
-//                four fit one wave up to 128 CTAs, clusters of six up to 96 (144 took two), eight never paid;
-//   tile kernel  rounds * (k-blocks * 294 + 5000) + 10600, a round being 74 tiles of 256 x 256.
-// Layers wider than L2 holds (64 MB of codes) pay a DRAM latency per wave here, which the persistent kernel hides.
-Plan mid_plan(int T, int N, int kbt) {
-    const long ch = (N + 2 * BM - 1) / (2 * BM);
-    const long tile_rounds = (ch * ((T + 255) / 256) + 73) / 74;
-    long best = tile_rounds * (kbt * 294L + 5000) + 10600;
-    const long wave_extra = static_cast<long>(N) * kbt * BK > (64L << 20) ? 4000 : 0;
-    Plan pl = {0, 0, 0, false};
-    for (int ntok = 256; ntok >= 32; ntok -= 32) {
-        const int nt = (T + ntok - 1) / ntok;
-        if (ntok > 32 && (T + ntok - 33) / (ntok - 32) == nt) continue;  // a narrower tile covers T with as many
-        const long c = ntok <= 128 ? 214 : ntok == 160 ? 222 : ntok == 192 ? 231 : ntok == 224 ? 250 : 297;
-        for (int s = 1; s <= 3; ++s) {
-            const long ctas = ch * nt * 2 * s;
-            if (s > 1 && (ctas > (s == 2 ? 128 : 96) || kbt < 4 * s)) break;
-            const long waves = s > 1 ? 1 : (ch * nt + 73) / 74;
-            const long one = (kbt + s - 1) / s * c + 3200 + 27L * ntok + (s == 2 ? 1200 + 5L * ntok : s == 3 ? 2200 + 6L * ntok : 0);
-            long t = waves * (one - 1500 + wave_extra) + 1500;
-            if (waves > 1) t += t / 20;  // a tie goes to the persistent kernel
-            if (t < best) {
-                best = t;
-                pl = {ntok, nt, s, true};
-            }
-        }
-    }
-    return pl;
-}
-
 }  // namespace
 
 cudaError_t launch_mixed_gemm_mid(int T, int N, int K, int r, const int8_t* x8, const int8_t* x4e, const float* s_x8,
@@ -354,7 +317,7 @@ cudaError_t launch_mixed_gemm_mid(int T, int N, int K, int r, const int8_t* x8, 
                                   cudaStream_t st, const float* z_x8, const float* z_x4, const int32_t* wsum8,
                                   const int32_t* wsum4) {
     const int K4 = K - r, kb8 = (r + BK - 1) / BK, kb4 = (K4 + BK - 1) / BK;
-    const Plan pl = mid_plan(T, N, kb4 + kb8);
+    const MidPlan pl = mid_plan(T, N, kb4 + kb8);
     if (!pl.use) return cudaErrorNotSupported;
     const bool asym = z_x8 != nullptr;  // then x8 / x4e hold unsigned codes
     static bool attr_set[64] = {};

@@ -1,0 +1,118 @@
+// Rules on the host that pick a kernel form from the sizes of a call.  Plain arithmetic, no CUDA: the launchers use them, and
+// the tests ask them which form a shape takes.
+#pragma once
+#include <cstddef>
+#include <cstdint>
+
+namespace resq {
+
+// ---- mixed GEMM beyond 16 tokens: which kernel (mixed_gemm_mid.cu; mixed_gemm.cu: the large tiles), token tile, split
+struct MidPlan {
+    int ntok, tok_tiles, splits;
+    bool use;  // false: the large tiles
+};
+
+// Which (token tile, split) and whether at all.  Modelled times in ns, fitted to measurements over six layer shapes
+// (2048 x 3072 to 14336 x 4096 and 4096 x 28672) and 17 to 2048 tokens, weights in L2:
+//   this kernel  waves * (k-blocks per pair * c(N) + 3200 + 27 N - 1500) + 1500, c = 214 up to N = 128, 297 at 256 (fewer
+//                stages fit), plus the exchange: 1200 + 5 N (S = 2), 2200 + 6 N (S = 3); one wave is 74 pairs; clusters of
+//                four fit one wave up to 128 CTAs, clusters of six up to 96 (144 took two), eight never paid;
+//   tile kernel  rounds * (k-blocks * 294 + 5000) + 10600, a round being 74 tiles of 256 x 256.
+// Layers wider than L2 holds (64 MB of codes) pay a DRAM latency per wave here, which the persistent kernel hides.
+inline MidPlan mid_plan(int T, int N, int kbt) {
+    const long ch = (N + 255) / 256;
+    const long tile_rounds = (ch * ((T + 255) / 256) + 73) / 74;
+    long best = tile_rounds * (kbt * 294L + 5000) + 10600;
+    const long wave_extra = static_cast<long>(N) * kbt * 128 > (64L << 20) ? 4000 : 0;
+    MidPlan pl = {0, 0, 0, false};
+    for (int ntok = 256; ntok >= 32; ntok -= 32) {
+        const int nt = (T + ntok - 1) / ntok;
+        if (ntok > 32 && (T + ntok - 33) / (ntok - 32) == nt) continue;  // a narrower tile covers T with as many
+        const long c = ntok <= 128 ? 214 : ntok == 160 ? 222 : ntok == 192 ? 231 : ntok == 224 ? 250 : 297;
+        for (int s = 1; s <= 3; ++s) {
+            const long ctas = ch * nt * 2 * s;
+            if (s > 1 && (ctas > (s == 2 ? 128 : 96) || kbt < 4 * s)) break;
+            const long waves = s > 1 ? 1 : (ch * nt + 73) / 74;
+            const long one = (kbt + s - 1) / s * c + 3200 + 27L * ntok + (s == 2 ? 1200 + 5L * ntok : s == 3 ? 2200 + 6L * ntok : 0);
+            long t = waves * (one - 1500 + wave_extra) + 1500;
+            if (waves > 1) t += t / 20;  // a tie goes to the persistent kernel
+            if (t < best) {
+                best = t;
+                pl = {ntok, nt, s, true};
+            }
+        }
+    }
+    return pl;
+}
+
+// ---- GPTQ packing (gptq.cu): rows per CTA, one CTA per SM.  As many as fit its shared memory (8 bytes per weight), then no
+// more than spread the rows evenly over the rounds this takes.
+constexpr int kGptqMaxRows = 8;                 // one rounding warp each
+constexpr size_t kGptqSmemPerCta = 225 * 1024;  // dynamic shared memory of a CTA
+
+inline int gptq_rows_per_cta(int N, int K) {
+    int R = static_cast<int>(kGptqSmemPerCta / (static_cast<size_t>(K) * 8));
+    if (R > kGptqMaxRows) R = kGptqMaxRows;
+    const int rounds = (N + 148 * R - 1) / (148 * R);
+    return (N + 148 * rounds - 1) / (148 * rounds);
+}
+
+// ---- causal run at d_head = 128 (kv_prefill.cu): tiles of 128 rows per CTA, CTAs of a cluster that split the steps
+struct PrefillPlan {
+    int tiles_per_cta, splits;
+    long long row_groups;  // groups of tiles_per_cta tiles; the grid is row_groups * Hkv * splits
+};
+
+inline PrefillPlan prefill_plan(int pos0, int T, int g, int Hkv) {
+    constexpr int kRows = 128, kStep = 64;
+    PrefillPlan pl;
+    // Two tiles per CTA share the expanded codes and fill each other's waits; one where single tiles do not fill the SMs.
+    const long long single = (static_cast<long long>(T) * g + kRows - 1) / kRows;
+    pl.tiles_per_cta = single * Hkv <= 148 ? 1 : 2;
+    pl.row_groups = (single + pl.tiles_per_cta - 1) / pl.tiles_per_cta;
+    const int steps = (pos0 + T + kStep - 1) / kStep;
+    // one CTA per SM is in flight; at least four steps per CTA of a cluster pay for the merge
+    pl.splits = 1;
+    while (pl.splits < 8 && pl.row_groups * Hkv * pl.splits * 2 <= 148 && steps >= 8 * pl.splits) pl.splits *= 2;
+    return pl;
+}
+
+// ---- attention at d_head = 64 (kv_d64.cu)
+enum Pack { kPackNever = 0, kPackIfShort = 1, kPackAlways = 2 };  // whether a CTA takes as many items as it has warps
+struct Attn64Plan {
+    int warps;        // per CTA
+    int splits;       // CTAs of a cluster that share an item or a tile
+    int pack;         // Pack (rows that are alone)
+    int short_steps;  // kPackIfShort: items of up to as many steps of 32 positions are packed
+    long long ctas;   // grid
+};
+
+// A causal run of one sequence: tiles of 64 rows, four warps each.
+inline Attn64Plan attention64_run_plan(int pos0, int T, int g, int Hkv) {
+    Attn64Plan pl{4, 1, kPackNever, 0, 0};
+    const long long tiles = (static_cast<long long>(T) * g + 63) / 64 * Hkv;
+    const int steps = (pos0 + T + 63) / 64;
+    // three CTAs per SM are in flight; at least four steps per CTA of a cluster
+    while (pl.splits < 8 && tiles * pl.splits * 2 <= 3 * 148 && steps >= 8 * pl.splits) pl.splits *= 2;
+    pl.ctas = tiles * pl.splits;
+    return pl;
+}
+
+// Query rows that are alone: one item per (row, KV head).  The lengths are on the device; the capacity stands in for them.
+inline Attn64Plan attention64_rows_plan(int rows, int Hkv, int capacity) {
+    const long long items = static_cast<long long>(rows) * Hkv;
+    if (items >= 2 * 3 * 148) {
+        // four rounds of full CTAs, three per SM: packed whatever the lengths
+        const int pack = items >= 4LL * 3 * 148 * 4 ? kPackAlways : kPackIfShort;
+        return {4, 1, pack, 4, pack == kPackAlways ? (items + 3) / 4 : items};
+    }
+    // twelve warps, one CTA per SM.  A round of CTAs with an item each takes about as long as one and a half steps of a
+    // packed CTA; three packed steps lost where lengths differ (512 items of 64 to 128 positions: 15 -> 19 us).
+    Attn64Plan pl{12, 1, items > 148 ? kPackIfShort : kPackNever, items > 2 * 148 ? 2 : 1, 0};
+    // at least two steps per warp
+    while (pl.splits < 8 && items * pl.splits * 2 <= 148 && capacity / 32 >= 4 * 12 * pl.splits) pl.splits *= 2;
+    pl.ctas = items * pl.splits;
+    return pl;
+}
+
+}  // namespace resq

@@ -9,6 +9,7 @@ import torch
 
 import synth
 from oracle import kv as okv
+from tests import plans
 from tests.gpu_util import bf16_to_dev, dev, host
 
 pytestmark = pytest.mark.gpu
@@ -221,3 +222,52 @@ def test_attention_beside_a_far_larger_value_scale(resq, kv, uc, outlier, k):
     kv.resq_attention_queries(cache, q16, dev(np.zeros(T, np.int32)), dev(lens.astype(np.int32)), many)
     assert np.abs(host(many) - ref).max() <= 2e-5 * vmax
     assert resq.resq_device_status() == resq.OK
+
+
+@pytest.mark.parametrize("rows,Hq,Hkv,longest,warps,pack", [
+    (148, 4, 1, 100, 12, 0),    # an item for every SM
+    (83, 16, 2, 130, 12, 1),    # 166 items: a CTA of twelve warps takes one, or twelve short ones; the last block has ten
+    (149, 15, 5, 100, 12, 1),   # 745: short is up to two steps; blocks span three rows
+    (445, 4, 2, 300, 4, 1),     # 890 items: one CTA of four warps each, or four short ones together
+    (891, 8, 1, 150, 4, 1),     # blocks of four rows, the last of three, lengths on both sides of short
+    (300, 24, 3, 40, 4, 1),     # all short, a row's heads in two blocks
+    (889, 8, 8, 60, 4, 2),      # 7112 items: four to a CTA whatever the lengths
+])
+def test_attention_of_many_short_rows(resq, kv, uc, rows, Hq, Hkv, longest, warps, pack):
+    """The many-query form where it hands a CTA several items, or one, by their lengths; empty prefixes, a length and a sequence
+    out of range among them.  The bound of test_attention_tile_edges."""
+    form = plans.rows64(rows, Hkv, (longest + 31) // 32 * 32)
+    assert (form.warps, form.pack) == (warps, pack)
+    W_C, wq, s_u = uc
+    S = (longest + 31) // 32 * 32
+    cache = kv.KvCache(2, Hkv, S, d_head=D)
+    cache.data.fill_(0xFF)
+    K_hat, V_hat = [], []
+    for b in range(2):
+        k = synth.head_vectors(S, Hkv, D, stream=1420 + b, lead=1.0, scale=1.5)
+        v = synth.head_vectors(S, Hkv, D, stream=1430 + b, lead=4.0, shift=0.3)
+        kv.resq_kv_append(cache, bf16_to_dev(synth.f32_to_bf16_bits(k)), bf16_to_dev(synth.f32_to_bf16_bits(v)),
+                          dev(np.full(S, b, np.int32)), dev(np.arange(S, dtype=np.int32)), wq, s_u)
+        hk, hv = _oracle_records(k, v, W_C)
+        dk, dv = okv.kv_dequantize(hk).reshape(S, Hkv, D), okv.kv_dequantize(hv).reshape(S, Hkv, D)
+        K_hat.append([dk[:, h] for h in range(Hkv)])
+        V_hat.append([dv[:, h] for h in range(Hkv)])
+    vmax = max(np.abs(x).max() for V in V_hat for x in V)
+    q16 = torch.empty((rows, Hq, D), dtype=torch.float16, device="cuda")
+    kv.resq_query_project(bf16_to_dev(synth.f32_to_bf16_bits(synth.head_vectors(rows, Hq, D, stream=1440, lead=1.0, scale=1.5))),
+                          wq, s_u, q16)
+    rng = np.random.default_rng(rows)
+    q_seq = rng.integers(0, 2, rows).astype(np.int32)
+    q_len = np.where(rng.random(rows) < 0.1, longest, rng.integers(0, 34, rows)).astype(np.int32)
+    out = torch.full((rows, Hq, D), float("nan"), dtype=torch.float32, device="cuda")
+    kv.resq_attention_queries(cache, q16, dev(q_seq), dev(q_len), out)
+    assert resq.resq_device_status() == resq.OK
+    ref = okv.attention_queries(host(q16), K_hat, V_hat, q_seq, q_len, Hq, Hkv)
+    assert np.abs(host(out) - ref).max() <= 2e-5 * vmax
+    q_len[7], q_seq[8] = S + 5, 9        # clamped to the capacity, unspecified; both reported
+    again = torch.full((rows, Hq, D), float("nan"), dtype=torch.float32, device="cuda")
+    kv.resq_attention_queries(cache, q16, dev(q_seq), dev(q_len), again)
+    assert resq.resq_device_status() == kv.ERR_INDEX
+    ref[7] = okv.attention_queries(host(q16[7:8]), K_hat, V_hat, q_seq[7:8], np.array([S]), Hq, Hkv)[0]
+    same = np.arange(rows) != 8
+    assert np.abs(host(again)[same] - ref[same]).max() <= 2e-5 * vmax
