@@ -12,18 +12,21 @@ struct MidPlan {
     bool use;  // false: the large tiles
 };
 
-// Which (token tile, split) and whether at all.  Modelled times in ns, fitted to measurements over six layer shapes
-// (2048 x 3072 to 14336 x 4096 and 4096 x 28672) and 17 to 2048 tokens, weights in L2:
+// Which (token tile, split) and whether at all.  Modelled times in ns:
 //   this kernel  waves * (k-blocks per pair * c(N) + 3200 + 27 N - 1500) + 1500, c = 214 up to N = 128, 297 at 256 (fewer
 //                stages fit), plus the exchange: 1200 + 5 N (S = 2), 2200 + 6 N (S = 3); one wave is 74 pairs; clusters of
 //                four fit one wave up to 128 CTAs, clusters of six up to 96 (144 took two), eight never paid;
-//   tile kernel  rounds * (k-blocks * 294 + 5000) + 10600, a round being 74 tiles of 256 x 256.
-// Layers wider than L2 holds (64 MB of codes) pay a DRAM latency per wave here, which the persistent kernel hides.
+//   tile kernel  rounds * (k-blocks * 295 + 4100) + 5800, a round being 74 tiles of 256 x 256 (within a tenth of 1214 times
+//                over 22 layer shapes, 1024 x 2048 to 28672 x 8192, and 17 to 4096 tokens, weights in L2 and not).
+// Where several waves follow one another the first line is short by 12 % and 1500 ns a wave, for the ends that the persistent
+// kernel overlaps.  Over those 1214 calls the choice is 0.1 % slower than the better kernel of each, at most 4 %; with
+// the tile kernel taken at rounds * (294 k-blocks + 5000) + 10600, as measured before its products were issued by a
+// converged warp, and 5 % for several waves, it was 2.1 % (4096 x 4096 at 3500 tokens 71 us instead of 51).
 inline MidPlan mid_plan(int T, int N, int kbt) {
-    const long ch = (N + 255) / 256;
-    const long tile_rounds = (ch * ((T + 255) / 256) + 73) / 74;
-    long best = tile_rounds * (kbt * 294L + 5000) + 10600;
-    const long wave_extra = static_cast<long>(N) * kbt * 128 > (64L << 20) ? 4000 : 0;
+    constexpr int kTile = 256;  // tokens and channels of a large tile
+    const long ch = (N + kTile - 1) / kTile;
+    const long tile_rounds = (ch * ((T + kTile - 1) / kTile) + 73) / 74;
+    long best = tile_rounds * (kbt * 295L + 4100) + 5800;
     MidPlan pl = {0, 0, 0, false};
     for (int ntok = 256; ntok >= 32; ntok -= 32) {
         const int nt = (T + ntok - 1) / ntok;
@@ -34,8 +37,8 @@ inline MidPlan mid_plan(int T, int N, int kbt) {
             if (s > 1 && (ctas > (s == 2 ? 128 : 96) || kbt < 4 * s)) break;
             const long waves = s > 1 ? 1 : (ch * nt + 73) / 74;
             const long one = (kbt + s - 1) / s * c + 3200 + 27L * ntok + (s == 2 ? 1200 + 5L * ntok : s == 3 ? 2200 + 6L * ntok : 0);
-            long t = waves * (one - 1500 + wave_extra) + 1500;
-            if (waves > 1) t += t / 20;  // a tie goes to the persistent kernel
+            long t = waves * (one - 1500) + 1500;
+            if (waves > 1) t += t * 12 / 100 + waves * 1500;
             if (t < best) {
                 best = t;
                 pl = {ntok, nt, s, true};

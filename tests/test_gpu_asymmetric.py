@@ -9,6 +9,7 @@ import torch
 import oracle
 import synth
 from tests.cases import synthetic_folded
+from tests import plans
 from tests.gpu_util import bf16_bits_from_dev, bf16_to_dev, dev, host
 
 pytestmark = pytest.mark.gpu
@@ -85,11 +86,15 @@ def _check_output(res, pw, y32_gpu, ybf_bits=None):
     (16, 512, 512, 64, False, True),
     (17, 512, 264, 64, False, True),      # ragged rows and columns
     (300, 2048, 520, 256, True, False),   # two pair tiles of rows, partial column tile, kernel expands packed weights
-    (2304, 1024, 2304, 128, False, True),  # 81 tiles on 74 CTA pairs: two rounds of the persistent grid
-    (1, 4096, 1024, 512, True, True),     # a single token through the tile kernel
+    (2304, 1024, 2304, 128, False, True),  # 81 large tiles on 74 CTA pairs: two rounds of the persistent grid
+    (225, 2080, 13320, 288, True, False),  # large tiles, ragged both ways, partial k-blocks
+    (1025, 544, 9480, 32, False, True),    # three rounds, a last tile row of one token
+    (300, 1056, 13320, 0, True, True),     # no INT8 blocks
+    (1, 4096, 1024, 512, True, True),     # a single token: streamed, and (codes one per byte) as a tile of 32 tokens
     (257, 1024, 768, 128, False, True),
 ])
 def test_asym_mixed_gemm_bit_exact(resq, T, K, N, r, fp16, w4i8):
+    assert T == 16 or plans.mid(T, K, N, r).use == (N < 2304)  # which of the kernels beyond 16 tokens
     C_bits = _shifted(T, K, 900 + T)
     _, Wp = synthetic_folded(2, K, N, r, seed_shift=T)
     pw = oracle.pack_weights(Wp, r, scale_fp16=fp16)
@@ -116,9 +121,11 @@ def test_asym_mixed_gemm_bit_exact(resq, T, K, N, r, fp16, w4i8):
     _check_output(res, pw, host(y32), bf16_bits_from_dev(ybf))
 
 
-def test_asym_extreme_codes(resq):
-    """All activation codes at 255 / 15 against weights at -128 / -8: largest accumulator magnitudes."""
-    T, K, N, r = 130, 1024, 256, 128
+@pytest.mark.parametrize("T,K,N,r", [(130, 1024, 256, 128), (225, 1056, 13320, 96)])
+def test_asym_extreme_codes(resq, T, K, N, r):
+    """All activation codes at 255 / 15 against weights at -128 / -8: largest accumulator magnitudes.  Both kernels beyond 16
+    tokens."""
+    assert plans.mid(T, K, N, r).use == (N == 256)
     K4 = K - r
     q8, q4 = np.full((N, r), -128, np.int8), np.full((N, K4), -8, np.int8)
     pw = oracle.PackedWeights(K, N, r, q8, q4, oracle.pack_nibbles(q4), np.full(N, 0.01, np.float32), np.full(N, 0.1, np.float32))

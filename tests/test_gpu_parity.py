@@ -13,6 +13,7 @@ import torch
 import oracle
 import synth
 from tests.cases import config1, config2_basis, synthetic_folded
+from tests import plans
 from tests.gpu_util import bf16_bits_from_dev, bf16_to_dev, dev, host
 
 pytestmark = pytest.mark.gpu
@@ -197,11 +198,17 @@ def oracle_case(T, K, N, r, fp16=False, seed_shift=0):
     (128, 4096, 1024, 512, True, True),   # k/v projection shape of the 8B model
     (1, 512, 512, 64, False, True),
     (4, 4096, 256, 512, True, True),
-    (2304, 1024, 2304, 128, False, True),   # 81 tiles on 74 CTA pairs: a second, thin round of the persistent grid
-    (2200, 2048, 2560, 256, True, True),    # 90 tiles, ragged last row tile
+    (2304, 1024, 2304, 128, False, True),   # large tiles, 81 on 74 CTA pairs: a second, thin round of the persistent grid
+    (2200, 2048, 2560, 256, True, True),    # large tiles, 90, ragged last row tile
     (2304, 1024, 2304, 0, False, True),     # the same with an empty INT8 segment
+    (225, 544, 13320, 32, True, False),     # large tiles, one row of them, ragged both ways; packed weights
+    (300, 2080, 13320, 288, False, True),   # partial k-blocks at the end of both segments
+    (1025, 544, 9480, 32, True, True),      # five k-blocks, three rounds, a last tile row of one token
+    (1030, 1056, 9480, 0, True, True),      # no INT8 blocks, a partial k-block
 ])
 def test_mixed_gemm_bit_exact(resq, T, K, N, r, fp16, w4i8):
+    large = T >= 2000 or N >= 9000  # which of the kernels beyond 16 tokens
+    assert T <= 16 or plans.mid(T, K, N, r).use == (not large)
     _, _, pw, res = oracle_case(T, K, N, r, fp16, seed_shift=T)
     a8, a4, y32, ybf = run_mixed_gemm(resq, pw, res, fp16, w4i8)
     assert (a8 == res.acc8).all()
@@ -210,17 +217,19 @@ def test_mixed_gemm_bit_exact(resq, T, K, N, r, fp16, w4i8):
 
 
 @pytest.mark.parametrize("T,K,N,r", [
-    (33, 6144, 264, 768),     # one token tile of 64, the reduction over three pairs, a channel tile of 8
+    (33, 6144, 264, 768),     # two token tiles, the reduction over three pairs, a channel tile of 8
     (70, 5792, 1032, 736),    # partial k-blocks at the end of both segments, token groups of 16 unevenly over the pairs
     (150, 2048, 4096, 0),     # no INT8 blocks
     (224, 8192, 2056, 4096),  # INT4 and INT8 blocks in both halves of the reduction
     (300, 1024, 6144, 128),   # no split: many narrow token tiles
     (700, 544, 3080, 32),     # five k-blocks
-    (1100, 2080, 3072, 288),  # more tiles than fit the GPU at once
+    (1100, 2080, 3072, 288),  # all SMs but four busy
+    (275, 1056, 10248, 96),   # more tiles than fit the GPU at once
 ])
 def test_mixed_gemm_token_counts_between(resq, T, K, N, r):
     """Token counts between the weight-streaming and the large-tile kernel: accumulators bit for bit at the edges of the
     token tiles, channel tiles, k-blocks and splits of the reduction."""
+    assert plans.mid(T, K, N, r).use
     _, _, pw, res = oracle_case(T, K, N, r, seed_shift=T)
     a8, a4, y32, ybf = run_mixed_gemm(resq, pw, res)
     assert (a8 == res.acc8).all()
@@ -228,9 +237,11 @@ def test_mixed_gemm_token_counts_between(resq, T, K, N, r):
     check_output(res, pw, y32, ybf)
 
 
-def test_mixed_gemm_extreme_codes(resq):
-    """All codes at the clip limits (-128 / -8): the accumulators reach their largest magnitudes."""
-    T, K, N, r = 130, 1024, 256, 128
+@pytest.mark.parametrize("T,K,N,r", [(130, 1024, 256, 128), (225, 1056, 13320, 96)])
+def test_mixed_gemm_extreme_codes(resq, T, K, N, r):
+    """All codes at the clip limits (-128 / -8): the accumulators reach their largest magnitudes.  Both kernels beyond 16
+    tokens."""
+    assert plans.mid(T, K, N, r).use == (N == 256)
     K4 = K - r
     x8 = np.full((T, r), -128, np.int8)
     x4 = np.full((T, K4), -8, np.int8)
@@ -296,17 +307,24 @@ def test_linear_d2048_pca_basis_end_to_end(resq):
     assert np.linalg.norm(host(y32) - ref) / np.linalg.norm(ref) < 0.25
 
 
-@pytest.mark.parametrize("T,K,N,r,fp16", [
-    (1280, 8192, 3840, 1024, False),   # 75 tiles on 74 CTA pairs: one tile in the last round
-    (1250, 8192, 3832, 1024, True),    # the same with ragged rows and columns
-    (1280, 8192, 3840, 6144, False),   # an INT8 segment three times as long as the INT4 one
-    (1280, 8192, 3840, 0, False),      # uniform INT4 over 64 K blocks
-    (2304, 8192, 2304, 1024, False),   # 81 tiles: seven in the last round
+@pytest.mark.parametrize("T,K,N,r,fp16,large", [
+    (1281, 8192, 6400, 1024, False, True),   # 150 tiles on 74 CTA pairs: two in the last round, a tile row of one token
+    (1281, 8192, 6152, 1024, True, True),    # the same with ragged columns
+    (1281, 8192, 6400, 6144, False, True),   # an INT8 segment three times as long as the INT4 one
+    (1281, 8192, 6400, 0, False, True),      # uniform INT4 over 64 K blocks
+    (1793, 8192, 4616, 1024, False, True),   # 152 tiles: four in the last round
+    (1280, 8192, 3840, 1024, False, False),  # the kernel for fewer tokens, two waves of its tiles
+    (1250, 8192, 3832, 1024, True, False),   # the same with ragged rows and columns
+    (1280, 8192, 3840, 6144, False, False),
+    (1280, 8192, 3840, 0, False, False),
+    (2304, 8192, 2304, 1024, False, False),
 ])
-def test_mixed_gemm_long_reduction_thin_last_round(resq, T, K, N, r, fp16):
-    """Reductions of 64 K blocks with a thin last round of the persistent grid (the accumulators reach their
+def test_mixed_gemm_long_reduction_thin_last_round(resq, T, K, N, r, fp16, large):
+    """Reductions of 64 K blocks with a thin last round of the persistent grid of large tiles, or of the waves of the kernel
+    for fewer tokens (the accumulators reach their
     largest magnitudes of the parity suite, the ring wraps ten times per tile): both accumulators bit for bit on
     the rows of the last tiles and on sampled rows elsewhere; two runs agree bit for bit."""
+    assert plans.mid(T, K, N, r).use == (not large)
     C_bits, Wp = synthetic_folded(T, K, N, r, seed_shift=300 + (r // 1024))
     pw = oracle.pack_weights(Wp, r, scale_fp16=fp16)
     q8, q4, s8, s4 = oracle.split_quantize(oracle.bf16_bits_to_f32(C_bits), r)
