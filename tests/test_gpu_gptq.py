@@ -7,6 +7,7 @@ import torch
 import oracle
 import synth
 from oracle import gptq
+from tests import plans
 from tests.gpu_util import bf16_bits_from_dev, bf16_to_dev, dev, host
 from tests.test_gpu_parity import check_output
 
@@ -52,17 +53,24 @@ def test_pack_weights_gptq_bit_exact(resq, N, K, r, fp16, dead_col):
         assert not host(W.w4_i8 if dead_col >= r else W.w8)[:, dead_col - r if dead_col >= r else dead_col].any()
 
 
-@pytest.mark.parametrize("N,K,r,kind", [
-    (1200, 288, 32, "dense"),    # several rows per CTA, a last CTA with fewer, a last block of one 32-column group
-    (600, 544, 512, "dense"),    # segment boundary on a block boundary
-    (8, 32, 0, "dense"),         # one group
-    (2400, 256, 64, "dense"),    # eight rows per CTA
-    (8, 14336, 1792, "sparse"),  # rows too wide for two CTAs per SM
-    (16, 512, 64, "ties"),       # quotients on half-integers, no feedback
-    (16, 512, 64, "tiny"),       # diagonal below the normal float range, zero rows
+@pytest.mark.parametrize("N,K,r,kind,R", [
+    (1200, 288, 32, "dense", 5),    # a last block of one 32-column group
+    (600, 544, 512, "dense", 5),    # segment boundary on a block boundary
+    (8, 32, 0, "dense", 1),         # one group
+    (2400, 256, 64, "dense", 6),    # two rounds of CTAs
+    (304, 288, 64, "dense", 3),     # a last CTA with one row of three
+    (592, 256, 32, "dense", 4),
+    (608, 320, 0, "dense", 5),      # three of five
+    (752, 256, 32, "dense", 6),     # two of six
+    (904, 544, 64, "dense", 7),     # one of seven
+    (1184, 512, 64, "dense", 8),    # as many rows as a CTA takes
+    (8, 14336, 1792, "sparse", 1),  # long rows
+    (16, 512, 64, "ties", 1),       # quotients on half-integers, no feedback
+    (16, 512, 64, "tiny", 1),       # diagonal below the normal float range, zero rows
 ])
-def test_pack_weights_gptq_edges(resq, N, K, r, kind):
-    """Bit for bit against the fp64 sweep where the kernel's tiling and its two division routes have edges."""
+def test_pack_weights_gptq_edges(resq, N, K, r, kind, R):
+    """Bit for bit against the fp64 sweep where the kernel's tiling (R rows per CTA) and its two division routes have edges."""
+    assert plans.gptq_rows(N, K) == R
     rng = np.random.default_rng(N + K)
     Wp = synth.projected_weights_direct(N, K, seed=900 + N)
     U = np.diag(rng.uniform(0.3, 3.0, K))
