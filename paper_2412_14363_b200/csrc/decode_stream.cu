@@ -207,9 +207,8 @@ mixed_gemm_stream_kernel(const __grid_constant__ CUtensorMap tmW8, const __grid_
     // Every weight byte is read once: mark the lines evict-first so that the activations, the scales
     // and whatever the neighbouring kernels keep in L2 stay there.
     const uint64_t stream_policy = l2_policy_evict_first();
-    // (w ^ kFlip) & kLo as ONE three-input logic op: the instruction takes a single immediate, so with two
-    // compile-time constants the assembler emits an XOR and an AND.  T is positive, which the compiler cannot know:
-    // the two words stay in registers.
+    // (w ^ kFlip) & kLo as one three-input logic instruction, which takes a single immediate: T is positive, which the
+    // compiler cannot know, so the two words are not constants to it and come from registers.
     const uint32_t never = p.T < 0 ? 1u : 0u;
     const uint32_t rflip = kFlip ^ never, rlo = kLo ^ never;
     auto even_codes = [&](uint32_t w) {

@@ -10,6 +10,7 @@
 #include <cfloat>
 #include <climits>
 
+#include "centred_codes.cuh"
 #include "internal.h"
 #include "plans.h"
 #include "ptx.cuh"
@@ -100,11 +101,6 @@ __device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], uint32_t addr) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
 }
-__device__ __forceinline__ float exp2_approx(float x) {
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
 __device__ __forceinline__ uint32_t h2_bits(__half2 v) { return *reinterpret_cast<const uint32_t*>(&v); }
 // The bits of a float that bf16 keeps.
 __device__ __forceinline__ float bf16_part(float x) { return __uint_as_float(__float_as_uint(x) & 0xFFFF0000u); }
@@ -117,26 +113,8 @@ __device__ __forceinline__ void split_bf16(float a, float b, uint32_t (&part)[3]
         b -= bf16_part(b);
     }
 }
-// Eight codes as halves minus their centre: `word` of nibbles (order 0 4 1 5 2 6 3 7), or eight bytes.
-__device__ __forceinline__ uint4 nibbles_centred(uint32_t word) {
-    const __half2 bias = __half2half2(__ushort_as_half(0x6408));  // 1024 + 8
-    uint32_t v[4];
-#pragma unroll
-    for (int m = 0; m < 4; ++m) {
-        const uint32_t b = ((word >> (4 * m)) & 0x000F000Fu) | 0x64006400u;
-        v[m] = h2_bits(__hsub2(*reinterpret_cast<const __half2*>(&b), bias));
-    }
-    return make_uint4(v[0], v[1], v[2], v[3]);
-}
-__device__ __forceinline__ uint4 bytes_centred(uint2 w) {
-    const __half2 bias = __half2half2(__ushort_as_half(0x6480));  // 1024 + 128
-    uint32_t v[4] = {__byte_perm(w.x, 0x64646464u, 0x4140), __byte_perm(w.x, 0x64646464u, 0x4342),
-                     __byte_perm(w.y, 0x64646464u, 0x4140), __byte_perm(w.y, 0x64646464u, 0x4342)};
-#pragma unroll
-    for (int m = 0; m < 4; ++m) v[m] = h2_bits(__hsub2(*reinterpret_cast<const __half2*>(&v[m]), bias));
-    return make_uint4(v[0], v[1], v[2], v[3]);
-}
-// The same as bf16, which holds 128 + (0..127) exactly: the bytes' upper bits move the centre.
+// Eight codes as bf16 minus their centre (centred_codes.cuh has them as halves).  bf16 holds 128 + (0..127) exactly: the
+// bytes' upper bits move the centre.
 __device__ __forceinline__ uint32_t minus_bf16(uint32_t v, uint32_t centre) {
     const __nv_bfloat162 d = __hsub2(*reinterpret_cast<const __nv_bfloat162*>(&v), *reinterpret_cast<const __nv_bfloat162*>(&centre));
     return *reinterpret_cast<const uint32_t*>(&d);

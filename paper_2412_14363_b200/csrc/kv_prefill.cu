@@ -32,6 +32,7 @@
 // step of 256 rows; not HBM, not the tensor pipe (42 %).  32 query / 8 KV heads, 2048 tokens behind 4096: 1310 us with
 // one 128-row tile per CTA whose phases follow one another in two passes, 404 us as it stands (431 with the products
 // issued by a thread alone in a branch).
+#include "centred_codes.cuh"
 #include "internal.h"
 #include "plans.h"
 #include "ptx.cuh"
@@ -137,32 +138,10 @@ __device__ __forceinline__ void arrived(uint32_t (&v)[8]) {
 #pragma unroll
     for (int i = 0; i < 8; ++i) asm volatile("" : "+r"(v[i]));
 }
-__device__ __forceinline__ float ex2(float x) {
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
 __device__ __forceinline__ uint32_t half_pair(f2 v) {
     const float2 f = unpack2(v);
     const __half2 h = __floats2half2_rn(f.x, f.y);
     return *reinterpret_cast<const uint32_t*>(&h);
-}
-
-// Eight codes as halves minus their centre: a word of nibbles (order 0 4 1 5 2 6 3 7), or eight bytes.
-__device__ __forceinline__ uint32_t centred(uint32_t biased, uint16_t bias) {
-    const __half2 v = __hsub2(*reinterpret_cast<const __half2*>(&biased), __half2half2(__ushort_as_half(bias)));
-    return *reinterpret_cast<const uint32_t*>(&v);
-}
-__device__ __forceinline__ uint4 nibbles_centred(uint32_t w) {
-    uint32_t v[4];
-#pragma unroll
-    for (int m = 0; m < 4; ++m) v[m] = centred(((w >> (4 * m)) & 0x000F000Fu) | 0x64006400u, 0x6408);  // 1024 + 8
-    return make_uint4(v[0], v[1], v[2], v[3]);
-}
-__device__ __forceinline__ uint4 bytes_centred(uint2 w) {
-    const uint16_t b = 0x6480;  // 1024 + 128
-    return make_uint4(centred(__byte_perm(w.x, 0x64646464u, 0x4140), b), centred(__byte_perm(w.x, 0x64646464u, 0x4342), b),
-                      centred(__byte_perm(w.y, 0x64646464u, 0x4140), b), centred(__byte_perm(w.y, 0x64646464u, 0x4342), b));
 }
 
 // One step of the expanding warps: thread = (position tid % 64, chunk parity tid / 64).  The constants of
@@ -263,7 +242,7 @@ __device__ __forceinline__ void step_weights(RowState& st, const f2 (&sc)[32], u
             const f2x2 s = lds_pairs(col_v + 2 * pr);
             const f2x2 z = lds_pairs(col_v + 2 * pr + 1);
             const float2 f = unpack2(sc[pr]);
-            const f2 e = pack2(ex2(f.x), ex2(f.y));
+            const f2 e = pack2(exp2_approx(f.x), exp2_approx(f.y));
             st.l = add2(st.l, e);
             st.z8 = fma2(e, z.x, st.z8);
             st.z4 = fma2(e, z.y, st.z4);
@@ -406,7 +385,7 @@ __global__ void __launch_bounds__(Geometry<NT>::kThreads, 1) attention_prefill_k
             const bool raise = mx > (st.m == -INFINITY ? -INFINITY : kSlack);
             if (__any_sync(0xffffffffu, raise)) {
                 const float d = raise ? mx : 0.f;
-                const float f = raise ? (st.m == -INFINITY ? 0.f : ex2(-d)) : 1.f;
+                const float f = raise ? (st.m == -INFINITY ? 0.f : exp2_approx(-d)) : 1.f;
                 const f2 d2 = pack2(-d, -d), ff = pack2(f, f);
 #pragma unroll
                 for (int i = 0; i < 32; ++i) sc[i] = add2(sc[i], d2);
@@ -579,7 +558,7 @@ __global__ void __launch_bounds__(Geometry<NT>::kThreads, 1) attention_prefill_k
                     const uint32_t a = cluster_map_addr(local, rk);
                     const float2 ml = ld_cluster_f2(a + 128 * 4);
                     const float4 o = ld_cluster_f4(a + c4 * 16);
-                    const float f = ex2(ml.x - M);
+                    const float f = exp2_approx(ml.x - M);
                     L = fmaf(ml.y, f, L);
                     acc = make_float4(fmaf(o.x, f, acc.x), fmaf(o.y, f, acc.y), fmaf(o.z, f, acc.z), fmaf(o.w, f, acc.w));
                 }

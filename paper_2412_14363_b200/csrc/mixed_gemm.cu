@@ -27,6 +27,7 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include "byte_map.h"
 #include "internal.h"
 #include "ptx.cuh"
 
@@ -166,8 +167,7 @@ mixed_gemm_kernel(const __grid_constant__ CUtensorMap tmA8, const __grid_constan
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer (even CTA only): the whole warp, converged,
-        // one lane issues (descriptors stay in uniform registers; a thread alone in a branch needs about as long to issue
-        // a k-block's four products as the tensor core to run them)
+        // one lane issues (4096 tokens, gate|up: 355 us; issued by a thread alone in a branch 388 us)
         if (rank == 0) {
             const bool leader = elect_one();
             const uint32_t idesc = ASYM ? make_idesc_u8s8(2 * BM, p.bn) : make_idesc_i8(2 * BM, p.bn);
@@ -319,23 +319,6 @@ mixed_gemm_kernel(const __grid_constant__ CUtensorMap tmA8, const __grid_constan
         tc_fence_after();
         tmem_dealloc_pair(tmem_base, kTmemCols);
     }
-}
-
-typedef CUresult (*EncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                             const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                             CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-// [rows][kbytes] uint8 matrix, box = 128 bytes x box_rows, 128-byte swizzle, zero fill out of range.
-bool make_map_u8(CUtensorMap* m, const void* base, uint64_t rows, uint64_t kbytes, uint32_t box_rows) {
-    EncodeFn enc = reinterpret_cast<EncodeFn>(tensor_map_encode_fn());
-    if (!enc) return false;
-    cuuint64_t dims[2] = {kbytes, rows};
-    cuuint64_t strides[1] = {kbytes};
-    cuuint32_t box[2] = {128, box_rows};
-    cuuint32_t estr[2] = {1, 1};
-    return enc(m, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<void*>(base), dims, strides, box, estr,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 }  // namespace
