@@ -31,9 +31,9 @@ constexpr int kC8 = 32 * R8, kC4 = 32 * (N4 / 2), kHalf = kC8 + kC4 + 512, kBloc
 //             NW = 12, one CTA per SM, for few items.  From 888 of them (two rounds of 3 x 148 CTAs) NW = 4, three CTAs
 //             per SM, which overlap each other's start and merge.  With more items than SMs, NW neighbouring ones whose
 //             lengths are short (the lengths are on the device) are taken by one CTA, a warp each; with NW = 4 all are
-//             once they fill four rounds that way.  us for rows of 32 positions, 8 KV heads, one / four heads per group, before and
-//             after: 110 rows 21 / 22 -> 11 / 12, 1000 rows 177 / 187 -> 21 / 24, 4096 rows 713 / 754 -> 74 / 82 (one warp per query head:
-//             13 / 15, 31 / 89, 92 / 333).
+//             once they fill four rounds that way.  us for rows of 32 positions, 8 KV heads, one / four heads per group,
+//             a CTA of twelve warps per item -> now: 110 rows 21 / 22 -> 11 / 12, 1000 rows 177 / 187 -> 21 / 24, 4096 rows
+//             713 / 754 -> 74 / 82 (one warp per query head: 13 / 15, 31 / 89, 92 / 333).
 // With few CTAs a cluster splits the steps further and rank 0 merges the sums through distributed shared memory, so
 // no global scratch is needed.
 //
@@ -53,7 +53,7 @@ constexpr int kC8 = 32 * R8, kC4 = 32 * (N4 / 2), kHalf = kC8 + kC4 + 512, kBloc
 // What bounds it: the softmax arithmetic and the operand conversions on the CUDA cores (about 20 instructions per score
 // of which two thirds per pair) and, for few rows, the latency of a step; not HBM, not the tensor pipe (26 % busy).
 // 32 query / 8 KV heads, project-and-append included: 1000 new tokens 1355 -> 71 us (two halves per weight: 68), a step of
-// 16 sequences of 1024-2048 positions 507 -> 21.1 us (20.6), against one warp per (row, query head) that dequantized each
+// 16 sequences of 1024-2048 positions 507 -> 21.7 us (20.6), against one warp per (row, query head) that dequantized each
 // position per head.
 struct Attn64Params {
     const uint8_t* cache;
@@ -240,7 +240,7 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? 3 : 1) attention64_kernel(c
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    if (tt == 0) bad[0] = bad[1] = INT_MAX;
+    if (TWO && tt == 0) bad[0] = bad[1] = INT_MAX;
     issue(first, 0);
     issue(first + stride, 1);
 
@@ -306,13 +306,13 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? 3 : 1) attention64_kernel(c
             m.y = fmaf(128.f, m.x, m.y);
             m.w = fmaf(8.f, m.z, m.w);
             if (is_v) {
-                // a value's constants that are not finite become 0 (they would turn a hidden position's weight of 0 into NaN);
-                // the first such position is noted for the rows that see it
-                if (!(fabsf(m.x) <= FLT_MAX && fabsf(m.y) <= FLT_MAX)) {
+                // A causal run: a value's constants that are not finite become 0 (they would turn a hidden position's weight of 0
+                // into NaN); the first such position is noted for the rows that see it.  Rows that are alone see every position.
+                if (TWO && !(fabsf(m.x) <= FLT_MAX && fabsf(m.y) <= FLT_MAX)) {
                     m.x = m.y = 0.f;
                     atomicMin(bad, j0 + pos);
                 }
-                if (!(fabsf(m.z) <= FLT_MAX && fabsf(m.w) <= FLT_MAX)) {
+                if (TWO && !(fabsf(m.z) <= FLT_MAX && fabsf(m.w) <= FLT_MAX)) {
                     m.z = m.w = 0.f;
                     atomicMin(bad + 1, j0 + pos);
                 }
@@ -437,7 +437,7 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? 3 : 1) attention64_kernel(c
     // ---- records of the warps (unnormalised sums with the zero-points, maximum, sum of weights), then the merge
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     team_sync();
-    const int bad8 = bad[0], bad4 = bad[1];
+    const int bad8 = TWO ? bad[0] : INT_MAX, bad4 = TWO ? bad[1] : INT_MAX;
     // over the warp's own tiles, or (TEAM = 4) over the CTA's: [row][kRecPitch]
     float* rec = reinterpret_cast<float*>(TEAM == 1 ? raw : smem64 + warp * C::kRows * kRecPitch * 4);
 #pragma unroll
@@ -451,7 +451,7 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? 3 : 1) attention64_kernel(c
         float* r = rec + (gr + 8 * h) * kRecPitch;
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-            const float z = pos_i[h] >= (j == 0 ? bad8 : bad4) ? NAN : j == 0 ? zs8[h] : zs4[h];
+            const float z = TWO && pos_i[h] >= (j == 0 ? bad8 : bad4) ? NAN : j == 0 ? zs8[h] : zs4[h];
             r[coef64(j, 2 * c)] = O[j][2 * h] + z;
             r[coef64(j, 2 * c + 1)] = O[j][2 * h + 1] + z;
         }
