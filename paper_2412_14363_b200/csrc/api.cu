@@ -646,7 +646,7 @@ int resq_attention_decode(const resq_kv_cache_t* cache, const void* q16, int n_q
     if (!aligned16(q16) || !aligned16(out) || !aligned16(workspace)) return RESQ_ERR_ALIGN;
     if (int e = check_arch()) return e;
     if (cache->d_head == 64)
-        return cuda_status(launch_attention64(*cache, q16, n_q_heads, cache->n_seqs, nullptr, seq_lens, -1, 0, out,
+        return cuda_status(launch_attention64(*cache, q16, n_q_heads, cache->n_seqs, nullptr, seq_lens, out,
                                               static_cast<cudaStream_t>(stream)));
     return cuda_status(launch_attention_decode(*cache, q16, n_q_heads, seq_lens, out, workspace,
                                                static_cast<cudaStream_t>(stream)));
@@ -669,7 +669,7 @@ int resq_attention_queries(const resq_kv_cache_t* cache, const void* q16, int n_
     if (!aligned16(q16) || !aligned16(out) || !aligned16(workspace)) return RESQ_ERR_ALIGN;
     if (int e = check_arch()) return e;
     if (cache->d_head == 64)
-        return cuda_status(launch_attention64(*cache, q16, n_q_heads, n_queries, q_seq, q_len, -1, 0, out,
+        return cuda_status(launch_attention64(*cache, q16, n_q_heads, n_queries, q_seq, q_len, out,
                                               static_cast<cudaStream_t>(stream)));
     return cuda_status(launch_attention_decode(*cache, q16, n_q_heads, q_len, out, workspace,
                                                static_cast<cudaStream_t>(stream), n_queries, q_seq));
@@ -683,10 +683,8 @@ int resq_attention_prefill(const resq_kv_cache_t* cache, const void* q16, int n_
     if (!q16 || !out) return RESQ_ERR_NULL;
     if (!aligned16(q16) || !aligned16(out)) return RESQ_ERR_ALIGN;
     if (int e = check_arch()) return e;
-    if (cache->d_head == 64)
-        return cuda_status(launch_attention64(*cache, q16, n_q_heads, T, nullptr, nullptr, seq, pos0, out,
-                                              static_cast<cudaStream_t>(stream)));
-    return cuda_status(launch_attention_prefill(*cache, q16, n_q_heads, seq, pos0, T, out, static_cast<cudaStream_t>(stream)));
+    return cuda_status(launch_attention_prefill(*cache, q16, n_q_heads, seq, pos0, T, out, static_cast<cudaStream_t>(stream),
+                                                cache->d_head));
 }
 
 const char* resq_last_cuda_error(void) { return cudaGetErrorString(g_last_cuda_error); }

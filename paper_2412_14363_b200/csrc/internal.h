@@ -117,17 +117,15 @@ cudaError_t launch_attention_decode(const resq_kv_cache_t& cache, const void* q1
                                     float* out, void* scratch, cudaStream_t st, int n_rows = -1,
                                     const int32_t* seq_map = nullptr);
 
-// Causal attention of T new tokens of sequence `seq` (positions pos0 .. pos0 + T - 1) on the tensor cores.
+// Causal attention of T new tokens of sequence `seq` (positions pos0 .. pos0 + T - 1) on the tensor cores, d_head 128 or 64.
 cudaError_t launch_attention_prefill(const resq_kv_cache_t& cache, const void* q16, int n_q_heads, int seq, int pos0,
-                                     int T, float* out, cudaStream_t st);
+                                     int T, float* out, cudaStream_t st, int d_head);
 
 // Attention at d_head = 64 (the cache format with every code array halved).
 size_t kv64_block_bytes();
-// Row i of q16 / out attends the first len_of_row[i] (null: len0 + i + 1) positions of sequence seq_of_row[i] (null:
-// seq_const if >= 0, else i).
+// Row i of q16 / out attends the first len_of_row[i] positions of sequence seq_of_row[i] (null: i).
 cudaError_t launch_attention64(const resq_kv_cache_t& cache, const void* q16, int n_q_heads, int rows,
-                               const int32_t* seq_of_row, const int32_t* len_of_row, int seq_const, int len0, float* out,
-                               cudaStream_t st);
+                               const int32_t* seq_of_row, const int32_t* len_of_row, float* out, cudaStream_t st);
 
 // Driver entry point for tensor-map encoding (resolved once, without linking libcuda).
 void* tensor_map_encode_fn();

@@ -60,18 +60,22 @@ inline int gptq_rows_per_cta(int N, int K) {
     return (N + 148 * rounds - 1) / (148 * rounds);
 }
 
-// ---- causal run at d_head = 128 (kv_prefill.cu): tiles of 128 rows per CTA, CTAs of a cluster that split the steps
+// ---- causal run (kv_prefill.cu): tiles of 128 rows per CTA, CTAs of a cluster that split the steps of 64 positions
 struct PrefillPlan {
     int tiles_per_cta, splits;
+    bool pair;             // the CTA's two tiles walk together, not one after the other
     long long row_groups;  // groups of tiles_per_cta tiles; the grid is row_groups * Hkv * splits
 };
 
-inline PrefillPlan prefill_plan(int pos0, int T, int g, int Hkv) {
+// Between one and two rounds of tiles a CTA takes a long and a short one in turn: one round, all CTAs equally long.  Beyond, two
+// neighbours together where there is a form for it (can_pair): they share the expanded codes and fill each other's waits.  32 / 8
+// heads of 128, one after the other / together, us: 2048 tokens 114 / 81, behind 4096 447 / 341; 1000 tokens 36 / 44.
+inline PrefillPlan prefill_plan(int pos0, int T, int g, int Hkv, bool can_pair = true) {
     constexpr int kRows = 128, kStep = 64;
     PrefillPlan pl;
-    // Two tiles per CTA share the expanded codes and fill each other's waits; one where single tiles do not fill the SMs.
     const long long single = (static_cast<long long>(T) * g + kRows - 1) / kRows;
-    pl.tiles_per_cta = single * Hkv <= 148 ? 1 : 2;
+    pl.pair = single * Hkv > 2 * 148 && can_pair;
+    pl.tiles_per_cta = single * Hkv > 148 && (pl.pair || single * Hkv <= 2 * 148) ? 2 : 1;
     pl.row_groups = (single + pl.tiles_per_cta - 1) / pl.tiles_per_cta;
     const int steps = (pos0 + T + kStep - 1) / kStep;
     // one CTA per SM is in flight; at least four steps per CTA of a cluster pay for the merge
@@ -88,16 +92,15 @@ struct Attn64Plan {
     int pack;         // Pack (rows that are alone)
     int short_steps;  // kPackIfShort: items of up to as many steps of 32 positions are packed
     long long ctas;   // grid
+    int tiles = 0;    // a causal run: tiles of 128 rows per CTA, one after the other
 };
 
-// A causal run of one sequence: tiles of 64 rows, four warps each.
+// A causal run of one sequence goes to kv_prefill.cu: sixteen softmax warps, four threads a row.  There is no form for two tiles
+// together (a thread would hold 32 outputs beside its scores).
 inline Attn64Plan attention64_run_plan(int pos0, int T, int g, int Hkv) {
-    Attn64Plan pl{4, 1, kPackNever, 0, 0};
-    const long long tiles = (static_cast<long long>(T) * g + 63) / 64 * Hkv;
-    const int steps = (pos0 + T + 63) / 64;
-    // three CTAs per SM are in flight; at least four steps per CTA of a cluster
-    while (pl.splits < 8 && tiles * pl.splits * 2 <= 3 * 148 && steps >= 8 * pl.splits) pl.splits *= 2;
-    pl.ctas = tiles * pl.splits;
+    const PrefillPlan run = prefill_plan(pos0, T, g, Hkv, false);
+    Attn64Plan pl{16, run.splits, kPackNever, 0, run.row_groups * Hkv * run.splits};
+    pl.tiles = run.tiles_per_cta;
     return pl;
 }
 
