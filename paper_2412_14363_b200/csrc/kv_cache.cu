@@ -2,11 +2,15 @@
 // projection of query and key head vectors, and the per-head asymmetric 8/4-bit quantizer that writes key and value
 // into the blocked cache.  A few MB per call at most.  Two forms, chosen by the number of head vectors (launch_project):
 //
-// kv_project_kernel (many): one warp owns 16 consecutive head vectors (rows) and contracts them on mma.sync s8
+// kv_project_kernel (many): one warp owns 16 head vectors (rows) at a time and contracts them on mma.sync s8
 // fragments taken straight from the global loads.  Lane (g, c) = (lane / 4, lane % 4) loads, for rows g and g + 8, the
-// elements [32 ks + 4c, +4) and [32 ks + 16 + 4c, +4): exactly the bytes of its A fragments of mma.m16n8k32, and 32
-// contiguous bytes per quad, so every sector fetched is used.
-//
+// elements [32 b + 8c, +8), 16 bytes at a time: the bytes of its A fragments of mma.m16n8k32, in an order of the reduction that
+// U_C's staged rows share.  The product's columns are dealt out in the same way (a permutation of U_C's rows, free with
+// ldmatrix), so outputs leave 16 bytes at a time too, and key and value share the cache quantizer.
+// What bounds it: instructions, about 700 per 16 vectors; 2048 tokens of 32 + 16 vectors take 27.8 us at d = 128 (before 32.0; the
+// 100 MB would take 15) and 13.8 at 64 (before 18.1).  Rows of a key or value tile are 16 tokens of one head: their records are
+// neighbours in the cache.  The next tile's rows are on their way during the products.  Roundings are checked for a whole lane
+// at once (two bracketing products, packed pairs) instead of one by one with a branch each.
 // head_vector_kernel (few, a generation step): one warp per head vector, lane l owning coefficients l + 32 i, dp4a
 // against U_C's codes in shared memory.  A step is latency: one vector's chain is shorter than a 16-vector tile's and so is
 // the code, which counts in a step, where every kernel runs once between others.  16 tokens (512 query, 256 key and value
@@ -17,6 +21,7 @@
 #include <type_traits>
 
 #include "internal.h"
+#include "packed_fp32.cuh"
 #include "ptx.cuh"
 #include "../../include/resq_kv.h"
 
@@ -30,15 +35,18 @@ struct Head {  // geometry of a head vector and of its cache block (resq_kv.h)
     static constexpr int kB4 = (D - kR8) / 2;                  // bytes of 4-bit codes
     static constexpr int kC8 = RESQ_KV_BLOCK * kR8, kC4 = RESQ_KV_BLOCK * kB4;
     static constexpr int kHalf = kC8 + kC4 + RESQ_KV_BLOCK * 16, kBlock = 2 * kHalf;
-    static constexpr int kWStride = D + 16;  // bytes per staged W_C row: the 8 rows of a B fragment hit 8 bank groups
-    static constexpr int kRec = kR8 + kB4 + 16;                // staged record: code bytes, 4 floats
+    static constexpr int kWStride = D + 16;  // bytes per W_C row as head_vector_kernel stages it: the lanes' rows hit all banks
 };
 static_assert(Head<128>::kBlock == RESQ_KV_BLOCK_BYTES, "block layout");
-// Head vectors of a call up to which one warp takes one of them.  Event times in us, one per warp / 16 per warp, 32 + 16
-// vectors per token: d = 128, 128 tokens 12.9 / 15.0, 256 tokens 16.8 / 16.8, 512 tokens 25.0 / 17.0; d = 64, 256 tokens
-// 10.9 / 12.7, 512 tokens 15.2 / 12.7.
-constexpr long long kFewVectors = 12288;
+// Head vectors of a call up to which one warp takes one of them.  Event times in us, one per warp / 16 per warp, 32 + 16 vectors per
+// token: d = 128, 100 tokens 7.9 / 9.0, 128 10.7 / 9.2, 256 15.0 / 10.1, but with cold caches, as in a step of a model, 128 tokens
+// 14.3 / 16.4, 192 16.4 / 16.4, 256 18.4 / 16.4: 9216 vectors.  d = 64: 80 tokens 5.2 / 5.4, 100
+// 5.7 / 5.4, 256 9.7 / 6.1; cold, 64 tokens 10.2 / 10.2, 128 12.3 / 10.2.
+template <int D>
+constexpr long long kFewVectors = D == 128 ? 9216 : 4096;
 constexpr float kMagic = 12582912.f;  // 1.5 * 2^23
+constexpr float kBracket = 9.5367431640625e-7f;  // 2^-20
+constexpr int kTileWarps = 8;            // of a kv_project_kernel CTA, two per SM
 
 // round-half-even(x / s) with the IEEE quotient's rounding: the product with inv = RN(1/s) lies within 2^-15
 // (|q| <= 127) / 2^-14 (|q| <= 255) of the quotient, so the two can only round apart when the product is that
@@ -58,21 +66,6 @@ __device__ __forceinline__ void mma_s8(int (&d)[4], const uint32_t (&a)[4], uint
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-// The lane's D / 4 elements of one row as fp32: v[8 ks + i] = x[32 ks + 4c + i], v[8 ks + 4 + i] = x[32 ks + 16 + 4c + i].
-template <int D>
-__device__ __forceinline__ void load_row(const __nv_bfloat16* row, int c, bool live, float (&v)[D / 4]) {
-#pragma unroll
-    for (int ks = 0; ks < D / 32; ++ks)
-#pragma unroll
-        for (int hf = 0; hf < 2; ++hf) {
-            uint2 u = make_uint2(0u, 0u);
-            if (live) u = *reinterpret_cast<const uint2*>(row + 32 * ks + 16 * hf + 4 * c);
-            float* o = v + 8 * ks + 4 * hf;
-            o[0] = __uint_as_float(u.x << 16); o[1] = __uint_as_float(u.x & 0xFFFF0000u);
-            o[2] = __uint_as_float(u.y << 16); o[3] = __uint_as_float(u.y & 0xFFFF0000u);
-        }
-}
-
 __device__ __forceinline__ float quad_max(float v) {
     v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 1));
     return fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 2));
@@ -90,7 +83,7 @@ struct Asym {
         z = lo;
         s = __fdiv_rn(__fsub_rn(hi, lo), qmax);
         inv = s > 0.f ? __frcp_rn(s) : 0.f;
-        exact = needs_division(inv);
+        exact = s > 0.f && needs_division(inv);
     }
     __device__ __forceinline__ uint32_t code(float x, float qmax) const {
         if (!(s > 0.f)) return 0u;
@@ -99,68 +92,18 @@ struct Asym {
     }
 };
 
-// Where the record of head vector `row` goes: (block index) * 32 + slot in the block, or -1.
-__device__ __forceinline__ long long cache_slot(long long row, int n_kv_heads, int n_seqs, int capacity,
-                                                const int32_t* seq_ids, const int32_t* positions, int* status) {
-    const long long t = row / n_kv_heads;
-    const int h = static_cast<int>(row - t * n_kv_heads);
+// Byte offset in the cache of the block that holds head h of token t, plus the token's slot in it (below 32; blocks are multiples
+// of 32 bytes), or -1.
+template <int D>
+__device__ __forceinline__ long long cache_slot(int t, int h, int n_kv_heads, int n_seqs, int capacity, const int32_t* seq_ids,
+                                                const int32_t* positions, int* status) {
     const int b = seq_ids[t], pos = positions[t];
     if (b < 0 || b >= n_seqs || pos < 0 || pos >= capacity) {
         atomicOr(status, kStatusBitIndex);
         return -1;
     }
     const long long blk = (static_cast<long long>(b) * n_kv_heads + h) * (capacity / RESQ_KV_BLOCK) + pos / RESQ_KV_BLOCK;
-    return blk * RESQ_KV_BLOCK + (pos % RESQ_KV_BLOCK);
-}
-
-// Copies the 16 staged records of a warp tile into the cache blocks (key: half 0, value: half 1).
-template <int D>
-__device__ __forceinline__ void flush_records(const uint8_t* rec, const long long* slot, uint8_t* cache, int half,
-                                              int lane) {
-    using H = Head<D>;
-    using Unit = typename std::conditional<D == 128, uint2, uint32_t>::type;  // what divides every part of a record
-    constexpr int kU = sizeof(Unit), kN8 = H::kR8 / kU, kN4 = H::kB4 / kU, kN = H::kRec / kU;
-    for (int u = lane; u < 16 * kN; u += 32) {
-        const int row = u / kN, part = u - row * kN;
-        const long long sl = slot[row];
-        if (sl < 0) continue;
-        uint8_t* blk = cache + (sl / RESQ_KV_BLOCK) * H::kBlock + half * H::kHalf;
-        const int p = static_cast<int>(sl % RESQ_KV_BLOCK);
-        uint8_t* dst = part < kN8         ? blk + p * H::kR8 + part * kU
-                       : part < kN8 + kN4 ? blk + H::kC8 + p * H::kB4 + (part - kN8) * kU
-                                          : blk + H::kC8 + H::kC4 + p * 16 + (part - kN8 - kN4) * kU;
-        *reinterpret_cast<Unit*>(dst) = *reinterpret_cast<const Unit*>(rec + row * H::kRec + part * kU);
-    }
-}
-
-// Symmetric INT8 codes of the lane's part of two rows, packed as the A fragments a[ks][0..3]; returns the scales.
-template <int D>
-__device__ __forceinline__ void sym8_fragments(const float (&xv)[2][D / 4], uint32_t (&a)[D / 32][4], float (&sx)[2]) {
-#pragma unroll
-    for (int rr = 0; rr < 2; ++rr) {
-        float m = 0.f;
-#pragma unroll
-        for (int i = 0; i < D / 4; ++i) m = fmaxf(m, fabsf(xv[rr][i]));
-        m = quad_max(m);
-        const float s = __fdiv_rn(m, 127.f);
-        const float inv = s > 0.f ? __frcp_rn(s) : 0.f;
-        const bool exact = needs_division(inv);
-        sx[rr] = s;
-#pragma unroll
-        for (int ks = 0; ks < D / 32; ++ks)
-#pragma unroll
-            for (int hf = 0; hf < 2; ++hf) {
-                uint32_t w = 0;
-                if (s > 0.f) {
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const float q = code_rn(xv[rr][8 * ks + 4 * hf + i], s, inv, exact, 0.5f - 0.000030517578125f);
-                        w |= (static_cast<uint32_t>(static_cast<int>(q)) & 0xFFu) << (8 * i);
-                    }
-                }
-                a[ks][2 * hf + rr] = w;  // a0: row g, k 4c..; a1: row g+8; a2: row g, k 16+4c..; a3: row g+8
-            }
-    }
+    return blk * Head<D>::kBlock + (pos % RESQ_KV_BLOCK);
 }
 
 struct ProjectParams {
@@ -178,21 +121,6 @@ struct ProjectParams {
     int* status;
 };
 
-// Ranges of the two segments of a row held by a quad: the lane's values 0 .. N8 - 1 are in the 8-bit segment where in8,
-// else in the 4-bit one with the rest.
-template <int N8, int N>
-__device__ __forceinline__ void quad_ranges(const float* v, bool in8, float (&lohi)[4]) {
-    float lo8 = 3.402823466e38f, hi8 = -3.402823466e38f, lo4 = lo8, hi4 = hi8;
-#pragma unroll
-    for (int i = N8; i < N; ++i) { lo4 = fminf(lo4, v[i]); hi4 = fmaxf(hi4, v[i]); }
-#pragma unroll
-    for (int i = 0; i < N8; ++i) {
-        if (in8) { lo8 = fminf(lo8, v[i]); hi8 = fmaxf(hi8, v[i]); }
-        else { lo4 = fminf(lo4, v[i]); hi4 = fmaxf(hi4, v[i]); }
-    }
-    lohi[0] = quad_min(lo8); lohi[1] = quad_max(hi8); lohi[2] = quad_min(lo4); lohi[3] = quad_max(hi4);
-}
-
 // W_C's codes and scales into shared memory.
 template <int D>
 __device__ __forceinline__ void stage_uc(const int8_t* wq, const float* s_u, uint8_t* w_s, float* su_s) {
@@ -203,132 +131,292 @@ __device__ __forceinline__ void stage_uc(const int8_t* wq, const float* s_u, uin
     for (int i = threadIdx.x; i < D; i += blockDim.x) su_s[i] = s_u[i];
 }
 
-// One warp per tile of 16 head vectors; the tiles of a call are the query tiles (projected, written as half),
-// then the key tiles (projected, quantized, appended), then the value tiles (quantized, appended).
+// Rounds N values x / s (after x - z) to codes 0 .. qmax or of either sign, t[i] = code + kMagic as bits: x v for the two factors
+// v = RN(inv (1 -+ 2^-20)) that bracket 1 / s, inv = RN(1 / s).  Where both products round to the same integer it is the rounded
+// IEEE quotient; else, or where one is NaN, the true divisions decide for all of the lane's values.
+template <int N>
+__device__ __forceinline__ void round_codes(const f2* d, float s, float inv, bool exact, float lo, float hi, uint32_t (&t)[N]) {
+    const float v_lo = fmaf(inv, -kBracket, inv), v_hi = fmaf(inv, kBracket, inv);
+    const f2 vl = pack2(v_lo, v_lo), vh = pack2(v_hi, v_hi), magic = pack2(kMagic, kMagic);
+    uint32_t differ = 0, seen = 0;
+#pragma unroll
+    for (int i = 0; i < N / 2; ++i) {
+        const float2 a = unpack2(fma2(d[i], vl, magic)), b = unpack2(fma2(d[i], vh, magic));
+        t[2 * i] = __float_as_uint(a.x);
+        t[2 * i + 1] = __float_as_uint(a.y);
+        differ |= t[2 * i] ^ __float_as_uint(b.x);
+        differ |= t[2 * i + 1] ^ __float_as_uint(b.y);
+        seen |= t[2 * i] | t[2 * i + 1];
+    }
+    if (exact || differ != 0 || (seen & 0x34000000u) != 0) {  // kMagic plus a code has none of these bits, NaN has
+#pragma unroll
+        for (int i = 0; i < N / 2; ++i) {
+            const float2 x = unpack2(d[i]);
+            const float qa = rintf(__fdiv_rn(x.x, s)), qb = rintf(__fdiv_rn(x.y, s));
+            t[2 * i] = __float_as_uint((qa == qa ? fminf(fmaxf(qa, lo), hi) : 0.f) + kMagic);  // NaN: 0
+            t[2 * i + 1] = __float_as_uint((qb == qb ? fminf(fmaxf(qb, lo), hi) : 0.f) + kMagic);
+        }
+    }
+}
+__device__ __forceinline__ uint32_t low_bytes(uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+    return __byte_perm(__byte_perm(a, b, 0x0040), __byte_perm(c, d, 0x0040), 0x5410);
+}
+
+// Staging of a warp's 16 records.
 template <int D>
-__global__ void __launch_bounds__(kWarps * 32) kv_project_kernel(const ProjectParams p) {
+struct Records {
+    alignas(16) uint8_t c8[16][Head<D>::kR8];
+    alignas(16) uint8_t c4[16][Head<D>::kB4];
+    float4 meta[16];
+    long long slot[16];
+};
+
+// The asymmetric 8/4-bit record of a row held by a quad, v[4 b + i]: columns 32 b + 8c + 2i and the next.
+template <int D>
+__device__ __forceinline__ void quantize_record(const f2 (&v)[D / 8], int c, Records<D>& rec, int row) {
+    const bool in8 = 8 * c < Head<D>::kR8;  // the lane's first eight values; the others are in the 4-bit segment for every lane
+    float hmin = 3.402823466e38f, hmax = -3.402823466e38f, lo4 = 3.402823466e38f, hi4 = -3.402823466e38f;
+#pragma unroll
+    for (int i = 0; i < D / 8; ++i) {
+        const float2 x = unpack2(v[i]);
+        float& lo = i < 4 ? hmin : lo4;
+        float& hi = i < 4 ? hmax : hi4;
+        lo = fminf(lo, fminf(x.x, x.y));
+        hi = fmaxf(hi, fmaxf(x.x, x.y));
+    }
+    const Asym q8(quad_min(in8 ? hmin : 3.402823466e38f), quad_max(in8 ? hmax : -3.402823466e38f), 255.f);
+    const Asym q4(quad_min(in8 ? lo4 : fminf(lo4, hmin)), quad_max(in8 ? hi4 : fmaxf(hi4, hmax)), 15.f);
+#pragma unroll
+    for (int b = 0; b < D / 32; ++b) {
+        const bool wide = b == 0 && in8;
+        const Asym& q = wide ? q8 : q4;
+        const f2 mz = pack2(-q.z, -q.z);
+        f2 d[4];
+        uint32_t t[8];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) d[i] = add2(v[4 * b + i], mz);
+        round_codes<8>(d, q.s, q.inv, q.exact, 0.f, wide ? 255.f : 15.f, t);
+        const uint32_t lo = q.s > 0.f ? low_bytes(t[0], t[1], t[2], t[3]) : 0u, hi = q.s > 0.f ? low_bytes(t[4], t[5], t[6], t[7]) : 0u;
+        if (wide) {
+            *reinterpret_cast<uint2*>(rec.c8[row] + 8 * c) = make_uint2(lo, hi);
+        } else {  // eight nibbles
+            const uint32_t x = lo & 0x0F0F0F0Fu, y = hi & 0x0F0F0F0Fu;
+            *reinterpret_cast<uint32_t*>(rec.c4[row] + 16 * b + 4 * c - Head<D>::kR8 / 2) = __byte_perm(x | (x >> 4), y | (y >> 4), 0x6420);
+        }
+    }
+    if (c == 0) rec.meta[row] = make_float4(q8.s, q8.z, q4.s, q4.z);
+}
+
+// Copies the 16 staged records into the cache (half 0: key, 1: value).
+template <int D>
+__device__ __forceinline__ void flush_records(const Records<D>& rec, uint8_t* cache, int half, int lane) {
     using H = Head<D>;
-    constexpr int KS = D / 32, NT = D / 8;
-    __shared__ __align__(16) uint8_t w_s[D * H::kWStride];
-    __shared__ float su_s[D];
-    __shared__ __align__(16) uint8_t rec_s[kWarps][16 * H::kRec];
-    __shared__ long long slot_s[kWarps][16];
+    using Byte8 = typename std::conditional<D == 128, uint4, uint2>::type;   // a record's 8-bit codes
+    using Unit = typename std::conditional<D == 128, uint2, uint32_t>::type;  // a seventh of its 4-bit codes
+    const int row = lane & 15;
+    const long long mine = rec.slot[row];
+    if (mine >= 0) {
+        uint8_t* blk = cache + (mine & ~31ll) + half * H::kHalf;
+        const int p = static_cast<int>(mine & 31);
+        if (lane < 16) *reinterpret_cast<Byte8*>(blk + p * H::kR8) = *reinterpret_cast<const Byte8*>(rec.c8[row]);
+        else *reinterpret_cast<float4*>(blk + H::kC8 + H::kC4 + p * 16) = rec.meta[row];
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int u = i * 32 + lane, r = u / 7, part = u - 7 * r;
+        if (u >= 112) break;
+        const long long sl = rec.slot[r];
+        if (sl < 0) continue;
+        uint8_t* dst = cache + (sl & ~31ll) + half * H::kHalf + H::kC8 + static_cast<int>(sl & 31) * H::kB4;
+        reinterpret_cast<Unit*>(dst)[part] = reinterpret_cast<const Unit*>(rec.c4[r])[part];
+    }
+}
+
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], uint32_t addr) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+
+// Tiles of 16 head vectors: the keys' (16 tokens of one head: projected, quantized, appended), the values' (quantized, appended), the
+// query's (16 rows: projected, written as half).  All warps go through them in this order, neighbours in different CTAs: longest first,
+// and at any time an SM's warps run one kind's code (2048 tokens of 32 + 16 vectors of 128: 27.8 us; queries before values 36.6).
+template <int D>
+__global__ void __launch_bounds__(kTileWarps * 32, 2) kv_project_kernel(const ProjectParams p) {
+    constexpr int KS = D / 32;  // k steps, blocks of 32 columns
+    __shared__ __align__(128) uint8_t w_s[D * D];  // chunk j of row n at chunk j ^ swizzle(n)
+    __shared__ __align__(16) float su_s[D];
+    __shared__ __align__(16) Records<D> rec_s[kTileWarps];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, c = lane & 3;
+    Records<D>& rec = rec_s[warp];
+    const int T = p.n_kv_heads ? static_cast<int>(p.kv_rows / p.n_kv_heads) : 0;
+    const long long kv_tiles = static_cast<long long>((T + 15) / 16) * p.n_kv_heads, q_tiles = (p.q_rows + 15) / 16;
+    const long long tiles = q_tiles + 2 * kv_tiles, stride = static_cast<long long>(gridDim.x) * kTileWarps;
+    // an ldmatrix reads rows 0 1 8 9 16 17 24 25 of 32 at once, or those plus 2, 4, 6
+    auto swizzle = [](int n) { return D == 128 ? (n & 1) | ((n >> 2) & 6) : (n >> 3) & 3; };
+
+    int kind = 0, t0 = 0, head = 0;  // 0 query, 1 key, 2 value; first token; head
+    const __nv_bfloat16* rows[2];
+    bool live[2];
+    uint4 raw[2][KS];
+    auto load = [&](long long tile) {
+        kind = tile < kv_tiles ? 1 : tile < 2 * kv_tiles ? 2 : 0;
+        if (kind == 0) {
+            const long long r0 = (tile - 2 * kv_tiles) * 16 + g;
+            t0 = static_cast<int>(tile - 2 * kv_tiles);
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                live[i] = r0 + 8 * i < p.q_rows;
+                rows[i] = p.q + (r0 + 8 * i) * D;
+            }
+        } else {
+            const unsigned kt = static_cast<unsigned>(kind == 1 ? tile : tile - kv_tiles);
+            t0 = static_cast<int>(kt / static_cast<unsigned>(p.n_kv_heads));
+            head = static_cast<int>(kt - static_cast<unsigned>(t0) * p.n_kv_heads);
+            t0 *= 16;
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const int t = t0 + g + 8 * i;
+                live[i] = t < T;
+                rows[i] = (kind == 1 ? p.k : p.v) + (static_cast<long long>(t) * p.n_kv_heads + head) * D;
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int b = 0; b < KS; ++b)
+                raw[i][b] = live[i] ? *reinterpret_cast<const uint4*>(rows[i] + 32 * b + 8 * c) : make_uint4(0u, 0u, 0u, 0u);
+    };
     griddep_wait();  // launched with programmatic stream serialization
     griddep_launch_dependents();
-    stage_uc<D>(p.wq, p.s_u, w_s, su_s);
+    long long tile = static_cast<long long>(warp) * gridDim.x + blockIdx.x;  // neighbours in different CTAs
+    if (tile < tiles) load(tile);  // on its way while U_C is staged
+    for (int i = threadIdx.x; i < D * (D / 16); i += kTileWarps * 32) {
+        // the reduction's order: of 32 bytes first the even words, then the odd ones
+        const int n = i / (D / 16), j = i % (D / 16);
+        const uint4* src = reinterpret_cast<const uint4*>(p.wq + n * D) + (j & ~1);
+        const uint4 x = src[0], y = src[1];
+        *reinterpret_cast<uint4*>(w_s + n * D + ((j ^ swizzle(n)) << 4)) = j & 1 ? make_uint4(x.y, x.w, y.y, y.w) : make_uint4(x.x, x.z, y.x, y.z);
+    }
+    for (int i = threadIdx.x; i < D; i += kTileWarps * 32) su_s[i] = p.s_u[i];
     __syncthreads();
+    const int w_row = 8 * ((lane & 7) >> 1) + (lane & 1) + 2 * (lane >> 4);  // of a block: the lane's ldmatrix row
+    uint32_t w_addr[2][KS];  // of block 0: products 0 and 1, or 2 and 3
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int ks = 0; ks < KS; ++ks)
+            w_addr[h][ks] = smem_u32(w_s) + (w_row + 4 * h) * D + (((2 * ks + ((lane >> 3) & 1)) ^ swizzle(w_row + 4 * h)) << 4);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, c = lane & 3;
-    const long long q_tiles = (p.q_rows + 15) / 16, kv_tiles = (p.kv_rows + 15) / 16, tiles = q_tiles + 2 * kv_tiles;
-    uint8_t* rec = rec_s[warp];
-    for (long long tile = static_cast<long long>(blockIdx.x) * kWarps + warp; tile < tiles;
-         tile += static_cast<long long>(gridDim.x) * kWarps) {
-        const int kind = tile < q_tiles ? 0 : (tile < q_tiles + kv_tiles ? 1 : 2);  // query, key, value
-        const long long t0 = kind == 0 ? tile : (kind == 1 ? tile - q_tiles : tile - q_tiles - kv_tiles);
-        const long long rows = kind == 0 ? p.q_rows : p.kv_rows;
-        const __nv_bfloat16* x = kind == 0 ? p.q : (kind == 1 ? p.k : p.v);
-        const long long r0 = t0 * 16 + g, r1 = r0 + 8;
-        const bool live0 = r0 < rows, live1 = r1 < rows;
-        float xv[2][D / 4];
-        load_row<D>(x + r0 * D, c, live0, xv[0]);
-        load_row<D>(x + r1 * D, c, live1, xv[1]);
-        if (kind != 0 && lane < 16) {
-            const long long r = t0 * 16 + lane;
-            slot_s[warp][lane] = r < rows ? cache_slot(r, p.n_kv_heads, p.n_seqs, p.capacity, p.seq_ids, p.positions, p.status) : -1;
+    while (tile < tiles) {
+        const int now = kind, tok = t0, h = head;
+        const bool ok0 = live[0], ok1 = live[1];
+        if (now != 0) {
+            if (lane < 16)
+                rec.slot[lane] = tok + lane < T ? cache_slot<D>(tok + lane, h, p.n_kv_heads, p.n_seqs, p.capacity, p.seq_ids, p.positions, p.status)
+                                                : -1;
         }
-        if (kind == 2) {
-            // ---- value: the bf16 head vectors quantized directly; elements 0-3 of the lane are columns
-            // [4c, 4c + 4): the 8-bit segment, of which D = 64 has only the quad's first two lanes
-            const bool in8 = 4 * c < H::kR8;
+        auto pairs_of = [](uint4 u, f2* x) {
+            const uint32_t w[4] = {u.x, u.y, u.z, u.w};
 #pragma unroll
-            for (int rr = 0; rr < 2; ++rr) {
-                float lohi[4];
-                quad_ranges<4, D / 4>(xv[rr], in8, lohi);
-                const Asym q8(lohi[0], lohi[1], 255.f), q4(lohi[2], lohi[3], 15.f);
-                uint8_t* rrow = rec + (g + 8 * rr) * H::kRec;
-                if (in8) {
-                    uint32_t w8 = 0;
+            for (int i = 0; i < 4; ++i) x[i] = pack2(__uint_as_float(w[i] << 16), __uint_as_float(w[i] & 0xFFFF0000u));
+        };
+        tile += stride;
+        if (now == 2) {
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) w8 |= q8.code(xv[rr][i], 255.f) << (8 * i);
-                    *reinterpret_cast<uint32_t*>(rrow + 4 * c) = w8;
-                }
+            for (int i = 0; i < 2; ++i) {
+                f2 x[D / 8];
 #pragma unroll
-                for (int ks = 0; ks < KS; ++ks)
-#pragma unroll
-                    for (int hf = 0; hf < 2; ++hf) {
-                        if (ks == 0 && hf == 0 && in8) continue;
-                        const float* e = xv[rr] + 8 * ks + 4 * hf;
-                        const int col = 32 * ks + 16 * hf + 4 * c;  // >= kR8
-                        *reinterpret_cast<uint16_t*>(rrow + H::kR8 + (col - H::kR8) / 2) = static_cast<uint16_t>(
-                            q4.code(e[0], 15.f) | (q4.code(e[1], 15.f) << 4) | (q4.code(e[2], 15.f) << 8) | (q4.code(e[3], 15.f) << 12));
-                    }
-                if (c == 0) {
-                    float* m = reinterpret_cast<float*>(rrow + H::kR8 + H::kB4);
-                    m[0] = q8.s; m[1] = q8.z; m[2] = q4.s; m[3] = q4.z;
-                }
+                for (int b = 0; b < KS; ++b) pairs_of(raw[i][b], x + 4 * b);
+                quantize_record<D>(x, c, rec, g + 8 * i);
             }
+            if (tile < tiles) load(tile);
             __syncwarp();
-            flush_records<D>(rec, slot_s[warp], p.cache, 1, lane);
+            flush_records<D>(rec, p.cache, 1, lane);
             __syncwarp();
             continue;
         }
-        float sx[2];
+        // ---- symmetric INT8 codes, packed as the A fragments: a[ks][0] row g, [1] row g + 8: the first four elements of eight;
+        // [2], [3]: the others
         uint32_t a[KS][4];
-        sym8_fragments<D>(xv, a, sx);
-        // ---- y = x W_C^T: column tiles of 8, exact int32
-        int acc[NT][4];
+        float sx[2];
 #pragma unroll
-        for (int nt = 0; nt < NT; ++nt) {
-            acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0;
-            const uint8_t* wrow = w_s + (8 * nt + g) * H::kWStride + 4 * c;
+        for (int i = 0; i < 2; ++i) {
+            f2 x[D / 8];
+            float m = 0.f;
+#pragma unroll
+            for (int b = 0; b < KS; ++b) pairs_of(raw[i][b], x + 4 * b);
+#pragma unroll
+            for (int j = 0; j < D / 8; ++j) {
+                const float2 u = unpack2(x[j]);
+                m = fmaxf(m, fmaxf(fabsf(u.x), fabsf(u.y)));
+            }
+            m = quad_max(m);
+            const float s = __fdiv_rn(m, 127.f), inv = s > 0.f ? __frcp_rn(s) : 0.f;
+            sx[i] = s;
+            const bool exact = s > 0.f && needs_division(inv);
+#pragma unroll
+            for (int b = 0; b < KS; b += 2) {
+                uint32_t t[16];
+                round_codes<16>(x + 4 * b, s, inv, exact, -128.f, 127.f, t);
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    a[b + (j >> 1)][2 * (j & 1) + i] = s > 0.f ? low_bytes(t[4 * j], t[4 * j + 1], t[4 * j + 2], t[4 * j + 3]) : 0u;
+            }
+        }
+        // ---- y = x W_C^T, a block of 32 columns at a time: the lane gets columns 32 b + 8c .. + 7 of rows g and g + 8
+        auto product = [&](int b, f2 (&y0)[4], f2 (&y1)[4]) {
+            const float4 u0 = *reinterpret_cast<const float4*>(su_s + 32 * b + 8 * c), u1 = *reinterpret_cast<const float4*>(su_s + 32 * b + 8 * c + 4);
+            const f2 u[4] = {pack2(u0.x, u0.y), pack2(u0.z, u0.w), pack2(u1.x, u1.y), pack2(u1.z, u1.w)};
+            const f2 s0 = pack2(sx[0], sx[0]), s1 = pack2(sx[1], sx[1]);
+            int acc[4][4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0;
 #pragma unroll
             for (int ks = 0; ks < KS; ++ks)
-                mma_s8(acc[nt], a[ks], *reinterpret_cast<const uint32_t*>(wrow + 32 * ks),
-                       *reinterpret_cast<const uint32_t*>(wrow + 32 * ks + 16));
-        }
-        // y[row g][8 nt + 2c + e] = acc[nt][e], y[row g + 8][...] = acc[nt][2 + e]
-        if (kind == 0) {
 #pragma unroll
-            for (int nt = 0; nt < NT; ++nt) {
-                const float u0 = su_s[8 * nt + 2 * c], u1 = su_s[8 * nt + 2 * c + 1];
-                if (live0)
-                    *reinterpret_cast<__half2*>(p.q_out + r0 * D + 8 * nt + 2 * c) = __floats2half2_rn(
-                        __fmul_rn(static_cast<float>(acc[nt][0]), __fmul_rn(sx[0], u0)),
-                        __fmul_rn(static_cast<float>(acc[nt][1]), __fmul_rn(sx[0], u1)));
-                if (live1)
-                    *reinterpret_cast<__half2*>(p.q_out + r1 * D + 8 * nt + 2 * c) = __floats2half2_rn(
-                        __fmul_rn(static_cast<float>(acc[nt][2]), __fmul_rn(sx[1], u0)),
-                        __fmul_rn(static_cast<float>(acc[nt][3]), __fmul_rn(sx[1], u1)));
+                for (int h = 0; h < 2; ++h) {
+                    uint32_t w[4];
+                    ldsm4(w, w_addr[h][ks] + b * 32 * D);
+                    mma_s8(acc[2 * h], a[ks], w[0], w[1]);
+                    mma_s8(acc[2 * h + 1], a[ks], w[2], w[3]);
+                }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                y0[j] = mul2(pack2(static_cast<float>(acc[j][0]), static_cast<float>(acc[j][1])), mul2(s0, u[j]));
+                y1[j] = mul2(pack2(static_cast<float>(acc[j][2]), static_cast<float>(acc[j][3])), mul2(s1, u[j]));
+            }
+        };
+        if (now == 0) {
+            if (tile < tiles) load(tile);
+            __half* dst = p.q_out + (static_cast<long long>(tok) * 16 + g) * D + 8 * c;
+#pragma unroll 1  // the code of a kind stays small
+            for (int b = 0; b < KS; ++b) {
+                f2 y[2][4];
+                product(b, y[0], y[1]);
+#pragma unroll
+                for (int i = 0; i < 2; ++i)
+                    if (i == 0 ? ok0 : ok1)
+                        *reinterpret_cast<uint4*>(dst + 8 * i * D + 32 * b) =
+                            make_uint4(half_pair(y[i][0]), half_pair(y[i][1]), half_pair(y[i][2]), half_pair(y[i][3]));
             }
             continue;
         }
-        // ---- key: asymmetric 8/4-bit codes of the fp32 coefficients (the first D / 64 column tiles are the 8-bit segment)
+        f2 y[2][D / 8];
 #pragma unroll
-        for (int rr = 0; rr < 2; ++rr) {
-            float y[D / 4];  // y[2 nt + e]
+        for (int b = 0; b < KS; ++b) {
+            f2 y0[4], y1[4];
+            product(b, y0, y1);
 #pragma unroll
-            for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-                for (int e = 0; e < 2; ++e)
-                    y[2 * nt + e] = __fmul_rn(static_cast<float>(acc[nt][2 * rr + e]), __fmul_rn(sx[rr], su_s[8 * nt + 2 * c + e]));
-            float lohi[4];
-            quad_ranges<2 * (D / 64), D / 4>(y, true, lohi);
-            const Asym q8(lohi[0], lohi[1], 255.f), q4(lohi[2], lohi[3], 15.f);
-            uint8_t* rrow = rec + (g + 8 * rr) * H::kRec;
-#pragma unroll
-            for (int nt = 0; nt < D / 64; ++nt)
-                *reinterpret_cast<uint16_t*>(rrow + 8 * nt + 2 * c) =
-                    static_cast<uint16_t>(q8.code(y[2 * nt], 255.f) | (q8.code(y[2 * nt + 1], 255.f) << 8));
-#pragma unroll
-            for (int nt = D / 64; nt < NT; ++nt)
-                rrow[H::kR8 + 4 * (nt - D / 64) + c] = static_cast<uint8_t>(q4.code(y[2 * nt], 15.f) | (q4.code(y[2 * nt + 1], 15.f) << 4));
-            if (c == 0) {
-                float* m = reinterpret_cast<float*>(rrow + H::kR8 + H::kB4);
-                m[0] = q8.s; m[1] = q8.z; m[2] = q4.s; m[3] = q4.z;
+            for (int j = 0; j < 4; ++j) {
+                y[0][4 * b + j] = y0[j];
+                y[1][4 * b + j] = y1[j];
             }
         }
+        quantize_record<D>(y[0], c, rec, g);
+        quantize_record<D>(y[1], c, rec, g + 8);
+        if (tile < tiles) load(tile);
         __syncwarp();
-        flush_records<D>(rec, slot_s[warp], p.cache, 0, lane);
+        flush_records<D>(rec, p.cache, 0, lane);
         __syncwarp();
     }
 }
@@ -344,7 +432,7 @@ __device__ __forceinline__ float warp_min(float v) {
     return v;
 }
 
-// One warp per head vector, lane l owning coefficients l + 32 i; items in the order of kv_project_kernel.
+// One warp per head vector, lane l owning coefficients l + 32 i; items: queries, keys, values.
 template <int D>
 __global__ void __launch_bounds__(kWarps * 32) head_vector_kernel(const ProjectParams p) {
     using H = Head<D>;
@@ -378,7 +466,11 @@ __global__ void __launch_bounds__(kWarps * 32) head_vector_kernel(const ProjectP
     for (; item < total; item += step) {
         long long slot = -1;
         if (kind != 0) {
-            if (lane == 0) slot = cache_slot(row, p.n_kv_heads, p.n_seqs, p.capacity, p.seq_ids, p.positions, p.status);
+            if (lane == 0) {
+                const unsigned t = static_cast<unsigned>(row) / static_cast<unsigned>(p.n_kv_heads);
+                slot = cache_slot<D>(static_cast<int>(t), static_cast<int>(row - static_cast<long long>(t) * p.n_kv_heads), p.n_kv_heads, p.n_seqs,
+                                     p.capacity, p.seq_ids, p.positions, p.status);
+            }
             slot = __shfl_sync(0xffffffffu, slot, 0);
         }
         float y[N];
@@ -422,8 +514,8 @@ __global__ void __launch_bounds__(kWarps * 32) head_vector_kernel(const ProjectP
             for (int i = 1; i < N; ++i) { lo4 = fminf(lo4, y[i]); hi4 = fmaxf(hi4, y[i]); }
             const Asym q8(warp_min(in8 ? y[0] : INFINITY), warp_max(in8 ? y[0] : -INFINITY), 255.f);
             const Asym q4(warp_min(lo4), warp_max(hi4), 15.f);
-            uint8_t* half = p.cache + (slot / RESQ_KV_BLOCK) * H::kBlock + (kind == 2 ? H::kHalf : 0);
-            const int ps = static_cast<int>(slot % RESQ_KV_BLOCK);
+            uint8_t* half = p.cache + (slot & ~31ll) + (kind == 2 ? H::kHalf : 0);
+            const int ps = static_cast<int>(slot & 31);
             uint8_t* c4 = half + H::kC8 + ps * H::kB4;
 #pragma unroll
             for (int i = 0; i < N; ++i) {  // a 4-bit coefficient j is nibble j - kR8; kR8 is even, so pairs start at even lanes
@@ -465,13 +557,13 @@ cudaError_t launch_project(const ProjectParams& p, cudaStream_t st) {
     const long long vectors = p.q_rows + 2 * p.kv_rows;
     if (vectors == 0) return cudaSuccess;
     count_launch();
-    const auto grid = [](long long warps) {
-        const long long ctas = (warps + kWarps - 1) / kWarps;
-        return static_cast<unsigned>(ctas < 148 * 8 ? ctas : 148 * 8);
-    };
-    if (vectors <= kFewVectors)
-        return launch_programmatic(head_vector_kernel<D>, grid(vectors), kWarps * 32, 0, st, p);
-    return launch_programmatic(kv_project_kernel<D>, grid((p.q_rows + 15) / 16 + 2 * ((p.kv_rows + 15) / 16)), kWarps * 32, 0, st, p);
+    if (vectors <= kFewVectors<D>) {
+        const long long ctas = (vectors + kWarps - 1) / kWarps;
+        return launch_programmatic(head_vector_kernel<D>, ctas < 148 * 8 ? ctas : 148 * 8, kWarps * 32, 0, st, p);
+    }
+    const long long T = p.n_kv_heads ? p.kv_rows / p.n_kv_heads : 0;
+    const long long tiles = (p.q_rows + 15) / 16 + 2 * ((T + 15) / 16) * p.n_kv_heads, ctas = (tiles + kTileWarps - 1) / kTileWarps;
+    return launch_programmatic(kv_project_kernel<D>, ctas < 148 * 2 ? ctas : 148 * 2, kTileWarps * 32, 0, st, p);
 }
 
 }  // namespace

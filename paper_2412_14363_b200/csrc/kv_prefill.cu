@@ -42,6 +42,7 @@
 // tokens 49 -> 36; d = 64, 1000 tokens 60 -> 38 (mma.sync tiles of 64 rows), 2048 behind 4096 828 -> 509.
 #include "centred_codes.cuh"
 #include "internal.h"
+#include "packed_fp32.cuh"
 #include "plans.h"
 #include "ptx.cuh"
 
@@ -129,33 +130,6 @@ __host__ __device__ constexpr uint32_t make_idesc_f16(int M, int N) {  // f16 x 
 }
 constexpr uint32_t kBNMajor = 1u << 16;
 
-// Packed fp32 pairs.
-using f2 = unsigned long long;
-__device__ __forceinline__ f2 pack2(float lo, float hi) {
-    f2 d;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
-    return d;
-}
-__device__ __forceinline__ float2 unpack2(f2 v) {
-    float2 d;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(d.x), "=f"(d.y) : "l"(v));
-    return d;
-}
-__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
-    f2 d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ f2 mul2(f2 a, f2 b) {
-    f2 d;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ f2 add2(f2 a, f2 b) {
-    f2 d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
 // Two pairs from shared memory, where the program has it (hoisted reads would not fit the registers).
 struct f2x2 {
     f2 x, y;
@@ -184,12 +158,6 @@ __device__ __forceinline__ void sts128(uint32_t addr, uint4 v) {
     asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
 __device__ __forceinline__ void sts_f(uint32_t addr, float v) { asm volatile("st.shared.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory"); }
-__device__ __forceinline__ uint32_t half_pair(f2 v) {
-    const float2 f = unpack2(v);
-    const __half2 h = __floats2half2_rn(f.x, f.y);
-    return *reinterpret_cast<const uint32_t*>(&h);
-}
-
 // Two floats as three pairs of bf16 that add up to all of their 24 bits: each part is what the ones before leave, rounded.
 __device__ __forceinline__ uint32_t bf16_pair(f2 v) {
     const float2 f = unpack2(v);
