@@ -199,30 +199,38 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? 3 : 1) attention64_kernel(c
         __syncwarp();  // the step's bytes are in place and nobody reads the previous tiles
         const uint8_t* rb = raw + buf * kBlock;
         const int j0 = s * kStep;
-        // ---- expand: chunks of eight coefficients, 0-7 of the keys then of the values; lane = position
+        // ---- expand: chunks of eight coefficients, lane = position.  Every word is read before the first chunk is written: one by one
+        // they would each wait for shared memory (16 rows of 2048 positions, 8 KV heads, with the append: 21.7 -> 19.7 us).
+        {
+            uint32_t w4[2][7];
+            uint2 w8[2];
+            float4 m[2];
 #pragma unroll
-        for (int ch = 0; ch < 16; ++ch) {
-            const uint8_t* half_base = rb + (ch >= 8 ? kHalf : 0);
-            const int j = ch & 7;
-            uint4 v;
-            if (j == 0) {
-                const uint2 w = *reinterpret_cast<const uint2*>(half_base + lane * R8);
-                v = ch >= 8 ? bytes_centred_bf16(w) : bytes_centred(w);
-            } else {
-                const uint32_t w = *reinterpret_cast<const uint32_t*>(half_base + kC8 + lane * (N4 / 2) + 4 * (j - 1));
-                v = ch >= 8 ? nibbles_centred_bf16(w) : nibbles_centred(w);
+            for (int is_v = 0; is_v < 2; ++is_v) {
+                const uint8_t* half_base = rb + is_v * kHalf;
+                w8[is_v] = *reinterpret_cast<const uint2*>(half_base + lane * R8);
+#pragma unroll
+                for (int j = 0; j < 7; ++j) w4[is_v][j] = *reinterpret_cast<const uint32_t*>(half_base + kC8 + lane * (N4 / 2) + 4 * j);
+                m[is_v] = *reinterpret_cast<const float4*>(half_base + kC8 + kC4 + lane * 16);
             }
-            *reinterpret_cast<uint4*>((ch >= 8 ? Vt : Kt) + lane * kPitch + j * 16) = v;
-        }
-        // ---- per-position constants; positions past the row's last hold anything and are zeroed by selection
+            uint4* krow = reinterpret_cast<uint4*>(Kt + lane * kPitch);
+            uint4* vrow = reinterpret_cast<uint4*>(Vt + lane * kPitch);
+            krow[0] = bytes_centred(w8[0]);
+            vrow[0] = bytes_centred_bf16(w8[1]);
 #pragma unroll
-        for (int is_v = 0; is_v < 2; ++is_v) {
-            float4 m = *reinterpret_cast<const float4*>(rb + (is_v ? kHalf : 0) + kC8 + kC4 + lane * 16);
-            if (j0 + lane >= limit) m = make_float4(0.f, 0.f, 0.f, 0.f);
-            m.y = fmaf(128.f, m.x, m.y);
-            m.w = fmaf(8.f, m.z, m.w);
-            if (is_v) colV[lane] = m;
-            else colK[lane] = make_float4(m.x * kScore, m.y * kScore, m.z * kScore, m.w * kScore);
+            for (int j = 0; j < 7; ++j) {
+                krow[1 + j] = nibbles_centred(w4[0][j]);
+                vrow[1 + j] = nibbles_centred_bf16(w4[1][j]);
+            }
+            // per-position constants; positions past the row's last hold anything and are zeroed by selection
+#pragma unroll
+            for (int is_v = 0; is_v < 2; ++is_v) {
+                if (j0 + lane >= limit) m[is_v] = make_float4(0.f, 0.f, 0.f, 0.f);
+                m[is_v].y = fmaf(128.f, m[is_v].x, m[is_v].y);
+                m[is_v].w = fmaf(8.f, m[is_v].z, m[is_v].w);
+            }
+            colK[lane] = make_float4(m[0].x * kScore, m[0].y * kScore, m[0].z * kScore, m[0].w * kScore);
+            colV[lane] = m[1];
         }
         __syncwarp();
         issue(s + 2 * stride, buf);  // everybody is done with this raw buffer
