@@ -9,6 +9,7 @@
 #include <cuda_fp16.h>
 
 #include "internal.h"
+#include "packed_fp32.cuh"
 #include "ptx.cuh"
 
 namespace resq {
@@ -209,12 +210,16 @@ __device__ __forceinline__ Chunk<F32> lds_chunk(const uint8_t* row, int c) {
 template <bool F32>
 __device__ __forceinline__ void fast_codes(const Chunk<F32>& ch, float s, float inv, bool exact_only, uint32_t (&t)[8]) {
     const float v_lo = fmaf(inv, -kBracket, inv), v_hi = fmaf(inv, kBracket, inv);
+    const f2 vl = pack2(v_lo, v_lo), vh = pack2(v_hi, v_hi), magic = pack2(kMagic, kMagic);
     uint32_t differ = 0;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const float x = ch.get(i);
-        t[i] = __float_as_uint(fmaf(x, v_lo, kMagic));
-        differ |= t[i] ^ __float_as_uint(fmaf(x, v_hi, kMagic));
+    for (int i = 0; i < 8; i += 2) {
+        const f2 x = pack2(ch.get(i), ch.get(i + 1));
+        const float2 a = unpack2(fma2(x, vl, magic)), b = unpack2(fma2(x, vh, magic));
+        t[i] = __float_as_uint(a.x);
+        t[i + 1] = __float_as_uint(a.y);
+        differ |= t[i] ^ __float_as_uint(b.x);
+        differ |= t[i + 1] ^ __float_as_uint(b.y);
     }
     if (exact_only || differ != 0) {
 #pragma unroll
@@ -229,13 +234,19 @@ template <bool F32>
 __device__ __forceinline__ void fast_codes_asym(const Chunk<F32>& ch, float z, float s, float inv, bool exact_only, float qmax,
                                                 uint32_t (&t)[8]) {
     const float v_lo = fmaf(inv, -kBracket, inv), v_hi = fmaf(inv, kBracket, inv);
+    const f2 vl = pack2(v_lo, v_lo), vh = pack2(v_hi, v_hi), magic = pack2(kMagic, kMagic), mz = pack2(-z, -z);
     uint32_t differ = 0;
     float d[8];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        d[i] = __fsub_rn(ch.get(i), z);
-        t[i] = __float_as_uint(fmaf(d[i], v_lo, kMagic));
-        differ |= t[i] ^ __float_as_uint(fmaf(d[i], v_hi, kMagic));
+    for (int i = 0; i < 8; i += 2) {
+        const f2 x = add2(pack2(ch.get(i), ch.get(i + 1)), mz);
+        const float2 u = unpack2(x), a = unpack2(fma2(x, vl, magic)), b = unpack2(fma2(x, vh, magic));
+        d[i] = u.x;
+        d[i + 1] = u.y;
+        t[i] = __float_as_uint(a.x);
+        t[i + 1] = __float_as_uint(a.y);
+        differ |= t[i] ^ __float_as_uint(b.x);
+        differ |= t[i + 1] ^ __float_as_uint(b.y);
     }
     if (exact_only || differ != 0) {
 #pragma unroll
@@ -503,6 +514,9 @@ __global__ void unpack_int4_kernel(const uint8_t* __restrict__ packed, int8_t* _
 // Sylvester butterflies up to five index bits per pass (32 values in registers),
 // scaled, and then quantized exactly as in the fast path above (absmax per segment, reciprocal-product
 // rounding with the exact fallback).  r = 0 gives the paper's uniform INT4 down_proj input.
+// What bounds it: instructions.  So the factor's p and m halves, neighbouring coefficients of a butterfly and of the code
+// rounding go two to an instruction, and through shared memory 8 bytes at a time: 1537 rows of 14336 45.2 -> 37.6 us, 4096
+// 114 -> 96 (the row quantizers above, which share the rounding: 4096 x 4096 24.5 -> 23.7).
 // Paley's second construction for a prime q = 1 (mod 4): H = S (x) [[1,1],[1,-1]] + I (x) [[1,-1],[-1,-1]] of order
 // 2 (q + 1), with S = [[0, 1^T], [1, chi(i - j)]] and chi the quadratic character of GF(q).  S is evaluated at compile
 // time, so the product with H is additions and subtractions only: with p_i = x_2i + x_2i+1 and m_i = x_2i - x_2i+1,
@@ -569,10 +583,60 @@ __device__ __forceinline__ void butterfly_pass(float* hrow, int K, int s, int ti
     }
 }
 
+// The same for M even, a thread taking coefficients b and b + 1 of its 2^NB groups as pairs: half the instructions.
+template <int M, int NT, int NB>
+__device__ __forceinline__ void butterfly_pairs(float* hrow, int K, int s, int tid, bool last, float inv_sqrt_k, int r, float& a8,
+                                                float& a4) {
+    constexpr int N = 1 << NB;
+    const int count = K >> (NB + 1);
+    const int stride = M << s;
+    for (int i = tid; i < count; i += NT) {
+        const int arest = i / (M / 2), b = 2 * (i - arest * (M / 2));
+        const int a0 = ((arest >> s) << (s + NB)) | (arest & ((1 << s) - 1));
+        f2* base = reinterpret_cast<f2*>(hrow + a0 * M + b);
+        f2 v[N];
+#pragma unroll
+        for (int j = 0; j < N; ++j) v[j] = base[j * (stride / 2)];
+#pragma unroll
+        for (int bit = 0; bit < NB; ++bit) {
+#pragma unroll
+            for (int j = 0; j < N; ++j) {
+                if (!(j & (1 << bit))) {
+                    const f2 lo = v[j], hi = v[j | (1 << bit)];
+                    v[j] = add2(lo, hi);
+                    v[j | (1 << bit)] = sub2(lo, hi);
+                }
+            }
+        }
+        if (last) {
+            const f2 scale = pack2(inv_sqrt_k, inv_sqrt_k);
+            const int e0 = a0 * M + b;  // r is a multiple of 8: a pair is in one segment
+#pragma unroll
+            for (int j = 0; j < N; ++j) v[j] = mul2(v[j], scale);
+            if (e0 >= r) {
+#pragma unroll
+                for (int j = 0; j < N; ++j) {
+                    const float2 x = unpack2(v[j]);
+                    a4 = fmaxf(a4, fmaxf(fabsf(x.x), fabsf(x.y)));
+                }
+            } else {
+#pragma unroll
+                for (int j = 0; j < N; ++j) {
+                    const float2 x = unpack2(v[j]);
+                    float& m = e0 + j * stride < r ? a8 : a4;
+                    m = fmaxf(m, fmaxf(fabsf(x.x), fabsf(x.y)));
+                }
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < N; ++j) base[j * (stride / 2)] = v[j];
+    }
+}
+
 // NT threads per row: 256 when rows outnumber the SMs (throughput: several CTAs per SM), 1024 for the few rows of a
 // generation step, where one row's chain of passes is all there is to wait for.
 template <int M, int NT>
-__global__ void __launch_bounds__(NT)
+__global__ void __launch_bounds__(NT, NT == kThreads ? (M > 1 ? 3 : 4) : 1)
 hadamard_quantize_kernel(const __nv_bfloat16* X, size_t rows, int K, int kbits, int r, float inv_sqrt_k,
                          int8_t* __restrict__ q8, uint8_t* __restrict__ q4, float* __restrict__ s8_out,
                          float* __restrict__ s4_out, int8_t* __restrict__ q4e) {
@@ -608,40 +672,46 @@ hadamard_quantize_kernel(const __nv_bfloat16* X, size_t rows, int K, int kbits, 
                 // M * 4 bytes is a multiple of 16: the group moves as float4s (conflict-free at this stride)
                 float4* gp = reinterpret_cast<float4*>(hrow + a * M);
                 const uint2* xg = reinterpret_cast<const uint2*>(X + row * static_cast<size_t>(K) + static_cast<size_t>(a) * M);
-                float x[M], y[M], ps[H2], ms[H2];
+                float y[M];
+                f2 pm[H2];  // (x_2i + x_2i+1, x_2i - x_2i+1)
 #pragma unroll
                 for (int i = 0; i < M / 4; ++i) {
                     const uint2 u = xg[i];
-                    x[4 * i] = __uint_as_float(u.x << 16); x[4 * i + 1] = __uint_as_float(u.x & 0xFFFF0000u);
-                    x[4 * i + 2] = __uint_as_float(u.y << 16); x[4 * i + 3] = __uint_as_float(u.y & 0xFFFF0000u);
-                }
 #pragma unroll
-                for (int i = 0; i < H2; ++i) {
-                    ps[i] = x[2 * i] + x[2 * i + 1];
-                    ms[i] = x[2 * i] - x[2 * i + 1];
+                    for (int h = 0; h < 2; ++h) {
+                        const uint32_t w = h ? u.y : u.x;
+                        const float lo = __uint_as_float(w << 16), hi = __uint_as_float(w & 0xFFFF0000u);
+                        pm[2 * i + h] = add2(pack2(lo, lo), pack2(hi, -hi));
+                    }
                 }
                 // S = [[0, 1^T], [1, Q]] with Q_ij = chi(i - j) circulant of order q = M / 2 - 1.  With t = sum of the
                 // q inner entries and R_j = sum over the quadratic residues k of entry (j + k) mod q, the non-residues
-                // sum to t - entry_j - R_j, so (Q v)_j = 2 R_j - t + v_j: (q - 1) / 2 + 2 operations instead of q - 1.
+                // sum to t - entry_j - R_j, so (Q v)_j = 2 R_j - t + v_j: (q - 1) / 2 + 2 operations instead of q - 1, on the
+                // p and m halves in one instruction.
                 constexpr int Q = H2 - 1;
-                float tp = ps[1], tm = ms[1];
+                const f2 two = pack2(2.f, 2.f);
+                f2 t = pm[1];
 #pragma unroll
-                for (int i = 2; i < H2; ++i) { tp += ps[i]; tm += ms[i]; }
-                y[0] = ms[0] + tp;
-                y[1] = tm - ps[0];
+                for (int i = 2; i < H2; ++i) t = add2(t, pm[i]);
+                const float2 first = unpack2(pm[0]), tt = unpack2(t);
+                y[0] = first.y + tt.x;
+                y[1] = tt.y - first.x;
 #pragma unroll
                 for (int jp = 0; jp < Q; ++jp) {
-                    float rp = 0.f, rm = 0.f;
+                    f2 res = 0ull;
+                    bool any = false;
 #pragma unroll
                     for (int k = 1; k < Q; ++k) {
                         if (conf.s[1 + k][1] > 0) {  // chi(k) = +1
-                            rp += ps[1 + (jp + k) % Q];
-                            rm += ms[1 + (jp + k) % Q];
+                            res = any ? add2(res, pm[1 + (jp + k) % Q]) : pm[1 + (jp + k) % Q];
+                            any = true;
                         }
                     }
-                    const float qp = fmaf(2.f, rp, ps[jp + 1] - tp), qm = fmaf(2.f, rm, ms[jp + 1] - tm);
-                    y[2 * (jp + 1)] = (ms[jp + 1] + ps[0]) + qp;
-                    y[2 * (jp + 1) + 1] = (ms[0] - ps[jp + 1]) + qm;
+                    const float2 own = unpack2(pm[jp + 1]);
+                    const f2 q = fma2(two, res, sub2(pm[jp + 1], t));
+                    const float2 o = unpack2(add2(add2(pack2(own.y, -own.x), pack2(first.x, first.y)), q));
+                    y[2 * (jp + 1)] = o.x;
+                    y[2 * (jp + 1) + 1] = o.y;
                 }
 #pragma unroll
                 for (int i = 0; i < M / 4; ++i) gp[i] = make_float4(y[4 * i], y[4 * i + 1], y[4 * i + 2], y[4 * i + 3]);
@@ -657,7 +727,13 @@ hadamard_quantize_kernel(const __nv_bfloat16* X, size_t rows, int K, int kbits, 
             const int left = kbits - s;
             const int nb = left <= kMaxBits ? left : (left <= 2 * kMaxBits ? (left + 1) / 2 : kMaxBits);
             const bool last = s + nb >= kbits;
-            if (nb == 1) butterfly_pass<M, NT, 1>(hrow, K, s, tid, last, inv_sqrt_k, r, a8, a4);
+            if constexpr (M > 1 && NT == kThreads) {  // 1024 threads have no registers for 32 pairs; M = 1 has odd neighbours in the first pass
+                if (nb == 1) butterfly_pairs<M, NT, 1>(hrow, K, s, tid, last, inv_sqrt_k, r, a8, a4);
+                else if (nb == 2) butterfly_pairs<M, NT, 2>(hrow, K, s, tid, last, inv_sqrt_k, r, a8, a4);
+                else if (nb == 3) butterfly_pairs<M, NT, 3>(hrow, K, s, tid, last, inv_sqrt_k, r, a8, a4);
+                else if (nb == 4) butterfly_pairs<M, NT, 4>(hrow, K, s, tid, last, inv_sqrt_k, r, a8, a4);
+                else butterfly_pairs<M, NT, 5>(hrow, K, s, tid, last, inv_sqrt_k, r, a8, a4);
+            } else if (nb == 1) butterfly_pass<M, NT, 1>(hrow, K, s, tid, last, inv_sqrt_k, r, a8, a4);
             else if (nb == 2) butterfly_pass<M, NT, 2>(hrow, K, s, tid, last, inv_sqrt_k, r, a8, a4);
             else if (nb == 3) butterfly_pass<M, NT, 3>(hrow, K, s, tid, last, inv_sqrt_k, r, a8, a4);
             else if constexpr (kMaxBits > 3) {
@@ -722,10 +798,8 @@ hadamard_quantize_kernel(const __nv_bfloat16* X, size_t rows, int K, int kbits, 
                 const int jj = (c - rchunks) * 8;
                 if (q4e_row) *reinterpret_cast<uint2*>(q4e_row + jj) = make_uint2(w0, w1);
                 if (q4row) {
-                    uint32_t packed = 0;
-#pragma unroll
-                    for (int k = 0; k < 8; ++k) packed |= (t[k] & 0xFu) << (4 * k);
-                    *reinterpret_cast<uint32_t*>(q4row + (jj >> 1)) = packed;
+                    const uint32_t x = w0 & 0x0F0F0F0Fu, y = w1 & 0x0F0F0F0Fu;
+                    *reinterpret_cast<uint32_t*>(q4row + (jj >> 1)) = __byte_perm(x | (x >> 4), y | (y >> 4), 0x6420);
                 }
             }
         }
