@@ -47,8 +47,8 @@
  * on the host before anything is enqueued.  d_head must be 128 or 64; capacity % 32 == 0;
  * n_q_heads / n_kv_heads must be an integer between 1 and 8.  d_head = 128 runs on mma.sync
  * fragments for the projection and the single-query pass and on tcgen05 tiles for the prefill form; d_head = 64 runs the
- * same arithmetic and cache format, attention on mma.sync tiles whose softmax weights keep all of fp32's bits (as three
- * bf16 parts) instead of being rounded to half. Indices that live on the device (seq_ids,
+ * same forms on the same cache format, with softmax weights that keep all of fp32's bits (as three bf16 parts) instead of
+ * being rounded to half. Indices that live on the device (seq_ids,
  * positions, seq_lens) are checked by the kernels: an out-of-range entry is skipped (a sequence length is
  * clamped to the capacity) and RESQ_ERR_INDEX is reported by resq_device_status.
  */

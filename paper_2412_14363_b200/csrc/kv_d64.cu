@@ -45,8 +45,8 @@ constexpr int kC8 = 32 * R8, kC4 = 32 * (N4 / 2), kHalf = kC8 + kC4 + 512, kBloc
 // pair); the query fragments are gathered in that order and the outputs put back.
 //
 // What bounds it: the latency of a step and the operand conversions on the CUDA cores; not HBM, not the tensor pipe.
-// 32 query / 8 KV heads, project-and-append included: a step of 16 sequences of 1024-2048 positions 507 -> 21.7 us (20.6 with two
-// halves per weight), against one warp per (row, query head) that dequantized each position per head.
+// 32 query / 8 KV heads, project-and-append included: a step of 16 sequences of 1024-2048 positions 507 -> 19.7 us (21.7 while the words
+// of a step were read and expanded one by one), against one warp per (row, query head) that dequantized each position per head.
 struct Attn64Params {
     const uint8_t* cache;
     const __half* q;   // [rows][Hq][64]
