@@ -636,7 +636,7 @@ __device__ __forceinline__ void butterfly_pairs(float* hrow, int K, int s, int t
 // NT threads per row: 256 when rows outnumber the SMs (throughput: several CTAs per SM), 1024 for the few rows of a
 // generation step, where one row's chain of passes is all there is to wait for.
 template <int M, int NT>
-__global__ void __launch_bounds__(NT, NT == kThreads ? (M > 1 ? 3 : 4) : 1)
+__global__ void __launch_bounds__(NT, NT == kThreads ? (M > 1 ? 3 : 5) : 1)
 hadamard_quantize_kernel(const __nv_bfloat16* X, size_t rows, int K, int kbits, int r, float inv_sqrt_k,
                          int8_t* __restrict__ q8, uint8_t* __restrict__ q4, float* __restrict__ s8_out,
                          float* __restrict__ s4_out, int8_t* __restrict__ q4e) {
