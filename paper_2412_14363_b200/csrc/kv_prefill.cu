@@ -700,7 +700,7 @@ __global__ void __launch_bounds__(Geometry<D, WAYS, PAIR>::kThreads, 1) attentio
             // ---- out = (O 2^E + zero-point sums) / sum of p; the row's outputs leave in the coefficients' own order
             const float2 l2 = unpack2(st.l), z8p = unpack2(st.z8), z4p = unpack2(st.z4);
             row_part[part][row] = make_float4(l2.x + l2.y, z8p.x + z8p.y, z4p.x + z4p.y, 0.f);
-            (void)group_any<32 * WAYS>(group, false);
+            if (group_any<32 * WAYS>(group, !ok)) ok = false;  // the warps of these rows leave together: they would meet at the next tile's barrier
             float l = 0.f, z8 = 0.f, z4 = 0.f;
 #pragma unroll
             for (int i = 0; i < WAYS; ++i) {

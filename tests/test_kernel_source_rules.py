@@ -84,3 +84,15 @@ def test_tensor_memory_is_reached_by_whole_warps(name):
             assert "__syncwarp();" in body[:m.start() - at], (name, text[m.start():m.start() + 60])
     for m in re.finditer(r"if \(!mbar_wait\(&sh->acc_full", text):
         raise AssertionError((name, text[m.start():m.start() + 80]))
+
+
+def test_warps_that_meet_at_a_barrier_leave_together():
+    """The softmax warps that share rows of the prefill kernel meet at a named barrier, which has no time limit.  A wait that runs out in
+    one of them is voted on at every such barrier and the outcome acted on, so that none goes on to a barrier where the others
+    will not come."""
+    text = _code("kv_prefill.cu")
+    kernel = next(body for head, body in _kernels(text) if "attention_prefill_kernel" in head)
+    votes = re.findall(r"([^;{}]*)\bgroup_any<32 \* WAYS>\(group, ([^;]*)", kernel)
+    assert len(votes) == 3
+    for before, predicate in votes:
+        assert "!ok" in predicate and "(void)" not in before and re.search(r"\bif \($|= $", before), (before, predicate)
