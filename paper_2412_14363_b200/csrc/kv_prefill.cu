@@ -58,6 +58,7 @@ constexpr int kRows = 128;          // rows of a tile = TMEM lanes
 constexpr int kStep = 64;           // cache positions per step
 constexpr int kStages = 3;          // expanded steps
 constexpr int kExpandWarps = 3;
+constexpr uint32_t kTmemCols = 512, kColS4 = 64;  // the 4-bit segment's scores behind the 8-bit one's
 constexpr float kSlack = 8.f;       // log2 of how far a score may rise above a row's first maximum before its reference is raised
 
 // What depends on the head width.  Operand tiles have rows of 128 bytes (64 coefficients of 16 bits).
@@ -77,7 +78,6 @@ struct Head {
     static constexpr int kRecPitch = D + 4;                                 // floats per row of a record: sums, reference, sum of weights
 };
 static_assert(Head<128>::kBlockBytes == RESQ_KV_BLOCK_BYTES && Head<128>::kOffVm == 5120, "block layout");
-constexpr uint32_t kTmemCols = 512, kColS4 = 64;  // the 4-bit segment's scores behind the 8-bit one's
 
 struct Shared {
     // per stage and pair of positions: keys (s8 s8 s4 s4) (z8 z8 z4 z4) times log2(e) / sqrt(d), the zero-points with the
@@ -94,7 +94,7 @@ struct Shared {
 };
 
 // WAYS: threads of a row, each with that share of a step's positions and of the output.  PAIR: two tiles in flight with one score
-// buffer each; otherwise one with two.
+// buffer each; otherwise two steps of one.
 template <int D, int WAYS, bool PAIR>
 struct Geometry {
     static constexpr int kGroupWarps = 4 * WAYS;  // of a tile
@@ -108,11 +108,10 @@ struct Geometry {
     static constexpr size_t kSmem = 1024 + kTiles + kOutStage + 2 * Head<D>::kRawBytes + sizeof(Shared);
     static_assert(kSmem <= 227 * 1024 && kMmaWarp < 20 && (!PAIR || WAYS == 2), "one CTA per SM");
     static_assert(kTiles >= static_cast<size_t>(kRows) * Head<D>::kRecPitch * 4, "records fit");
-    // TMEM: per score buffer 8-bit and 4-bit segment, the weights over them, then the output products: one per buffer, but for a single
-    // tile at D = 128, whose output is behind both
-    static constexpr uint32_t kBufCols = PAIR ? 256 : D == 128 ? 128 : 192;
-    static constexpr bool kOneOutput = !PAIR && D == 128;
-    static constexpr uint32_t kColOut = kOneOutput ? 256 : 128;
+    // TMEM: score buffers (8-bit and 4-bit segment, the weights over them; PAIR: one per tile, else one per stage), then the outputs:
+    // PAIR: one per tile; D = 128: one, which the tensor core adds up; D = 64: two, by turns
+    static constexpr uint32_t kBufCols = 128, kColOut = (PAIR ? 2 : kStages) * kBufCols, kOutPitch = PAIR ? 128 : D == 128 ? 0 : 64;
+    static_assert(kColOut + kOutPitch + D <= kTmemCols, "TMEM");
 };
 
 struct PrefillParams {
@@ -576,11 +575,11 @@ __global__ void __launch_bounds__(Geometry<D, WAYS, PAIR>::kThreads, 1) attentio
     int stage = 0, stage_parity = 0;  // of the role's next step
     if (softmax) {
         const uint32_t tmem_row = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16);
-        auto buffer = [&](int N) { return PAIR ? buf0 : N & 1; };  // of step N, and the parity of its barriers
+        auto buffer = [&](int N) { return PAIR ? buf0 : N & 1; };  // whose barriers (and output) step N uses, and their parity
         auto parity = [&](int N) { return PAIR ? N & 1 : N >> 1 & 1; };
-        auto out_columns = [&](int N) { return tmem_row + G::kColOut + part * G::kOutCols + (G::kOneOutput ? 0 : buffer(N) * G::kBufCols); };
+        auto out_columns = [&](int N) { return tmem_row + G::kColOut + part * G::kOutCols + buffer(N) * G::kOutPitch; };
         constexpr int kLag = PAIR ? 1 : 2;               // steps after which an output product is complete without a wait
-        constexpr bool kLastOnly = PAIR && D == 128;     // only the last one is told of: the next scores' product follows it
+        constexpr bool kLastOnly = PAIR && D == 128;     // only the last one is waited for: the next scores are behind the others
         const uint32_t cols_k = smem_u32(sh->col_k) + part * (G::kPart * 16), cols_v = smem_u32(sh->col_v) + part * (G::kPart * 16);
         for (int ti = 0, done = 0; ti < tiles && ok; ++ti) {  // done: steps of the tiles before
             const Tile tile = tile_of(ti);
@@ -593,9 +592,10 @@ __global__ void __launch_bounds__(Geometry<D, WAYS, PAIR>::kThreads, 1) attentio
 #pragma unroll
                 for (int i = 0; i < G::kOutCols / 2; ++i) O[i] = 0ull;
             }
-            // Waits for the output product of the CTA's step N, counted over its tiles; but for kLastOnly every one of a buffer's in turn.
+            // Waits for the output product of the CTA's step N, counted over its tiles; of those that are not behind the scores seen last
+            // every one of a buffer's in turn.
             auto output_ready = [&](int N) {
-                ok = mbar_wait(&sh->pv_done[buffer(N)], kLastOnly ? 0 : parity(N), &sh->abort_flag, p.status);
+                ok = mbar_wait(&sh->pv_done[buffer(N)], parity(N), &sh->abort_flag, p.status);
                 ok = !__any_sync(0xffffffffu, !ok);
                 tc_fence_after();
                 return ok;
@@ -617,7 +617,7 @@ __global__ void __launch_bounds__(Geometry<D, WAYS, PAIR>::kThreads, 1) attentio
                 const int N = done + n;
                 const int j0 = (tile.first + n) * kStep + part * G::kPart;
                 const uint32_t col_k = cols_k + stage * (kStep * 16), col_v = cols_v + stage * (kStep * 16);
-                const uint32_t tmem_s = tmem_row + buffer(N) * G::kBufCols;
+                const uint32_t tmem_s = tmem_row + (PAIR ? buf0 : stage) * G::kBufCols;
                 f2 sc[G::kPairs];
                 const float m_use = st.m == -INFINITY ? 0.f : st.m;
                 float mx = -INFINITY;
@@ -690,7 +690,7 @@ __global__ void __launch_bounds__(Geometry<D, WAYS, PAIR>::kThreads, 1) attentio
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&sh->p_full[buffer(N)]);
             }
-            for (int n = max(n_steps - 2, 0); n < n_steps && ok; ++n)
+            for (int n = max(n_steps - (kLastOnly ? 1 : 2), 0); n < n_steps && ok; ++n)
                 if (output_ready(done + n) && !(added && n == n_steps - 2)) add_output(done + n);
             // a row that sees a value whose constants are not finite gets NaN in that segment
             if (pos_i >= sh->bad8) st.z8 = pack2(NAN, NAN);
@@ -812,7 +812,7 @@ __global__ void __launch_bounds__(Geometry<D, WAYS, PAIR>::kThreads, 1) attentio
             tc_fence_after();
             return ok;
         };
-        auto score_product = [&](int q_tile, int buf, int st) {
+        auto score_product = [&](int q_tile, int buf, int st, int bar) {
             const uint32_t idS = make_idesc_f16(kRows, kStep);
             const uint32_t q = smem_u32(Qs) + q_tile * H::kQBytes, k = smem_u32(stages) + st * H::kStageBytes;
             const uint64_t q0 = make_smem_desc_k128(q), k0 = make_smem_desc_k128(k), k1 = make_smem_desc_k128(k + H::kTile);
@@ -829,13 +829,13 @@ __global__ void __launch_bounds__(Geometry<D, WAYS, PAIR>::kThreads, 1) attentio
 #pragma unroll
                 for (int i = 0; i < 4; ++i) mma_f16_ss_if(leader, d + kColS4, q0 + 2 * i, k0 + 2 * i, idS, i > 0);
             }
-            tc_commit_if(leader, &sh->s_full[buf]);
+            tc_commit_if(leader, &sh->s_full[bar]);
         };
-        auto output_product = [&](int buf, bool fresh, int st) {
+        auto output_product = [&](int buf, int out, bool fresh, int st) {
             const uint32_t v = smem_u32(stages) + st * H::kStageBytes + H::kOffStageV4;
             const uint64_t v4 = make_smem_desc_mn128(v, H::kTile);
             const uint32_t w = tmem + buf * G::kBufCols;  // the weights
-            const uint32_t d = (G::kOneOutput ? tmem : w) + G::kColOut;
+            const uint32_t d = tmem + G::kColOut + out * G::kOutPitch;
             if constexpr (D == 128) {
                 const uint64_t v8 = make_smem_desc_mn128(v + H::kOffStageV8 - H::kOffStageV4, H::kTile);
                 const uint32_t id8 = make_idesc_f16(kRows, 16) | kBNMajor, id4 = make_idesc_f16(kRows, 112) | kBNMajor;
@@ -865,22 +865,26 @@ __global__ void __launch_bounds__(Geometry<D, WAYS, PAIR>::kThreads, 1) attentio
                 stage_parity ^= 1;
             }
         };
+        // Scores go over the weights of an earlier output product, which has to be complete: two products are ordered by their issue only
+        // if they share accumulator and shape.  PAIR: a wait (2 % of a long walk).  Otherwise a stage has its score buffer, and its keys
+        // are in place only after the output product of the step that had the stage before has freed it.
         int out_stage = 0;
         if constexpr (PAIR) {
             if (total_steps > 0 && keys_ready()) {
-                for (int t = 0; t < 2; ++t) score_product(t, t, stage);
+                for (int t = 0; t < 2; ++t) score_product(t, t, stage, t);
                 next_stage();
             }
             for (int n = 0; n < total_steps && ok; ++n) {
 #pragma unroll
                 for (int t = 0; t < 2; ++t) {
                     if (!wait(&sh->p_full[t], n & 1)) break;
-                    output_product(t, n == 0, out_stage);
-                    if (D == 64 || n == total_steps - 1) tc_commit_if(leader, &sh->pv_done[t]);
+                    output_product(t, t, n == 0, out_stage);
+                    tc_commit_if(leader, &sh->pv_done[t]);
                     if (t == 1) tc_commit_if(leader, &sh->kv_empty[out_stage]);
-                    if (n + 1 < total_steps) {  // over the weights: products execute in the order of their issue
+                    if (n + 1 < total_steps) {
                         if (t == 0 && !keys_ready()) break;
-                        score_product(t, t, stage);
+                        if (!wait(&sh->pv_done[t], n & 1)) break;
+                        score_product(t, t, stage, t);
                     }
                 }
                 if (++out_stage == kStages) out_stage = 0;
@@ -889,17 +893,17 @@ __global__ void __launch_bounds__(Geometry<D, WAYS, PAIR>::kThreads, 1) attentio
         } else {
             auto scores = [&](int N) {
                 if (!keys_ready()) return;
-                score_product(N >= tile0.n_steps, N & 1, stage);
+                score_product(N >= tile0.n_steps, stage, stage, N & 1);
                 next_stage();
             };
             for (int N = 0; N < min(2, total_steps) && ok; ++N) scores(N);
             for (int N = 0; N < total_steps && ok; ++N) {
                 if (!wait(&sh->p_full[N & 1], (N >> 1) & 1)) break;
-                output_product(N & 1, N == 0 || N == tile0.n_steps, out_stage);
+                output_product(out_stage, N & 1, N == 0 || N == tile0.n_steps, out_stage);
                 tc_commit_if(leader, &sh->pv_done[N & 1]);
                 tc_commit_if(leader, &sh->kv_empty[out_stage]);
                 if (++out_stage == kStages) out_stage = 0;
-                if (N + 2 < total_steps) scores(N + 2);  // over the weights: products execute in the order of their issue
+                if (N + 2 < total_steps) scores(N + 2);
             }
         }
         if (!ok) {  // products in flight finish before TMEM and shared memory are given back (bounded)

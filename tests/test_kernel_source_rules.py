@@ -96,3 +96,22 @@ def test_warps_that_meet_at_a_barrier_leave_together():
     assert len(votes) == 3
     for before, predicate in votes:
         assert "!ok" in predicate and "(void)" not in before and re.search(r"\bif \($|= $", before), (before, predicate)
+
+
+def test_scores_go_over_weights_only_behind_the_product_that_reads_them():
+    """The weights of an output product lie in TMEM where later scores go.  Products are ordered by their issue only if they share
+    accumulator and shape, which these two do not.  So the scores are issued behind a wait for the other's completion, or
+    into the buffer of their stage, whose keys are awaited: expansion fills a stage only after the product that read it has freed it."""
+    text = _code("kv_prefill.cu")
+    kernel = next(body for head, body in _kernels(text) if "attention_prefill_kernel" in head)
+    pair_at = kernel.index("if constexpr (PAIR)", kernel.index("int out_stage"))
+    pair = _block(kernel, pair_at)
+    one = _block(kernel, kernel.index("else", pair_at + len(pair)))
+    loop = _block(pair, pair.index("for (int n = 0"))
+    between = loop[loop.index("output_product("):loop.index("score_product(")]
+    assert between.index("tc_commit_if(leader, &sh->pv_done[t])") < between.index("wait(&sh->pv_done[t], n & 1)"), between
+    scores = _block(one, one.index("auto scores"))
+    assert scores.index("!keys_ready()) return;") < scores.index("score_product(") and "stage, stage, N & 1)" in scores
+    assert "output_product(out_stage, N & 1," in one and "tc_commit_if(leader, &sh->kv_empty[out_stage])" in one
+    expand = kernel[kernel.index("for (; N < total_steps; ++N)"):kernel.index("expand_step<D>")]
+    assert "mbar_wait(&sh->kv_empty[stage]" in expand
