@@ -171,11 +171,12 @@ struct Records {
     long long slot[16];
 };
 
-// The asymmetric 8/4-bit record of a row held by a quad, v[4 b + i]: columns 32 b + 8c + 2i and the next.
+// The asymmetric 8/4-bit record of a row held by a quad, v[4 b + i]: columns 32 b + 8c + 2i and the next.  Values that are
+// all NaN (a key with an infinity has them) leave z = inf and s = -inf, as in head_vector_kernel.
 template <int D>
 __device__ __forceinline__ void quantize_record(const f2 (&v)[D / 8], int c, Records<D>& rec, int row) {
     const bool in8 = 8 * c < Head<D>::kR8;  // the lane's first eight values; the others are in the 4-bit segment for every lane
-    float hmin = 3.402823466e38f, hmax = -3.402823466e38f, lo4 = 3.402823466e38f, hi4 = -3.402823466e38f;
+    float hmin = INFINITY, hmax = -INFINITY, lo4 = INFINITY, hi4 = -INFINITY;
 #pragma unroll
     for (int i = 0; i < D / 8; ++i) {
         const float2 x = unpack2(v[i]);
@@ -184,7 +185,7 @@ __device__ __forceinline__ void quantize_record(const f2 (&v)[D / 8], int c, Rec
         lo = fminf(lo, fminf(x.x, x.y));
         hi = fmaxf(hi, fmaxf(x.x, x.y));
     }
-    const Asym q8(quad_min(in8 ? hmin : 3.402823466e38f), quad_max(in8 ? hmax : -3.402823466e38f), 255.f);
+    const Asym q8(quad_min(in8 ? hmin : INFINITY), quad_max(in8 ? hmax : -INFINITY), 255.f);
     const Asym q4(quad_min(in8 ? lo4 : fminf(lo4, hmin)), quad_max(in8 ? hi4 : fmaxf(hi4, hmax)), 15.f);
 #pragma unroll
     for (int b = 0; b < D / 32; ++b) {

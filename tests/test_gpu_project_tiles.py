@@ -30,9 +30,13 @@ def test_tiles_write_what_single_vectors_write(d, T, Hq, Hkv, part):
     for i, n in enumerate(part):
         x = synth.head_vectors(T, Hq if n == "q" else Hkv, d, stream=900 + i, lead=4.0, scale=0.7)
         x[T - 1, -1] = 0.0
-        if n == "q":
-            x[17, 0, 3] = np.inf
-            x[18, 0, d - 1] = np.nan
+        x[17, 0, 3] = np.inf                 # a key: every projected value is NaN
+        x[18, 0, d - 1] = np.nan
+        x[21, 0, d // 8:] = np.inf           # a value: the whole 4-bit segment, the 8-bit one below
+        x[22, 0, :d // 8] = -np.inf
+        x[23, 0] = np.nan
+        x[24, 0, ::2] = np.inf
+        x[24, 0, 1::2] = -np.inf
         x[19, 0] *= 1e-36
         x[20, 0] *= 1e36
         heads[n] = bf16_to_dev(synth.f32_to_bf16_bits(x))
