@@ -19,8 +19,10 @@
 // all R rows through the chain at once, four lanes per row, and hands the group's errors on through named barriers.
 // An updated block comes back in the slots its errors will take.
 // K = N = 4096: 65.1 ms right-looking, 11.5 ms left-looking with all warps waiting for the chain (two CTAs per
-// SM), 7.2 ms with a rounding warp per row, 6.2 ms as it stands (3.7 ms if the fp64 pipe were always busy; the
-// updates alone take 71 cycles per column and seven rows where the pipe needs 56: broadcasts of e, U from L2).
+// SM), 7.2 ms with a rounding warp per row, 6.2 ms as it stands (3.7 ms if the fp64 pipe were always busy).  U comes from DRAM where it
+// does not stay in L2 (the first call on it, K above 4096), later than the loads a thread has on their way: with few rows
+// the updating warps ask L2 for it 256 rows ahead.  K = 4096, 592 rows, caches cold: 2.06 ms without, 1.16 with; K = 8192, 1184 rows: 18.9, 10.3; but
+// K = N = 4096 (seven rows per CTA) 6.2, 6.4.
 #include <cuda_fp16.h>
 
 #include "internal.h"
@@ -34,6 +36,8 @@ constexpr int kWarps = kThreads / 32;
 constexpr int kAhead = 32;        // columns of U a thread requests ahead of their use (L2 latency)
 constexpr int kCtaThreads = 2 * kThreads;  // eight updating, eight rounding warps
 static_assert(kGptqMaxRows * 4 <= 32, "four lanes per row");
+constexpr int kFar = 256;         // rows of U a warp asks L2 for ahead of their use (DRAM latency; a multiple of 32)
+constexpr int kAskRows = 5;       // up to as many rows (K above 4800 has no more): with six and seven the updates take longer than DRAM does
 constexpr int kPf = 4;            // steps by which a rounding warp requests U ahead
 constexpr int kHandOver = 9, kInBlock = 10;  // named barriers behind those of the groups (1-8): a block, its groups by turns
 constexpr size_t kRowLimit = 200 * 1024;   // accepted rows: 9 bytes per weight within this (the documented bound)
@@ -167,6 +171,7 @@ __device__ __forceinline__ void feed_back(double (&acc)[R], const float (&u)[n],
     }
 }
 
+__device__ __forceinline__ void prefetch_l2(const float* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 __device__ __forceinline__ void named_sync(int id, int threads) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
@@ -245,11 +250,22 @@ __global__ void __launch_bounds__(kCtaThreads, 1) gptq_rows_kernel(const Params 
                 if (live && p.dead && p.dead[col]) w = 0.f;
                 acc[rr] = static_cast<double>(w);
             }
+            // Lane i asks L2 for the warp's 128 bytes of row kFar + i, then 32 rows on.  CTAs share this out: an eighth of the grid asks for a row.
+            const unsigned share = gridDim.x >= 64 ? 7u : 0u;
+            const float* ask = U + static_cast<size_t>(kFar + lane) * K + min(c0 + 32 * warp, K - 1);
+            int ask_row = kFar + lane;
+            auto request_rows = [&] {
+                if constexpr (R > kAskRows) return;
+                if ((((ask_row >> 5) + blockIdx.x) & share) == 0 && ask_row < K) prefetch_l2(ask);
+                ask_row += 32;
+                ask += static_cast<size_t>(32) * K;
+            };
             const int known = max(c0 - kThreads, 0);  // columns rounded for certain: all blocks but the previous one
             float u_next[kAhead];
 #pragma unroll
             for (int i = 0; i < kAhead; ++i) u_next[i] = ucol[static_cast<size_t>(i) * K];
             for (int j = 0; j < known; j += kAhead) {
+                request_rows();
                 float u[kAhead];
 #pragma unroll
                 for (int i = 0; i < kAhead; ++i) u[i] = u_next[i];
@@ -261,6 +277,7 @@ __global__ void __launch_bounds__(kCtaThreads, 1) gptq_rows_kernel(const Params 
             if (c0 > 0) {
                 for (int g = 0; g < kWarps; ++g) {  // the previous block, group by group as it is rounded
                     const int j0 = known + 32 * g;
+                    request_rows();  // the diagonal block's
                     float u[32];
 #pragma unroll
                     for (int i = 0; i < 32; ++i) u[i] = ucol[static_cast<size_t>(j0 + i) * K];
