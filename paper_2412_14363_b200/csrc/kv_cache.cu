@@ -22,6 +22,7 @@
 
 #include "internal.h"
 #include "packed_fp32.cuh"
+#include "plans.h"
 #include "ptx.cuh"
 #include "../../include/resq_kv.h"
 
@@ -119,6 +120,7 @@ struct ProjectParams {
     const int32_t* seq_ids;
     const int32_t* positions;
     int* status;
+    bool together;  // append_tiles_together
 };
 
 // W_C's codes and scales into shared memory.
@@ -239,8 +241,10 @@ __device__ __forceinline__ void ldsm4(uint32_t (&r)[4], uint32_t addr) {
 }
 
 // Tiles of 16 head vectors: the keys' (16 tokens of one head: projected, quantized, appended), the values' (quantized, appended), the
-// query's (16 rows: projected, written as half).  All warps go through them in this order, neighbours in different CTAs: longest first,
-// and at any time an SM's warps run one kind's code (2048 tokens of 32 + 16 vectors of 128: 27.8 us; queries before values 36.6).
+// query's (16 rows: projected, written as half).  All warps go through them in this order: longest first, and at any time an SM's
+// warps run one kind's code (2048 tokens of 32 + 16 vectors of 128: 27.8 us; queries before values 36.6).  Neighbours are in
+// different CTAs, or (append_tiles_together) in the warps of one, which start each round together; a last round that is
+// not full is spread over the CTAs either way.
 template <int D>
 __global__ void __launch_bounds__(kTileWarps * 32, 2) kv_project_kernel(const ProjectParams p) {
     constexpr int KS = D / 32;  // k steps, blocks of 32 columns
@@ -250,8 +254,8 @@ __global__ void __launch_bounds__(kTileWarps * 32, 2) kv_project_kernel(const Pr
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, c = lane & 3;
     Records<D>& rec = rec_s[warp];
     const int T = p.n_kv_heads ? static_cast<int>(p.kv_rows / p.n_kv_heads) : 0;
-    const long long kv_tiles = static_cast<long long>((T + 15) / 16) * p.n_kv_heads, q_tiles = (p.q_rows + 15) / 16;
-    const long long tiles = q_tiles + 2 * kv_tiles, stride = static_cast<long long>(gridDim.x) * kTileWarps;
+    const int kv_tiles = (T + 15) / 16 * p.n_kv_heads, q_tiles = static_cast<int>((p.q_rows + 15) / 16);
+    const int tiles = q_tiles + 2 * kv_tiles, stride = static_cast<int>(gridDim.x) * kTileWarps;  // 2^31 tiles would be terabytes
     // an ldmatrix reads rows 0 1 8 9 16 17 24 25 of 32 at once, or those plus 2, 4, 6
     auto swizzle = [](int n) { return D == 128 ? (n & 1) | ((n >> 2) & 6) : (n >> 3) & 3; };
 
@@ -259,11 +263,11 @@ __global__ void __launch_bounds__(kTileWarps * 32, 2) kv_project_kernel(const Pr
     const __nv_bfloat16* rows[2];
     bool live[2];
     uint4 raw[2][KS];
-    auto load = [&](long long tile) {
+    auto load = [&](int tile) {
         kind = tile < kv_tiles ? 1 : tile < 2 * kv_tiles ? 2 : 0;
         if (kind == 0) {
-            const long long r0 = (tile - 2 * kv_tiles) * 16 + g;
-            t0 = static_cast<int>(tile - 2 * kv_tiles);
+            const long long r0 = static_cast<long long>(tile - 2 * kv_tiles) * 16 + g;
+            t0 = tile - 2 * kv_tiles;
 #pragma unroll
             for (int i = 0; i < 2; ++i) {
                 live[i] = r0 + 8 * i < p.q_rows;
@@ -289,7 +293,9 @@ __global__ void __launch_bounds__(kTileWarps * 32, 2) kv_project_kernel(const Pr
     };
     griddep_wait();  // launched with programmatic stream serialization
     griddep_launch_dependents();
-    long long tile = static_cast<long long>(warp) * gridDim.x + blockIdx.x;  // neighbours in different CTAs
+    const int apart = warp * static_cast<int>(gridDim.x) + static_cast<int>(blockIdx.x);
+    const int full = p.together ? tiles / stride * stride : 0;  // the rounds in which every warp has a tile
+    int tile = p.together ? static_cast<int>(blockIdx.x) * kTileWarps + warp : apart;
     if (tile < tiles) load(tile);  // on its way while U_C is staged
     for (int i = threadIdx.x; i < D * (D / 16); i += kTileWarps * 32) {
         // the reduction's order: of 32 bytes first the even words, then the odd ones
@@ -309,6 +315,7 @@ __global__ void __launch_bounds__(kTileWarps * 32, 2) kv_project_kernel(const Pr
             w_addr[h][ks] = smem_u32(w_s) + (w_row + 4 * h) * D + (((2 * ks + ((lane >> 3) & 1)) ^ swizzle(w_row + 4 * h)) << 4);
 
     while (tile < tiles) {
+        if (tile < full) __syncthreads();  // together: all of the CTA's warps are in the round
         const int now = kind, tok = t0, h = head;
         const bool ok0 = live[0], ok1 = live[1];
         if (now != 0) {
@@ -321,7 +328,7 @@ __global__ void __launch_bounds__(kTileWarps * 32, 2) kv_project_kernel(const Pr
 #pragma unroll
             for (int i = 0; i < 4; ++i) x[i] = pack2(__uint_as_float(w[i] << 16), __uint_as_float(w[i] & 0xFFFF0000u));
         };
-        tile += stride;
+        tile = tile < full && tile + stride >= full ? full + apart : tile + stride;
         if (now == 2) {
 #pragma unroll
             for (int i = 0; i < 2; ++i) {
@@ -563,8 +570,12 @@ cudaError_t launch_project(const ProjectParams& p, cudaStream_t st) {
         return launch_programmatic(head_vector_kernel<D>, ctas < 148 * 8 ? ctas : 148 * 8, kWarps * 32, 0, st, p);
     }
     const long long T = p.n_kv_heads ? p.kv_rows / p.n_kv_heads : 0;
-    const long long tiles = (p.q_rows + 15) / 16 + 2 * ((T + 15) / 16) * p.n_kv_heads, ctas = (tiles + kTileWarps - 1) / kTileWarps;
-    return launch_programmatic(kv_project_kernel<D>, ctas < 148 * 2 ? ctas : 148 * 2, kTileWarps * 32, 0, st, p);
+    const long long kv_tiles = 2 * ((T + 15) / 16) * p.n_kv_heads, tiles = (p.q_rows + 15) / 16 + kv_tiles;
+    const long long ctas = (tiles + kTileWarps - 1) / kTileWarps;
+    ProjectParams tp = p;
+    tp.together = append_tiles_together(D, kv_tiles, tiles);
+    static_assert(kTileWarps * 148 * 2 == kAppendWarps, "a round");
+    return launch_programmatic(kv_project_kernel<D>, ctas < 148 * 2 ? ctas : 148 * 2, kTileWarps * 32, 0, st, tp);
 }
 
 }  // namespace

@@ -60,6 +60,17 @@ inline int gptq_rows_per_cta(int N, int K) {
     return (N + 148 * rounds - 1) / (148 * rounds);
 }
 
+// ---- query projection and cache append (kv_cache.cu), tiles of 16 head vectors: whether the warps of a CTA go through tiles together
+constexpr long long kAppendWarps = 148 * 2 * 8;  // of the grid: tiles of a round
+// Each kind of tile is tens of KB of straight code, and an SM whose warps are at different places of it waits for instructions.  As
+// long as each kind is within a round the warps keep pace by themselves.  us, d = 128, 16 heads each, apart / together: 2600 tokens (2.2
+// rounds of keys and values) 57.6 / 34.5, 3000 75 / 41 and without a query 46 / 31 (four of five cycles of a warp's wait);
+// 32 / 8 heads, 2600 tokens (1.1) 36.3 / 32.4, 2048 (0.9) 27.2 / 29.0.  One round of keys and values and no second one beside: 1500
+// tokens of 16 heads (1.3 + 0.6) 24.7 / 29.0.  d = 64, half the code: 2600 tokens of 16 heads 23.8 / 17.7, 2300 (1.95) 15.4 / 15.8.
+inline bool append_tiles_together(int d, long long kv_tiles, long long tiles) {
+    return kv_tiles > (d == 128 ? 1 : 2) * kAppendWarps && tiles >= 2 * kAppendWarps;
+}
+
 // ---- causal run (kv_prefill.cu): tiles of 128 rows per CTA, CTAs of a cluster that split the steps of 64 positions
 struct PrefillPlan {
     int tiles_per_cta, splits;

@@ -6,6 +6,7 @@ import pytest
 import torch
 
 import synth
+from tests import plans
 from tests.gpu_util import bf16_to_dev, dev, host
 
 pytestmark = pytest.mark.gpu
@@ -20,10 +21,14 @@ pytestmark = pytest.mark.gpu
     (1231, 0, 5, "kv"),       # keys and values alone
     (9217, 1, 0, "q"),        # one vector more than the other form takes at 128
     (4097, 1, 0, "q"),        # and at 64
+    (2400, 16, 16, "qkv"),    # a CTA's warps go through tiles together: three rounds and a few
+    (2007, 13, 19, "qkv"),    # two and most of a third, of queries and the last values
+    (2200, 0, 18, "kv"),      # two and a few of the last values
 ])
 def test_tiles_write_what_single_vectors_write(d, T, Hq, Hkv, part):
     import paper_2412_14363_b200 as resq
     from paper_2412_14363_b200 import kv
+    assert plans.append_together(d, T, Hq, Hkv) == (T >= 2000 and Hkv > 1)
     wq, s_u = kv.resq_uc_quantize(dev(np.ascontiguousarray(synth.haar_orthogonal(d).T.astype(np.float32))))
     seq_ids, positions = dev((np.arange(T) % 3).astype(np.int32)), dev((np.arange(T) // 3).astype(np.int32))
     heads = {}
