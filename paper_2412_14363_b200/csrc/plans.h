@@ -78,15 +78,31 @@ struct PrefillPlan {
     long long row_groups;  // groups of tiles_per_cta tiles; the grid is row_groups * Hkv * splits
 };
 
-// Between one and two rounds of tiles a CTA takes a long and a short one in turn: one round, all CTAs equally long.  Beyond, two
-// neighbours together where there is a form for it (can_pair): they share the expanded codes and fill each other's waits.  32 / 8
-// heads of 128, one after the other / together, us: 2048 tokens 114 / 81, behind 4096 447 / 341; 1000 tokens 36 / 44.
+// Between one and two rounds of tiles a CTA takes two of them, d_head = 128 in one of two forms.  In turn, a long and a short one:
+// all CTAs are equally long, but each walks what both tiles see twice.  Together, two neighbours: they share the expanded codes and
+// fill each other's waits.  So in turn is better for a prompt and together behind a prefix of about its length.  Measured (32 / 8 heads, 608
+// to 1184 tokens behind 0 to 8 times as many, within 3 % but for one round more), ns: in turn 1330 a step and 13500, together 2080
+// a step of two tiles and 10000; CTAs beyond 148 are a part of the last row group and follow another part of it.  1024 tokens, us in
+// turn / together: at 0 36 / 44, behind 512 57 / 60, 1024 79 / 77, 4096 205 / 176, 8192 376 / 310.  Beyond two rounds
+// together: 2048 tokens 114 / 82, behind 4096 447 / 349.
+inline bool prefill_together(int pos0, int T, int g, int Hkv, long long single) {
+    auto steps = [=](long long tile) -> long long {  // of 64 positions, up to the last one that the tile's rows see
+        const long long last = (tile * 128 + 127) / g;
+        return (pos0 + (last < T ? last + 1 : T) + 63) / 64;
+    };
+    const bool behind = (single + 1) / 2 * Hkv > 148;  // a CTA of the last row group follows another one
+    const long long one = 2 * (1330 * steps(single / 2) + 8500), turn = 1330 * (steps(single - 1) + steps(0)) + 13500;
+    const long long two = 2 * (2080 * steps(1) + 10000), pair = 2080 * steps(single - 1) + 10000;
+    return (behind && two > pair ? two : pair) < (behind && one > turn ? one : turn);
+}
+
 inline PrefillPlan prefill_plan(int pos0, int T, int g, int Hkv, bool can_pair = true) {
     constexpr int kRows = 128, kStep = 64;
     PrefillPlan pl;
     const long long single = (static_cast<long long>(T) * g + kRows - 1) / kRows;
-    pl.pair = single * Hkv > 2 * 148 && can_pair;
-    pl.tiles_per_cta = single * Hkv > 148 && (pl.pair || single * Hkv <= 2 * 148) ? 2 : 1;
+    const bool fits = single * Hkv <= 148, two_rounds = !fits && single * Hkv <= 2 * 148;
+    pl.pair = can_pair && !fits && (!two_rounds || prefill_together(pos0, T, g, Hkv, single));
+    pl.tiles_per_cta = pl.pair || two_rounds ? 2 : 1;
     pl.row_groups = (single + pl.tiles_per_cta - 1) / pl.tiles_per_cta;
     const int steps = (pos0 + T + kStep - 1) / kStep;
     // one CTA per SM is in flight; at least four steps per CTA of a cluster pay for the merge
