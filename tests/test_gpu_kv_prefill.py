@@ -60,7 +60,7 @@ def _fill(kv, uc, cache, b, n, Hkv, stream, v_scale=1.0, v_shift=0.3):
     (260, 1, 8, 2, 1.0),       # a single new token (a generation step written as a prefill)
     (2000, 40, 8, 2, 1.0),     # few CTAs, many steps: the steps are split over a cluster of eight
     (600, 100, 12, 4, 30.0),   # a cluster of two, a group of three
-    (1, 600, 32, 8, 1.0),      # two tiles per CTA, the last CTA's second tile empty
+    (1, 600, 32, 8, 1.0),      # two tiles in turn, the middle one of nineteen alone
 ])
 def test_attention_prefill_against_the_oracle(resq, kv, uc, prefix, T, Hq, Hkv, v_scale):
     S = prefix + T
@@ -90,7 +90,7 @@ def test_attention_prefill_against_the_oracle(resq, kv, uc, prefix, T, Hq, Hkv, 
 
 @pytest.mark.parametrize("prefix,T,Hq,Hkv,tiles,splits", [
     (0, 400, 8, 2, 1, 1), (900, 60, 4, 4, 1, 2), (0, 300, 32, 16, 1, 1),
-    (0, 600, 32, 8, 2, 1),      # two tiles in flight
+    (0, 600, 32, 8, 2, 1),      # two tiles in turn
     (1000, 256, 8, 4, 1, 4),
     (0, 2048, 1, 1, 1, 8),      # the first tile has two steps for eight CTAs: ranks without any
 ])
@@ -98,7 +98,7 @@ def test_attention_prefill_with_scores_that_keep_growing(resq, kv, uc, prefix, T
     """Keys that grow with the position: a row's maximum rises by far more than 2^8 over
     its steps, so the output accumulator is rescaled along the way, in one-tile, two-tile and split forms."""
     form = plans.prefill(prefix, T, Hq, Hkv)
-    assert (form.tiles_per_cta, form.splits) == (tiles, splits)
+    assert (form.tiles_per_cta, form.splits, form.pair) == (tiles, splits, 0)  # (together: test_gpu_prefill_many_tiles.py)
     S = prefix + T
     W_C, wq, s_u = uc
     cache = kv.KvCache(1, Hkv, (S + 31) // 32 * 32)
