@@ -329,7 +329,7 @@ __device__ __forceinline__ float step_scores(f2 (&sc)[PAIRS], uint32_t tmem_s, u
         f2x2 s[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) s[i] = pair_scales(col_k, 4 * part + i);
-        tmem_ld8x2_now(tmem_s + 8 * part, tmem_s + kColS4 + 8 * part, a8, a4);
+        tmem_ld8x2(tmem_s + 8 * part, tmem_s + kColS4 + 8 * part, a8, a4);
 #pragma unroll
         for (int i = 0; i < 4; ++i)
             sc[4 * part + i] = fma2(s[i].y, pack2(__uint_as_float(a4[2 * i]), __uint_as_float(a4[2 * i + 1])), sc[4 * part + i]);
@@ -606,7 +606,7 @@ __global__ void __launch_bounds__(Geometry<D, WAYS, PAIR>::kThreads, 1) attentio
                     for (int c = 0; c < G::kOutCols / 16; ++c) {
                         uint32_t o[16];
                         __syncwarp();
-                        tmem_ld16_now(out_columns(N) + 16 * c, o);
+                        tmem_ld16(out_columns(N) + 16 * c, o);
 #pragma unroll
                         for (int i = 0; i < 8; ++i) O[8 * c + i] = add2(O[8 * c + i], pack2(__uint_as_float(o[2 * i]), __uint_as_float(o[2 * i + 1])));
                     }
@@ -676,7 +676,7 @@ __global__ void __launch_bounds__(Geometry<D, WAYS, PAIR>::kThreads, 1) attentio
                         for (int c = 0; c < G::kOutCols / 16; ++c) {
                             uint32_t o[16];
                             __syncwarp();
-                            tmem_ld16_now(out_columns(N) + 16 * c, o);
+                            tmem_ld16(out_columns(N) + 16 * c, o);
 #pragma unroll
                             for (int i = 0; i < 16; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * f);
                             tmem_st16(out_columns(N) + 16 * c, o);
@@ -734,8 +734,8 @@ __global__ void __launch_bounds__(Geometry<D, WAYS, PAIR>::kThreads, 1) attentio
                 } else {
                     uint32_t u[2][16];
                     __syncwarp();
-                    tmem_ld16_now(out_columns(0) + 32 * c, u[0]);
-                    tmem_ld16_now(out_columns(0) + 32 * c + 16, u[1]);
+                    tmem_ld16(out_columns(0) + 32 * c, u[0]);
+                    tmem_ld16(out_columns(0) + 32 * c + 16, u[1]);
 #pragma unroll
                     for (int i = 0; i < 32; ++i) o[i] = __uint_as_float(u[i >> 4][i & 15]);
                 }

@@ -240,11 +240,9 @@ mixed_gemm_kernel(const __grid_constant__ CUtensorMap tmA8, const __grid_constan
             tc_fence_after();
             const uint32_t lane_addr = tmem_base + (static_cast<uint32_t>(quad * 32) << 16) + ch * (BN / 2);
             // Phase 1: the INT4 accumulator values of this thread's 128 columns, raw, into registers.
-            uint32_t a4[4][32];
+            uint32_t a4[128];
             __syncwarp();
-#pragma unroll
-            for (int c = 0; c < 4; ++c) tmem_ld32(lane_addr + BN + c * 32, a4[c]);
-            tmem_ld_wait();
+            tmem_ld128(lane_addr + BN, a4);
             tc_fence_before();
             mbar_arrive_cluster(cluster_map(&sh->acc4_empty, 0));
             // Phase 2: the INT8 accumulator, the scales, the store -- 16 columns at a time.
@@ -253,14 +251,13 @@ mixed_gemm_kernel(const __grid_constant__ CUtensorMap tmA8, const __grid_constan
                 uint32_t a8[16];
                 __syncwarp();
                 tmem_ld16(lane_addr + c * 16, a8);
-                tmem_ld_wait();
                 if (p.kb8 == 0) {  // uniform INT4: the INT8 accumulator was never written
 #pragma unroll
                     for (int j = 0; j < 16; ++j) a8[j] = 0;
                 }
                 const int cb = ch * (BN / 2) + c * 16;  // first column of the chunk inside the tile
                 const int nb = n0 + cb;
-                const uint32_t* a4c = &a4[c >> 1][(c & 1) * 16];
+                const uint32_t* a4c = &a4[c * 16];
                 if (row_ok) {
                     const size_t off = static_cast<size_t>(row) * p.N + nb;
                     if (p.dbg8) {

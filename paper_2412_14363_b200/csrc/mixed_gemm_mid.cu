@@ -201,14 +201,12 @@ mixed_gemm_mid_kernel(const __grid_constant__ CUtensorMap tmW8, const __grid_con
                 uint32_t a[16];
                 if (w4) {
                     tmem_ld16(lane_addr + kColAcc4 + 16 * g, a);
-                    tmem_ld_wait();
 #pragma unroll
                     for (int q = 0; q < 4; ++q)
                         *reinterpret_cast<uint4*>(dst + q * (BM * 16)) = make_uint4(a[4 * q], a[4 * q + 1], a[4 * q + 2], a[4 * q + 3]);
                 }
                 if (w8) {
                     tmem_ld16(lane_addr + 16 * g, a);
-                    tmem_ld_wait();
 #pragma unroll
                     for (int q = 0; q < 4; ++q)
                         *reinterpret_cast<uint4*>(dst + part8 + q * (BM * 16)) =
@@ -234,9 +232,7 @@ mixed_gemm_mid_kernel(const __grid_constant__ CUtensorMap tmW8, const __grid_con
             const int g = pair + k * p.splits;  // g % splits == pair
             uint32_t a4[16], a8[16];
             __syncwarp();  // TMEM loads are for the whole, converged warp; lanes beyond the channels only skip their stores
-            tmem_ld16(lane_addr + kColAcc4 + 16 * g, a4);
-            tmem_ld16(lane_addr + 16 * g, a8);
-            tmem_ld_wait();
+            tmem_ld16x2(lane_addr + kColAcc4 + 16 * g, lane_addr + 16 * g, a4, a8);
             if (!w4)
 #pragma unroll
                 for (int j = 0; j < 16; ++j) a4[j] = 0;

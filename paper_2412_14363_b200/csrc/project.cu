@@ -270,7 +270,6 @@ project_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_c
                 uint32_t v[32];
                 __syncwarp();
                 tmem_ld32(lane_addr + c * 32, v);
-                tmem_ld_wait();
                 const int nb = it.n0 + c * 32;
                 if (!it.bounded || it.m0 + lrow < p.T) {
                     float* cp = it.dst + static_cast<size_t>(lrow) * it.ld + c * 32;
@@ -445,7 +444,6 @@ project_gemm_few_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_co
                 uint32_t v[16];
                 __syncwarp();
                 tmem_ld16(lane_addr + c * 16, v);
-                tmem_ld_wait();
                 if (col_ok) {
 #pragma unroll
                     for (int i = 0; i < 16; ++i)

@@ -60,6 +60,19 @@ def test_what_another_grid_may_still_write_is_not_read_as_read_only(name):
 
 
 @pytest.mark.parametrize("name", SOURCES)
+def test_a_tensor_memory_load_and_its_wait_are_one_statement(name):
+    """Registers of a load on its way may be written at any time: between it and a wait of its own the compiler could move one."""
+    text = _code(name)
+    for m in re.finditer(r"\basm (?:volatile)?\(", text):
+        end, depth = m.end(), 1
+        while depth:
+            depth += {"(": 1, ")": -1}.get(text[end], 0)
+            end += 1
+        statement = text[m.start():end]
+        assert ("tcgen05.ld." in statement) == ("tcgen05.wait::ld" in statement), (name, statement[:80])
+
+
+@pytest.mark.parametrize("name", SOURCES)
 def test_tensor_memory_is_reached_by_whole_warps(name):
     """A TMEM load or store is for all 32 lanes at once.  A loop in which lanes may part ways (rows, columns or outputs that some
     lanes do not have) brings them together again before the next iteration's access, and no lane goes on past a wait that
