@@ -59,6 +59,10 @@ def test_what_another_grid_may_still_write_is_not_read_as_read_only(name):
             assert not re.search(r"const\s+\w+\s*\*\s*__restrict__", head), head
 
 
+TMEM_ACCESS = r"(?<!__forceinline__ void )\btmem_(?:ld|st)\d\w*\("
+TMEM_ACCESSES = {"kv_prefill.cu": 7, "mixed_gemm.cu": 2, "mixed_gemm_mid.cu": 3, "project.cu": 2}
+
+
 @pytest.mark.parametrize("name", SOURCES)
 def test_a_tensor_memory_load_and_its_wait_are_one_statement(name):
     """Registers of a load on its way may be written at any time: between it and a wait of its own the compiler could move one."""
@@ -78,7 +82,9 @@ def test_tensor_memory_is_reached_by_whole_warps(name):
     lanes do not have) brings them together again before the next iteration's access, and no lane goes on past a wait that
     ran out for another."""
     text = _code(name)
-    for m in re.finditer(r"tmem_(?:ld|st)\d+\(", text):
+    found = list(re.finditer(TMEM_ACCESS, text))
+    assert len(found) >= TMEM_ACCESSES.get(name, 0)  # a new name of the wrappers does not empty the rule
+    for m in found:
         loops = [f for f in re.finditer(r"\bfor \(", text[:m.start()])]
         enclosing = None
         for f in loops:
