@@ -6,7 +6,7 @@
 // sequence in steps of 64 positions (two cache blocks).  Roles:
 //   expand   3 warps: raw blocks (bulk copies, two steps ahead) -> operand tiles [position][coefficient], keys K-major, values
 //            N-major (so neither is transposed), and the step's per-position constants; three stages.  The codes become exact
-//            halves, centred (code - 128, code - 8); values at d = 64 become s (code - centre) + z' as three bf16 parts.
+//            halves, centred (code - 128, code - 8); values at d = 64 become s (code - centre) as three bf16 parts.
 //   mma      one warp: S8 and S4, the products of the two segments, into TMEM; later the output product with the weights taken
 //            from TMEM.
 //   softmax  2 or 4 threads per row, each with a share of the step's positions: score = s8 S8 + s4 S4 + (z8 + 128 s8) sum(q8) +
@@ -15,12 +15,14 @@
 // d = 128: P8 = half(p s8_v 2^-E), P4 = half(p s4_v 2^-E) times the exact codes, sums of p and of p (z + c0 s) in fp32.  2^E is the
 // largest finite value scale of the positions the CTA visits (read ahead of the walk), so the products stay in half's normal
 // range.  The outputs are accumulated in TMEM.
-// d = 64, whose outputs keep fp32's precision: p as three bf16 parts of all its 24 bits (bf16 has fp32's range: a value scale 2^28
-// above the others' beside next to no weight costs nothing) times the values' parts, six products, those left out below 2^-26.  The
-// tensor core truncates its fp32 sums, so a step's product is added to the thread's registers, with rounding.
+// d = 64, whose outputs keep fp32's precision (relative error against 64 bits 0.8e-7 to 2.6e-7; the mma.sync tiles before 0.9e-7 to 3.3e-7):
+// p as three bf16 parts of all its 24 bits (bf16 has fp32's range: a value scale 2^28 above the others' beside next to no weight
+// costs nothing) times the parts of the values without their zero-points, six products, those left out below 2^-26.  The tensor core
+// truncates its fp32 sums, so a step's product is added to the thread's registers, with rounding, and the zero-points, in which a
+// common mean of the values lies, are summed in fp32.  The row's reference comes off a score last, when it is small.
 // The reference of a row is the maximum of its first step and is raised only when a score exceeds it by 2^8; in that rare step the
 // row's outputs are rescaled.  So there is one pass over the cache, and weights are no smaller against the row's maximum than
-// 2^-8 of those with an exact one (d = 64: the reference lies 2^8 above the maximum, so weights are at most 1).
+// 2^-8 of those with an exact one (d = 64: values are taken times 2^-8, so that no sum is larger than with weights up to 1).
 // Two things are in flight, so that the products of one run under the softmax of the other: two steps of one tile, or (PAIR, d = 128,
 // where there are tiles enough) two tiles.  A CTA may take a long and a short tile in turn; the roles run on from one to the other.
 // With few CTAs a cluster splits the steps, and every rank merges the sums of a share of the rows through distributed shared memory.
@@ -193,8 +195,9 @@ __device__ __forceinline__ void expand_step(uint32_t raw, uint32_t stage, uint32
     auto constants = [&](float4 c, int blk, bool is_v, float fs, float fz) {
         const int j = 32 * blk + lane;
         if (j >= n_valid) c = make_float4(0.f, 0.f, 0.f, 0.f);
-        c.y = fmaf(128.f, c.x, c.y);
-        c.w = fmaf(8.f, c.z, c.w);
+        const float up = D == 64 && is_v ? 0.5f : 0.f;  // value_parts
+        c.y = fmaf(128.f - up, c.x, c.y);
+        c.w = fmaf(8.f - up, c.z, c.w);
         if (is_v && !(fabsf(c.x) <= FLT_MAX && fabsf(c.y) <= FLT_MAX)) {
             c.x = c.y = 0.f;
             atomicMin(bad8, j0 + j);
@@ -212,11 +215,13 @@ __device__ __forceinline__ void expand_step(uint32_t raw, uint32_t stage, uint32
         sts_f(dst + 16, c.y);
         sts_f(dst + 24, c.w);
     };
-    // D = 64: eight values, s (code - centre) + z', as three chunks of bf16
-    auto value_parts = [&](uint32_t at, const f2 (&code)[4], float scale, float zero) {
+    // D = 64: eight values without their zero-point, s (code - centre), as three chunks of bf16.  The centre is half a code lower, in the
+    // middle of the codes: sums that the tensor core truncates shall not lean to one side.
+    auto value_parts = [&](uint32_t at, const f2 (&code)[4], float scale) {
         uint32_t p[3][4];
+        const f2 half = pack2(0.5f * scale, 0.5f * scale);
 #pragma unroll
-        for (int m = 0; m < 4; ++m) split_bf16(fma2(code[m], pack2(scale, scale), pack2(zero, zero)), p[0][m], p[1][m], p[2][m]);
+        for (int m = 0; m < 4; ++m) split_bf16(fma2(code[m], pack2(scale, scale), half), p[0][m], p[1][m], p[2][m]);
 #pragma unroll
         for (int k = 0; k < 3; ++k) sts128(at + k * H::kTile, make_uint4(p[k][0], p[k][1], p[k][2], p[k][3]));
     };
@@ -234,7 +239,7 @@ __device__ __forceinline__ void expand_step(uint32_t raw, uint32_t stage, uint32
         } else {
             f2 code[4];
             centred_floats(nibbles_centred(word), code);
-            value_parts((row ^ (w << 4)) + H::kOffStageV4, code, c.z, c.w);
+            value_parts((row ^ (w << 4)) + H::kOffStageV4, code, c.z);
         }
     };
     if (warp < 2) {
@@ -256,7 +261,7 @@ __device__ __forceinline__ void expand_step(uint32_t raw, uint32_t stage, uint32
         if (D == 64) {
             sts128(row + H::kTile, bytes_centred(k8));
             store_constants(col_k, warp, constants(mk, warp, false, kScore, kScore));
-            mv = constants(mv, warp, true, 1.f, 1.f);
+            mv = constants(mv, warp, true, p_scale, p_scale);
         }
 #pragma unroll
         for (int w = 0; w < kFirst; ++w) value_word(row, w, v[w], mv);
@@ -276,11 +281,9 @@ __device__ __forceinline__ void expand_step(uint32_t raw, uint32_t stage, uint32
             if (D == 128) k8[c] = lds64(src + lane * H::kR8 + 8 * c);
             v8[c] = lds64(src + lane * H::kR8 + H::kOffV8 + 8 * c);
         }
-        mv = constants(mv, blk, true, p_scale, 1.f);
-        if (D == 128) {
-            store_constants(col_k, blk, constants(mk, blk, false, kScore, kScore));
-            store_constants(col_v, blk, mv);
-        }
+        mv = constants(mv, blk, true, p_scale, D == 128 ? 1.f : p_scale);
+        if (D == 128) store_constants(col_k, blk, constants(mk, blk, false, kScore, kScore));
+        store_constants(col_v, blk, mv);
 #pragma unroll
         for (int w = kFirst; w < kWords; ++w) value_word(row, w, v[w - kFirst], mv);
         if constexpr (D == 128) {
@@ -292,7 +295,7 @@ __device__ __forceinline__ void expand_step(uint32_t raw, uint32_t stage, uint32
         } else {
             f2 code[4];
             centred_floats(bytes_centred(v8[0]), code);
-            value_parts((row ^ (7 << 4)) + H::kOffStageV4, code, mv.x, mv.y);
+            value_parts((row ^ (7 << 4)) + H::kOffStageV4, code, mv.x);
         }
     }
 }
@@ -307,21 +310,24 @@ struct RowState {
 __device__ __forceinline__ f2x2 pair_scales(uint32_t col, int pair) { return lds_pairs(col + 32 * pair); }
 __device__ __forceinline__ f2x2 pair_zeros(uint32_t col, int pair) { return lds_pairs(col + 32 * pair + 16); }
 
-// What the zero-points give to the scores of the thread's positions, minus the row's reference, as pairs: known before the products.
-template <int PAIRS>
+// What the zero-points give to the scores of the thread's positions (D = 128: minus the row's reference), as pairs: known before the
+// products.
+template <int D, int PAIRS>
 __device__ __forceinline__ void step_offsets(f2 (&sc)[PAIRS], uint32_t col_k, f2 q8, f2 q4, float neg_m) {
     const f2 nm = pack2(neg_m, neg_m);
 #pragma unroll
     for (int pr = 0; pr < PAIRS; ++pr) {
         const f2x2 z = pair_zeros(col_k, pr);
-        sc[pr] = fma2(z.x, q8, fma2(z.y, q4, nm));
+        sc[pr] = fma2(z.x, q8, D == 128 ? fma2(z.y, q4, nm) : mul2(z.y, q4));
     }
 }
 
-// The scores on top of that; returns their maximum.  tmem_s, col_k: at the first of the positions; those beyond `last` are hidden
-// from the row.
-template <bool MASKED, int PAIRS>
-__device__ __forceinline__ float step_scores(f2 (&sc)[PAIRS], uint32_t tmem_s, uint32_t col_k, int last) {
+// The scores on top of that, against the row's reference; returns their maximum.  D = 64 takes the reference off last: what is left of
+// the scores that count is small and so is its rounding.  tmem_s, col_k: at the first of the positions; those beyond `last` are
+// hidden from the row.
+template <int D, bool MASKED, int PAIRS>
+__device__ __forceinline__ float step_scores(f2 (&sc)[PAIRS], uint32_t tmem_s, uint32_t col_k, float neg_m, int last) {
+    const f2 nm = pack2(neg_m, neg_m);
     float mx = -INFINITY;
 #pragma unroll
     for (int part = 0; part < PAIRS / 4; ++part) {  // eight positions
@@ -337,6 +343,7 @@ __device__ __forceinline__ float step_scores(f2 (&sc)[PAIRS], uint32_t tmem_s, u
         for (int i = 0; i < 4; ++i) {
             const int pr = 4 * part + i;
             sc[pr] = fma2(s[i].x, pack2(__uint_as_float(a8[2 * i]), __uint_as_float(a8[2 * i + 1])), sc[pr]);
+            if (D == 64) sc[pr] = add2(sc[pr], nm);
         }
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
@@ -360,12 +367,12 @@ template <int D, int PAIRS>
 __device__ __forceinline__ void step_weights(RowState& st, f2 (&sc)[PAIRS], uint32_t tmem_p, uint32_t col_v) {
     constexpr int kStore = 4;  // pairs per store
     f2x2 s[2], z[2];
-    if constexpr (D == 128) {
+    RowState sum{0.f, 0ull, 0ull, 0ull};  // D = 64: of the step, so that most of the additions round small sums
+    RowState& to = D == 128 ? st : sum;
 #pragma unroll
-        for (int i = 0; i < 2; ++i) {
-            s[i] = pair_scales(col_v, i);
-            z[i] = pair_zeros(col_v, i);
-        }
+    for (int i = 0; i < 2; ++i) {
+        if (D == 128) s[i] = pair_scales(col_v, i);
+        z[i] = pair_zeros(col_v, i);
     }
 #pragma unroll
     for (int pr = 0; pr < PAIRS; ++pr) {
@@ -378,22 +385,25 @@ __device__ __forceinline__ void step_weights(RowState& st, f2 (&sc)[PAIRS], uint
 #pragma unroll
         for (int i = 0; i < kStore; ++i) {
             const int pr = kStore * g + i, b = pr & 1;
-            st.l = add2(st.l, sc[pr]);
+            to.l = add2(to.l, sc[pr]);
+            to.z8 = fma2(sc[pr], z[b].x, to.z8);
+            to.z4 = fma2(sc[pr], z[b].y, to.z4);
             if constexpr (D == 128) {
-                st.z8 = fma2(sc[pr], z[b].x, st.z8);
-                st.z4 = fma2(sc[pr], z[b].y, st.z4);
                 w[0][i] = half_pair(mul2(sc[pr], s[b].x));
                 w[1][i] = half_pair(mul2(sc[pr], s[b].y));
-                if (pr + 2 < PAIRS) {
-                    s[b] = pair_scales(col_v, pr + 2);
-                    z[b] = pair_zeros(col_v, pr + 2);
-                }
+                if (pr + 2 < PAIRS) s[b] = pair_scales(col_v, pr + 2);
             } else {
                 split_bf16(sc[pr], w[0][i], w[1][i], w[2][i]);
             }
+            if (pr + 2 < PAIRS) z[b] = pair_zeros(col_v, pr + 2);
         }
 #pragma unroll
         for (int k = 0; k < Head<D>::kWeights; ++k) tmem_st4(tmem_p + 32 * k + kStore * g, w[k]);
+    }
+    if (D == 64) {
+        st.l = add2(st.l, sum.l);
+        st.z8 = add2(st.z8, sum.z8);
+        st.z4 = add2(st.z4, sum.z4);
     }
 }
 
@@ -410,6 +420,7 @@ template <int D, int WAYS, bool PAIR>
 __global__ void __launch_bounds__(Geometry<D, WAYS, PAIR>::kThreads, 1) attention_prefill_kernel(const PrefillParams p) {
     using H = Head<D>;
     using G = Geometry<D, WAYS, PAIR>;
+    constexpr float kUnit = D == 128 ? 1.f : 256.f;  // of the outputs before their division
     constexpr int kThreads = G::kThreads, kSoftmaxWarps = G::kSoftmaxWarps, kMmaWarp = G::kMmaWarp;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* base = smem_raw + (-smem_u32(smem_raw) & 1023u);  // (through an integer the compiler would lose that it is shared memory)
@@ -496,7 +507,7 @@ __global__ void __launch_bounds__(Geometry<D, WAYS, PAIR>::kThreads, 1) attentio
     if (loader)
         for (int N = 0; N < min(2, total_steps); ++N) issue_load(N);
     // ---- D = 128: the largest value scale of the positions visited
-    float p_scale = 1.f, out_scale = 1.f;
+    float p_scale = D == 128 ? 1.f : 0.00390625f, out_scale = 1.f;
     if (D == 128) {
         float vmax = 0.f;
         const int limit = positions_seen(long_tile), end = min(limit, first_step(limit, rank + 1) * kStep);
@@ -624,7 +635,7 @@ __global__ void __launch_bounds__(Geometry<D, WAYS, PAIR>::kThreads, 1) attentio
                 ok = mbar_wait(&sh->kv_full[stage], stage_parity, &sh->abort_flag, p.status);
                 ok = !__any_sync(0xffffffffu, !ok);
                 const float2 q = sh->row_sum[PAIR ? buf0 : ti][row];  // read again each step: cheaper than its registers
-                step_offsets(sc, col_k, pack2(q.x, q.x), pack2(q.y, q.y), -m_use);  // under the wait for the products
+                step_offsets<D>(sc, col_k, pack2(q.x, q.x), pack2(q.y, q.y), -m_use);  // under the wait for the products
                 if (++stage == kStages) {
                     stage = 0;
                     stage_parity ^= 1;
@@ -637,14 +648,13 @@ __global__ void __launch_bounds__(Geometry<D, WAYS, PAIR>::kThreads, 1) attentio
                 if (ok) {
                     const bool masked = j0 + G::kPart - 1 > pos_first;
                     const int last = pos_i - j0;  // the last of these positions that this row sees
-                    if (masked) mx = step_scores<true>(sc, tmem_s + part * G::kPart, col_k, last);
-                    else mx = step_scores<false>(sc, tmem_s + part * G::kPart, col_k, last);
+                    if (masked) mx = step_scores<D, true>(sc, tmem_s + part * G::kPart, col_k, -m_use, last);
+                    else mx = step_scores<D, false>(sc, tmem_s + part * G::kPart, col_k, -m_use, last);
                 }
                 // ---- raise the reference where a score leaves it too far behind (and set it at the first position seen).  Behind
                 // the barrier all warps of the rows have read the scores that the weights go over, and all leave if a wait of one failed
-                const float top = D == 128 ? kSlack : 0.f;
                 tc_fence_before();
-                const bool rare = group_any<32 * WAYS>(group, !ok || mx > (st.m == -INFINITY ? -INFINITY : top));
+                const bool rare = group_any<32 * WAYS>(group, !ok || mx > (st.m == -INFINITY ? -INFINITY : kSlack));
                 tc_fence_after();
                 if (rare) {
                     row_part[part][row].w = mx;
@@ -658,8 +668,8 @@ __global__ void __launch_bounds__(Geometry<D, WAYS, PAIR>::kThreads, 1) attentio
                     }
 #pragma unroll
                     for (int i = 0; i < WAYS; ++i) mx = fmaxf(mx, row_part[i][row].w);
-                    const bool raise = mx > (st.m == -INFINITY ? -INFINITY : top);
-                    const float d = raise ? mx + (D == 128 ? 0.f : kSlack) : 0.f;
+                    const bool raise = mx > (st.m == -INFINITY ? -INFINITY : kSlack);
+                    const float d = raise ? mx : 0.f;
                     const float f = raise ? (st.m == -INFINITY ? 0.f : exp2_approx(-d)) : 1.f;
                     const f2 d2 = pack2(-d, -d), ff = pack2(f, f);
 #pragma unroll
@@ -712,7 +722,7 @@ __global__ void __launch_bounds__(Geometry<D, WAYS, PAIR>::kThreads, 1) attentio
             // A block of the warp's columns goes through shared memory (to a split walk's record, or a patch of the warp's own): stored
             // from rows, every 16 bytes would be a line of their own (2 us per tile).
             float* record = reinterpret_cast<float*>(base) + row * H::kRecPitch;  // over the tiles: every product of the CTA is done
-            const float inv = splits > 1 ? 1.f : l > 0.f ? 1.f / l : 0.f;
+            const float inv = splits > 1 ? 1.f : l > 0.f ? kUnit / l : 0.f;
             if (splits > 1 && part == 0 && ok) {
                 record[D] = st.m;
                 record[D + 1] = l;
@@ -945,7 +955,7 @@ __global__ void __launch_bounds__(Geometry<D, WAYS, PAIR>::kThreads, 1) attentio
                 L = fmaf(ml[rk].y, f, L);
                 acc = make_float4(fmaf(o[rk].x, f, acc.x), fmaf(o[rk].y, f, acc.y), fmaf(o[rk].z, f, acc.z), fmaf(o[rk].w, f, acc.w));
             }
-            const float inv = L > 0.f ? 1.f / L : 0.f;
+            const float inv = L > 0.f ? kUnit / L : 0.f;
             *reinterpret_cast<float4*>(p.out + head_vector(Ro) * D + 4 * c4) =
                 make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv);
         }
