@@ -635,7 +635,11 @@ __device__ __forceinline__ void butterfly_pairs(float* hrow, int K, int s, int t
 
 // NT threads per row: 256 when rows outnumber the SMs (throughput: several CTAs per SM), 1024 for the few rows of a
 // generation step, where one row's chain of passes is all there is to wait for.
-template <int M, int NT>
+// PAIRS: butterflies of two neighbours to a thread, for rows of kPairWidth and more.  Narrower ones have fewer pairs than threads: with
+// M = 12 and 28 and pairs, rows of 384 to 896 took 2 to 6 % longer than now (1537 rows of 384 9.7 us, 9.0 now; 1000 rows of 1536
+// 8.2, 8.1; of 1792 8.5, singly 9.1).
+constexpr int kPairWidth = 1792;
+template <int M, int NT, bool PAIRS = (M > 1 && NT == kThreads)>
 __global__ void __launch_bounds__(NT, NT == kThreads ? (M > 1 ? 3 : 5) : 1)
 hadamard_quantize_kernel(const __nv_bfloat16* X, size_t rows, int K, int kbits, int r, float inv_sqrt_k,
                          int8_t* __restrict__ q8, uint8_t* __restrict__ q4, float* __restrict__ s8_out,
@@ -727,7 +731,7 @@ hadamard_quantize_kernel(const __nv_bfloat16* X, size_t rows, int K, int kbits, 
             const int left = kbits - s;
             const int nb = left <= kMaxBits ? left : (left <= 2 * kMaxBits ? (left + 1) / 2 : kMaxBits);
             const bool last = s + nb >= kbits;
-            if constexpr (M > 1 && NT == kThreads) {  // 1024 threads have no registers for 32 pairs; M = 1 has odd neighbours in the first pass
+            if constexpr (PAIRS) {  // 1024 threads have no registers for 32 pairs; M = 1 has odd neighbours in the first pass
                 if (nb == 1) butterfly_pairs<M, NT, 1>(hrow, K, s, tid, last, inv_sqrt_k, r, a8, a4);
                 else if (nb == 2) butterfly_pairs<M, NT, 2>(hrow, K, s, tid, last, inv_sqrt_k, r, a8, a4);
                 else if (nb == 3) butterfly_pairs<M, NT, 3>(hrow, K, s, tid, last, inv_sqrt_k, r, a8, a4);
@@ -930,7 +934,8 @@ cudaError_t launch_hadamard_quantize(const void* X, size_t rows, int K, int r, i
     if (dev < 64 && !ready[dev]) {
         // Once per device: the shared-memory limit of the kernels.
         for (auto k : {hadamard_quantize_kernel<1, kThreads>, hadamard_quantize_kernel<12, kThreads>,
-                       hadamard_quantize_kernel<28, kThreads>, hadamard_quantize_kernel<1, kWideThreads>,
+                       hadamard_quantize_kernel<28, kThreads>, hadamard_quantize_kernel<12, kThreads, false>,
+                       hadamard_quantize_kernel<28, kThreads, false>, hadamard_quantize_kernel<1, kWideThreads>,
                        hadamard_quantize_kernel<12, kWideThreads>, hadamard_quantize_kernel<28, kWideThreads>})
             if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024)) != cudaSuccess)
                 return e;
@@ -945,9 +950,9 @@ cudaError_t launch_hadamard_quantize(const void* X, size_t rows, int K, int r, i
     auto kern = wide ? (m == 1    ? hadamard_quantize_kernel<1, kWideThreads>
                         : m == 12 ? hadamard_quantize_kernel<12, kWideThreads>
                                   : hadamard_quantize_kernel<28, kWideThreads>)
-                     : (m == 1    ? hadamard_quantize_kernel<1, kThreads>
-                        : m == 12 ? hadamard_quantize_kernel<12, kThreads>
-                                  : hadamard_quantize_kernel<28, kThreads>);
+                : m == 1         ? hadamard_quantize_kernel<1, kThreads>
+                : K < kPairWidth ? (m == 12 ? hadamard_quantize_kernel<12, kThreads, false> : hadamard_quantize_kernel<28, kThreads, false>)
+                                 : (m == 12 ? hadamard_quantize_kernel<12, kThreads> : hadamard_quantize_kernel<28, kThreads>);
     count_launch();
     return launch_programmatic(kern, grid, wide ? kWideThreads : kThreads, smem, st, x, rows, K, kbits, r, inv_sqrt_k, q8, q4,
                                s8, s4, q4_i8);
