@@ -105,9 +105,12 @@ inline PrefillPlan prefill_plan(int pos0, int T, int g, int Hkv, bool can_pair =
     pl.tiles_per_cta = pl.pair || two_rounds ? 2 : 1;
     pl.row_groups = (single + pl.tiles_per_cta - 1) / pl.tiles_per_cta;
     const int steps = (pos0 + T + kStep - 1) / kStep;
-    // one CTA per SM is in flight; at least four steps per CTA of a cluster pay for the merge
+    // One CTA per SM is in flight; at least four steps per CTA of a cluster pay for the merge.  15 clusters of eight run at the same time; one
+    // more makes a second round.  At d_head = 64 that is what the tiles of 64 rows before took (32 / 8 heads, 64 tokens behind 4000: 39.2
+    // us, 40.1 with eight CTAs each, 32.8 with four); at 128 (74 before, 42 and 31) the limit is still that of single CTAs.
+    const int eights = can_pair ? 148 : 15 * 8;
     pl.splits = 1;
-    while (pl.splits < 8 && pl.row_groups * Hkv * pl.splits * 2 <= 148 && steps >= 8 * pl.splits) pl.splits *= 2;
+    while (pl.splits < 8 && pl.row_groups * Hkv * pl.splits * 2 <= (pl.splits == 4 ? eights : 148) && steps >= 8 * pl.splits) pl.splits *= 2;
     return pl;
 }
 

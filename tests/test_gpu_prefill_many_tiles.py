@@ -77,7 +77,7 @@ def test_runs_of_many_tiles_against_the_oracle(D, prefix, T, Hq, Hkv, tiles, for
 
 @pytest.mark.parametrize("D,prefix,T,Hq,Hkv,form,splits", [
     (128, 3, 1200, 32, 32, TOGETHER, 1), (128, 1400, 700, 28, 7, TOGETHER, 1), (128, 0, 1660, 12, 4, TURN, 1),
-    (64, 0, 400, 8, 2, ONE, 1), (64, 900, 60, 4, 4, ONE, 2), (64, 0, 2048, 1, 1, ONE, 8), (64, 0, 1000, 32, 8, TURN, 1),
+    (64, 0, 400, 8, 2, ONE, 1), (64, 900, 60, 4, 4, ONE, 2), (64, 200, 1900, 1, 1, ONE, 8), (64, 0, 1000, 32, 8, TURN, 1),
     (64, 150, 1660, 12, 4, TURN, 1), (64, 0, 1200, 32, 32, ONE, 1),
 ])
 def test_scores_that_keep_growing(D, prefix, T, Hq, Hkv, form, splits):

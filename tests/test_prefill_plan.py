@@ -32,3 +32,9 @@ def test_forms_outside_that_range():
         assert form.tiles_per_cta == 2 and form.pair
     assert plans.run64(8192, 1024, 32, 8).tiles == 2                    # d_head = 64 has no form for two tiles together
     assert plans.run64(0, 1200, 32, 8).tiles == 1
+
+
+@pytest.mark.parametrize("T, prefix, Hq, Hkv, splits", [(32, 4000, 60, 15, 8), (32, 4000, 64, 16, 4), (64, 4000, 32, 8, 4), (32, 1200, 128, 32, 4)])
+def test_clusters_of_eight_run_at_the_same_time_at_d_head_64(T, prefix, Hq, Hkv, splits):
+    """Up to 15 of them: a second round costs more than the split gives."""
+    assert plans.run64(prefix, T, Hq, Hkv).splits == splits
