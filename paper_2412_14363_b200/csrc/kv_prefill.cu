@@ -108,7 +108,7 @@ struct Geometry {
     static constexpr size_t kOutStage = D == 128 ? 0 : kSoftmaxWarps * kOutBytes;
     static_assert(D == 64 || kGroupWarps * kOutBytes <= Head<D>::kQBytes, "outputs fit");
     static constexpr size_t kSmem = 1024 + kTiles + kOutStage + 2 * Head<D>::kRawBytes + sizeof(Shared);
-    static_assert(kSmem <= 227 * 1024 && kMmaWarp < 20 && (!PAIR || WAYS == 2), "one CTA per SM");
+    static_assert(kSmem <= 227 * 1024 && kMmaWarp < 20 && (!PAIR || (D == 128 && WAYS == 2)), "one CTA per SM");
     static_assert(kTiles >= static_cast<size_t>(kRows) * Head<D>::kRecPitch * 4, "records fit");
     // TMEM: score buffers (8-bit and 4-bit segment, the weights over them; PAIR: one per tile, else one per stage), then the outputs:
     // PAIR: one per tile; D = 128: one, which the tensor core adds up; D = 64: two, by turns
@@ -589,8 +589,6 @@ __global__ void __launch_bounds__(Geometry<D, WAYS, PAIR>::kThreads, 1) attentio
         auto buffer = [&](int N) { return PAIR ? buf0 : N & 1; };  // whose barriers (and output) step N uses, and their parity
         auto parity = [&](int N) { return PAIR ? N & 1 : N >> 1 & 1; };
         auto out_columns = [&](int N) { return tmem_row + G::kColOut + part * G::kOutCols + buffer(N) * G::kOutPitch; };
-        constexpr int kLag = PAIR ? 1 : 2;               // steps after which an output product is complete without a wait
-        constexpr bool kLastOnly = PAIR && D == 128;     // only the last one is waited for: the next scores are behind the others
         const uint32_t cols_k = smem_u32(sh->col_k) + part * (G::kPart * 16), cols_v = smem_u32(sh->col_v) + part * (G::kPart * 16);
         for (int ti = 0, done = 0; ti < tiles && ok; ++ti) {  // done: steps of the tiles before
             const Tile tile = tile_of(ti);
@@ -603,8 +601,8 @@ __global__ void __launch_bounds__(Geometry<D, WAYS, PAIR>::kThreads, 1) attentio
 #pragma unroll
                 for (int i = 0; i < G::kOutCols / 2; ++i) O[i] = 0ull;
             }
-            // Waits for the output product of the CTA's step N, counted over its tiles; of those that are not behind the scores seen last
-            // every one of a buffer's in turn.
+            // Waits for the output product of the CTA's step N, counted over its tiles: of a buffer's every one in turn (PAIR: the last
+            // alone; the next scores are behind the others).
             auto output_ready = [&](int N) {
                 ok = mbar_wait(&sh->pv_done[buffer(N)], parity(N), &sh->abort_flag, p.status);
                 ok = !__any_sync(0xffffffffu, !ok);
@@ -640,7 +638,7 @@ __global__ void __launch_bounds__(Geometry<D, WAYS, PAIR>::kThreads, 1) attentio
                     stage = 0;
                     stage_parity ^= 1;
                 }
-                if (!kLastOnly && n >= kLag && ok && output_ready(N - kLag) && !added) add_output(N - kLag);
+                if (!PAIR && n >= 2 && ok && output_ready(N - 2) && !added) add_output(N - 2);
                 added = false;
                 ok = ok && mbar_wait(&sh->s_full[buffer(N)], parity(N), &sh->abort_flag, p.status);
                 ok = !__any_sync(0xffffffffu, !ok);
@@ -700,7 +698,7 @@ __global__ void __launch_bounds__(Geometry<D, WAYS, PAIR>::kThreads, 1) attentio
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&sh->p_full[buffer(N)]);
             }
-            for (int n = max(n_steps - (kLastOnly ? 1 : 2), 0); n < n_steps && ok; ++n)
+            for (int n = max(n_steps - (PAIR ? 1 : 2), 0); n < n_steps && ok; ++n)
                 if (output_ready(done + n) && !(added && n == n_steps - 2)) add_output(done + n);
             // a row that sees a value whose constants are not finite gets NaN in that segment
             if (pos_i >= sh->bad8) st.z8 = pack2(NAN, NAN);
@@ -729,7 +727,7 @@ __global__ void __launch_bounds__(Geometry<D, WAYS, PAIR>::kThreads, 1) attentio
             }
             constexpr int kCols = G::kOutBlock, kQuads = kCols / 4;
             auto coefficient = [&](int n0) { return n0 >= D - H::kR8 ? n0 - (D - H::kR8) : H::kR8 + n0; };  // of the first of eight columns
-            uint8_t* patch = (D == 128 ? Qs + (PAIR ? buf0 : ti) * H::kQBytes : out_stage_d64) + (PAIR ? warp & 7 : warp) * G::kOutBytes;
+            uint8_t* patch = D == 128 ? Qs + (PAIR ? buf0 : ti) * H::kQBytes + (warp & 7) * G::kOutBytes : out_stage_d64 + warp * G::kOutBytes;
 #pragma unroll
             for (int c = 0; c < G::kOutCols / kCols; ++c) {
                 if (R0 + (warp & 3) * 32 >= p.T * p.g && splits == 1) break;  // none of the warp's rows exists
@@ -1020,16 +1018,11 @@ cudaError_t launch_attention_prefill(const resq_kv_cache_t& cache, const void* q
     p.g_inv = static_cast<unsigned>(((1ull << 32) + p.g - 1) / p.g);
     p.pos0 = pos0;
     p.status = device_status_ptr();
-    if (d_head == 64) {
-        const Attn64Plan pl = attention64_run_plan(pos0, T, p.g, p.Hkv);
-        p.splits = pl.splits;
-        p.tiles = pl.tiles;
-        return launch_prefill<64, 4, false>(p, pl.ctas, st);
-    }
-    const PrefillPlan pl = prefill_plan(pos0, T, p.g, p.Hkv);
+    const PrefillPlan pl = prefill_plan(pos0, T, p.g, p.Hkv, d_head);
     p.splits = pl.splits;
     p.tiles = pl.tiles_per_cta;
     const long long ctas = pl.row_groups * p.Hkv * pl.splits;
+    if (d_head == 64) return launch_prefill<64, 4, false>(p, ctas, st);
     return pl.pair ? launch_prefill<128, 2, true>(p, ctas, st) : launch_prefill<128, 2, false>(p, ctas, st);
 }
 

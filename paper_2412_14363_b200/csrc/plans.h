@@ -76,7 +76,7 @@ struct PrefillPlan {
     int tiles_per_cta, splits;
     bool pair;             // the CTA's two tiles walk together, not one after the other
     long long row_groups;  // groups of tiles_per_cta tiles; the grid is row_groups * Hkv * splits
-};
+};  // d_head = 64 has no form for two tiles together (a thread would hold 32 outputs beside its scores)
 
 // Between one and two rounds of tiles a CTA takes two of them, d_head = 128 in one of two forms.  In turn, a long and a short one:
 // all CTAs are equally long, but each walks what both tiles see twice.  Together, two neighbours: they share the expanded codes and
@@ -96,43 +96,33 @@ inline bool prefill_together(int pos0, int T, int g, int Hkv, long long single) 
     return (behind && two > pair ? two : pair) < (behind && one > turn ? one : turn);
 }
 
-inline PrefillPlan prefill_plan(int pos0, int T, int g, int Hkv, bool can_pair = true) {
+inline PrefillPlan prefill_plan(int pos0, int T, int g, int Hkv, int d_head) {
     constexpr int kRows = 128, kStep = 64;
     PrefillPlan pl;
     const long long single = (static_cast<long long>(T) * g + kRows - 1) / kRows;
     const bool fits = single * Hkv <= 148, two_rounds = !fits && single * Hkv <= 2 * 148;
-    pl.pair = can_pair && !fits && (!two_rounds || prefill_together(pos0, T, g, Hkv, single));
+    pl.pair = d_head == 128 && !fits && (!two_rounds || prefill_together(pos0, T, g, Hkv, single));
     pl.tiles_per_cta = pl.pair || two_rounds ? 2 : 1;
     pl.row_groups = (single + pl.tiles_per_cta - 1) / pl.tiles_per_cta;
     const int steps = (pos0 + T + kStep - 1) / kStep;
     // One CTA per SM is in flight; at least four steps per CTA of a cluster pay for the merge.  15 clusters of eight run at the same time; one
     // more makes a second round.  At d_head = 64 that is what the tiles of 64 rows before took (32 / 8 heads, 64 tokens behind 4000: 39.2
     // us, 40.1 with eight CTAs each, 32.8 with four); at 128 (74 before, 42 and 31) the limit is still that of single CTAs.
-    const int eights = can_pair ? 148 : 15 * 8;
+    const int eights = d_head == 128 ? 148 : 15 * 8;
     pl.splits = 1;
     while (pl.splits < 8 && pl.row_groups * Hkv * pl.splits * 2 <= (pl.splits == 4 ? eights : 148) && steps >= 8 * pl.splits) pl.splits *= 2;
     return pl;
 }
 
-// ---- attention at d_head = 64 (kv_d64.cu)
+// ---- attention at d_head = 64, rows that are alone (kv_d64.cu)
 enum Pack { kPackNever = 0, kPackIfShort = 1, kPackAlways = 2 };  // whether a CTA takes as many items as it has warps
 struct Attn64Plan {
     int warps;        // per CTA
-    int splits;       // CTAs of a cluster that share an item or a tile
-    int pack;         // Pack (rows that are alone)
+    int splits;       // CTAs of a cluster that share an item
+    int pack;         // Pack
     int short_steps;  // kPackIfShort: items of up to as many steps of 32 positions are packed
     long long ctas;   // grid
-    int tiles = 0;    // a causal run: tiles of 128 rows per CTA, one after the other
 };
-
-// A causal run of one sequence goes to kv_prefill.cu: sixteen softmax warps, four threads a row.  There is no form for two tiles
-// together (a thread would hold 32 outputs beside its scores).
-inline Attn64Plan attention64_run_plan(int pos0, int T, int g, int Hkv) {
-    const PrefillPlan run = prefill_plan(pos0, T, g, Hkv, false);
-    Attn64Plan pl{16, run.splits, kPackNever, 0, run.row_groups * Hkv * run.splits};
-    pl.tiles = run.tiles_per_cta;
-    return pl;
-}
 
 // Query rows that are alone: one item per (row, KV head).  The lengths are on the device; the capacity stands in for them.
 inline Attn64Plan attention64_rows_plan(int rows, int Hkv, int capacity) {

@@ -15,18 +15,15 @@ extern "C" {
 void mid(int T, int N, int kbt, int* o) { MidPlan p = mid_plan(T, N, kbt); o[0] = p.use; o[1] = p.ntok; o[2] = p.tok_tiles; o[3] = p.splits; }
 int together(int d, int kv_tiles, int tiles) { return append_tiles_together(d, kv_tiles, tiles); }
 int gptq(int N, int K) { return gptq_rows_per_cta(N, K); }
-void prefill(int pos0, int T, int g, int Hkv, int* o) {
-    PrefillPlan p = prefill_plan(pos0, T, g, Hkv); o[0] = p.tiles_per_cta; o[1] = p.splits; o[2] = (int)p.row_groups; o[3] = p.pair; }
-void run64(int pos0, int T, int g, int Hkv, int* o) {
-    Attn64Plan p = attention64_run_plan(pos0, T, g, Hkv);
-    o[0] = p.warps; o[1] = p.splits; o[2] = p.pack; o[3] = p.short_steps; o[4] = (int)p.ctas; o[5] = p.tiles; }
+void prefill(int pos0, int T, int g, int Hkv, int d, int* o) {
+    PrefillPlan p = prefill_plan(pos0, T, g, Hkv, d); o[0] = p.tiles_per_cta; o[1] = p.splits; o[2] = (int)p.row_groups; o[3] = p.pair; }
 void rows64(int rows, int Hkv, int capacity, int* o) {
-    Attn64Plan p = attention64_rows_plan(rows, Hkv, capacity); o[0] = p.warps; o[1] = p.splits; o[2] = p.pack; o[3] = p.short_steps; o[4] = (int)p.ctas; o[5] = p.tiles; }
+    Attn64Plan p = attention64_rows_plan(rows, Hkv, capacity); o[0] = p.warps; o[1] = p.splits; o[2] = p.pack; o[3] = p.short_steps; o[4] = (int)p.ctas; }
 }
 """
 Mid = namedtuple("Mid", "use ntok tok_tiles splits")
 Prefill = namedtuple("Prefill", "tiles_per_cta splits row_groups pair")
-Attn64 = namedtuple("Attn64", "warps splits pack short_steps ctas tiles")
+Attn64 = namedtuple("Attn64", "warps splits pack short_steps ctas")
 
 
 @functools.lru_cache(None)
@@ -63,12 +60,8 @@ def append_together(d, T, Hq, Hkv):
     return bool(_lib().together(d, kv_tiles, kv_tiles + -(-T * Hq // 16)))
 
 
-def prefill(pos0, T, Hq, Hkv):
-    return _call("prefill", Prefill, pos0, T, Hq // Hkv, Hkv)
-
-
-def run64(pos0, T, Hq, Hkv):
-    return _call("run64", Attn64, pos0, T, Hq // Hkv, Hkv)
+def prefill(pos0, T, Hq, Hkv, d=128):
+    return _call("prefill", Prefill, pos0, T, Hq // Hkv, Hkv, d)
 
 
 def rows64(rows, Hkv, capacity):

@@ -19,9 +19,7 @@ TURN, TOGETHER, ONE = (2, 0), (2, 1), (1, 0)  # tiles of a CTA, whether they wal
 
 
 def _form(D, prefix, T, Hq, Hkv):
-    if D == 64:
-        return plans.run64(prefix, T, Hq, Hkv).tiles, 0
-    form = plans.prefill(prefix, T, Hq, Hkv)
+    form = plans.prefill(prefix, T, Hq, Hkv, D)
     return form.tiles_per_cta, form.pair
 
 
@@ -82,5 +80,5 @@ def test_runs_of_many_tiles_against_the_oracle(D, prefix, T, Hq, Hkv, tiles, for
 ])
 def test_scores_that_keep_growing(D, prefix, T, Hq, Hkv, form, splits):
     assert _form(D, prefix, T, Hq, Hkv) == form
-    assert (plans.run64 if D == 64 else plans.prefill)(prefix, T, Hq, Hkv).splits == splits
+    assert plans.prefill(prefix, T, Hq, Hkv, D).splits == splits
     _check(D, prefix, T, Hq, Hkv, growing=True)

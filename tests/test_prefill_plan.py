@@ -30,11 +30,12 @@ def test_forms_outside_that_range():
     for prefix in (0, 4096):                                            # 304 tiles: together whatever the prefix
         form = plans.prefill(prefix, 1200, 32, 8)
         assert form.tiles_per_cta == 2 and form.pair
-    assert plans.run64(8192, 1024, 32, 8).tiles == 2                    # d_head = 64 has no form for two tiles together
-    assert plans.run64(0, 1200, 32, 8).tiles == 1
+    form = plans.prefill(8192, 1024, 32, 8, 64)                         # d_head = 64 has no form for two tiles together
+    assert form.tiles_per_cta == 2 and not form.pair
+    assert plans.prefill(0, 1200, 32, 8, 64).tiles_per_cta == 1
 
 
 @pytest.mark.parametrize("T, prefix, Hq, Hkv, splits", [(32, 4000, 60, 15, 8), (32, 4000, 64, 16, 4), (64, 4000, 32, 8, 4), (32, 1200, 128, 32, 4)])
 def test_clusters_of_eight_run_at_the_same_time_at_d_head_64(T, prefix, Hq, Hkv, splits):
     """Up to 15 of them: a second round costs more than the split gives."""
-    assert plans.run64(prefix, T, Hq, Hkv).splits == splits
+    assert plans.prefill(prefix, T, Hq, Hkv, 64).splits == splits
