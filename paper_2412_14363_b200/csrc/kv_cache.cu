@@ -7,8 +7,8 @@
 // elements [32 b + 8c, +8), 16 bytes at a time: the bytes of its A fragments of mma.m16n8k32, in an order of the reduction that
 // U_C's staged rows share.  The product's columns are dealt out in the same way (a permutation of U_C's rows, free with
 // ldmatrix), so outputs leave 16 bytes at a time too, and key and value share the cache quantizer.
-// What bounds it: instructions, about 700 per 16 vectors; 2048 tokens of 32 + 16 vectors take 27.8 us at d = 128 (before 32.0; the
-// 100 MB would take 15) and 13.8 at 64 (before 18.1).  Rows of a key or value tile are 16 tokens of one head: their records are
+// What bounds it: instructions, their fetch first (120 KB of straight code at d = 128, 70 at 64); 2048 tokens of 32 + 16 vectors take
+// 27.2 us at d = 128 (before 32.0; the 100 MB would take 15) and 13.6 at 64 (before 18.1).  128 registers at d = 128 spill 76 bytes.  Rows of a key or value tile are 16 tokens of one head: their records are
 // neighbours in the cache.  The next tile's rows are on their way during the products.  Roundings are checked for a whole lane
 // at once (two bracketing products, packed pairs) instead of one by one with a branch each.
 // head_vector_kernel (few, a generation step): one warp per head vector, lane l owning coefficients l + 32 i, dp4a

@@ -35,13 +35,14 @@
 // tokens, may hold anything.  All waits are bounded; after a failed wait every role leaves its loop, copies and products in
 // flight are waited for, and TMEM is freed.
 //
-// What bounds it: the instructions of softmax and expansion (57 % of the issue slots at d = 128) and the latency of their chains.
-// Cycles per step: d = 128, two tiles of 128 rows 3800 (4300 with one thread per row and four expanding warps); d = 64, one
-// tile 2100.  The expansion set the pace while its words were read, converted and written one by one: 290 cycles per piece of
-// 32 positions against 65 with addresses of a register and a constant and all words on their way first.  Divisions by the
-// group size took 5 us of a call, outputs stored row by row 2 us.
-// us, 32 query / 8 KV heads: d = 128, 2048 tokens behind 4096 400 -> 340 (1310 with one 128-row tile per CTA in two passes), 1000
-// tokens 49 -> 36; d = 64, 1000 tokens 60 -> 38 (mma.sync tiles of 64 rows), 2048 behind 4096 828 -> 509.
+// What bounds it: the instructions of softmax and expansion (60 % of the issue slots, 63 at d = 64) and the latency of their chains.
+// us per step: d = 128, two tiles together 2.08, one tile 1.33; d = 64, one tile 1.87 (1.62 with the zero-points inside the values'
+// parts).  The expansion sets the pace where its words are read, converted and written one by one; so all words are on their way
+// first, with addresses of a register and a constant.  Divisions by the group size took 5 us of a call, outputs stored row by row 2 us.
+// us, 32 query / 8 KV heads: d = 128, 2048 tokens behind 4096 400 -> 349 (1310 with one 128-row tile per CTA in two passes), 1000
+// tokens 49 -> 37; d = 64, 1000 tokens 60 -> 43 (mma.sync tiles of 64 rows), 2048 behind 4096 828 -> 580.  A run of one step (32
+// tokens of 8 / 8 heads at position 0: 7.2 -> 8.0) and, at d = 64, of a few tokens there (5.6 -> 6.9) is slower than before: more of it
+// is set-up.
 #include "centred_codes.cuh"
 #include "internal.h"
 #include "packed_fp32.cuh"
