@@ -18,6 +18,11 @@
 // (movmatrix) to become the second product's B fragments.  Scores, the running softmax and all sums are
 // fp32; the weights p_j s_j are scaled by a power of two taken from the value scales so that they stay in
 // half's range whatever the magnitude of V.
+//
+// What bounds it: the stream (5.3 TB/s over the 27 us between a run's first block and the last end) and what is not stream.  16 ragged sequences of up to 8192
+// positions, 32 / 8 heads, 142 MB: 41.4 -> 37.4 us, of which 1.5 us until the copies are asked for (5.7 to the first block's
+// arithmetic, now 2.6: two scans of the lengths with 64-bit divisions, and query loads behind 30 MB of copies), 2 us of uneven ends (runs of 14 or
+// 15 blocks), 1 us to the merge kernel and 2 to 3.6 in it.
 #include <cuda_fp16.h>
 
 #include "internal.h"
@@ -54,34 +59,64 @@ __device__ __forceinline__ int clamped_len(const int32_t* seq_lens, int b, int c
     return len < 0 ? 0 : (len > capacity ? capacity : len);
 }
 
-// Whole warp: returns the number of blocks per head summed over all sequences.  If target >= 0, also finds the
-// sequence that holds global block `target` (the list has n_kv_heads times the per-head blocks of each
-// sequence) and the per-head blocks of all sequences before it.
-__device__ __forceinline__ long long scan_blocks(const AttnParams& p, int lane, long long target, int* b_out,
-                                                 long long* before_out) {
-    long long base = 0;
-    bool found = false;
-    for (int b0 = 0; b0 < p.n_seqs; b0 += 32) {
-        const int b = b0 + lane;
-        const int t = b < p.n_seqs ? (clamped_len(p.seq_lens, b, p.capacity) + 31) >> 5 : 0;
-        int incl = t;
+// First block of run w: floor(total w / kNumWarps).
+__device__ __forceinline__ long long run_start(long long total, int w) {
+    if (total >> 31) return total * w / kNumWarps;
+    const unsigned t = static_cast<unsigned>(total), q = t / kNumWarps, r = t % kNumWarps;  // 64-bit divisions are long
+    return static_cast<long long>(q) * w + r * static_cast<unsigned>(w) / kNumWarps;
+}
+
+// Blocks per head of sequences b0 .. b0 + 31, one per lane, and their running sum.
+struct Scan {
+    int len, blocks, incl;
+};
+__device__ __forceinline__ Scan scan_32(const AttnParams& p, int b0, int lane) {
+    Scan s;
+    s.len = b0 + lane < p.n_seqs ? clamped_len(p.seq_lens, b0 + lane, p.capacity) : 0;
+    s.blocks = s.incl = (s.len + 31) >> 5;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int v = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += v;
-        }
-        if (target >= 0 && !found) {
-            const unsigned m = __ballot_sync(0xffffffffu, (base + incl) * p.n_kv_heads > target);
-            if (m) {
-                const int l = __ffs(m) - 1;
-                *b_out = b0 + l;
-                *before_out = base + __shfl_sync(0xffffffffu, incl - t, l);
-                found = true;
-            }
-        }
-        base += __shfl_sync(0xffffffffu, incl, 31);
+    for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, s.incl, o);
+        if (lane >= o) s.incl += v;
     }
-    return base;
+    return s;
+}
+
+// Whole warp: run w of the block list (the list has n_kv_heads times the per-head blocks of each sequence).  Returns its number of
+// blocks; where it is not 0, also the sequence of its first block, that one's length and blocks, and the block's number within the sequence.
+struct Run {
+    int n, b, len, nblk;
+    unsigned local;
+};
+__device__ __forceinline__ Run find_run(const AttnParams& p, int lane, int w) {
+    Run r{0, 0, 0, 0, 0};
+    Scan s = scan_32(p, 0, lane);
+    long long total = __shfl_sync(0xffffffffu, s.incl, 31);
+    for (int b0 = 32; b0 < p.n_seqs; b0 += 32) {
+        s = scan_32(p, b0, lane);
+        total += __shfl_sync(0xffffffffu, s.incl, 31);
+    }
+    total *= p.n_kv_heads;
+    const long long start = run_start(total, w);
+    r.n = static_cast<int>(run_start(total, w + 1) - start);
+    if (r.n <= 0) return r;
+    long long before = 0;
+    for (int b0 = 0; b0 < p.n_seqs; b0 += 32) {  // start < total: some lane finds it
+        if (p.n_seqs > 32) s = scan_32(p, b0, lane);  // else still at hand
+        const unsigned m = __ballot_sync(0xffffffffu, (before + s.incl) * p.n_kv_heads > start);
+        if (m) {
+            const int l = __ffs(m) - 1;
+            r.b = b0 + l;
+            r.len = __shfl_sync(0xffffffffu, s.len, l);
+            r.nblk = __shfl_sync(0xffffffffu, s.blocks, l);
+            before += __shfl_sync(0xffffffffu, s.incl, l) - r.nblk;
+            r.local = static_cast<unsigned>(start - before * p.n_kv_heads);
+            return r;
+        }
+        before += __shfl_sync(0xffffffffu, s.incl, 31);
+    }
+    r.n = 0;
+    return r;
 }
 
 struct Cursor {  // one block of the global list
@@ -146,17 +181,9 @@ __device__ __forceinline__ uint32_t pack_h2(float lo, float hi) {
 __device__ __forceinline__ uint32_t lds32(const uint8_t* p) { return *reinterpret_cast<const uint32_t*>(p); }
 __device__ __forceinline__ uint32_t lds16(const uint8_t* p) { return *reinterpret_cast<const uint16_t*>(p); }
 
-// Coefficient index behind entry e (k = 2c, 2c + 1, 2c + 8, 2c + 9) of contraction step j of the score product,
-// as the key-side extraction delivers them: step 0 is the 8-bit segment (bytes 4c..4c+3 of the position's 16),
-// steps 1-6 take two steps per 32-bit word c + 4i of the 4-bit codes (nibbles (0,4),(1,5) then (2,6),(3,7)),
-// step 7 the nibbles (0,2),(1,3) of half-word 24 + c.
-__device__ __forceinline__ int kdim(int j, int c, int e) {
-    if (j == 0) return 4 * c + e;
-    if (j == 7) return 112 + 4 * c + ((e & 1) << 1) + (e >> 1);
-    const int i = (j - 1) >> 1, sub = (j - 1) & 1;
-    return 16 + 8 * (c + 4 * i) + 2 * sub + ((e & 1) << 2) + (e >> 1);
-}
-
+// Coefficients behind the entries (k = 2c, 2c + 1, 2c + 8, 2c + 9) of a contraction step of the score product, as the key-side
+// extraction delivers them: step 0 is the 8-bit segment (bytes 4c..4c+3 of the position's 16), steps 1-6 take two steps per
+// 32-bit word c + 4i of the 4-bit codes (nibbles (0,4),(1,5) then (2,6),(3,7)), step 7 the nibbles (0,2),(1,3) of half-word 24 + c.
 struct ValueScale {  // per position: value scales times 2^-E (E: the block's exponent), zero-points
     float sn8, sn4, z8, z4;
 };
@@ -194,22 +221,16 @@ __global__ void __launch_bounds__(kWarps * 32, 1) attention_decode_kernel(const 
     griddep_launch_dependents();  // the merge kernel may be scheduled as SMs free up; it waits for this grid itself
 
     // ---- this warp's run of the global block list
-    const long long wg = static_cast<long long>(blockIdx.x) * kWarps + warp;
-    int b_first = 0;
-    long long before = 0;
-    const long long total = scan_blocks(p, lane, -1, &b_first, &before) * p.n_kv_heads;
-    const long long start = total * wg / kNumWarps, end = total * (wg + 1) / kNumWarps, n = end - start;
+    const int wg = blockIdx.x * kWarps + warp;
+    const Run run = find_run(p, lane, wg);
+    const int n = run.n;
     if (n <= 0) return;
-    scan_blocks(p, lane, start, &b_first, &before);
     Cursor cons;
-    cons.b = b_first;
-    cons.len = clamped_len(p.seq_lens, b_first, p.capacity);
-    cons.nblk = (cons.len + 31) >> 5;
-    {
-        const long long local = start - before * p.n_kv_heads;
-        cons.h = static_cast<int>(local / cons.nblk);
-        cons.blk = static_cast<int>(local - static_cast<long long>(cons.h) * cons.nblk);
-    }
+    cons.b = run.b;
+    cons.len = run.len;
+    cons.nblk = run.nblk;
+    cons.h = static_cast<int>(run.local / static_cast<unsigned>(run.nblk));
+    cons.blk = static_cast<int>(run.local) - cons.h * run.nblk;
     Cursor prod = cons;
     const int blocks_cap = p.capacity / RESQ_KV_BLOCK;
     auto issue = [&](int stage) {  // lane 0 copies the producer cursor's block; every lane moves the cursor
@@ -227,8 +248,23 @@ __global__ void __launch_bounds__(kWarps * 32, 1) attention_decode_kernel(const 
         }
         advance(prod, p);
     };
-    long long issued = 0;
-    for (; issued < n && issued < kStages; ++issued) issue(static_cast<int>(issued));
+    // Contiguous pieces of the lane's query row, dealt to the fragments below (as single halves they are 32 loads).  The first record's are
+    // asked for before the copies: behind 30 MB of them they arrive 2 us later.
+    uint2 q0, q7;
+    uint4 qw[3];
+    auto load_query = [&] {
+        q0 = q7 = make_uint2(0u, 0u);
+        qw[0] = qw[1] = qw[2] = make_uint4(0u, 0u, 0u, 0u);
+        if (g >= p.group) return;
+        const __half* qrow = p.q + (static_cast<long long>(cons.b) * p.n_kv_heads * p.group + cons.h * p.group + g) * kD;
+        q0 = *reinterpret_cast<const uint2*>(qrow + 4 * c);
+#pragma unroll
+        for (int i3 = 0; i3 < 3; ++i3) qw[i3] = *reinterpret_cast<const uint4*>(qrow + 16 + 8 * (c + 4 * i3));
+        q7 = *reinterpret_cast<const uint2*>(qrow + 112 + 4 * c);
+    };
+    load_query();
+    int issued = 0;
+    for (; issued < n && issued < kStages; ++issued) issue(issued);
 
     // capacity is positive; the compiler cannot know, so the four words stay in registers (see NibbleConsts)
     const uint32_t never = p.capacity < 0 ? 1u : 0u;
@@ -237,23 +273,30 @@ __global__ void __launch_bounds__(kWarps * 32, 1) attention_decode_kernel(const 
     float kq8[2], kq4[2], ko8[2], ko4[2], m_run[2], l[2], z8[2], z4[2], acc[8][4], ones8[4], ones4[4], wx8[2], wx4[2];
     bool fresh = true, ok = true;
     int rec_blk0 = 0;  // block of the (sequence, head) at which the current record began
-    long long i = 0;
-    int stage = 0;
+    int i = 0, stage = 0;
     uint32_t phase = 0;
     for (; i < n; ++i) {
         if (fresh) {  // a new (sequence, KV head): query fragments of its group, empty running state
             fresh = false;
             rec_blk0 = cons.blk;
-            const __half* qrow = p.q + (static_cast<long long>(cons.b) * p.n_kv_heads * p.group + cons.h * p.group + g) * kD;
+            if (i > 0) load_query();
             float s8 = 0.f, s4 = 0.f, o4 = 0.f;  // sums of q over the segments; offset-weighted sum of the 4-bit part
+            qf[0][0] = q0.x;
+            qf[0][1] = q0.y;
+            qf[7][0] = __byte_perm(q7.x, q7.y, 0x5410);
+            qf[7][1] = __byte_perm(q7.x, q7.y, 0x7632);
+#pragma unroll
+            for (int i3 = 0; i3 < 3; ++i3) {
+                qf[1 + 2 * i3][0] = __byte_perm(qw[i3].x, qw[i3].z, 0x5410);
+                qf[1 + 2 * i3][1] = __byte_perm(qw[i3].x, qw[i3].z, 0x7632);
+                qf[2 + 2 * i3][0] = __byte_perm(qw[i3].y, qw[i3].w, 0x5410);
+                qf[2 + 2 * i3][1] = __byte_perm(qw[i3].y, qw[i3].w, 0x7632);
+            }
 #pragma unroll
             for (int j = 0; j < 8; ++j)
 #pragma unroll
                 for (int hf = 0; hf < 2; ++hf) {
-                    __half2 v = __floats2half2_rn(0.f, 0.f);
-                    if (g < p.group) v = __halves2half2(qrow[kdim(j, c, 2 * hf)], qrow[kdim(j, c, 2 * hf + 1)]);
-                    qf[j][hf] = *reinterpret_cast<const uint32_t*>(&v);
-                    const float2 f = __half22float2(v);
+                    const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&qf[j][hf]));
                     if (j == 0) s8 += f.x + f.y;
                     else { s4 += f.x + f.y; o4 += (hf == 0 ? kOffLo : kOffHi) * (f.x + f.y); }  // entries 0-1 lo, 2-3 hi
                 }
@@ -458,8 +501,8 @@ __global__ void __launch_bounds__(kWarps * 32, 1) attention_decode_kernel(const 
         advance(cons, p);
     }
     if (!ok) {  // a wait ran out: let this warp's copies in flight land (bounded), then report
-        for (long long k = i; k < issued; ++k) {
-            const int stage = static_cast<int>(k % kStages);
+        for (int k = i; k < issued; ++k) {
+            const int stage = k % kStages;
             const uint32_t phase = static_cast<uint32_t>(k / kStages) & 1u;
             for (int spin = 0; spin < (1 << 20) && !mbar_try_wait(&full[stage], phase); ++spin) {}
         }
@@ -469,25 +512,22 @@ __global__ void __launch_bounds__(kWarps * 32, 1) attention_decode_kernel(const 
 
 // Merges the partial records of one (sequence, query head): out = sum_i 2^(m_i - M) o_i / sum_i 2^(m_i - M) l_i.
 // The warps that hold a record of this (sequence, KV head) are those whose runs meet its range of the block
-// list.  The CTA has 128 x G threads: candidates are taken blockDim at a time (thread t reads (m, l) of candidate
-// t, the block agrees on the maximum), then group g adds the weighted records g, g + G, ... eight at a time, one
-// output coefficient per thread, and the G partial sums are added in group order.  G = 4 when few (sequence, head)
-// pairs share the grid's warps (long contexts: hundreds of records each), else 1.  Launched so that it may start
+// list.  The CTA has 128 x G threads, one output coefficient each: group g takes records 16 g .. 16 g + 15, then those G * 16 on, and the
+// groups' sums meet in shared memory.  G = 4 when few (sequence, head)
+// pairs share the grid's warps (long contexts: hundreds of records each), else 1.  What bounds it is latency: a thread asks for its
+// coefficient and for reference and sum of sixteen records at once, a single trip to memory (with the references first, a vote on their
+// maximum and then the records: 5.1 us from the end of the wait to the last output, now 3.6).  Launched so that it may start
 // while the attention kernel drains: everything before griddepcontrol.wait reads only the sequence lengths, which are
 // complete (the attention kernel lets its dependents start after its own wait).
-constexpr int kMaxGroups = 4;
+constexpr int kMaxGroups = 4, kChunk = 16;
 __global__ void __launch_bounds__(kD * kMaxGroups) attention_combine_kernel(const AttnParams p) {
     __shared__ long long red[2][kD * kMaxGroups / 32];
-    __shared__ float redf[2][kD * kMaxGroups / 32];
-    extern __shared__ __align__(16) uint8_t merge_smem[];  // rec_s [nthr] long long, f_s [nthr] float, num_s [groups][128] float
+    __shared__ float part_s[kMaxGroups][kD], ml_s[kMaxGroups][2];  // of the groups
     const int n_q_heads = p.n_kv_heads * p.group;
     const int b = blockIdx.x / n_q_heads, hq = blockIdx.x - b * n_q_heads;
     const int hk = hq / p.group, hg = hq - hk * p.group;
-    const int tid = threadIdx.x, nthr = blockDim.x, nwarp = nthr >> 5, warp = tid >> 5;
+    const int tid = threadIdx.x, nthr = blockDim.x, nwarp = nthr >> 5, warp = tid >> 5, lane = tid & 31;
     const int d = tid & (kD - 1), grp = tid >> 7, groups = nthr >> 7;
-    long long* rec_s = reinterpret_cast<long long*>(merge_smem);
-    float* f_s = reinterpret_cast<float*>(rec_s + nthr);
-    float* num_s = f_s + nthr;
     long long before = 0, total = 0;
     for (int i = tid; i < p.n_seqs; i += nthr) {
         const int len = p.seq_lens[i];
@@ -502,13 +542,29 @@ __global__ void __launch_bounds__(kD * kMaxGroups) attention_combine_kernel(cons
         before += __shfl_xor_sync(0xffffffffu, before, o);
         total += __shfl_xor_sync(0xffffffffu, total, o);
     }
-    if ((tid & 31) == 0) { red[0][warp] = before; red[1][warp] = total; }
+    if (lane == 0) { red[0][warp] = before; red[1][warp] = total; }
     __syncthreads();
     before = total = 0;
     for (int w = 0; w < nwarp; ++w) { before += red[0][w]; total += red[1][w]; }
     total *= p.n_kv_heads;
     float* out = p.out + (static_cast<long long>(b) * n_q_heads + hq) * kD;
     const int nblk = (clamped_len(p.seq_lens, b, p.capacity) + 31) >> 5;
+    const long long lo = before * p.n_kv_heads + static_cast<long long>(hk) * nblk, hi = lo + nblk;  // [lo, hi)
+    int w_first = 0, w_last = 0;
+    if (nblk > 0) {
+        w_first = static_cast<int>(((lo + 1) * kNumWarps - 1) / total);
+        w_last = static_cast<int>((hi * kNumWarps - 1) / total);
+    }
+    auto records = [&](int w0) {  // which of the sixteen candidates from w0 on hold a record: non-empty runs that meet [lo, hi)
+        const int w = w0 + (lane & (kChunk - 1));
+        bool have = false;
+        if (w <= w_last) {
+            const long long rs = run_start(total, w), re = run_start(total, w + 1);
+            have = re > rs && re > lo && rs < hi;
+        }
+        return __ballot_sync(0xffffffffu, have);
+    };
+    unsigned mask = records(w_first + kChunk * grp);
     // Every CTA waits for the attention grid before it returns, also those with nothing to merge: this grid was
     // launched as a programmatic dependent, so the next kernel of the stream is ordered against THIS grid only,
     // and it must not retire while the attention grid is still writing `out`.
@@ -517,60 +573,53 @@ __global__ void __launch_bounds__(kD * kMaxGroups) attention_combine_kernel(cons
         if (grp == 0) out[d] = 0.f;
         return;
     }
-    const long long lo = before * p.n_kv_heads + static_cast<long long>(hk) * nblk, hi = lo + nblk;  // [lo, hi)
-    constexpr long long nw = kNumWarps;
-    const int w_first = static_cast<int>(((lo + 1) * nw - 1) / total), w_last = static_cast<int>((hi * nw - 1) / total);
     if (w_first == w_last) return;  // one warp saw the whole (sequence, head) and wrote the output itself
     const long long s = static_cast<long long>(b) * p.n_kv_heads + hk;
-    float M = -INFINITY, num = 0.f, den = 0.f;  // num: this group's share; den: a per-thread partial until the end
-    for (int w0 = w_first; w0 <= w_last; w0 += nthr) {
-        const int w = w0 + tid;
-        bool have = false;
-        if (w <= w_last) {  // a non-empty run that meets [lo, hi)
-            const long long rs = total * w / nw, re = total * (w + 1) / nw;
-            have = re > rs && re > lo && rs < hi;
-        }
-        const long long off = (w + s) * kRecFloats + hg * (kD + 2);
-        float m = -INFINITY, lw = 0.f;
-        if (have) { m = __ldcg(p.partial + off); lw = __ldcg(p.partial + off + 1); }
-        float mx = m;
+    float M = -INFINITY, num = 0.f, den = 0.f;  // this group's share
+    for (int w0 = w_first + kChunk * grp; w0 <= w_last;) {
+        const float* rec = p.partial + (w0 + s) * kRecFloats + hg * (kD + 2);
+        float2 ml[kChunk];
+        float v[kChunk];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        __syncthreads();  // the previous chunk's f_s / rec_s / redf are no longer read
-        if ((tid & 31) == 0) redf[0][warp] = mx;
-        __syncthreads();
-        float Mn = M;
-        for (int k = 0; k < nwarp; ++k) Mn = fmaxf(Mn, redf[0][k]);
-        const float resc = ex2(M - Mn);  // 0 on the first chunk
-        M = Mn;
-        const float f = have ? ex2(m - M) : 0.f;
-        f_s[tid] = f;
-        rec_s[tid] = have ? off + 2 : -1;
-        num *= resc;
-        den = fmaf(f, lw, den * resc);
-        __syncthreads();
-        const int cnt = min(nthr, w_last - w0 + 1);
-        for (int i0 = 8 * grp; i0 < cnt; i0 += 8 * groups) {
-            float v[8];
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                const long long r = i0 + k < cnt ? rec_s[i0 + k] : -1;
-                v[k] = r >= 0 ? __ldcg(p.partial + r + d) : 0.f;
+        for (int k = 0; k < kChunk; ++k) {
+            ml[k] = make_float2(-INFINITY, 0.f);
+            v[k] = 0.f;
+            if (mask >> k & 1u) {
+                ml[k] = __ldcg(reinterpret_cast<const float2*>(rec + k * kRecFloats));
+                v[k] = __ldcg(rec + k * kRecFloats + 2 + d);
             }
-#pragma unroll
-            for (int k = 0; k < 8; ++k) num = fmaf(i0 + k < cnt ? f_s[i0 + k] : 0.f, v[k], num);
         }
-    }
+        float Mn = M;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) den += __shfl_xor_sync(0xffffffffu, den, o);
-    __syncthreads();
-    if ((tid & 31) == 0) redf[1][warp] = den;
-    num_s[grp * kD + d] = num;
+        for (int k = 0; k < kChunk; ++k) Mn = fmaxf(Mn, ml[k].x);
+        const float resc = M == -INFINITY ? 0.f : ex2(M - Mn);
+        num *= resc;
+        den *= resc;
+        M = Mn;
+#pragma unroll
+        for (int k = 0; k < kChunk; ++k) {
+            const float f = mask >> k & 1u ? ex2(ml[k].x - Mn) : 0.f;
+            num = fmaf(f, v[k], num);
+            den = fmaf(f, ml[k].y, den);
+        }
+        w0 += kChunk * groups;
+        if (w0 <= w_last) mask = records(w0);
+    }
+    if (groups == 1) {
+        out[d] = num / den;
+        return;
+    }
+    part_s[grp][d] = num;
+    if (d == 0) { ml_s[grp][0] = M; ml_s[grp][1] = den; }
     __syncthreads();
     if (grp == 0) {
-        float dsum = 0.f, nsum = 0.f;
-        for (int k = 0; k < nwarp; ++k) dsum += redf[1][k];
-        for (int g = 0; g < groups; ++g) nsum += num_s[g * kD + d];
+        float Mn = M, nsum = 0.f, dsum = 0.f;
+        for (int g = 1; g < groups; ++g) Mn = fmaxf(Mn, ml_s[g][0]);
+        for (int g = 0; g < groups; ++g) {
+            const float f = ml_s[g][0] == -INFINITY ? 0.f : ex2(ml_s[g][0] - Mn);  // -INF: no record
+            nsum = fmaf(f, part_s[g][d], nsum);
+            dsum = fmaf(f, ml_s[g][1], dsum);
+        }
         out[d] = nsum / dsum;
     }
 }
@@ -614,7 +663,6 @@ cudaError_t launch_attention_decode(const resq_kv_cache_t& cache, const void* q1
     // few (sequence, head) pairs share the grid's warps: each has many records, so four groups of threads add them
     const int merge_threads = n_rows * cache.n_kv_heads <= 64 ? kD * kMaxGroups : kD;
     cfg.blockDim = dim3(merge_threads, 1, 1);
-    cfg.dynamicSmemBytes = static_cast<size_t>(merge_threads) * (sizeof(long long) + sizeof(float)) + (merge_threads / kD) * kD * sizeof(float);
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
