@@ -512,15 +512,17 @@ __global__ void __launch_bounds__(kWarps * 32, 1) attention_decode_kernel(const 
 
 // Merges the partial records of one (sequence, query head): out = sum_i 2^(m_i - M) o_i / sum_i 2^(m_i - M) l_i.
 // The warps that hold a record of this (sequence, KV head) are those whose runs meet its range of the block
-// list.  The CTA has 128 x G threads, one output coefficient each: group g takes records 16 g .. 16 g + 15, then those G * 16 on, and the
-// groups' sums meet in shared memory.  G = 4 when few (sequence, head)
-// pairs share the grid's warps (long contexts: hundreds of records each), else 1.  What bounds it is latency: a thread asks for its
-// coefficient and for reference and sum of sixteen records at once, a single trip to memory (with the references first, a vote on their
-// maximum and then the records: 5.1 us from the end of the wait to the last output, now 3.6).  Launched so that it may start
-// while the attention kernel drains: everything before griddepcontrol.wait reads only the sequence lengths, which are
+// list.  The CTA has 128 x G threads, an output coefficient each: group g adds records CHUNK g .. CHUNK (g + 1) - 1, then those
+// G * CHUNK on, and the groups' sums meet in shared memory.  G = 4 when few (sequence, head) pairs share the grid's warps (long contexts:
+// hundreds of records each), else 1.  What bounds it is latency: a thread asks for coefficient, reference and sum of a whole chunk of
+// records at once, a single trip to memory (with the references first, a vote on their maximum and then the records: 5.1 us from the
+// end of the wait to the last output, now 3.6; references by lanes and shuffles: slower).  CHUNK is what a pair has by the sizes: a chunk of 16
+// takes 103 registers, and with four CTAs per SM 8192 merges of two or three records take 5 us longer (74 us of a call) than with chunks of four.
+// Launched so that it may start while the attention kernel drains: everything before griddepcontrol.wait reads only the sequence lengths, which are
 // complete (the attention kernel lets its dependents start after its own wait).
-constexpr int kMaxGroups = 4, kChunk = 16;
-__global__ void __launch_bounds__(kD * kMaxGroups) attention_combine_kernel(const AttnParams p) {
+constexpr int kMaxGroups = 4;
+template <int CHUNK>
+__global__ void __launch_bounds__(kD * kMaxGroups, CHUNK == 4 ? 3 : 1) attention_combine_kernel(const AttnParams p) {
     __shared__ long long red[2][kD * kMaxGroups / 32];
     __shared__ float part_s[kMaxGroups][kD], ml_s[kMaxGroups][2];  // of the groups
     const int n_q_heads = p.n_kv_heads * p.group;
@@ -555,8 +557,8 @@ __global__ void __launch_bounds__(kD * kMaxGroups) attention_combine_kernel(cons
         w_first = static_cast<int>(((lo + 1) * kNumWarps - 1) / total);
         w_last = static_cast<int>((hi * kNumWarps - 1) / total);
     }
-    auto records = [&](int w0) {  // which of the sixteen candidates from w0 on hold a record: non-empty runs that meet [lo, hi)
-        const int w = w0 + (lane & (kChunk - 1));
+    auto records = [&](int w0) {  // which of the CHUNK candidates from w0 on hold a record: non-empty runs that meet [lo, hi)
+        const int w = w0 + (lane & (CHUNK - 1));
         bool have = false;
         if (w <= w_last) {
             const long long rs = run_start(total, w), re = run_start(total, w + 1);
@@ -564,7 +566,7 @@ __global__ void __launch_bounds__(kD * kMaxGroups) attention_combine_kernel(cons
         }
         return __ballot_sync(0xffffffffu, have);
     };
-    unsigned mask = records(w_first + kChunk * grp);
+    unsigned mask = w_first < w_last ? records(w_first + CHUNK * grp) : 0u;
     // Every CTA waits for the attention grid before it returns, also those with nothing to merge: this grid was
     // launched as a programmatic dependent, so the next kernel of the stream is ordered against THIS grid only,
     // and it must not retire while the attention grid is still writing `out`.
@@ -576,12 +578,12 @@ __global__ void __launch_bounds__(kD * kMaxGroups) attention_combine_kernel(cons
     if (w_first == w_last) return;  // one warp saw the whole (sequence, head) and wrote the output itself
     const long long s = static_cast<long long>(b) * p.n_kv_heads + hk;
     float M = -INFINITY, num = 0.f, den = 0.f;  // this group's share
-    for (int w0 = w_first + kChunk * grp; w0 <= w_last;) {
+    for (int w0 = w_first + CHUNK * grp; w0 <= w_last;) {
         const float* rec = p.partial + (w0 + s) * kRecFloats + hg * (kD + 2);
-        float2 ml[kChunk];
-        float v[kChunk];
+        float2 ml[CHUNK];
+        float v[CHUNK];
 #pragma unroll
-        for (int k = 0; k < kChunk; ++k) {
+        for (int k = 0; k < CHUNK; ++k) {
             ml[k] = make_float2(-INFINITY, 0.f);
             v[k] = 0.f;
             if (mask >> k & 1u) {
@@ -591,18 +593,18 @@ __global__ void __launch_bounds__(kD * kMaxGroups) attention_combine_kernel(cons
         }
         float Mn = M;
 #pragma unroll
-        for (int k = 0; k < kChunk; ++k) Mn = fmaxf(Mn, ml[k].x);
+        for (int k = 0; k < CHUNK; ++k) Mn = fmaxf(Mn, ml[k].x);
         const float resc = M == -INFINITY ? 0.f : ex2(M - Mn);
         num *= resc;
         den *= resc;
         M = Mn;
 #pragma unroll
-        for (int k = 0; k < kChunk; ++k) {
+        for (int k = 0; k < CHUNK; ++k) {
             const float f = mask >> k & 1u ? ex2(ml[k].x - Mn) : 0.f;
             num = fmaf(f, v[k], num);
             den = fmaf(f, ml[k].y, den);
         }
-        w0 += kChunk * groups;
+        w0 += CHUNK * groups;
         if (w0 <= w_last) mask = records(w0);
     }
     if (groups == 1) {
@@ -660,16 +662,16 @@ cudaError_t launch_attention_decode(const resq_kv_cache_t& cache, const void* q1
     if (cudaError_t e = launch_programmatic(attention_decode_kernel, 148, kWarps * 32, kSmem, st, p); e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(n_rows * n_q_heads, 1, 1);
-    // few (sequence, head) pairs share the grid's warps: each has many records, so four groups of threads add them
-    const int merge_threads = n_rows * cache.n_kv_heads <= 64 ? kD * kMaxGroups : kD;
-    cfg.blockDim = dim3(merge_threads, 1, 1);
+    const int pairs = n_rows * cache.n_kv_heads, records = kNumWarps / pairs + 2;  // of a pair, if all are equally long
+    // groups of threads for more than a chunk of them; four leave one CTA on an SM
+    cfg.blockDim = dim3(kD * (records <= 16 ? 1 : n_rows * n_q_heads <= 148 ? kMaxGroups : 2), 1, 1);
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, attention_combine_kernel, p);
+    return cudaLaunchKernelEx(&cfg, records <= 4 ? attention_combine_kernel<4> : records <= 9 ? attention_combine_kernel<8> : attention_combine_kernel<16>, p);
 }
 
 }  // namespace resq
