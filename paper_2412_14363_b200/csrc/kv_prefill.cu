@@ -36,7 +36,7 @@
 // flight are waited for, and TMEM is freed.
 //
 // What bounds it: the instructions of softmax and expansion (60 % of the issue slots, 63 at d = 64) and the latency of their chains.
-// us per step: d = 128, two tiles together 2.08, one tile 1.33; d = 64, one tile 1.87 (1.62 with the zero-points inside the values'
+// us per step: d = 128, two tiles together 2.03, one tile 1.33; d = 64, one tile 1.87 (1.62 with the zero-points inside the values'
 // parts).  The expansion sets the pace where its words are read, converted and written one by one; so all words are on their way
 // first, with addresses of a register and a constant.  Divisions by the group size took 5 us of a call, outputs stored row by row 2 us.
 // us, 32 query / 8 KV heads: d = 128, 2048 tokens behind 4096 400 -> 349 (1310 with one 128-row tile per CTA in two passes), 1000
@@ -91,7 +91,7 @@ struct Shared {
     float4 row_part[4][kRows];
     float warp_max[20];           // one per warp
     int bad8, bad4;  // the first position visited whose value constants of the 8-bit / 4-bit segment are infinite or NaN
-    uint64_t raw_full[2], kv_full[kStages], kv_empty[kStages], s_full[2], p_full[2], pv_done[2], drain;
+    uint64_t raw_full[2], kv_full[kStages], kv_empty[kStages], s_full[2], s_read[2], p_full[2], pv_done[2], drain;
     uint32_t tmem_base;
     int abort_flag;
 };
@@ -478,6 +478,7 @@ __global__ void __launch_bounds__(Geometry<D, WAYS, PAIR>::kThreads, 1) attentio
         for (int i = 0; i < 2; ++i) {
             mbar_init(&sh->raw_full[i], 1);
             mbar_init(&sh->s_full[i], 1);
+            mbar_init(&sh->s_read[i], G::kGroupWarps);
             mbar_init(&sh->p_full[i], G::kGroupWarps);
             mbar_init(&sh->pv_done[i], 1);
         }
@@ -650,6 +651,11 @@ __global__ void __launch_bounds__(Geometry<D, WAYS, PAIR>::kThreads, 1) attentio
                     if (masked) mx = step_scores<D, true>(sc, tmem_s + part * G::kPart, col_k, -m_use, last);
                     else mx = step_scores<D, false>(sc, tmem_s + part * G::kPart, col_k, -m_use, last);
                 }
+                if constexpr (PAIR) {  // the 4-bit segment's next scores may come: the weights go over the other's only
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&sh->s_read[buf0]);
+                }
                 // ---- raise the reference where a score leaves it too far behind (and set it at the first position seen).  Behind
                 // the barrier all warps of the rows have read the scores that the weights go over, and all leave if a wait of one failed
                 tc_fence_before();
@@ -821,24 +827,25 @@ __global__ void __launch_bounds__(Geometry<D, WAYS, PAIR>::kThreads, 1) attentio
             tc_fence_after();
             return ok;
         };
-        auto score_product = [&](int q_tile, int buf, int st, int bar) {
+        auto score_product = [&](int q_tile, int buf, int st, bool seg4, bool seg8) {  // of a segment or both
             const uint32_t idS = make_idesc_f16(kRows, kStep);
             const uint32_t q = smem_u32(Qs) + q_tile * H::kQBytes, k = smem_u32(stages) + st * H::kStageBytes;
             const uint64_t q0 = make_smem_desc_k128(q), k0 = make_smem_desc_k128(k), k1 = make_smem_desc_k128(k + H::kTile);
             const uint32_t d = tmem + buf * G::kBufCols;
             if constexpr (D == 128) {
                 const uint64_t q1 = make_smem_desc_k128(q + kRows * 128);
-                mma_f16_ss_if(leader, d, q0, k0, idS, 0);
+                if (seg8) mma_f16_ss_if(leader, d, q0, k0, idS, 0);
+                if (seg4) {
 #pragma unroll
-                for (int i = 1; i < 4; ++i) mma_f16_ss_if(leader, d + kColS4, q0 + 2 * i, k0 + 2 * i, idS, i > 1);
+                    for (int i = 1; i < 4; ++i) mma_f16_ss_if(leader, d + kColS4, q0 + 2 * i, k0 + 2 * i, idS, i > 1);
 #pragma unroll
-                for (int i = 0; i < 4; ++i) mma_f16_ss_if(leader, d + kColS4, q1 + 2 * i, k1 + 2 * i, idS, 1);
+                    for (int i = 0; i < 4; ++i) mma_f16_ss_if(leader, d + kColS4, q1 + 2 * i, k1 + 2 * i, idS, 1);
+                }
             } else {  // each segment's keys are 0 where the other's coefficients are
                 mma_f16_ss_if(leader, d, q0, k1, idS, 0);
 #pragma unroll
                 for (int i = 0; i < 4; ++i) mma_f16_ss_if(leader, d + kColS4, q0 + 2 * i, k0 + 2 * i, idS, i > 0);
             }
-            tc_commit_if(leader, &sh->s_full[bar]);
         };
         auto output_product = [&](int buf, int out, bool fresh, int st) {
             const uint32_t v = smem_u32(stages) + st * H::kStageBytes + H::kOffStageV4;
@@ -875,34 +882,46 @@ __global__ void __launch_bounds__(Geometry<D, WAYS, PAIR>::kThreads, 1) attentio
             }
         };
         // Scores go over the weights of an earlier output product, which has to be complete: two products are ordered by their issue only
-        // if they share accumulator and shape.  PAIR: a wait (2 % of a long walk).  Otherwise a stage has its score buffer, and its keys
+        // if they share accumulator and shape.  PAIR: the weights lie over the 8-bit segment's scores, so only that product, one
+        // instruction, waits for the output product; the 4-bit segment's follow as soon as the softmax has read the ones before, under
+        // its weights (2048 tokens behind 4096: 338.6 us; both products behind it 346.6).  Otherwise a stage has its score buffer, and its keys
         // are in place only after the output product of the step that had the stage before has freed it.
         int out_stage = 0;
         if constexpr (PAIR) {
             if (total_steps > 0 && keys_ready()) {
-                for (int t = 0; t < 2; ++t) score_product(t, t, stage, t);
+                for (int t = 0; t < 2; ++t) {
+                    score_product(t, t, stage, true, true);
+                    tc_commit_if(leader, &sh->s_full[t]);
+                }
                 next_stage();
             }
             for (int n = 0; n < total_steps && ok; ++n) {
+                const bool more = n + 1 < total_steps;
 #pragma unroll
                 for (int t = 0; t < 2; ++t) {
+                    if (more) {
+                        if (t == 0 && !keys_ready()) break;
+                        if (!wait(&sh->s_read[t], n & 1)) break;
+                        score_product(t, t, stage, true, false);
+                    }
                     if (!wait(&sh->p_full[t], n & 1)) break;
                     output_product(t, t, n == 0, out_stage);
                     tc_commit_if(leader, &sh->pv_done[t]);
                     if (t == 1) tc_commit_if(leader, &sh->kv_empty[out_stage]);
-                    if (n + 1 < total_steps) {
-                        if (t == 0 && !keys_ready()) break;
+                    if (more) {
                         if (!wait(&sh->pv_done[t], n & 1)) break;
-                        score_product(t, t, stage, t);
+                        score_product(t, t, stage, false, true);
+                        tc_commit_if(leader, &sh->s_full[t]);
                     }
                 }
                 if (++out_stage == kStages) out_stage = 0;
-                if (n + 1 < total_steps) next_stage();
+                if (more) next_stage();
             }
         } else {
             auto scores = [&](int N) {
                 if (!keys_ready()) return;
-                score_product(N >= tile0.n_steps, stage, stage, N & 1);
+                score_product(N >= tile0.n_steps, stage, stage, true, true);
+                tc_commit_if(leader, &sh->s_full[N & 1]);
                 next_stage();
             };
             for (int N = 0; N < min(2, total_steps) && ok; ++N) scores(N);
