@@ -827,25 +827,32 @@ __global__ void __launch_bounds__(Geometry<D, WAYS, PAIR>::kThreads, 1) attentio
             tc_fence_after();
             return ok;
         };
-        auto score_product = [&](int q_tile, int buf, int st, bool seg4, bool seg8) {  // of a segment or both
-            const uint32_t idS = make_idesc_f16(kRows, kStep);
+        const uint32_t idS = make_idesc_f16(kRows, kStep);
+        // the 4-bit segment's scores at d = 128, beside the weights
+        auto segment4_scores = [&](int q_tile, int buf, int st) {
+            const uint32_t q = smem_u32(Qs) + q_tile * H::kQBytes, k = smem_u32(stages) + st * H::kStageBytes;
+            const uint64_t q0 = make_smem_desc_k128(q), k0 = make_smem_desc_k128(k), k1 = make_smem_desc_k128(k + H::kTile);
+            const uint64_t q1 = make_smem_desc_k128(q + kRows * 128);
+            const uint32_t d = tmem + buf * G::kBufCols + kColS4;
+#pragma unroll
+            for (int i = 1; i < 4; ++i) mma_f16_ss_if(leader, d, q0 + 2 * i, k0 + 2 * i, idS, i > 1);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) mma_f16_ss_if(leader, d, q1 + 2 * i, k1 + 2 * i, idS, 1);
+        };
+        // the scores that the weights lie over (PAIR: the 8-bit segment's alone, behind the others), then all of them are announced
+        auto score_product = [&](int q_tile, int buf, int st, int bar) {
             const uint32_t q = smem_u32(Qs) + q_tile * H::kQBytes, k = smem_u32(stages) + st * H::kStageBytes;
             const uint64_t q0 = make_smem_desc_k128(q), k0 = make_smem_desc_k128(k), k1 = make_smem_desc_k128(k + H::kTile);
             const uint32_t d = tmem + buf * G::kBufCols;
             if constexpr (D == 128) {
-                const uint64_t q1 = make_smem_desc_k128(q + kRows * 128);
-                if (seg8) mma_f16_ss_if(leader, d, q0, k0, idS, 0);
-                if (seg4) {
-#pragma unroll
-                    for (int i = 1; i < 4; ++i) mma_f16_ss_if(leader, d + kColS4, q0 + 2 * i, k0 + 2 * i, idS, i > 1);
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) mma_f16_ss_if(leader, d + kColS4, q1 + 2 * i, k1 + 2 * i, idS, 1);
-                }
+                mma_f16_ss_if(leader, d, q0, k0, idS, 0);
+                if constexpr (!PAIR) segment4_scores(q_tile, buf, st);
             } else {  // each segment's keys are 0 where the other's coefficients are
                 mma_f16_ss_if(leader, d, q0, k1, idS, 0);
 #pragma unroll
                 for (int i = 0; i < 4; ++i) mma_f16_ss_if(leader, d + kColS4, q0 + 2 * i, k0 + 2 * i, idS, i > 0);
             }
+            tc_commit_if(leader, &sh->s_full[bar]);
         };
         auto output_product = [&](int buf, int out, bool fresh, int st) {
             const uint32_t v = smem_u32(stages) + st * H::kStageBytes + H::kOffStageV4;
@@ -890,8 +897,8 @@ __global__ void __launch_bounds__(Geometry<D, WAYS, PAIR>::kThreads, 1) attentio
         if constexpr (PAIR) {
             if (total_steps > 0 && keys_ready()) {
                 for (int t = 0; t < 2; ++t) {
-                    score_product(t, t, stage, true, true);
-                    tc_commit_if(leader, &sh->s_full[t]);
+                    segment4_scores(t, t, stage);
+                    score_product(t, t, stage, t);
                 }
                 next_stage();
             }
@@ -902,7 +909,7 @@ __global__ void __launch_bounds__(Geometry<D, WAYS, PAIR>::kThreads, 1) attentio
                     if (more) {
                         if (t == 0 && !keys_ready()) break;
                         if (!wait(&sh->s_read[t], n & 1)) break;
-                        score_product(t, t, stage, true, false);
+                        segment4_scores(t, t, stage);
                     }
                     if (!wait(&sh->p_full[t], n & 1)) break;
                     output_product(t, t, n == 0, out_stage);
@@ -910,8 +917,7 @@ __global__ void __launch_bounds__(Geometry<D, WAYS, PAIR>::kThreads, 1) attentio
                     if (t == 1) tc_commit_if(leader, &sh->kv_empty[out_stage]);
                     if (more) {
                         if (!wait(&sh->pv_done[t], n & 1)) break;
-                        score_product(t, t, stage, false, true);
-                        tc_commit_if(leader, &sh->s_full[t]);
+                        score_product(t, t, stage, t);
                     }
                 }
                 if (++out_stage == kStages) out_stage = 0;
@@ -920,8 +926,7 @@ __global__ void __launch_bounds__(Geometry<D, WAYS, PAIR>::kThreads, 1) attentio
         } else {
             auto scores = [&](int N) {
                 if (!keys_ready()) return;
-                score_product(N >= tile0.n_steps, stage, stage, true, true);
-                tc_commit_if(leader, &sh->s_full[N & 1]);
+                score_product(N >= tile0.n_steps, stage, stage, N & 1);
                 next_stage();
             };
             for (int N = 0; N < min(2, total_steps) && ok; ++N) scores(N);
