@@ -348,6 +348,12 @@ int resq_linear(const resq_layer_desc_t* d, int T, const void* X, const void* P,
     float* s_x8 = reinterpret_cast<float*>(ws + map.sx8);
     float* s_x4 = reinterpret_cast<float*>(ws + map.sx4);
     const bool tiles = T > kDecodeMaxT;
+    if (!P && !tiles) {  // few rows: quantized by the product itself where that is the shorter way
+        const cudaError_t e = launch_mixed_gemm_stream(T, d->n_out, d->K, d->r, nullptr, nullptr, nullptr, nullptr, W->w8, W->w4, W->s_w8, W->s_w4,
+                                                       d->w_scale_dtype == RESQ_SCALE_FP16, Y, y_dtype, nullptr, nullptr,
+                                                       static_cast<cudaStream_t>(stream), false, nullptr, nullptr, nullptr, nullptr, X);
+        if (e != cudaErrorNotSupported) return cuda_status(e);
+    }
     int8_t* x4e = tiles ? reinterpret_cast<int8_t*>(ws + map.x4e) : nullptr;
     // The tile kernel consumes the one-code-per-byte layout, the streaming kernel the packed one.
     if (int e = resq_project_quantize(X, P, T, d->K, d->r, x8, tiles ? nullptr : x4, s_x8, s_x4, x4e, ws + map.panel,
@@ -508,6 +514,12 @@ int resq_linear_asym(const resq_layer_desc_t* d, int T, const void* X, const voi
     float* s_x4 = reinterpret_cast<float*>(ws + map.sx4);
     float* z_x8 = reinterpret_cast<float*>(ws + map.zx8);
     float* z_x4 = reinterpret_cast<float*>(ws + map.zx4);
+    if (!P && T <= kDecodeMaxT) {  // few rows: quantized by the product itself where that is the shorter way
+        const cudaError_t e = launch_mixed_gemm_stream(T, d->n_out, d->K, d->r, nullptr, nullptr, nullptr, nullptr, W->w8, W->w4, W->s_w8, W->s_w4,
+                                                       d->w_scale_dtype == RESQ_SCALE_FP16, Y, y_dtype, nullptr, nullptr,
+                                                       static_cast<cudaStream_t>(stream), false, nullptr, nullptr, wsum8, wsum4, X);
+        if (e != cudaErrorNotSupported) return cuda_status(e);
+    }
     // Few tokens: the streaming kernel wants the packed codes as well (the tile kernel, its fallback, the others).
     uint8_t* u4 = T <= kDecodeMaxT ? reinterpret_cast<uint8_t*>(ws + map.x4) : nullptr;
     if (int e = resq_project_quantize_asym(X, P, T, d->K, d->r, u8, u4, s_x8, s_x4, z_x8, z_x4, u4e, ws + map.panel,

@@ -37,12 +37,18 @@
 // Overlap with the preceding kernel.  The weights do not depend on it, so with the launch attribute
 // for programmatic stream serialization every warp fills its ring at once and only then waits
 // (griddepcontrol.wait) for the activations.
+//
+// QUANT: the rows come as bf16 and every CTA quantizes all of them itself while its first weights are on their way, instead of reading the
+// codes that a kernel before this one wrote.  That kernel costs a launch on the host (2.4 us) and 2 to 3 us on the device, against
+// T K / 256 values per thread here.  A call of one token, 2048 x 3072: 6.6 -> 5.4 us on the device, 8.5 -> 5.8 on the host; where the rule lies: plans.h.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
 #include "internal.h"
+#include "plans.h"
 #include "ptx.cuh"
+#include "row_codes.cuh"
 
 namespace resq {
 namespace {
@@ -58,6 +64,7 @@ constexpr int kSmemLimit = 227 * 1024;
 constexpr int kControlBytes = kWarps > 8 ? 2048 : 1024;
 constexpr int kSlotInts = 2 * 2 * 128;  // [token group][acc8 | acc4][fragment element]: one shared item
 constexpr int kSlotBytes = kWarps * kSlotInts * 4;
+constexpr int kQuantChunks = 8;  // QUANT: chunks of eight values that a thread keeps
 constexpr uint32_t kHi = 0xF0F0F0F0u, kLo = 0x0F0F0F0Fu, kFlip = 0x08080808u;
 
 struct Params {
@@ -84,6 +91,7 @@ struct Params {
     int y_dtype;
     int32_t* dbg8;
     int32_t* dbg4;
+    const __nv_bfloat16* X;  // QUANT: the rows
     int* status;
     // Work split: CTA b owns units [b * uq + floor(b * urem / grid), ...): uq or uq + 1 of them; tab[0] / tab[1] hold the warps' run
     // boundaries (run_boundary) for those two sizes.
@@ -96,6 +104,8 @@ struct __align__(16) Control {
     int s_even[16];  // per token: sum of the even-position INT4 activation codes
     int arrived[kWarps];  // per slot: warps that have added their part
     int abort_flag;
+    float token[4][8];      // QUANT: scales (INT8, INT4) and zero-points of the tokens
+    float extrema[4][kWarps];  // QUANT: of a warp's share of a row: largest and smallest, INT8 and INT4 segment
     uint64_t act_bar[kWarps];  // per warp: completion of the bulk copies it issued to stage activation rows (packed staging only)
 };
 static_assert(sizeof(Control) <= kControlBytes, "control block");
@@ -160,11 +170,12 @@ inline int run_boundary(int w, int items, int c8, int c4) {
 //         activations then enter as their even / odd codes themselves (no factor 16), so
 //         acc4 = accO / 16 + accE - 8 * S_even[t], and the epilogue adds the zero-point terms
 //         z_x8[t] * s_w8[n] * wsum8[n] + z_x4[t] * s_w4[n] * wsum4[n].
-template <int TT, int CS, bool kSplit, bool ASYM>
+template <int TT, int CS, bool kSplit, bool ASYM, bool QUANT>
 __global__ void __launch_bounds__(kThreads, 1)
 mixed_gemm_stream_kernel(const __grid_constant__ CUtensorMap tmW8, const __grid_constant__ CUtensorMap tmW4,
                          const __grid_constant__ CUtensorMap tmH8, const __grid_constant__ CUtensorMap tmH4,
                          const Params p) {
+    static_assert(!QUANT || (TT == 1 && kSplit), "rows of up to 8 tokens, staged as split codes");
     extern __shared__ __align__(128) uint8_t smem[];
     constexpr int kChunkBytes = CS * 64;
     constexpr int kStageBytes = kItemRows * kChunkBytes;
@@ -254,17 +265,158 @@ mixed_gemm_stream_kernel(const __grid_constant__ CUtensorMap tmW8, const __grid_
     // (and g + 8) and holds the sums of tokens 2 tig, 2 tig + 1 (and + 8).  Their scales and zero-points:
     const bool a_ok = g < p.T, b_ok = TT == 2 && g + 8 < p.T;
     float sx8t[TT][2], sx4t[TT][2], zx8t[TT][2], zx4t[TT][2];
+    const float* s_x8 = QUANT ? ctl->token[0] : p.s_x8;
+    const float* s_x4 = QUANT ? ctl->token[1] : p.s_x4;
+    const float* z_x8 = QUANT ? ctl->token[2] : p.z_x8;
+    const float* z_x4 = QUANT ? ctl->token[3] : p.z_x4;
+    auto token_scales = [&] {
 #pragma unroll
-    for (int tt = 0; tt < TT; ++tt)
+        for (int tt = 0; tt < TT; ++tt)
 #pragma unroll
-        for (int e = 0; e < 2; ++e) {
-            const int t = 8 * tt + 2 * tig + e;
-            const bool t_ok = t < p.T;
-            sx8t[tt][e] = t_ok ? p.s_x8[t] : 0.f;
-            sx4t[tt][e] = t_ok ? p.s_x4[t] : 0.f;
-            zx8t[tt][e] = ASYM && t_ok ? p.z_x8[t] : 0.f;
-            zx4t[tt][e] = ASYM && t_ok ? p.z_x4[t] : 0.f;
+            for (int e = 0; e < 2; ++e) {
+                const int t = 8 * tt + 2 * tig + e;
+                const bool t_ok = t < p.T;
+                sx8t[tt][e] = t_ok ? s_x8[t] : 0.f;
+                sx4t[tt][e] = t_ok ? s_x4[t] : 0.f;
+                zx8t[tt][e] = ASYM && t_ok ? z_x8[t] : 0.f;
+                zx4t[tt][e] = ASYM && t_ok ? z_x4[t] : 0.f;
+            }
+    };
+    if constexpr (!QUANT) token_scales();
+    if constexpr (QUANT) {
+        // ---- codes of all rows from their bf16 values: a power of two of threads per row, the same in every CTA
+        const int K = p.r + 2 * p.row4, nchunks8 = K >> 3;
+        const int tpr = kThreads >> (p.T > 4 ? 3 : p.T > 2 ? 2 : p.T > 1 ? 1 : 0);  // threads of a row
+        const int t = threadIdx.x / tpr, j = threadIdx.x - t * tpr, wpr = tpr >> 5, w0 = t * wpr;
+        const bool live = t < p.T;
+        const void* row = p.X + static_cast<size_t>(live ? t : 0) * K;
+        Chunk<false> ch[kQuantChunks];
+#pragma unroll
+        for (int i = 0; i < kQuantChunks; ++i)
+            if (j + i * tpr < nchunks8) ch[i] = load_chunk<false>(row, j + i * tpr);
+        if (lane == 0) {  // the ring behind the rows' loads
+            for (int s = issued; s < first_burst; ++s) issue(s);
+            issued = first_burst;
         }
+        // zeros behind the data of a row, and the zero row
+        const int end8 = p.r, end4 = p.row4;
+        for (int i = 16 * threadIdx.x; i < p.T * p.pitch8; i += 16 * kThreads)
+            if (i % p.pitch8 >= end8) *reinterpret_cast<uint4*>(act8 + i) = make_uint4(0, 0, 0, 0);
+        for (int i = 16 * threadIdx.x; i < p.T * p.pitch4; i += 16 * kThreads)
+            if (i % p.pitch4 >= end4) {
+                *reinterpret_cast<uint4*>(act4 + i) = make_uint4(0, 0, 0, 0);
+                *reinterpret_cast<uint4*>(act4 + static_cast<size_t>(TR) * p.pitch4 + i) = make_uint4(0, 0, 0, 0);
+            }
+        if (TR > p.T) {
+            for (int i = 16 * threadIdx.x; i < p.pitch8; i += 16 * kThreads) *reinterpret_cast<uint4*>(act8 + p.T * p.pitch8 + i) = make_uint4(0, 0, 0, 0);
+            for (int i = 16 * threadIdx.x; i < p.pitch4; i += 16 * kThreads) {
+                *reinterpret_cast<uint4*>(act4 + p.T * p.pitch4 + i) = make_uint4(0, 0, 0, 0);
+                *reinterpret_cast<uint4*>(act4 + static_cast<size_t>(TR + p.T) * p.pitch4 + i) = make_uint4(0, 0, 0, 0);
+            }
+        }
+        if (threadIdx.x < 16) ctl->s_even[threadIdx.x] = 0;
+        // ---- the largest magnitude of the two segments (hi8, hi4), or their ranges ([lo8, hi8], [lo4, hi4])
+        constexpr float kBig = 3.402823466e38f;
+        float hi8 = ASYM ? -kBig : 0.f, hi4 = hi8, lo8 = kBig, lo4 = kBig;
+        if constexpr (ASYM) {
+            const uint32_t big = 0x7F7F7F7Fu, small = 0xFF7FFF7Fu;  // the largest finite bf16, and its negative
+            __nv_bfloat162 l8 = *reinterpret_cast<const __nv_bfloat162*>(&big), h8 = *reinterpret_cast<const __nv_bfloat162*>(&small);
+            __nv_bfloat162 l4 = l8, h4 = h8;
+#pragma unroll
+            for (int i = 0; i < kQuantChunks; ++i) {
+                const int c = j + i * tpr;
+                if (c >= nchunks8) continue;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const __nv_bfloat162 x = *reinterpret_cast<const __nv_bfloat162*>(&ch[i].w[k]);
+                    if (8 * c < p.r) {
+                        l8 = __hmin2(l8, x);
+                        h8 = __hmax2(h8, x);
+                    } else {
+                        l4 = __hmin2(l4, x);
+                        h4 = __hmax2(h4, x);
+                    }
+                }
+            }
+            lo8 = fminf(__low2float(l8), __high2float(l8)); hi8 = fmaxf(__low2float(h8), __high2float(h8));
+            lo4 = fminf(__low2float(l4), __high2float(l4)); hi4 = fmaxf(__low2float(h4), __high2float(h4));
+        } else {
+#pragma unroll
+            for (int i = 0; i < kQuantChunks; ++i) {
+                const int c = j + i * tpr;
+                if (c >= nchunks8) continue;
+                const float m = chunk_absmax(ch[i]);
+                if (8 * c < p.r) hi8 = fmaxf(hi8, m);
+                else hi4 = fmaxf(hi4, m);
+            }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            hi8 = fmaxf(hi8, __shfl_xor_sync(0xffffffffu, hi8, o));
+            hi4 = fmaxf(hi4, __shfl_xor_sync(0xffffffffu, hi4, o));
+            if (ASYM) {
+                lo8 = fminf(lo8, __shfl_xor_sync(0xffffffffu, lo8, o));
+                lo4 = fminf(lo4, __shfl_xor_sync(0xffffffffu, lo4, o));
+            }
+        }
+        if (lane == 0) {
+            ctl->extrema[0][warp] = hi8;
+            ctl->extrema[1][warp] = hi4;
+            ctl->extrema[2][warp] = lo8;
+            ctl->extrema[3][warp] = lo4;
+        }
+        __syncthreads();
+        for (int w = w0; w < w0 + wpr; ++w) {
+            hi8 = fmaxf(hi8, ctl->extrema[0][w]);
+            hi4 = fmaxf(hi4, ctl->extrema[1][w]);
+            if (ASYM) {
+                lo8 = fminf(lo8, ctl->extrema[2][w]);
+                lo4 = fminf(lo4, ctl->extrema[3][w]);
+            }
+        }
+        if (ASYM && p.r == 0) lo8 = hi8 = 0.f;  // an empty INT8 segment has s = 0, z = 0
+        const float s8 = ASYM ? __fdiv_rn(__fsub_rn(hi8, lo8), 255.f) : __fdiv_rn(hi8, 127.f);
+        const float s4 = ASYM ? __fdiv_rn(__fsub_rn(hi4, lo4), 15.f) : __fdiv_rn(hi4, 7.f);
+        const ScaleInv i8(s8), i4(s4);
+        if (live && j == 0) {
+            ctl->token[0][t] = s8;
+            ctl->token[1][t] = s4;
+            ctl->token[2][t] = lo8;
+            ctl->token[3][t] = lo4;
+        }
+        int even = 0;
+#pragma unroll
+        for (int i = 0; i < kQuantChunks; ++i) {
+            const int c = j + i * tpr;
+            if (c >= nchunks8 || !live) continue;
+            const bool seg8 = 8 * c < p.r;
+            const float s = seg8 ? s8 : s4, z = seg8 ? lo8 : lo4;
+            const ScaleInv& si = seg8 ? i8 : i4;
+            uint32_t q[8];
+            if (s > 0.f) {
+                if constexpr (ASYM) fast_codes_asym(ch[i], z, s, si.inv, si.exact, seg8 ? 255.f : 15.f, q);
+                else fast_codes(ch[i], s, si.inv, si.exact, q);
+            } else {
+#pragma unroll
+                for (int k = 0; k < 8; ++k) q[k] = 0;
+            }
+            if (seg8) {
+                *reinterpret_cast<uint2*>(act8 + static_cast<size_t>(t) * p.pitch8 + 8 * c) =
+                    make_uint2(pack_low_bytes(q[0], q[1], q[2], q[3]), pack_low_bytes(q[4], q[5], q[6], q[7]));
+            } else {  // codes 2 j and 2 j + 1 of byte j apart, as the products take them
+                uint32_t e = pack_low_bytes(q[0], q[2], q[4], q[6]), o = pack_low_bytes(q[1], q[3], q[5], q[7]);
+                e = ASYM ? e & kLo : (e << 4) & kHi;
+                o = ASYM ? o & kLo : (o << 4) & kHi;
+                uint8_t* dst = act4 + static_cast<size_t>(t) * p.pitch4 + ((8 * c - p.r) >> 1);
+                *reinterpret_cast<uint32_t*>(dst) = e;
+                *reinterpret_cast<uint32_t*>(dst + static_cast<size_t>(TR) * p.pitch4) = o;
+                even = __dp4a(static_cast<int>(e), 0x01010101, even);
+            }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) even += __shfl_xor_sync(0xffffffffu, even, o);
+        if (lane == 0 && live) atomicAdd(&ctl->s_even[t], ASYM ? even : even >> 4);  // signed codes: the lanes held 16 x the codes
+    } else
     // Stage the activation codes of the T tokens, zero padded to the pitch (the weights arrive as zeros there, but an
     // even INT4 weight code enters the product as code + 8), and the zero row.  The first batch of INT8 and
     // of INT4 vectors is loaded before anything is stored (one round trip to L2 for the usual sizes); the rest of
@@ -425,6 +577,7 @@ mixed_gemm_stream_kernel(const __grid_constant__ CUtensorMap tmW8, const __grid_
         }
     }
     __syncthreads();
+    if constexpr (QUANT) token_scales();
     bool ok = true;
     if constexpr (!kSplit) {  // the staged rows have landed
 #pragma unroll 1
@@ -669,9 +822,9 @@ bool make_map_rows(CUtensorMap* m, const void* base, uint64_t rows, uint64_t row
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int TT, int CS, bool SPLIT, bool ASYM>
+template <int TT, int CS, bool SPLIT, bool ASYM, bool QUANT = false>
 cudaError_t launch_variant(const CUtensorMap (&tm)[4], const Params& p, int grid, size_t smem, cudaStream_t st) {
-    auto kern = mixed_gemm_stream_kernel<TT, CS, SPLIT, ASYM>;
+    auto kern = mixed_gemm_stream_kernel<TT, CS, SPLIT, ASYM, QUANT>;
     static bool attr_set[64] = {};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -752,14 +905,15 @@ cudaError_t launch_mixed_gemm_stream(int T, int N, int K, int r, const int8_t* x
                                      const float* s_x8, const float* s_x4, const int8_t* w8, const uint8_t* w4,
                                      const void* s_w8, const void* s_w4, bool w_scale_fp16, void* Y, int y_dtype,
                                      int32_t* dbg8, int32_t* dbg4, cudaStream_t st, bool after_quantizer,
-                                     const float* z_x8, const float* z_x4, const int32_t* wsum8, const int32_t* wsum4) {
-    const bool asym = z_x8 != nullptr;  // then x8 / x4 hold unsigned codes
+                                     const float* z_x8, const float* z_x4, const int32_t* wsum8, const int32_t* wsum4,
+                                     const void* X) {
+    const bool asym = wsum8 != nullptr;  // then x8 / x4 hold unsigned codes
     int dev = 0, sms = 148;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const Plan pl = make_plan(T, N, K, r, sms);
-    if (!pl.ok) return cudaErrorNotSupported;
+    if (!pl.ok || (X && !(pl.TT == 1 && pl.split && quantizes_rows(T, K)))) return cudaErrorNotSupported;
     Params p;
     p.T = T; p.N = N; p.r = r; p.row4 = (K - r) / 2;
     p.TR = pl.TR;
@@ -772,6 +926,7 @@ cudaError_t launch_mixed_gemm_stream(int T, int N, int K, int r, const int8_t* x
     p.w_fp16 = w_scale_fp16 ? 1 : 0;
     p.z_x8 = z_x8; p.z_x4 = z_x4; p.wsum8 = wsum8; p.wsum4 = wsum4;
     p.Y = Y; p.y_dtype = y_dtype; p.dbg8 = dbg8; p.dbg4 = dbg8 ? dbg4 : nullptr;
+    p.X = static_cast<const __nv_bfloat16*>(X);
     p.status = device_status_ptr();
 
     // Maps: [0], [1] INT8 / INT4 weights with the 16-row box of an item, [2], [3] the same with the 8-row box of a
@@ -786,6 +941,13 @@ cudaError_t launch_mixed_gemm_stream(int T, int N, int K, int r, const int8_t* x
     } else {
         t8 = t4;  // uniform INT4: no INT8 chunks are ever requested
         tm[2] = tm[3];
+    }
+    if (X) {
+        if (pl.cs == 5)
+            return asym ? launch_variant<1, 5, true, true, true>(tm, p, pl.grid, pl.smem, st)
+                        : launch_variant<1, 5, true, false, true>(tm, p, pl.grid, pl.smem, st);
+        return asym ? launch_variant<1, 3, true, true, true>(tm, p, pl.grid, pl.smem, st)
+                    : launch_variant<1, 3, true, false, true>(tm, p, pl.grid, pl.smem, st);
     }
     const int variant = (pl.TT == 2 ? 4 : 0) + (pl.cs == 5 ? 2 : 0) + pl.split;
 #define RESQ_STREAM_CASE(v, tt, c, sp)                                                               \

@@ -92,8 +92,9 @@ cudaError_t launch_mixed_gemm_stream(int T, int N, int K, int r, const int8_t* x
                                      const void* s_w8, const void* s_w4, bool w_scale_fp16, void* Y, int y_dtype,
                                      int32_t* dbg8, int32_t* dbg4, cudaStream_t st, bool after_quantizer = false,
                                      const float* z_x8 = nullptr, const float* z_x4 = nullptr,
-                                     const int32_t* wsum8 = nullptr, const int32_t* wsum4 = nullptr);
-// z_x8 != NULL: asymmetric, unsigned codes.  after_quantizer: the kernel enqueued just before is one of the row
+                                     const int32_t* wsum8 = nullptr, const int32_t* wsum4 = nullptr, const void* X = nullptr);
+// wsum8 != NULL: asymmetric, unsigned codes.  X != NULL: the bf16 rows, which the kernel quantizes itself (x8 .. s_x4, z_x8, z_x4 are not
+// read); cudaErrorNotSupported, with nothing launched, where its rule leaves that to a quantizer.  after_quantizer: the kernel enqueued just before is one of the row
 // quantizers above, which lets a dependent start only once everything before IT is complete: the weights may be streamed
 // while it runs.
 void set_decode_early_weights(int on);

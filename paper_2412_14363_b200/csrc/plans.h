@@ -48,6 +48,16 @@ inline MidPlan mid_plan(int T, int N, int kbt) {
     return pl;
 }
 
+// ---- products of up to eight tokens (decode_stream.cu): whether every CTA quantizes the rows itself.  A row's share of the CTA's threads keeps
+// its values in registers: up to 64 each, where all or half of the threads share a row, else 32.  us on the device, a quantizer before / in the
+// product (K x N, symmetric): one row 1024 x 1024 6.8 / 4.8, 2048 x 3072 6.6 / 5.4, 4096 x 28672 14.1 / 13.2, 14336 x 4096 12.1 / 10.7; two rows
+// 2048 x 3072 6.9 / 6.0, 8192 x 8192 12.2 / 11.9; four rows 2048 x 3072 7.3 / 6.7, but 4096 x 6144 9.0 / 9.8; six rows 1024 x 1024 6.6 / 6.4, but
+// 2048 x 3072 7.4 / 8.2.
+inline bool quantizes_rows(int T, int K) {
+    const int threads = T > 4 ? 32 : T > 2 ? 64 : T > 1 ? 128 : 256;  // of a row
+    return T <= 8 && K <= (T > 2 ? 32 : 64) * threads;
+}
+
 // ---- GPTQ packing (gptq.cu): rows per CTA, one CTA per SM.  As many as fit its shared memory (8 bytes per weight), then no
 // more than spread the rows evenly over the rounds this takes.
 constexpr int kGptqMaxRows = 8;                 // one rounding warp each

@@ -11,56 +11,13 @@
 #include "internal.h"
 #include "packed_fp32.cuh"
 #include "ptx.cuh"
+#include "row_codes.cuh"
 
 namespace resq {
 namespace {
 
 constexpr int kThreads = 256;
 constexpr int kMaxChunks = 8;  // register-cached chunks per thread: rows up to 8*8*256 = 16384 wide
-
-// A chunk is kept in registers in its storage format: 4 words of bf16 pairs, or 8 fp32 words.
-template <bool F32>
-struct Chunk {
-    uint32_t w[F32 ? 8 : 4];
-    __device__ __forceinline__ float get(int i) const {
-        if constexpr (F32) return __uint_as_float(w[i]);
-        else return (i & 1) ? __uint_as_float(w[i >> 1] & 0xFFFF0000u) : __uint_as_float(w[i >> 1] << 16);
-    }
-};
-
-template <bool F32>
-__device__ __forceinline__ Chunk<F32> load_chunk(const void* row, int c) {
-    Chunk<F32> o;
-    if constexpr (F32) {
-        const uint4* p = reinterpret_cast<const uint4*>(row) + 2 * c;
-        uint4 a = p[0], b = p[1];
-        o.w[0] = a.x; o.w[1] = a.y; o.w[2] = a.z; o.w[3] = a.w;
-        o.w[4] = b.x; o.w[5] = b.y; o.w[6] = b.z; o.w[7] = b.w;
-    } else {
-        uint4 u = reinterpret_cast<const uint4*>(row)[c];
-        o.w[0] = u.x; o.w[1] = u.y; o.w[2] = u.z; o.w[3] = u.w;
-    }
-    return o;
-}
-
-template <bool F32>
-__device__ __forceinline__ float chunk_absmax(const Chunk<F32>& c) {
-    if constexpr (F32) {
-        float m = 0.f;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) m = fmaxf(m, fabsf(c.get(i)));
-        return m;
-    } else {
-        // bf16 pairs: clear the signs, then compare as packed bf16 (exact: max selects one of its inputs)
-        __nv_bfloat162 m = __floats2bfloat162_rn(0.f, 0.f);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const uint32_t a = c.w[i] & 0x7FFF7FFFu;
-            m = __hmax2(m, *reinterpret_cast<const __nv_bfloat162*>(&a));
-        }
-        return fmaxf(__low2float(m), __high2float(m));
-    }
-}
 
 // code = clamp(round-half-even(x / s)); IEEE division, no reciprocal.
 __device__ __forceinline__ int quant1(float x, float s, float lo, float hi) {
@@ -178,19 +135,9 @@ split_quantize_kernel(const void* __restrict__ in, size_t in_row_bytes, size_t r
 // flight at once and several CTAs per SM keep HBM busy while others compute.  Each row is then read
 // twice from shared memory: once for the two absmax values, once for the codes.
 //
-// Rounding.  The definition is code = round-half-even(fl(x / s)) with an IEEE division.  Here
-// t = fma(x, v, M) with M = 1.5 * 2^23 rounds the exact product x * v to the nearest integer (ties to
-// even) in one instruction, and the low byte of t's bit pattern is the two's-complement code.  It is
-// evaluated for two factors that bracket 1 / s, v_lo = RN(inv (1 - 2^-20)) and v_hi = RN(inv (1 + 2^-20))
-// with inv = RN(1 / s): fl(x / s) lies between x * v_lo and x * v_hi (the division and the reciprocal
-// are each off by at most 2^-24 relative, the bracket is 2^-21 wide at least on either side), rounding to
-// nearest is monotone, so when both products round to the same integer, that integer is the defined code;
-// when they differ (the quotient is within |x / s| * 2^-19 of a half-integer, ties included) the chunk is
-// redone with the true division.
+// Rounding: row_codes.cuh.
 constexpr int kFastGroupBytes = 32 * 1024;
 constexpr int kFastMaxRowBytes = 200 * 1024;
-constexpr float kMagic = 12582912.f;                    // 1.5 * 2^23
-constexpr float kBracket = 9.5367431640625e-07f;        // 2^-20
 
 template <bool F32>
 __device__ __forceinline__ Chunk<F32> lds_chunk(const uint8_t* row, int c) {
@@ -205,58 +152,6 @@ __device__ __forceinline__ Chunk<F32> lds_chunk(const uint8_t* row, int c) {
         o.w[0] = u.x; o.w[1] = u.y; o.w[2] = u.z; o.w[3] = u.w;
     }
     return o;
-}
-
-template <bool F32>
-__device__ __forceinline__ void fast_codes(const Chunk<F32>& ch, float s, float inv, bool exact_only, uint32_t (&t)[8]) {
-    const float v_lo = fmaf(inv, -kBracket, inv), v_hi = fmaf(inv, kBracket, inv);
-    const f2 vl = pack2(v_lo, v_lo), vh = pack2(v_hi, v_hi), magic = pack2(kMagic, kMagic);
-    uint32_t differ = 0;
-#pragma unroll
-    for (int i = 0; i < 8; i += 2) {
-        const f2 x = pack2(ch.get(i), ch.get(i + 1));
-        const float2 a = unpack2(fma2(x, vl, magic)), b = unpack2(fma2(x, vh, magic));
-        t[i] = __float_as_uint(a.x);
-        t[i + 1] = __float_as_uint(a.y);
-        differ |= t[i] ^ __float_as_uint(b.x);
-        differ |= t[i + 1] ^ __float_as_uint(b.y);
-    }
-    if (exact_only || differ != 0) {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) t[i] = __float_as_uint(rintf(__fdiv_rn(ch.get(i), s)) + kMagic);
-    }
-}
-
-// The asymmetric form (Eq. 1, second form): code = round-half-even(fl(fl(x - z) / s)) clamped to [0, qmax].  The same
-// bracket around 1 / s on d = fl(x - z): quotients reach 255, where a bracketed product still rounds to an integer in one
-// fma and the argument above is about relative errors only.
-template <bool F32>
-__device__ __forceinline__ void fast_codes_asym(const Chunk<F32>& ch, float z, float s, float inv, bool exact_only, float qmax,
-                                                uint32_t (&t)[8]) {
-    const float v_lo = fmaf(inv, -kBracket, inv), v_hi = fmaf(inv, kBracket, inv);
-    const f2 vl = pack2(v_lo, v_lo), vh = pack2(v_hi, v_hi), magic = pack2(kMagic, kMagic), mz = pack2(-z, -z);
-    uint32_t differ = 0;
-    float d[8];
-#pragma unroll
-    for (int i = 0; i < 8; i += 2) {
-        const f2 x = add2(pack2(ch.get(i), ch.get(i + 1)), mz);
-        const float2 u = unpack2(x), a = unpack2(fma2(x, vl, magic)), b = unpack2(fma2(x, vh, magic));
-        d[i] = u.x;
-        d[i + 1] = u.y;
-        t[i] = __float_as_uint(a.x);
-        t[i + 1] = __float_as_uint(a.y);
-        differ |= t[i] ^ __float_as_uint(b.x);
-        differ |= t[i + 1] ^ __float_as_uint(b.y);
-    }
-    if (exact_only || differ != 0) {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) t[i] = __float_as_uint(fminf(fmaxf(rintf(__fdiv_rn(d[i], s)), 0.f), qmax) + kMagic);
-    }
-}
-
-// Low bytes of four words -> one word.
-__device__ __forceinline__ uint32_t pack_low_bytes(uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
-    return __byte_perm(__byte_perm(a, b, 0x0040), __byte_perm(c, d, 0x0040), 0x5410);
 }
 
 // ASYM: asymmetric codes (unsigned), with the zero-points z8_out / z4_out; else symmetric ones.
@@ -434,10 +329,9 @@ split_quantize_fast_kernel(const void* in, size_t in_row_bytes, size_t rows, int
             if (ASYM && rchunks == 0) lo8 = a8 = 0.f;  // uniform 4-bit layer: the empty INT8 segment has s = 0, z = 0
             const float s8 = ASYM ? __fdiv_rn(__fsub_rn(a8, lo8), 255.f) : __fdiv_rn(a8, 127.f);
             const float s4 = ASYM ? __fdiv_rn(__fsub_rn(a4, lo4), 15.f) : __fdiv_rn(a4, 7.f);
-            const float inv8 = s8 > 0.f ? __frcp_rn(s8) : 0.f, inv4 = s4 > 0.f ? __frcp_rn(s4) : 0.f;
-            // The product form needs a finite, normal reciprocal; otherwise every chunk takes the division.
-            const bool exact8 = s8 > 0.f && !(inv8 >= 1.1754944e-38f && inv8 <= 3.0e38f);
-            const bool exact4 = s4 > 0.f && !(inv4 >= 1.1754944e-38f && inv4 <= 3.0e38f);
+            const ScaleInv i8(s8), i4(s4);
+            const float inv8 = i8.inv, inv4 = i4.inv;
+            const bool exact8 = i8.exact, exact4 = i4.exact;
             if (j == 0) {
                 s8_out[row] = s8;
                 s4_out[row] = s4;

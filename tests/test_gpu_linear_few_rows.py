@@ -1,0 +1,61 @@
+"""resq_linear and resq_linear_asym of up to eight tokens, whose rows the product quantizes itself: the bits of the row quantizer and the
+product in two calls, at the edges of the rule, with rows that are zero, constant, half-way between codes, infinite or NaN."""
+import pytest
+import torch
+
+from tests import plans
+
+
+def test_rule_for_quantizing_rows():
+    for T, widest in ((1, 16384), (2, 8192), (3, 2048), (4, 2048), (5, 1024), (8, 1024)):
+        assert plans.quantizes_rows(T, widest) and not plans.quantizes_rows(T, widest + 32), T
+    assert not plans.quantizes_rows(9, 64)
+
+
+def _rows(T, K, g):
+    x = torch.randn(T, K, device="cuda", generator=g) * torch.exp2(torch.randint(-6, 7, (T, 1), device="cuda", generator=g))
+    x[:, :: 97] *= 20
+    return x.to(torch.bfloat16)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("asym", [False, True])
+@pytest.mark.parametrize("T,K,r,N", [
+    (1, 2048, 256, 3072), (1, 64, 32, 8), (1, 16384, 2048, 1024), (1, 16416, 2048, 64),  # the last: a quantizer of its own
+    (2, 8192, 1024, 264), (2, 4096, 0, 40), (2, 8224, 32, 8), (3, 2048, 256, 2000), (4, 2048, 2016, 1184), (4, 2080, 32, 64), (5, 1024, 128, 2048),
+    (6, 1056, 32, 136), (6, 992, 32, 136), (7, 800, 224, 3072), (8, 1024, 256, 6144), (8, 512, 0, 8), (9, 1024, 256, 512)])
+def test_linear_of_few_rows(T, K, r, N, asym):
+    import paper_2412_14363_b200 as resq
+
+    g = torch.Generator(device="cuda").manual_seed(T * K + r)
+    desc = resq.layer_desc(K, N, r, resq.SCALE_FP16 if T % 2 else resq.SCALE_FP32)
+    W = resq.resq_pack_weights(desc, torch.randn(N, K, device="cuda", generator=g), with_w4_i8=asym)
+    wsum = resq.resq_weight_row_sums(W) if asym else None
+    ws = (resq.alloc_workspace_asym if asym else resq.alloc_workspace)(desc, T, False, asym)
+    X = _rows(T, K, g)
+    forms = [X, X.clone(), X.clone()]
+    forms[1][0] = 0
+    forms[1][-1, r:] = 3.0                                       # a constant segment
+    forms[1][T // 2] = (torch.arange(K, device="cuda") % 15 - 7) * 0.5  # quotients on half-integers
+    forms[1][T // 2, 0] = 7
+    forms[2][0, K // 2] = float("inf")
+    forms[2][-1, K - 1] = float("nan")
+    z = lambda n, dt=torch.float32: torch.zeros(n, dtype=dt, device="cuda")
+    for X in forms:
+        for dt in (torch.bfloat16, torch.float32):
+            Y, want = (torch.full((T, N), 5.0, dtype=dt, device="cuda") for _ in range(2))
+            s = [z(T) for _ in range(4)]
+            x4 = z((T, (K - r) // 2), torch.uint8)
+            if asym:
+                resq.resq_linear_asym(W, *wsum, X, None, Y, ws)
+                u8 = z((T, max(r, 1)), torch.uint8) if r else None
+                resq.resq_project_quantize_asym(X, None, r, u8, x4, *s)
+                resq.resq_mixed_gemm_asym(W, *wsum, u8, x4, *s, want, ws)
+            else:
+                resq.resq_linear(W, X, None, Y, ws)
+                x8 = z((T, r), torch.int8) if r else None
+                resq.resq_project_quantize(X, None, r, x8, x4, s[0], s[1])
+                resq.resq_mixed_gemm(W, x8, x4, s[0], s[1], want, ws)
+            assert resq.resq_device_status() == resq.OK
+            same = (Y == want) | (Y.isnan() & want.isnan())
+            assert same.all(), (X is forms[2], dt, (~same).sum().item())
