@@ -31,22 +31,24 @@ constexpr int kC8 = 32 * R8, kC4 = 32 * (N4 / 2), kHalf = kC8 + kC4 + 512, kBloc
 // With few CTAs a cluster splits the steps further and rank 0 merges the sums through distributed shared memory, so
 // no global scratch is needed.
 //
-// A step: the raw blocks arrive by cp.async two steps ahead; the codes are expanded, centred (code - 128, code - 8), in two
-// tiles [position][64 coefficients], keys as exact halves, values as exact bf16; K fragments come from ldmatrix, V
-// fragments from ldmatrix.trans, P straight from the score accumulators.  Scales and zero-points act in fp32 on the
-// accumulators:
+// A step: a block arrives by cp.async three steps ahead.  Positions are the rows of the score product and heads its columns, coefficients the
+// rows of the second product; both take their codes straight from the block's bytes, a lane reading the pieces of the positions
+// and coefficients that are its own in the fragments, centred (code - 128, code - 8), keys as exact halves, values as exact bf16:
+// expanded into shared memory and read back with ldmatrix, a step moved 236 shared-memory wavefronts, three quarters of what twelve
+// warps had of them, and now some 140.  The weights become the second product's columns by 8 x 8 transposes.  Scales and
+// zero-points act in fp32 on the accumulators:
 //   score = s8 S8 + s4 S4 + (z8 + 128 s8) sum(q8) + (z4 + 8 s4) sum(q4)         (q half, codes exact: products exact)
 //   out   = sum_j p_j s_j (c_j - c0) + sum_j p_j (z_j + c0 s_j)
 // The weights p_j s_j enter the second product as they are in fp32: as three bf16 values of 8 bits each, which add up to
-// all 24, in two products per fragment, since the rows fill half of one.  (Two halves under a common power of
+// all 24.  (Two halves under a common power of
 // two hold 22 bits of the largest weight only: a value scale 2^20 above the others, on a position with next to no
-// weight, left 2e-5 of the rest.)
-// The eight coefficients of a 32-bit word of nibbles are stored in the order 0 4 1 5 2 6 3 7 (one shift and mask per
-// pair); the query fragments are gathered in that order and the outputs put back.
+// weight, left 2e-5 of the rest.)  A head's reference is raised when a score exceeds it by 2^2; against 64 bits the outputs are as far off as with
+// an exact maximum (1.2 to 4.2e-7 over seven distributions, the form before 1.2 to 4.2e-7; with 2^8 and one chain for all parts up to 11 % more).
 //
-// What bounds it: the latency of a step and the operand conversions on the CUDA cores; not HBM, not the tensor pipe.
-// 32 query / 8 KV heads, project-and-append included: a step of 16 sequences of 1024-2048 positions 507 -> 19.7 us (21.7 while the words
-// of a step were read and expanded one by one), against one warp per (row, query head) that dequantized each position per head.
+// What bounds it: shared memory and issue slots about equally; not HBM, not the tensor pipe.
+// 32 query / 8 KV heads, project-and-append included: a step of 16 sequences of 1024-2048 positions 507 us (one warp per (row, query head) that
+// dequantized each position per head) -> 19.7 -> 18.0; the attention alone 15.2 -> 13.4; 64 sequences of 1000 positions 35.1 -> 30.6, with eight heads in a
+// group 36.9 -> 31.0.
 struct Attn64Params {
     const uint8_t* cache;
     const __half* q;   // [rows][Hq][64]
@@ -58,12 +60,13 @@ struct Attn64Params {
     int* status;
 };
 
-constexpr int kPitch = 144;        // bytes per position of an expanded tile: 64 halves + 16 (ldmatrix without conflicts)
 constexpr int kRecPitch = 68;      // floats per row of a record: 64 sums, maximum, sum of weights
 
-constexpr int kStep = 32, kNT = kStep / 8;  // positions of a step, score fragments
-constexpr int kWarpBytes = 2 * kBlock + 2 * kStep * kPitch + 2 * kStep * 16;  // of a warp's shared memory
+constexpr int kStep = 32;          // positions of a step: a cache block
+constexpr int kStages = 3;         // blocks of a warp's ring
+constexpr int kWarpBytes = kStages * kBlock;  // of a warp's shared memory
 static_assert(kWarpBytes >= 8 * kRecPitch * 4 && kWarpBytes % 16 == 0, "records fit");
+constexpr float kSlack = 2.f;      // log2 of the largest weight before the reference is raised
 
 __device__ __forceinline__ void mma16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
     asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
@@ -77,14 +80,14 @@ __device__ __forceinline__ void mma8(float (&d)[4], uint32_t a0, uint32_t a1, ui
     asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%0,%1,%2,%3};"
                  : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a0), "r"(a1), "r"(b0));
 }
-__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], uint32_t addr) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+__device__ __forceinline__ uint32_t movmatrix_trans(uint32_t x) {
+    uint32_t d;
+    asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(d) : "r"(x));
+    return d;
 }
-__device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], uint32_t addr) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
-}
+__device__ __forceinline__ uint32_t lds32(const uint8_t* p) { return *reinterpret_cast<const uint32_t*>(p); }
+__device__ __forceinline__ uint32_t lds16(const uint8_t* p) { return *reinterpret_cast<const uint16_t*>(p); }
+__device__ __forceinline__ float4 lds_f4(const uint8_t* p) { return *reinterpret_cast<const float4*>(p); }
 __device__ __forceinline__ uint32_t h2_bits(__half2 v) { return *reinterpret_cast<const uint32_t*>(&v); }
 // The bits of a float that bf16 keeps.
 __device__ __forceinline__ float bf16_part(float x) { return __uint_as_float(__float_as_uint(x) & 0xFFFF0000u); }
@@ -97,9 +100,6 @@ __device__ __forceinline__ void split_bf16(float a, float b, uint32_t (&part)[3]
         b -= bf16_part(b);
     }
 }
-// Coefficient at element e (0..7) of chunk j (0: the 8-bit segment, 1..7: words of nibbles).
-__device__ __forceinline__ int coef64(int j, int e) { return j == 0 ? e : 8 * j + (e >> 1) + ((e & 1) << 2); }
-
 // Sequence and attended positions of query row `row`; out-of-range entries are clamped and, if asked, reported.
 __device__ __forceinline__ int row_length(const Attn64Params& p, int row, bool report, int& b) {
     b = p.seq_of_row ? p.seq_of_row[row] : row;
@@ -121,10 +121,6 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? 3 : 1) attention64_kernel(c
     extern __shared__ __align__(128) uint8_t smem64[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gr = lane >> 2, c = lane & 3;
     uint8_t* raw = smem64 + static_cast<size_t>(warp) * kWarpBytes;
-    uint8_t* Kt = raw + 2 * kBlock;
-    uint8_t* Vt = Kt + kStep * kPitch;
-    float4* colK = reinterpret_cast<float4*>(Vt + kStep * kPitch);
-    float4* colV = colK + kStep;
     const int rank = static_cast<int>(blockIdx.x % p.splits);
     int item = static_cast<int>(blockIdx.x / p.splits);
     griddep_wait();  // launched with programmatic stream serialization
@@ -163,183 +159,239 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? 3 : 1) attention64_kernel(c
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    issue(first, 0);
-    issue(first + stride, 1);
+#pragma unroll
+    for (int i = 0; i < kStages; ++i) issue(first + i * stride, i);
 
-    // ---- query fragments: chunk 0 (m16n8k8), chunks 1-6 as three k16 pairs, chunk 7 (m16n8k8); sums per segment
+    // ---- the query as the products' column operand: column gr is head gr; coefficients in the order in which the keys' pieces come (below)
     uint32_t qa[8];
     float qs8 = 0.f, qs4 = 0.f;
-    const __half* qrow = p.q + (static_cast<size_t>(row) * p.Hq + kvh * p.g + (gr < p.g ? gr : 0)) * D;
+    {
+        const __half* qrow = p.q + (static_cast<size_t>(row) * p.Hq + kvh * p.g + (gr < p.g ? gr : 0)) * D;
+        uint32_t q0 = 0u, q3 = 0u;
+        uint4 q1 = make_uint4(0u, 0u, 0u, 0u);
+        uint2 q2 = make_uint2(0u, 0u);
+        if (gr < p.g) {
+            q0 = *reinterpret_cast<const uint32_t*>(qrow + 2 * c);
+            q1 = *reinterpret_cast<const uint4*>(qrow + R8 + 8 * c);
+            q2 = *reinterpret_cast<const uint2*>(qrow + R8 + 32 + 4 * c);
+            q3 = *reinterpret_cast<const uint32_t*>(qrow + R8 + 48 + 2 * c);
+        }
+        qa[0] = q0;
+        qa[1] = __byte_perm(q1.x, q1.z, 0x5410);  // 0 4 | 1 5, then 2 6 | 3 7 of a word of nibbles
+        qa[2] = __byte_perm(q1.x, q1.z, 0x7632);
+        qa[3] = __byte_perm(q1.y, q1.w, 0x5410);
+        qa[4] = __byte_perm(q1.y, q1.w, 0x7632);
+        qa[5] = __byte_perm(q2.x, q2.y, 0x5410);  // 0 2 | 1 3 of two bytes
+        qa[6] = __byte_perm(q2.x, q2.y, 0x7632);
+        qa[7] = q3;
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        __half2 v = __floats2half2_rn(0.f, 0.f);
-        if (gr < p.g) v = __halves2half2(qrow[coef64(j, 2 * c)], qrow[coef64(j, 2 * c + 1)]);
-        qa[j] = h2_bits(v);
-        const float2 f = __half22float2(v);
-        if (j == 0) qs8 += f.x + f.y;
-        else qs4 += f.x + f.y;
+        for (int j = 0; j < 8; ++j) {
+            const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&qa[j]));
+            if (j == 0) qs8 += f.x + f.y;
+            else qs4 += f.x + f.y;
+        }
     }
+    const float kScore = 1.4426950408889634f * 0.125f;  // log2(e) / sqrt(64)
+    float kq8[2], kq4[2];  // of heads 2 c, 2 c + 1, the columns of a lane's scores
 #pragma unroll
     for (int o = 1; o < 4; o <<= 1) {
         qs8 += __shfl_xor_sync(0xffffffffu, qs8, o);
         qs4 += __shfl_xor_sync(0xffffffffu, qs4, o);
     }
-    const uint32_t none = 0u;  // rows 8-15 of a fragment
-
-    float O[8][2], m_run = -INFINITY, l = 0.f, zs8 = 0.f, zs4 = 0.f;
 #pragma unroll
-    for (int j = 0; j < 8; ++j) O[j][0] = O[j][1] = 0.f;
-    const float kScore = 1.4426950408889634f * 0.125f;  // log2(e) / sqrt(64)
-    const uint32_t k_addr = smem_u32(Kt) + (lane & 7) * kPitch + (lane >> 3) * 16;
-    const uint32_t v_addr = smem_u32(Vt) + ((lane & 7) + ((lane >> 3) & 1) * 8) * kPitch + (lane >> 4) * 16;
-
-    int buf = 0;
-    for (int s = first; s < n_steps; s += stride, buf ^= 1) {
-        asm volatile("cp.async.wait_group 1;" ::: "memory");
-        __syncwarp();  // the step's bytes are in place and nobody reads the previous tiles
-        const uint8_t* rb = raw + buf * kBlock;
-        const int j0 = s * kStep;
-        // ---- expand: chunks of eight coefficients, lane = position.  Every word is read before the first chunk is written: one by one
-        // they would each wait for shared memory (16 rows of 2048 positions, 8 KV heads, with the append: 21.7 -> 19.7 us).
-        {
-            uint32_t w4[2][7];
-            uint2 w8[2];
-            float4 m[2];
-#pragma unroll
-            for (int is_v = 0; is_v < 2; ++is_v) {
-                const uint8_t* half_base = rb + is_v * kHalf;
-                w8[is_v] = *reinterpret_cast<const uint2*>(half_base + lane * R8);
-#pragma unroll
-                for (int j = 0; j < 7; ++j) w4[is_v][j] = *reinterpret_cast<const uint32_t*>(half_base + kC8 + lane * (N4 / 2) + 4 * j);
-                m[is_v] = *reinterpret_cast<const float4*>(half_base + kC8 + kC4 + lane * 16);
-            }
-            uint4* krow = reinterpret_cast<uint4*>(Kt + lane * kPitch);
-            uint4* vrow = reinterpret_cast<uint4*>(Vt + lane * kPitch);
-            krow[0] = bytes_centred(w8[0]);
-            vrow[0] = bytes_centred_bf16(w8[1]);
-#pragma unroll
-            for (int j = 0; j < 7; ++j) {
-                krow[1 + j] = nibbles_centred(w4[0][j]);
-                vrow[1 + j] = nibbles_centred_bf16(w4[1][j]);
-            }
-            // per-position constants; positions past the row's last hold anything and are zeroed by selection
-#pragma unroll
-            for (int is_v = 0; is_v < 2; ++is_v) {
-                if (j0 + lane >= limit) m[is_v] = make_float4(0.f, 0.f, 0.f, 0.f);
-                m[is_v].y = fmaf(128.f, m[is_v].x, m[is_v].y);
-                m[is_v].w = fmaf(8.f, m[is_v].z, m[is_v].w);
-            }
-            colK[lane] = make_float4(m[0].x * kScore, m[0].y * kScore, m[0].z * kScore, m[0].w * kScore);
-            colV[lane] = m[1];
-        }
-        __syncwarp();
-        issue(s + 2 * stride, buf);  // everybody is done with this raw buffer
-
-        // ---- scores
-        float sc[kNT][2];
-        float mx = -INFINITY;
-        const bool masked = j0 + kStep > limit;
-#pragma unroll
-        for (int nt = 0; nt < kNT; ++nt) {
-            uint32_t k0[4], k1[4];
-            ldsm4(k0, k_addr + nt * 8 * kPitch);
-            ldsm4(k1, k_addr + nt * 8 * kPitch + 64);
-            float s8[4] = {0.f, 0.f, 0.f, 0.f}, s4[4] = {0.f, 0.f, 0.f, 0.f};
-            mma8(s8, qa[0], none, k0[0]);
-            mma16(s4, qa[1], none, qa[2], none, k0[1], k0[2]);
-            mma16(s4, qa[3], none, qa[4], none, k0[3], k1[0]);
-            mma16(s4, qa[5], none, qa[6], none, k1[1], k1[2]);
-            mma8(s4, qa[7], none, k1[3]);
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const int pos = 8 * nt + 2 * c + e;
-                const float4 k = colK[pos];
-                float x = fmaf(k.x, s8[e], fmaf(k.z, s4[e], fmaf(k.y, qs8, k.w * qs4)));
-                if (masked && j0 + pos >= limit) x = -INFINITY;
-                sc[nt][e] = x;
-                mx = fmaxf(mx, x);
-            }
-        }
-        // ---- running maximum
-        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-        const float m_new = fmaxf(m_run, mx), m_use = m_new == -INFINITY ? 0.f : m_new;
-        const float corr = exp2_approx(m_run - m_use);
-        const bool moved = m_new != m_run;
-        m_run = m_new;
-        if (__any_sync(0xffffffffu, moved)) {
-            l *= corr;
-            zs8 *= corr;
-            zs4 *= corr;
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                O[j][0] *= corr;
-                O[j][1] *= corr;
-            }
-        }
-        // ---- weights and the second product: the tensor core's fp32 sums are truncated, so a chain of products runs over
-        // 32 positions only and is then added to the running sums with rounding.  The middle part of a weight takes the unused rows
-        // of the first one's product.
-        uint32_t p8[2][2][4], p4[2][2][4];
-#pragma unroll
-        for (int t = 0; t < 4; ++t) {
-            const int pos = 8 * t + 2 * c, i = 2 * (t & 1);
-            const float4 va = colV[pos], vb = colV[pos + 1];
-            uint32_t w8[3], w4[3];
-            const float pa = exp2_approx(sc[t][0] - m_use), pb = exp2_approx(sc[t][1] - m_use);
-            l += pa + pb;
-            zs8 = fmaf(pa, va.y, fmaf(pb, vb.y, zs8));
-            zs4 = fmaf(pa, va.w, fmaf(pb, vb.w, zs4));
-            split_bf16(pa * va.x, pb * vb.x, w8);
-            split_bf16(pa * va.z, pb * vb.z, w4);
-            p8[t >> 1][0][i] = w8[0];
-            p8[t >> 1][0][i + 1] = w8[1];
-            p8[t >> 1][1][i] = w8[2];
-            p4[t >> 1][0][i] = w4[0];
-            p4[t >> 1][0][i + 1] = w4[1];
-            p4[t >> 1][1][i] = w4[2];
-            p8[t >> 1][1][i + 1] = p4[t >> 1][1][i + 1] = none;
-        }
-#pragma unroll
-        for (int j = 0; j < 8; j += 2) {
-            float d0[4] = {0.f, 0.f, 0.f, 0.f}, d1[4] = {0.f, 0.f, 0.f, 0.f};
-            uint32_t v[2][4];
-            ldsm4t(v[0], v_addr + j * 16);
-            ldsm4t(v[1], v_addr + 16 * kPitch + j * 16);
-#pragma unroll
-            for (int k = 1; k >= 0; --k)  // the small parts first
-#pragma unroll
-                for (int ks = 0; ks < 2; ++ks) {
-                    mma16_bf16(d0, j == 0 ? p8[ks][k] : p4[ks][k], v[ks][0], v[ks][1]);
-                    mma16_bf16(d1, p4[ks][k], v[ks][2], v[ks][3]);
-                }
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                O[j][e] += d0[e] + d0[2 + e];
-                O[j + 1][e] += d1[e] + d1[2 + e];
-            }
-        }
+    for (int e = 0; e < 2; ++e) {
+        kq8[e] = kScore * __shfl_sync(0xffffffffu, qs8, 4 * (2 * c + e));
+        kq4[e] = kScore * __shfl_sync(0xffffffffu, qs4, 4 * (2 * c + e));
     }
 
-    // ---- records of the warps (unnormalised sums with the zero-points, maximum, sum of weights) over their tiles, then the merge
+    // Outputs: rows are coefficients (gr, gr + 8), columns heads 2 c, 2 c + 1.  O[0]: the 8-bit segment in rows 0-7; O[1 + 2 i + t]: byte t of
+    // half-word gr + 8 i of the 4-bit codes (i = 1: rows 6 and 7 are nobody's), the low nibble in row gr, the high one in row gr + 8.
+    float O[5][4], m_run[2], l[2], zs8[2], zs4[2];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        m_run[e] = -INFINITY;
+        l[e] = zs8[e] = zs4[e] = 0.f;
+    }
+#pragma unroll
+    for (int j = 0; j < 5; ++j) O[j][0] = O[j][1] = O[j][2] = O[j][3] = 0.f;
+
+    int buf = 0;
+    for (int s = first; s < n_steps; s += stride) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(kStages - 1) : "memory");
+        __syncwarp();  // the step's bytes are in place
+        const uint8_t* kb = raw + buf * kBlock;
+        const uint8_t* vb = kb + kHalf;
+        const int j0 = s * kStep;
+        const bool masked = j0 + kStep > limit;
+
+        // ---- scores of two tiles of 16 positions: row gr is position 2 gr of the tile, row gr + 8 the one behind it
+        float sc[2][2][2];  // [tile][position][head]
+        float mx[2] = {-INFINITY, -INFINITY};
+#pragma unroll
+        for (int m = 0; m < 2; ++m) {
+            const int tok = 16 * m + 2 * gr;
+            const uint8_t* k4 = kb + kC8 + tok * (N4 / 2);
+            uint32_t w[2], h[2], x[2], y[2];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                w[i] = lds32(k4 + i * (N4 / 2) + 4 * c);
+                h[i] = lds16(k4 + i * (N4 / 2) + 16 + 2 * c);
+                y[i] = k4[i * (N4 / 2) + 24 + c];
+                x[i] = lds16(kb + (tok + i) * R8 + 2 * c);
+            }
+            const uint4 va = nibbles_centred(w[0]), vn = nibbles_centred(w[1]);
+            float s8[4] = {0.f, 0.f, 0.f, 0.f}, s4[4] = {0.f, 0.f, 0.f, 0.f};
+            mma8(s8, centred(__byte_perm(x[0], 0x64646464u, 0x4140), 0x6480), centred(__byte_perm(x[1], 0x64646464u, 0x4140), 0x6480), qa[0]);
+            mma16(s4, va.x, vn.x, va.y, vn.y, qa[1], qa[2]);
+            mma16(s4, va.z, vn.z, va.w, vn.w, qa[3], qa[4]);
+            const uint2 ha = byte_pair_centred(__byte_perm(h[0], 0u, 0x4140)), hn = byte_pair_centred(__byte_perm(h[1], 0u, 0x4140));
+            mma16(s4, ha.x, hn.x, ha.y, hn.y, qa[5], qa[6]);
+            mma8(s4, centred(((y[0] * 0x1001u) & 0x000F000Fu) | 0x64006400u, 0x6408), centred(((y[1] * 0x1001u) & 0x000F000Fu) | 0x64006400u, 0x6408), qa[7]);
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                float4 k = lds_f4(kb + kC8 + kC4 + (tok + i) * 16);
+                const bool hidden = masked && j0 + tok + i >= limit;
+                if (hidden) k = make_float4(0.f, 0.f, 0.f, 0.f);
+                k.y = fmaf(128.f, k.x, k.y);
+                k.w = fmaf(8.f, k.z, k.w);
+                k.x *= kScore;
+                k.z *= kScore;
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const float v = fmaf(k.x, s8[2 * i + e], fmaf(k.z, s4[2 * i + e], fmaf(k.y, kq8[e], k.w * kq4[e])));
+                    sc[m][i][e] = hidden ? -INFINITY : v;
+                    mx[e] = fmaxf(mx[e], sc[m][i][e]);
+                }
+            }
+        }
+        // ---- reference of a head, the same in the lanes that share it: raised only when a score exceeds it by kSlack (and at first)
+        if (__any_sync(0xffffffffu, mx[0] > m_run[0] + kSlack || mx[1] > m_run[1] + kSlack)) {
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                float v = mx[e];
+#pragma unroll
+                for (int o = 4; o < 32; o <<= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+                const float m_new = fmaxf(m_run[e], v);
+                const float f = exp2_approx(m_run[e] - (m_new == -INFINITY ? 0.f : m_new));
+                m_run[e] = m_new;
+                l[e] *= f;
+                zs8[e] *= f;
+                zs4[e] *= f;
+#pragma unroll
+                for (int j = 0; j < 5; ++j) {
+                    O[j][e] *= f;
+                    O[j][2 + e] *= f;
+                }
+            }
+        }
+        // ---- weights times the value scales as three bf16 parts, transposed into the second product's column operand
+        uint32_t w8[2][3][2], w4[2][3][2];  // [tile][part][positions 0 2 | 1 3 of the lane's four]
+#pragma unroll
+        for (int m = 0; m < 2; ++m)
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const int tok = 16 * m + 2 * gr + i;
+                float4 v = lds_f4(vb + kC8 + kC4 + tok * 16);
+                if (masked && j0 + tok >= limit) v = make_float4(0.f, 0.f, 0.f, 0.f);
+                v.y = fmaf(128.f, v.x, v.y);
+                v.w = fmaf(8.f, v.z, v.w);
+                float pw[2];
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    pw[e] = exp2_approx(sc[m][i][e] - (m_run[e] == -INFINITY ? 0.f : m_run[e]));
+                    l[e] += pw[e];
+                    zs8[e] = fmaf(pw[e], v.y, zs8[e]);
+                    zs4[e] = fmaf(pw[e], v.w, zs4[e]);
+                }
+                uint32_t part[3];
+                split_bf16(pw[0] * v.x, pw[1] * v.x, part);
+#pragma unroll
+                for (int k = 0; k < 3; ++k) w8[m][k][i] = movmatrix_trans(part[k]);
+                split_bf16(pw[0] * v.z, pw[1] * v.z, part);
+#pragma unroll
+                for (int k = 0; k < 3; ++k) w4[m][k][i] = movmatrix_trans(part[k]);
+            }
+        // ---- the second product: the tensor core's fp32 sums are truncated, so a chain of products runs over
+        // 32 positions only and is then added to the running sums with rounding; the first parts in a chain of their own.
+        auto add_product = [&](float (&o)[4], const uint32_t (&a)[2][4], const uint32_t (&b)[2][3][2]) {
+            float d[4] = {0.f, 0.f, 0.f, 0.f}, rest[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+            for (int m = 0; m < 2; ++m) mma16_bf16(rest, a[m], b[m][2][0], b[m][2][1]);
+#pragma unroll
+            for (int m = 0; m < 2; ++m) {
+                mma16_bf16(rest, a[m], b[m][1][0], b[m][1][1]);
+                mma16_bf16(d, a[m], b[m][0][0], b[m][0][1]);
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) o[i] += d[i] + rest[i];
+        };
+        {
+            uint32_t a[2][4];
+#pragma unroll
+            for (int m = 0; m < 2; ++m) {
+                const uint8_t* v8 = vb + (16 * m + 4 * c) * R8 + gr;
+                a[m][0] = byte_pair_bf16(__byte_perm(v8[0], v8[2 * R8], 0x5410));
+                a[m][2] = byte_pair_bf16(__byte_perm(v8[R8], v8[3 * R8], 0x5410));
+                a[m][1] = a[m][3] = 0u;
+            }
+            add_product(O[0], a, w8);
+        }
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            uint32_t w02[2], w13[2];
+#pragma unroll
+            for (int m = 0; m < 2; ++m) {
+                const uint8_t* v4 = vb + kC8 + (16 * m + 4 * c) * (N4 / 2) + 2 * (i == 0 ? gr : 8 + min(gr, 5));
+                w02[m] = __byte_perm(lds16(v4), lds16(v4 + N4), 0x5410);
+                w13[m] = __byte_perm(lds16(v4 + N4 / 2), lds16(v4 + 3 * (N4 / 2)), 0x5410);
+            }
+#pragma unroll
+            for (int t = 0; t < 2; ++t) {
+                uint32_t a[2][4];
+#pragma unroll
+                for (int m = 0; m < 2; ++m) {
+                    a[m][0] = nibble_pair_bf16(w02[m] >> (8 * t));
+                    a[m][1] = nibble_pair_bf16(w02[m] >> (8 * t + 4));
+                    a[m][2] = nibble_pair_bf16(w13[m] >> (8 * t));
+                    a[m][3] = nibble_pair_bf16(w13[m] >> (8 * t + 4));
+                }
+                add_product(O[1 + 2 * i + t], a, w4);
+            }
+        }
+        __syncwarp();  // everybody is done with this block
+        issue(s + kStages * stride, buf);
+        if (++buf == kStages) buf = 0;
+    }
+
+    // ---- records of the warps (unnormalised sums with the zero-points, reference, sum of weights) over their rings, then the merge
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncwarp();
 #pragma unroll
-    for (int o = 1; o < 4; o <<= 1) {
-        l += __shfl_xor_sync(0xffffffffu, l, o);
-        zs8 += __shfl_xor_sync(0xffffffffu, zs8, o);
-        zs4 += __shfl_xor_sync(0xffffffffu, zs4, o);
-    }
-    float* r = reinterpret_cast<float*>(raw) + gr * kRecPitch;
+    for (int e = 0; e < 2; ++e)
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        const float z = j == 0 ? zs8 : zs4;
-        r[coef64(j, 2 * c)] = O[j][0] + z;
-        r[coef64(j, 2 * c + 1)] = O[j][1] + z;
-    }
-    if (c == 0) {
-        r[D] = m_run;
-        r[D + 1] = l;
+        for (int o = 4; o < 32; o <<= 1) {
+            l[e] += __shfl_xor_sync(0xffffffffu, l[e], o);
+            zs8[e] += __shfl_xor_sync(0xffffffffu, zs8[e], o);
+            zs4[e] += __shfl_xor_sync(0xffffffffu, zs4[e], o);
+        }
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        float* r = reinterpret_cast<float*>(raw) + (2 * c + e) * kRecPitch;
+        r[gr] = O[0][e] + zs8[e];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            if (i == 1 && gr >= 6) continue;
+            float* q = r + R8 + 4 * (gr + 8 * i);
+#pragma unroll
+            for (int t = 0; t < 2; ++t) {
+                q[2 * t] = O[1 + 2 * i + t][e] + zs4[e];
+                q[2 * t + 1] = O[1 + 2 * i + t][2 + e] + zs4[e];
+            }
+        }
+        if (gr == 0) {
+            r[D] = m_run[e];
+            r[D + 1] = l[e];
+        }
     }
     __syncwarp();
     if (p.splits > 1) cluster_sync_all();
