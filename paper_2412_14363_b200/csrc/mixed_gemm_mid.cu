@@ -14,7 +14,7 @@
 // no persistence.  The rule that picks this kernel, N and S is mid_plan (plans.h).  All waits are bounded.
 //
 // What bounds it: the latency of the TMA ring up to N = 128 (0.21 us per k-block of 24 KB, 8 stages), operand delivery beyond,
-// and about 7 us of launch, first copies, epilogue and drain.  us, tile kernel -> this one: 4096 x 6144 at 17 / 128 / 300 /
+// and about 6 us of launch, first copies, epilogue and drain.  us, tile kernel -> this one: 4096 x 6144 at 17 / 128 / 300 /
 // 700 tokens 17.5 -> 8.7, 24 -> 12.3, 24.7 -> 14.3, 24.9 -> 19.6; 14336 x 4096 at 17 / 300 / 1537 tokens 41 -> 15.3, 47 -> 23,
 // 89 -> 68.5.  Products issued by a thread alone in a branch: 0.27 us per k-block whatever N.
 #include <cuda.h>
@@ -35,6 +35,7 @@ constexpr int A_BYTES = BM * BK;
 constexpr int kRingBytes = 6 * (A_BYTES + 128 * BK);  // a stage holds 128 channel rows and ntok / 2 token rows (at most 128)
 constexpr int kThreads = 320;
 constexpr uint32_t kTmemCols = 512, kColAcc4 = 256;
+constexpr int kTok = 8;  // tokens that an epilogue thread finishes at a time
 constexpr int kGroupBytes = 16 * BM * 4;  // partial sums of 16 tokens x 128 channels
 
 struct Params {
@@ -56,13 +57,16 @@ struct Params {
     int* status;
 };
 
-struct __align__(8) Shared {
+struct __align__(16) Shared {
     uint64_t full[kMaxStages];
     uint64_t empty[kMaxStages];
     uint64_t acc_full;
     uint32_t tmem_base;
     int abort_flag;
-    float sx8[256], sx4[256], zx8[256], zx4[256];
+    alignas(16) float sx8[256];  // of the tile's tokens, 0 behind the last
+    alignas(16) float sx4[256];
+    alignas(16) float zx8[256];
+    alignas(16) float zx4[256];
 };
 
 constexpr size_t kSmemBytes = 1024 + kRingBytes + sizeof(Shared);
@@ -70,6 +74,14 @@ constexpr size_t kSmemBytes = 1024 + kRingBytes + sizeof(Shared);
 __device__ __forceinline__ float load_scale(const void* p, int i, int fp16) {
     return fp16 ? __half2float(reinterpret_cast<const __half*>(p)[i]) : reinterpret_cast<const float*>(p)[i];
 }
+
+template <int S>
+struct Count {
+    static constexpr int value = S;
+};
+
+__device__ __forceinline__ void put_value(float* dst, float y) { *dst = y; }
+__device__ __forceinline__ void put_value(__nv_bfloat16* dst, float y) { *dst = __float2bfloat16_rn(y); }
 
 // Slot of 16-token group g among the groups that pair `owner` of `splits` does not finish itself.
 __device__ __forceinline__ int slot_of(int g, int owner, int splits) { return g - (g + splits - 1 - owner) / splits; }
@@ -126,6 +138,10 @@ mixed_gemm_mid_kernel(const __grid_constant__ CUtensorMap tmW8, const __grid_con
     auto has8 = [&](int i) { return kbt * (i + 1) / p.splits > p.kb4; };
     const uint32_t part8 = static_cast<uint32_t>(groups - groups / p.splits) * kGroupBytes;  // INT8 sums behind the INT4 ones
     bool ok = true;
+    // An epilogue thread's channel, and its scales: asked for before the products are awaited.
+    const int n = n0 + row;
+    const bool n_in = warp >= 2 && n < p.N;
+    float sw8 = 0.f, sw4 = 0.f, zc8 = 0.f, zc4 = 0.f;
 
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer
@@ -190,6 +206,14 @@ mixed_gemm_mid_kernel(const __grid_constant__ CUtensorMap tmW8, const __grid_con
             sh->zx8[et] = zx8;
             sh->zx4[et] = zx4;
         }
+        if (n_in) {
+            sw8 = load_scale(p.s_w8, n, p.w_fp16);
+            sw4 = load_scale(p.s_w4, n, p.w_fp16);
+            if (ASYM) {
+                zc8 = static_cast<float>(p.wsum8[n]) * sw8;
+                zc4 = static_cast<float>(p.wsum4[n]) * sw4;
+            }
+        }
         ok = mbar_wait(&sh->acc_full, 0, abort_flag, p.status);
         ok = !__any_sync(0xffffffffu, !ok);
         tc_fence_after();
@@ -221,59 +245,100 @@ mixed_gemm_mid_kernel(const __grid_constant__ CUtensorMap tmW8, const __grid_con
 
     if (warp >= 2) {
         // ------------------------------------------------------------ epilogue, second half: sums, scales, stores
-        const int n = n0 + row;
-        const bool n_ok = n < p.N && ok;
-        const float sw8 = n_ok ? load_scale(p.s_w8, n, p.w_fp16) : 0.f;
-        const float sw4 = n_ok ? load_scale(p.s_w4, n, p.w_fp16) : 0.f;
-        const float zc8 = ASYM && n_ok ? static_cast<float>(p.wsum8[n]) * sw8 : 0.f;
-        const float zc4 = ASYM && n_ok ? static_cast<float>(p.wsum4[n]) * sw4 : 0.f;
-        const bool w4 = has4(pair), w8 = has8(pair);
-        for (int k = part; pair + k * p.splits < groups; k += 2) {
-            const int g = pair + k * p.splits;  // g % splits == pair
-            uint32_t a4[16], a8[16];
-            __syncwarp();  // TMEM loads are for the whole, converged warp; lanes beyond the channels only skip their stores
-            tmem_ld16x2(lane_addr + kColAcc4 + 16 * g, lane_addr + 16 * g, a4, a8);
-            if (!w4)
+        const int tokens = n_in && ok ? min(p.ntok, p.T - t0) : 0;
+        // What bounds it is the fetch of instructions: two warps a scheduler cannot hide a jump, and each skipped body (a split's sums, the sums to
+        // write out, the other output type) cost 30 to 100 cycles a pass.  So one loop a split count and output type, its body straight: 8 tokens
+        // take 550 cycles (two warps a scheduler, fp32 results with zero-points), 16 in one pass with those branches took 1750; the steps from
+        // the last product to the last store: 128 tokens 4.2 -> 3.0 us, 192 tokens 5.1 -> 3.6.  The time of the layer, us: 4096 x 6144 at 17 / 300 /
+        // 512 tokens 12.1 -> 11.4, 21.2 -> 19.8, 23.7 -> 20.7; 14336 x 4096 at 300 / 1537 tokens 32.6 -> 29.8, 94.9 -> 90.8.  The next sums asked for
+        // before the stores: 0.98 of that; two passes unrolled: the same; fewer registers (112, 96): 0.99.
+        auto finish = [&](auto splits, auto* Y) {
+            constexpr int S = decltype(splits)::value;
+            const bool w4 = has4(pair), w8 = has8(pair);
+            uint32_t src[S];  // another pair's sums of this pair's first group; the next group is S - 1 slots further
+            bool r4[S], r8[S];
 #pragma unroll
-                for (int j = 0; j < 16; ++j) a4[j] = 0;
-            if (!w8)
+            for (int o = 0; o < S - 1; ++o) {
+                const int i = o + (o >= pair ? 1 : 0);
+                src[o] = cluster_map(smem + slot_of(pair, i, S) * kGroupBytes + part * (kTok / 4 * BM * 16) + row * 16, 2 * i + h);
+                r4[o] = has4(i);
+                r8[o] = has8(i);
+            }
+            if (S == 1) {  // a segment without channels has no sums: its columns hold anything
+                if (!w4) sw4 = 0.f;
+                if (!w8) sw8 = 0.f;
+            }
+            // kTok tokens' sums over the pairs, from column t on.
+            auto sums = [&](int t, uint32_t (&a4)[kTok], uint32_t (&a8)[kTok]) {
+                __syncwarp();  // TMEM loads are for the whole, converged warp; lanes beyond the channels only skip their stores
+                tmem_ld8x2(lane_addr + kColAcc4 + t, lane_addr + t, a4, a8);
+                if (S > 1)
 #pragma unroll
-                for (int j = 0; j < 16; ++j) a8[j] = 0;
-            for (int i = 0; i < p.splits; ++i) {
-                if (i == pair) continue;
-                const uint32_t src = cluster_map(smem + slot_of(g, i, p.splits) * kGroupBytes + row * 16, 2 * i + h);
-                const bool r4 = has4(i), r8 = has8(i);
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    if (r4) {
-                        const uint4 v = ld_cluster_u4(src + q * (BM * 16));
-                        a4[4 * q] += v.x; a4[4 * q + 1] += v.y; a4[4 * q + 2] += v.z; a4[4 * q + 3] += v.w;
+                    for (int j = 0; j < kTok; ++j) {
+                        a4[j] = w4 ? a4[j] : 0;
+                        a8[j] = w8 ? a8[j] : 0;
                     }
-                    if (r8) {
-                        const uint4 v = ld_cluster_u4(src + part8 + q * (BM * 16));
-                        a8[4 * q] += v.x; a8[4 * q + 1] += v.y; a8[4 * q + 2] += v.z; a8[4 * q + 3] += v.w;
+                const uint32_t at = static_cast<uint32_t>(t / (16 * S) * (S - 1)) * kGroupBytes;
+#pragma unroll
+                for (int o = 0; o < S - 1; ++o)
+#pragma unroll
+                    for (int q = 0; q < kTok / 4; ++q) {
+                        const uint4 v4 = ld_cluster_u4_if(r4[o], src[o] + at + q * (BM * 16));
+                        const uint4 v8 = ld_cluster_u4_if(r8[o], src[o] + at + part8 + q * (BM * 16));
+                        a4[4 * q] += v4.x; a4[4 * q + 1] += v4.y; a4[4 * q + 2] += v4.z; a4[4 * q + 3] += v4.w;
+                        a8[4 * q] += v8.x; a8[4 * q + 1] += v8.y; a8[4 * q + 2] += v8.z; a8[4 * q + 3] += v8.w;
+                    }
+            };
+            const size_t step = static_cast<size_t>(p.N);
+            const int first = 16 * pair + kTok * part;
+            Y += static_cast<size_t>(t0) * step + n;
+#pragma unroll 1
+            for (int t = first; t < p.ntok; t += 16 * S) {
+                uint32_t a4[kTok], a8[kTok];
+                sums(t, a4, a8);
+                float y[kTok];
+#pragma unroll
+                for (int q = 0; q < kTok / 4; ++q) {
+                    const float4 s8 = reinterpret_cast<const float4*>(sh->sx8 + t)[q], s4 = reinterpret_cast<const float4*>(sh->sx4 + t)[q];
+                    const float f8[4] = {s8.x, s8.y, s8.z, s8.w}, f4[4] = {s4.x, s4.y, s4.z, s4.w};
+                    float4 z8 = {0.f, 0.f, 0.f, 0.f}, z4 = z8;
+                    if (ASYM) z8 = reinterpret_cast<const float4*>(sh->zx8 + t)[q], z4 = reinterpret_cast<const float4*>(sh->zx4 + t)[q];
+                    const float g8[4] = {z8.x, z8.y, z8.z, z8.w}, g4[4] = {z4.x, z4.y, z4.z, z4.w};
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const int j = 4 * q + i;
+                        const float t8 = static_cast<float>(static_cast<int>(a8[j])) * (f8[i] * sw8);
+                        const float t4 = static_cast<float>(static_cast<int>(a4[j])) * (f4[i] * sw4);
+                        y[j] = t8 + t4;
+                        if (ASYM) y[j] += g8[i] * zc8 + g4[i] * zc4;
                     }
                 }
-            }
-            if (n_ok) {
+                auto* dst = Y + static_cast<size_t>(t) * step;
 #pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    const int tt = 16 * g + j, t = t0 + tt;
-                    if (t >= p.T) break;
-                    const size_t off = static_cast<size_t>(t) * p.N + n;
-                    const float t8 = static_cast<float>(static_cast<int>(a8[j])) * (sh->sx8[tt] * sw8);
-                    const float t4 = static_cast<float>(static_cast<int>(a4[j])) * (sh->sx4[tt] * sw4);
-                    float y = t8 + t4;
-                    if (ASYM) y += sh->zx8[tt] * zc8 + sh->zx4[tt] * zc4;
-                    if (p.y_dtype == RESQ_Y_BF16) reinterpret_cast<__nv_bfloat16*>(p.Y)[off] = __float2bfloat16_rn(y);
-                    else reinterpret_cast<float*>(p.Y)[off] = y;
-                    if (p.dbg8) {
-                        p.dbg8[off] = static_cast<int>(a8[j]);
-                        p.dbg4[off] = static_cast<int>(a4[j]);
-                    }
-                }
+                for (int j = 0; j < kTok; ++j, dst += step)
+                    if (t + j < tokens) put_value(dst, y[j]);
             }
-        }
+            if (p.dbg8)
+#pragma unroll 1
+                for (int t = first; t < p.ntok; t += 16 * S) {
+                    uint32_t a4[kTok], a8[kTok];
+                    sums(t, a4, a8);
+#pragma unroll
+                    for (int j = 0; j < kTok; ++j)
+                        if (t + j < tokens) {
+                            const size_t off = static_cast<size_t>(t0 + t + j) * step + n;
+                            p.dbg8[off] = w8 || S > 1 ? static_cast<int>(a8[j]) : 0;
+                            p.dbg4[off] = w4 || S > 1 ? static_cast<int>(a4[j]) : 0;
+                        }
+                }
+        };
+        auto finish_as = [&](auto splits) {
+            if (p.y_dtype == RESQ_Y_BF16) finish(splits, reinterpret_cast<__nv_bfloat16*>(p.Y));
+            else finish(splits, reinterpret_cast<float*>(p.Y));
+        };
+        if (p.splits == 1) finish_as(Count<1>());
+        else if (p.splits == 2) finish_as(Count<2>());
+        else finish_as(Count<3>());
     }
 
     // ---------------------------------------------------------------- teardown
