@@ -27,6 +27,8 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include <type_traits>
+
 #include "byte_map.h"
 #include "internal.h"
 #include "ptx.cuh"
@@ -38,8 +40,9 @@ constexpr int BM = 128, BN = 256, BK = 128;  // BK in bytes == int8 elements
 constexpr int STAGES = 6;
 constexpr int BN_HALF = BN / 2;  // weight rows staged by each CTA of the pair
 constexpr int A_BYTES = BM * BK, B_BYTES = BN_HALF * BK;
-constexpr int kThreads = 320;
 constexpr int kEpiThreads = 256;
+constexpr int kThreads = 64 + kEpiThreads;
+constexpr int kCols = BN * BM / kEpiThreads;  // of a tile row that an epilogue thread finishes
 constexpr uint32_t kTmemCols = 512;
 
 struct Params {
@@ -57,13 +60,13 @@ struct Params {
     const int32_t* wsum8;
     const int32_t* wsum4;
     void* Y;
-    int y_dtype;
+    int wide;  // rows of Y start on 32 bytes
     int32_t* dbg8;
     int32_t* dbg4;
     int* status;
 };
 
-struct __align__(8) Shared {
+struct __align__(16) Shared {
     uint64_t full[STAGES];
     uint64_t empty[STAGES];
     uint64_t acc4_full;
@@ -73,10 +76,10 @@ struct __align__(8) Shared {
     uint32_t tmem_base;
     int abort_flag;
     int epi_stop;
-    float sw8[BN];
-    float sw4[BN];
-    float zc8[BN];  // asymmetric activations: (float)wsum8[n] * sw8[n], the column factor of the zero-point term
-    float zc4[BN];
+    alignas(16) float sw8[BN];
+    alignas(16) float sw4[BN];
+    alignas(16) float zc8[BN];  // asymmetric activations: (float)wsum8[n] * sw8[n], the column factor of the zero-point term
+    alignas(16) float zc4[BN];
 };
 
 constexpr size_t kSmemBytes = 1024 + STAGES * (A_BYTES + B_BYTES) + sizeof(Shared);
@@ -89,7 +92,7 @@ __device__ __forceinline__ void epi_barrier() { asm volatile("bar.sync 1, %0;" :
 
 // ASYM: the activation codes are unsigned (u8 x s8 products) and every output gets the rank-one
 // zero-point terms z_x8[t] * s_w8[n] * wsum8[n] + z_x4[t] * s_w4[n] * wsum4[n] (Eq. 1, second form).
-template <bool ASYM>
+template <bool ASYM, bool BF16>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 mixed_gemm_kernel(const __grid_constant__ CUtensorMap tmA8, const __grid_constant__ CUtensorMap tmA4,
                   const __grid_constant__ CUtensorMap tmB8, const __grid_constant__ CUtensorMap tmB4,
@@ -234,7 +237,7 @@ mixed_gemm_kernel(const __grid_constant__ CUtensorMap tmA8, const __grid_constan
             if (sh->epi_stop) break;
             const int row = m0 + quad * 32 + lane;
             const bool row_ok = row < p.T;
-            const float sx8 = row_ok ? p.s_x8[row] : 0.f;
+            const float sx8 = row_ok && p.kb8 ? p.s_x8[row] : 0.f;  // uniform INT4: the INT8 accumulator was never written
             const float sx4 = row_ok ? p.s_x4[row] : 0.f;
             const float zx8 = ASYM && row_ok ? p.z_x8[row] : 0.f;
             const float zx4 = ASYM && row_ok ? p.z_x4[row] : 0.f;
@@ -242,8 +245,8 @@ mixed_gemm_kernel(const __grid_constant__ CUtensorMap tmA8, const __grid_constan
             // Whole warps go on together; if a wait ran out, the flag is set: leave at the next sample.
             if (__any_sync(0xffffffffu, !mbar_wait(&sh->acc4_full, acc_phase, abort_flag, p.status))) continue;
             tc_fence_after();
-            const uint32_t lane_addr = tmem_base + (static_cast<uint32_t>(quad * 32) << 16) + ch * (BN / 2);
-            uint32_t a4[128];
+            const uint32_t lane_addr = tmem_base + (static_cast<uint32_t>(quad * 32) << 16) + ch * kCols;
+            uint32_t a4[kCols];
             __syncwarp();
             tmem_ld128(lane_addr + BN, a4);
             tc_fence_before();
@@ -251,62 +254,82 @@ mixed_gemm_kernel(const __grid_constant__ CUtensorMap tmA8, const __grid_constan
             if (__any_sync(0xffffffffu, !mbar_wait(&sh->acc_full, acc_phase, abort_flag, p.status))) continue;
             acc_phase ^= 1;
             tc_fence_after();
-            // Phase 2: the INT8 accumulator, the scales, the store -- 16 columns at a time.
+            // Phase 2: the INT8 accumulator, the scales, the store -- 32 bytes of a row at a time, a whole sector, where rows start on 32 bytes.
+            // With two warps a scheduler it is the fetch of instructions and spilled registers that bound it, and for short reductions or fp32
+            // results it bounds the kernel: 16 columns loaded, scaled and stored 16 bytes at a time, with the branches on the output type and on
+            // the sums to write out in each pass, took longer than the next tile's INT4 segment.  Now the kernel has the type, a load 8 columns.
+            // us, before / now: 3000 tokens 2048 x 16384 bf16 108 / 90, fp32 with zero-points 154 / 124; 4096 x 28672 241 / 235 and 314 / 255;
+            // 14336 x 4096 150 / 148 and 153 / 148; with stores of 16 bytes 112 and 153, with 16 warps of 64 columns (96 registers) 95 and 127.
+            const int cols = row_ok ? n_end - n0 - ch * kCols : 0;  // that this thread stores
+            const size_t off = static_cast<size_t>(row) * p.N + n0 + ch * kCols;
+            if (p.dbg8) {
 #pragma unroll
-            for (int c = 0; c < 8; ++c) {
-                uint32_t a8[16];
-                __syncwarp();
-                tmem_ld16(lane_addr + c * 16, a8);
-                if (p.kb8 == 0) {  // uniform INT4: the INT8 accumulator was never written
+                for (int c = 0; c < kCols / 16; ++c) {
+                    uint32_t a8[16];
+                    __syncwarp();
+                    tmem_ld16(lane_addr + c * 16, a8);
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) a8[j] = 0;
-                }
-                const int cb = ch * (BN / 2) + c * 16;  // first column of the chunk inside the tile
-                const int nb = n0 + cb;
-                const uint32_t* a4c = &a4[c * 16];
-                if (row_ok) {
-                    const size_t off = static_cast<size_t>(row) * p.N + nb;
-                    if (p.dbg8) {
-#pragma unroll
-                        for (int g = 0; g < 4; ++g)
-                            if (nb + g * 4 < n_end) {
-                                reinterpret_cast<uint4*>(p.dbg8 + off)[g] =
-                                    make_uint4(a8[4 * g], a8[4 * g + 1], a8[4 * g + 2], a8[4 * g + 3]);
-                                reinterpret_cast<uint4*>(p.dbg4 + off)[g] =
-                                    make_uint4(a4c[4 * g], a4c[4 * g + 1], a4c[4 * g + 2], a4c[4 * g + 3]);
-                            }
-                    }
-                    float y[16];
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        const float t8 = static_cast<float>(static_cast<int>(a8[j])) * (sx8 * sh->sw8[cb + j]);
-                        const float t4 = static_cast<float>(static_cast<int>(a4c[j])) * (sx4 * sh->sw4[cb + j]);
-                        y[j] = t8 + t4;
-                        if (ASYM) y[j] += zx8 * sh->zc8[cb + j] + zx4 * sh->zc4[cb + j];
-                    }
-                    if (p.y_dtype == RESQ_Y_BF16) {
-                        __nv_bfloat16* yp = reinterpret_cast<__nv_bfloat16*>(p.Y) + off;
-#pragma unroll
-                        for (int g = 0; g < 2; ++g)
-                            if (nb + g * 8 < n_end) {
-                                uint32_t w[4];
-#pragma unroll
-                                for (int q = 0; q < 4; ++q) {
-                                    __nv_bfloat162 h = __floats2bfloat162_rn(y[g * 8 + 2 * q], y[g * 8 + 2 * q + 1]);
-                                    w[q] = *reinterpret_cast<uint32_t*>(&h);
-                                }
-                                reinterpret_cast<uint4*>(yp)[g] = make_uint4(w[0], w[1], w[2], w[3]);
-                            }
-                    } else {
-                        float* yp = reinterpret_cast<float*>(p.Y) + off;
-#pragma unroll
-                        for (int g = 0; g < 4; ++g)
-                            if (nb + g * 4 < n_end)
-                                reinterpret_cast<float4*>(yp)[g] =
-                                    make_float4(y[4 * g], y[4 * g + 1], y[4 * g + 2], y[4 * g + 3]);
-                    }
+                    for (int g = 0; g < 4; ++g)
+                        if (c * 16 + g * 4 < cols) {
+                            reinterpret_cast<uint4*>(p.dbg8 + off)[4 * c + g] =
+                                p.kb8 ? make_uint4(a8[4 * g], a8[4 * g + 1], a8[4 * g + 2], a8[4 * g + 3]) : make_uint4(0, 0, 0, 0);
+                            reinterpret_cast<uint4*>(p.dbg4 + off)[4 * c + g] =
+                                make_uint4(a4[16 * c + 4 * g], a4[16 * c + 4 * g + 1], a4[16 * c + 4 * g + 2], a4[16 * c + 4 * g + 3]);
+                        }
                 }
             }
+            auto finish = [&](auto wide) {
+#pragma unroll
+                for (int c = 0; c < kCols / 16; ++c) {
+                    uint32_t w[8];  // 32 bytes of the row: the chunk in bf16, half of it in fp32
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        uint32_t a8[8];
+                        __syncwarp();
+                        tmem_ld8(lane_addr + c * 16 + e * 8, a8);
+                        const int cb = ch * kCols + c * 16 + e * 8;  // the first of these columns inside the tile
+#pragma unroll
+                        for (int q = 0; q < 2; ++q) {
+                            const float4 v8 = reinterpret_cast<const float4*>(sh->sw8 + cb)[q], v4 = reinterpret_cast<const float4*>(sh->sw4 + cb)[q];
+                            const float w8[4] = {v8.x, v8.y, v8.z, v8.w}, w4[4] = {v4.x, v4.y, v4.z, v4.w};
+                            float4 u8 = {0.f, 0.f, 0.f, 0.f}, u4 = u8;
+                            if (ASYM) u8 = reinterpret_cast<const float4*>(sh->zc8 + cb)[q], u4 = reinterpret_cast<const float4*>(sh->zc4 + cb)[q];
+                            const float c8[4] = {u8.x, u8.y, u8.z, u8.w}, c4[4] = {u4.x, u4.y, u4.z, u4.w};
+                            float y[4];
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) {
+                                const float t8 = static_cast<float>(static_cast<int>(a8[4 * q + i])) * (sx8 * w8[i]);
+                                const float t4 = static_cast<float>(static_cast<int>(a4[16 * c + 8 * e + 4 * q + i])) * (sx4 * w4[i]);
+                                y[i] = t8 + t4;
+                                if (ASYM) y[i] += zx8 * c8[i] + zx4 * c4[i];
+                            }
+                            if (BF16) {
+#pragma unroll
+                                for (int i = 0; i < 2; ++i) {
+                                    const __nv_bfloat162 h = __floats2bfloat162_rn(y[2 * i], y[2 * i + 1]);
+                                    w[4 * e + 2 * q + i] = *reinterpret_cast<const uint32_t*>(&h);
+                                }
+                            } else {
+#pragma unroll
+                                for (int i = 0; i < 4; ++i) w[4 * q + i] = __float_as_uint(y[i]);
+                            }
+                        }
+                        if (BF16 && e == 0) continue;
+                        const int col = c * 16 + (BF16 ? 0 : 8 * e);  // of the first word
+                        char* yp = reinterpret_cast<char*>(p.Y) + (off + col) * (BF16 ? 2 : 4);
+                        if (decltype(wide)::value) {
+                            if (col < cols) st_global_8(yp, w);
+                        } else {
+#pragma unroll
+                            for (int g = 0; g < 2; ++g)
+                                if (col + g * (BF16 ? 8 : 4) < cols)
+                                    reinterpret_cast<uint4*>(yp)[g] = make_uint4(w[4 * g], w[4 * g + 1], w[4 * g + 2], w[4 * g + 3]);
+                        }
+                    }
+                }
+            };
+            if (p.wide) finish(std::true_type());
+            else finish(std::false_type());
             tc_fence_before();
             mbar_arrive_cluster(cluster_map(&sh->acc8_empty, 0));
         }
@@ -336,17 +359,16 @@ cudaError_t launch_mixed_gemm_tiles(int T, int N, int K, int r, const int8_t* x8
         em != cudaErrorNotSupported)
         return em;
     const bool asym = z_x8 != nullptr;  // then x8 / x4e hold unsigned codes
+    using Kernel = decltype(&mixed_gemm_kernel<false, false>);
+    const Kernel kernels[4] = {mixed_gemm_kernel<false, false>, mixed_gemm_kernel<false, true>, mixed_gemm_kernel<true, false>,
+                               mixed_gemm_kernel<true, true>};
     static bool attr_set[64] = {};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 64 && !attr_set[dev]) {
-        e = cudaFuncSetAttribute(mixed_gemm_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 static_cast<int>(kSmemBytes));
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(mixed_gemm_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 static_cast<int>(kSmemBytes));
-        if (e != cudaSuccess) return e;
+        for (const Kernel k : kernels)
+            if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSmemBytes))) != cudaSuccess) return e;
         attr_set[dev] = true;
     }
     const int K4 = K - r;
@@ -372,12 +394,14 @@ cudaError_t launch_mixed_gemm_tiles(int T, int N, int K, int r, const int8_t* x8
     p.s_x8 = s_x8; p.s_x4 = s_x4; p.s_w8 = s_w8; p.s_w4 = s_w4;
     p.w_fp16 = w_scale_fp16 ? 1 : 0;
     p.z_x8 = z_x8; p.z_x4 = z_x4; p.wsum8 = wsum8; p.wsum4 = wsum4;
-    p.Y = Y; p.y_dtype = y_dtype; p.dbg8 = dbg8; p.dbg4 = dbg8 ? dbg4 : nullptr;
+    const bool bf16 = y_dtype == RESQ_Y_BF16;
+    p.Y = Y; p.wide = (reinterpret_cast<uintptr_t>(Y) | static_cast<uintptr_t>(N) * (bf16 ? 2 : 4)) % 32 == 0;
+    p.dbg8 = dbg8; p.dbg4 = dbg8 ? dbg4 : nullptr;
     p.status = device_status_ptr();
     const int tiles = p.m_tiles * p.n_tiles;
     const int pairs = tiles < sms / 2 ? tiles : sms / 2;
     count_launch();
-    return launch_programmatic(asym ? mixed_gemm_kernel<true> : mixed_gemm_kernel<false>, 2 * pairs, kThreads, kSmemBytes, st,
+    return launch_programmatic(kernels[2 * asym + bf16], 2 * pairs, kThreads, kSmemBytes, st,
                                tA8, tA4, tB8, tB4, p);
 }
 

@@ -245,6 +245,12 @@ __device__ __forceinline__ void cluster_sync_all() {  // every thread of every C
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 // Address, in the cluster's shared-memory window, of `local` as seen in the CTA of rank `rank`.
+// 32 bytes to global memory, aligned to 32.
+__device__ __forceinline__ void st_global_8(void* p, const uint32_t* v) {
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]),
+                 "r"(v[5]), "r"(v[6]), "r"(v[7])
+                 : "memory");
+}
 __device__ __forceinline__ uint32_t cluster_map(const void* local, uint32_t rank) {
     uint32_t a;
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(local)), "r"(rank));
@@ -340,6 +346,14 @@ __device__ __forceinline__ void tc_commit_pair_if(bool issue, uint64_t* bar, uin
 // TMEM -> registers: this warp's 32 lanes, that many consecutive 32-bit columns at one or each of two addresses; thread i gets lane i.
 // A load and its wait are one statement: the registers are written at any time between the two, so the compiler may not be given
 // a place between them for something that moves one (a copy, a spill).
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&v)[8]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+        : "r"(taddr)
+        : "memory");
+}
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x16.b32 {"

@@ -18,7 +18,7 @@ def _unpack(w4, K4):
 @pytest.mark.parametrize("T,K,r,N,splits", [
     (17, 512, 64, 200, 1), (33, 256, 32, 264, 1), (300, 1024, 96, 520, 1), (40, 256, 224, 8, 1), (1537, 14336, 0, 4096, 1),
     (17, 8192, 1024, 8192, 2), (250, 14336, 0, 2184, 2), (23, 6144, 6112, 256, 3), (61, 14336, 1792, 1032, 3), (257, 14336, 32, 2048, 3),
-    (1700, 256, 32, 3000, 0), (2049, 512, 480, 2056, 0), (1793, 384, 0, 4104, 0)])  # 0: 256 x 256 tiles
+    (1700, 256, 32, 3000, 0), (2049, 512, 480, 2056, 0), (1793, 384, 0, 4104, 0), (2100, 256, 128, 2064, 0)])  # 0: 256 x 256 tiles
 def test_sums_and_scales(T, K, r, N, splits, asym):
     import paper_2412_14363_b200 as resq
 
@@ -48,7 +48,8 @@ def test_sums_and_scales(T, K, r, N, splits, asym):
     for dt in (torch.float32, torch.bfloat16):
         outs = []
         for dbg in (False, True):
-            Y = torch.full((T + 1, N), 9.0, dtype=dt, device="cuda")
+            skip = 16 // dt.itemsize if dbg else 0  # once on 32 bytes, once 16 behind
+            Y = torch.full((skip + (T + 1) * N,), 9.0, dtype=dt, device="cuda")[skip:].view(T + 1, N)
             d = [torch.full((T, N), 77, dtype=torch.int32, device="cuda") if dbg else None for _ in range(2)]
             if asym:
                 resq.resq_mixed_gemm_asym(W, *wsum, x8, x4, s8, s4, z8, z4, Y[:T], ws, *d)
