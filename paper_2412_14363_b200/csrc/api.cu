@@ -222,13 +222,14 @@ int resq_project_quantize(const void* X, const void* P, int T, int K, int r, int
     for (int t0 = 0; t0 < T; t0 += kPanelRows) {
         const int rows = T - t0 < kPanelRows ? T - t0 : kPanelRows;
         const char* Xp = static_cast<const char*>(X) + static_cast<size_t>(t0) * K * 2;
-        if (cudaError_t e = launch_project_gemm(Xp, P, rows, K, panel, st, scratch, project_split_scratch_bytes());
+        const RowCodes out = {r, x8 + static_cast<size_t>(t0) * r, x4 ? x4 + static_cast<size_t>(t0) * K4 / 2 : nullptr,
+                              x4_i8 ? x4_i8 + static_cast<size_t>(t0) * K4 : nullptr, s_x8 + t0, s_x4 + t0, nullptr, nullptr};
+        bool coded = false;
+        if (cudaError_t e = launch_project_gemm(Xp, P, rows, K, panel, st, scratch, project_split_scratch_bytes(), &out, &coded);
             e != cudaSuccess)
             return cuda_status(e);
-        if (cudaError_t e = launch_split_quantize(panel, true, rows, K, r, x8 + static_cast<size_t>(t0) * r,
-                                                  x4 ? x4 + static_cast<size_t>(t0) * K4 / 2 : nullptr, s_x8 + t0,
-                                                  s_x4 + t0, false,
-                                                  x4_i8 ? x4_i8 + static_cast<size_t>(t0) * K4 : nullptr,
+        if (coded) continue;
+        if (cudaError_t e = launch_split_quantize(panel, true, rows, K, r, out.q8, out.q4, out.s8, out.s4, false, out.q4e,
                                                   static_cast<size_t>(K) * 4, st);
             e != cudaSuccess)
             return cuda_status(e);
@@ -400,13 +401,16 @@ int resq_project_quantize_asym(const void* X, const void* P, int T, int K, int r
     for (int t0 = 0; t0 < T; t0 += kPanelRows) {
         const int rows = T - t0 < kPanelRows ? T - t0 : kPanelRows;
         const char* Xp = static_cast<const char*>(X) + static_cast<size_t>(t0) * K * 2;
-        if (cudaError_t e = launch_project_gemm(Xp, P, rows, K, panel, st, scratch, project_split_scratch_bytes());
+        uint8_t* const p8 = u8 + static_cast<size_t>(t0) * r;
+        uint8_t* const p4 = u4 ? u4 + static_cast<size_t>(t0) * K4 / 2 : nullptr;
+        uint8_t* const p4e = u4_u8 ? u4_u8 + static_cast<size_t>(t0) * K4 : nullptr;
+        const RowCodes out = {r, reinterpret_cast<int8_t*>(p8), p4, reinterpret_cast<int8_t*>(p4e), s_x8 + t0, s_x4 + t0, z_x8 + t0, z_x4 + t0};
+        bool coded = false;
+        if (cudaError_t e = launch_project_gemm(Xp, P, rows, K, panel, st, scratch, project_split_scratch_bytes(), &out, &coded);
             e != cudaSuccess)
             return cuda_status(e);
-        if (cudaError_t e = launch_split_quantize_asym(panel, true, rows, K, r, u8 + static_cast<size_t>(t0) * r,
-                                                       u4 ? u4 + static_cast<size_t>(t0) * K4 / 2 : nullptr, s_x8 + t0,
-                                                       s_x4 + t0, z_x8 + t0, z_x4 + t0,
-                                                       u4_u8 ? u4_u8 + static_cast<size_t>(t0) * K4 : nullptr,
+        if (coded) continue;
+        if (cudaError_t e = launch_split_quantize_asym(panel, true, rows, K, r, p8, p4, s_x8 + t0, s_x4 + t0, z_x8 + t0, z_x4 + t0, p4e,
                                                        static_cast<size_t>(K) * 4, st);
             e != cudaSuccess)
             return cuda_status(e);

@@ -102,8 +102,17 @@ void set_decode_early_weights(int on);
 // Online projection C = X·P (bf16 x bf16 -> fp32) on tcgen05 kind::f16, CTA pairs; writes fp32 C [T][K].
 // scratch (optional, project_split_scratch_bytes() bytes): lets a thinly filled last round of tiles be cut along K.
 size_t project_split_scratch_bytes();
+// With `codes`, a product of few rows whose reduction is cut quantizes its rows as it sums the slices: *coded is set, C stays unwritten.
+struct RowCodes {  // of Eq. 1: symmetric, or with zero-points the asymmetric form; q4 (packed) or q4e (bytes) may be null
+    int r;
+    int8_t* q8;
+    uint8_t* q4;
+    int8_t* q4e;
+    float *s8, *s4, *z8, *z4;
+};
 cudaError_t launch_project_gemm(const void* X, const void* P, int T, int K, float* C, cudaStream_t st,
-                                void* scratch = nullptr, size_t scratch_bytes = 0);
+                                void* scratch = nullptr, size_t scratch_bytes = 0, const RowCodes* codes = nullptr,
+                                bool* coded = nullptr);
 
 // ---- attention-block path (declared in resq_kv.h) ----
 cudaError_t launch_uc_quantize(const float* W_C, int d_head, int8_t* wq, float* s_u, cudaStream_t st);

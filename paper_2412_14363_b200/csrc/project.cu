@@ -21,6 +21,7 @@
 
 #include "internal.h"
 #include "ptx.cuh"
+#include "row_codes.cuh"
 
 namespace resq {
 namespace {
@@ -146,6 +147,137 @@ __global__ void __launch_bounds__(256) project_reduce_kernel(const Params p) {
     }
     if (m0 + row < p.T && n0 + 4 * c4 < p.K)
         *reinterpret_cast<float4*>(p.C + static_cast<size_t>(m0 + row) * p.K + n0 + 4 * c4) = a;
+}
+
+// The same sum for rows that are quantized next (few tokens), and their codes: a cluster of eight CTAs takes a row, a thread one or two
+// chunks of eight coefficients, which stay in its registers between the row's extrema (through the CTAs' shared memory) and the codes.  The
+// coefficients never go to memory, and a launch and a trip to memory fall away.  Same coefficients, same codes as in two kernels.
+// What bounds it: the latency of three trips (partial tiles, extrema, codes out).
+// A whole layer, us, two kernels / one: 2048 x 2048 at 3 tokens 14.0 / 12.4, 4096 x 4096 at 1 / 16 tokens 17.4 / 15.5, 20.1 / 18.8; 8192 x 2048 at
+// 8 tokens 37.5 / 34.3, 14336 x 4096 at 3 / 64 tokens 84.5 / 81.4, 97.6 / 97.7.
+constexpr int kCodeCtas = 8, kCodeThreads = 256, kCodeChunks = 2;
+constexpr int kCodeMaxK = 8 * kCodeCtas * kCodeThreads * kCodeChunks;
+
+template <bool ASYM>
+__global__ void __cluster_dims__(kCodeCtas, 1, 1) __launch_bounds__(kCodeThreads)
+project_reduce_codes_kernel(const Params p, const RowCodes o) {
+    __shared__ float red[4][kCodeThreads / 32];
+    __shared__ __align__(16) float4 mine;
+    griddep_wait();
+    griddep_launch_dependents();  // behind the wait: a dependent that runs finds everything before this grid complete
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int rank = static_cast<int>(cluster_ctarank()), row = blockIdx.x / kCodeCtas;
+    const int nchunks = p.K >> 3, rchunks = o.r >> 3, per = (nchunks + kCodeCtas - 1) / kCodeCtas;
+    const size_t step = static_cast<size_t>(p.prows) * BN / 4;  // from slice to slice of a tile, in float4
+    constexpr float kBig = 3.402823466e38f;
+    float a8 = ASYM ? -kBig : 0.f, a4 = a8, lo8 = kBig, lo4 = kBig;
+    Chunk<true> v[kCodeChunks];
+    auto chunk = [&](int i) { return i * kCodeThreads + tid < per ? rank * per + i * kCodeThreads + tid : nchunks; };
+#pragma unroll
+    for (int i = 0; i < kCodeChunks; ++i) {
+        const int c = chunk(i);
+        if (c >= nchunks) continue;
+        const int col = c * 8, tile = col / BN;
+        const float4* part = reinterpret_cast<const float4*>(
+            p.partial + (static_cast<size_t>(tile) * p.splits * p.prows + row) * BN + (col - tile * BN));
+        float4 s[2];
+        for (int s0 = 0; s0 < p.splits; s0 += 4) {
+            float4 u[4][2];
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+                    u[k][h] = s0 + k < p.splits ? __ldcg(part + static_cast<size_t>(s0 + k) * step + h) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (s0 + k < p.splits)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        if (s0 + k == 0) s[h] = u[k][h];
+                        else { s[h].x += u[k][h].x; s[h].y += u[k][h].y; s[h].z += u[k][h].z; s[h].w += u[k][h].w; }
+                    }
+        }
+        const float f[8] = {s[0].x, s[0].y, s[0].z, s[0].w, s[1].x, s[1].y, s[1].z, s[1].w};
+        float lo = kBig, hi = ASYM ? -kBig : 0.f;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            v[i].w[k] = __float_as_uint(f[k]);
+            if (ASYM) lo = fminf(lo, f[k]);
+            hi = fmaxf(hi, ASYM ? f[k] : fabsf(f[k]));
+        }
+        if (c < rchunks) { a8 = fmaxf(a8, hi); lo8 = fminf(lo8, lo); }
+        else { a4 = fmaxf(a4, hi); lo4 = fminf(lo4, lo); }
+    }
+    auto fold = [&](int m) {
+        a8 = fmaxf(a8, __shfl_xor_sync(0xffffffffu, a8, m));
+        a4 = fmaxf(a4, __shfl_xor_sync(0xffffffffu, a4, m));
+        if (ASYM) {
+            lo8 = fminf(lo8, __shfl_xor_sync(0xffffffffu, lo8, m));
+            lo4 = fminf(lo4, __shfl_xor_sync(0xffffffffu, lo4, m));
+        }
+    };
+#pragma unroll
+    for (int m = 16; m > 0; m >>= 1) fold(m);
+    if (lane == 0) {
+        red[0][warp] = a8;
+        red[1][warp] = a4;
+        red[2][warp] = lo8;
+        red[3][warp] = lo4;
+    }
+    __syncthreads();
+    if (warp == 0) {
+        a8 = red[0][lane & 7]; a4 = red[1][lane & 7]; lo8 = red[2][lane & 7]; lo4 = red[3][lane & 7];
+#pragma unroll
+        for (int m = 4; m > 0; m >>= 1) fold(m);
+        if (lane == 0) mine = make_float4(a8, a4, lo8, lo4);
+        __syncwarp();
+    }
+    cluster_sync_all();
+    const float4 other = ld_cluster_f4(cluster_map(&mine, lane & 7));
+    a8 = other.x; a4 = other.y; lo8 = other.z; lo4 = other.w;
+#pragma unroll
+    for (int m = 4; m > 0; m >>= 1) fold(m);
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");  // no CTA leaves before all have read its extrema
+
+    if (ASYM && rchunks == 0) lo8 = a8 = 0.f;  // uniform 4-bit layer: the empty INT8 segment has s = 0, z = 0
+    const float s8 = ASYM ? __fdiv_rn(__fsub_rn(a8, lo8), 255.f) : __fdiv_rn(a8, 127.f);
+    const float s4 = ASYM ? __fdiv_rn(__fsub_rn(a4, lo4), 15.f) : __fdiv_rn(a4, 7.f);
+    const ScaleInv i8(s8), i4(s4);
+    if (rank == 0 && tid == 0) {
+        o.s8[row] = s8;
+        o.s4[row] = s4;
+        if (ASYM) {
+            o.z8[row] = lo8;
+            o.z4[row] = lo4;
+        }
+    }
+    const int K4 = p.K - o.r;
+#pragma unroll
+    for (int i = 0; i < kCodeChunks; ++i) {
+        const int c = chunk(i);
+        if (c >= nchunks) continue;
+        const bool seg8 = c < rchunks;
+        const float s = seg8 ? s8 : s4, inv = seg8 ? i8.inv : i4.inv;
+        const bool exact = seg8 ? i8.exact : i4.exact;
+        uint32_t t[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+        if (s > 0.f) {
+            if constexpr (ASYM) fast_codes_asym(v[i], seg8 ? lo8 : lo4, s, inv, exact, seg8 ? 255.f : 15.f, t);
+            else fast_codes(v[i], s, inv, exact, t);
+        }
+        const uint32_t lo = pack_low_bytes(t[0], t[1], t[2], t[3]), hi = pack_low_bytes(t[4], t[5], t[6], t[7]);
+        if (seg8) {
+            *reinterpret_cast<uint2*>(o.q8 + static_cast<size_t>(row) * o.r + c * 8) = make_uint2(lo, hi);
+        } else {
+            const int jj = (c - rchunks) * 8;
+            if (o.q4e) *reinterpret_cast<uint2*>(o.q4e + static_cast<size_t>(row) * K4 + jj) = make_uint2(lo, hi);
+            if (o.q4) {
+                const uint32_t xl = lo & 0x0F0F0F0Fu, xh = hi & 0x0F0F0F0Fu;
+                *reinterpret_cast<uint32_t*>(o.q4 + static_cast<size_t>(row) * (K4 / 2) + (jj >> 1)) =
+                    __byte_perm(xl | (xl >> 4), xh | (xh >> 4), 0x6420);
+            }
+        }
+    }
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
@@ -510,7 +642,7 @@ cudaError_t launch_reduce(const Params& p, cudaStream_t st) {
 // slices 74.3 / 67.7 / 69.6 / 70.3 / 79.4 us (25 is what the count without the 3 takes); K = 8192, T = 2: 2 / 9 / 16 slices
 // 25.9 / 28.2 / 30.8 us.
 cudaError_t launch_project_few(const void* X, const void* P, int T, int K, float* C, cudaStream_t st, void* scratch,
-                               size_t scratch_bytes, int dev) {
+                               size_t scratch_bytes, int dev, const RowCodes* codes, bool* coded) {
     static bool attr_set[64] = {};
     if (dev < 64 && !attr_set[dev]) {
         if (cudaError_t e = cudaFuncSetAttribute(project_gemm_few_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -560,10 +692,12 @@ cudaError_t launch_project_few(const void* X, const void* P, int T, int K, float
     if (cudaError_t e = launch_programmatic(project_gemm_few_kernel, 2 * pairs, kThreads, kFewSmemBytes, st, tX, tP, p, ntok);
         e != cudaSuccess)
         return e;
-    if (p.split_tiles > 0) {
-        return launch_reduce(p, st);
-    }
-    return cudaSuccess;
+    if (p.split_tiles == 0) return cudaSuccess;
+    if (!codes || K > kCodeMaxK) return launch_reduce(p, st);
+    *coded = true;
+    count_launch();
+    return launch_programmatic(codes->z8 ? project_reduce_codes_kernel<true> : project_reduce_codes_kernel<false>, static_cast<size_t>(T) * kCodeCtas,
+                               kCodeThreads, 0, st, p, *codes);
 }
 
 }  // namespace
@@ -571,7 +705,7 @@ cudaError_t launch_project_few(const void* X, const void* P, int T, int K, float
 size_t project_split_scratch_bytes() { return static_cast<size_t>(74) * (2 * BM) * BN * sizeof(float); }
 
 cudaError_t launch_project_gemm(const void* X, const void* P, int T, int K, float* C, cudaStream_t st, void* scratch,
-                                size_t scratch_bytes) {
+                                size_t scratch_bytes, const RowCodes* codes, bool* coded) {
     static bool attr_set[64] = {};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -582,7 +716,7 @@ cudaError_t launch_project_gemm(const void* X, const void* P, int T, int K, floa
         if (e != cudaSuccess) return e;
         attr_set[dev] = true;
     }
-    if (T <= kFewMaxT) return launch_project_few(X, P, T, K, C, st, scratch, scratch_bytes, dev);
+    if (T <= kFewMaxT) return launch_project_few(X, P, T, K, C, st, scratch, scratch_bytes, dev, codes, coded);
     CUtensorMap tX, tP;
     if (!make_map_bf16(&tX, X, T, K, BM) || !make_map_bf16(&tP, P, K, K, BK)) return cudaErrorInvalidValue;
     Params p;

@@ -244,13 +244,13 @@ __device__ __forceinline__ uint32_t cluster_ctarank() {
 __device__ __forceinline__ void cluster_sync_all() {  // every thread of every CTA of the cluster
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-// Address, in the cluster's shared-memory window, of `local` as seen in the CTA of rank `rank`.
 // 32 bytes to global memory, aligned to 32.
 __device__ __forceinline__ void st_global_8(void* p, const uint32_t* v) {
     asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]),
                  "r"(v[5]), "r"(v[6]), "r"(v[7])
                  : "memory");
 }
+// Address, in the cluster's shared-memory window, of `local` as seen in the CTA of rank `rank`.
 __device__ __forceinline__ uint32_t cluster_map(const void* local, uint32_t rank) {
     uint32_t a;
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(local)), "r"(rank));
