@@ -8,6 +8,8 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include <type_traits>
+
 #include "internal.h"
 #include "packed_fp32.cuh"
 #include "ptx.cuh"
@@ -527,12 +529,73 @@ __device__ __forceinline__ void butterfly_pairs(float* hrow, int K, int s, int t
     }
 }
 
+// Rows of 2^k with PAIRS: the first four index bits are the "small factor", groups of M = 16 coefficients.  Group a's 16-byte quarters sit
+// in the order q ^ (a >> 1 & 3), so that eight groups' quarters, which eight threads write together, cover all banks (in order: 4 ways).
+__device__ __forceinline__ int quarter_at(int a, int q) { return 16 * a + 4 * (q ^ ((a >> 1) & 3)); }
+
+// butterfly_pairs over these groups.  FIRST: s = 0, and the threads' groups are whole runs of 2^NB, NB >= 3, so the order of quarters
+// follows from j; later passes have s >= 3, and it is the same for all j.
+template <int NT, int NB, bool FIRST>
+__device__ __forceinline__ void butterfly_sixteens(float* hrow, int K, int s, int tid, bool last, float inv_sqrt_k, int r, float& a8, float& a4) {
+    constexpr int N = 1 << NB;
+    const int count = K >> (NB + 1);
+    for (int i = tid; i < count; i += NT) {
+        const int arest = i >> 3, b = 2 * (i & 7);
+        const int a0 = FIRST ? arest << NB : ((arest >> s) << (s + NB)) | (arest & ((1 << s) - 1));
+        const int stride = FIRST ? 16 : 16 << s;
+        float* at[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) at[c] = hrow + quarter_at(a0, (b >> 2) ^ (FIRST ? c : 0)) + (b & 2);
+        auto place = [&](int j) { return reinterpret_cast<f2*>(at[FIRST ? (j >> 1) & 3 : 0] + j * stride); };
+        f2 v[N];
+#pragma unroll
+        for (int j = 0; j < N; ++j) v[j] = *place(j);
+#pragma unroll
+        for (int bit = 0; bit < NB; ++bit) {
+#pragma unroll
+            for (int j = 0; j < N; ++j) {
+                if (!(j & (1 << bit))) {
+                    const f2 lo = v[j], hi = v[j | (1 << bit)];
+                    v[j] = add2(lo, hi);
+                    v[j | (1 << bit)] = sub2(lo, hi);
+                }
+            }
+        }
+        if (last) {
+            const f2 scale = pack2(inv_sqrt_k, inv_sqrt_k);
+            const int e0 = a0 * 16 + b;  // r is a multiple of 8: a pair is in one segment
+#pragma unroll
+            for (int j = 0; j < N; ++j) v[j] = mul2(v[j], scale);
+            if (e0 >= r) {
+#pragma unroll
+                for (int j = 0; j < N; ++j) {
+                    const float2 x = unpack2(v[j]);
+                    a4 = fmaxf(a4, fmaxf(fabsf(x.x), fabsf(x.y)));
+                }
+            } else {
+#pragma unroll
+                for (int j = 0; j < N; ++j) {
+                    const float2 x = unpack2(v[j]);
+                    float& m = e0 + j * stride < r ? a8 : a4;
+                    m = fmaxf(m, fmaxf(fabsf(x.x), fabsf(x.y)));
+                }
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < N; ++j) *place(j) = v[j];
+    }
+}
+
 // NT threads per row: 256 when rows outnumber the SMs (throughput: several CTAs per SM), 1024 for the few rows of a
 // generation step, where one row's chain of passes is all there is to wait for.
 // PAIRS: butterflies of two neighbours to a thread, for rows of kPairWidth and more.  Narrower ones have fewer pairs than threads: with
 // M = 12 and 28 and pairs, rows of 384 to 896 took 2 to 6 % longer than now (1537 rows of 384 9.7 us, 9.0 now; 1000 rows of 1536
 // 8.2, 8.1; of 1792 8.5, singly 9.1).
 constexpr int kPairWidth = 1792;
+// Rows of 2^k: groups of sixteen from here on, for any number of rows, 256 threads a row.  us, three index bits a pass (of 1024 threads a row up to
+// 148 rows) / groups: 1537 rows of 1024 11.6 / 10.0, 2048 16.9 / 11.1, 8192 56.5 / 23.9, 32768 285 / 168; one row of 1024 4.2 / 2.9, 8192
+// 8.5 / 4.6; but 1537 rows of 512 8.6 / 9.8.  One row of 512, 1024 / 256 threads: 3.8 / 2.8.
+constexpr int kSixteensWidth = 1024;
 template <int M, int NT, bool PAIRS = (M > 1 && NT == kThreads)>
 __global__ void __launch_bounds__(NT, NT == kThreads ? (M > 1 ? 3 : 5) : 1)
 hadamard_quantize_kernel(const __nv_bfloat16* X, size_t rows, int K, int kbits, int r, float inv_sqrt_k,
@@ -563,7 +626,34 @@ hadamard_quantize_kernel(const __nv_bfloat16* X, size_t rows, int K, int kbits, 
         if constexpr (M == 1) __syncthreads();
         // 2. the small factor, one group of M consecutive coefficients per thread: bf16 from global memory (M * 2 bytes
         //    per group, a multiple of 8), fp32 result to the row buffer
-        if constexpr (M > 1) {
+        if constexpr (M == 16) {  // bits 0 to 3 of a row of 2^k
+            for (int a = tid; a < (K >> 4); a += NT) {
+                const uint4* xg = xp + 2 * a;
+                const uint4 u0 = xg[0], u1 = xg[1];
+                const uint32_t w[8] = {u0.x, u0.y, u0.z, u0.w, u1.x, u1.y, u1.z, u1.w};
+                f2 v[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const float lo = __uint_as_float(w[i] << 16), hi = __uint_as_float(w[i] & 0xFFFF0000u);
+                    v[i] = add2(pack2(lo, lo), pack2(hi, -hi));
+                }
+#pragma unroll
+                for (int bit = 1; bit < 8; bit *= 2)
+#pragma unroll
+                    for (int i = 0; i < 8; ++i)
+                        if (!(i & bit)) {
+                            const f2 lo = v[i], hi = v[i | bit];
+                            v[i] = add2(lo, hi);
+                            v[i | bit] = sub2(lo, hi);
+                        }
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const float2 lo = unpack2(v[2 * q]), hi = unpack2(v[2 * q + 1]);
+                    *reinterpret_cast<float4*>(hrow + quarter_at(a, q)) = make_float4(lo.x, lo.y, hi.x, hi.y);
+                }
+            }
+            __syncthreads();
+        } else if constexpr (M > 1) {
             constexpr Conference<M> conf{};
             constexpr int H2 = M / 2;
             for (int a = tid; a < (K / M); a += NT) {
@@ -625,7 +715,19 @@ hadamard_quantize_kernel(const __nv_bfloat16* X, size_t rows, int K, int kbits, 
             const int left = kbits - s;
             const int nb = left <= kMaxBits ? left : (left <= 2 * kMaxBits ? (left + 1) / 2 : kMaxBits);
             const bool last = s + nb >= kbits;
-            if constexpr (PAIRS) {  // 1024 threads have no registers for 32 pairs; M = 1 has odd neighbours in the first pass
+            if constexpr (M == 16) {
+                auto pass = [&](auto bits, auto first) {
+                    butterfly_sixteens<NT, decltype(bits)::value, decltype(first)::value>(hrow, K, s, tid, last, inv_sqrt_k, r, a8, a4);
+                };
+                using std::integral_constant;
+                if (s == 0) {
+                    if (nb == 3) pass(integral_constant<int, 3>(), std::true_type());
+                    else if (nb == 4) pass(integral_constant<int, 4>(), std::true_type());
+                    else pass(integral_constant<int, 5>(), std::true_type());
+                } else if (nb == 3) pass(integral_constant<int, 3>(), std::false_type());
+                else if (nb == 4) pass(integral_constant<int, 4>(), std::false_type());
+                else pass(integral_constant<int, 5>(), std::false_type());
+            } else if constexpr (PAIRS) {  // 1024 threads have no registers for 32 pairs; M = 1 has odd neighbours in the first pass
                 if (nb == 1) butterfly_pairs<M, NT, 1>(hrow, K, s, tid, last, inv_sqrt_k, r, a8, a4);
                 else if (nb == 2) butterfly_pairs<M, NT, 2>(hrow, K, s, tid, last, inv_sqrt_k, r, a8, a4);
                 else if (nb == 3) butterfly_pairs<M, NT, 3>(hrow, K, s, tid, last, inv_sqrt_k, r, a8, a4);
@@ -684,7 +786,18 @@ hadamard_quantize_kernel(const __nv_bfloat16* X, size_t rows, int K, int kbits, 
             uint32_t t[8];
             const bool seg8 = c < rchunks;
             const float s = seg8 ? s8 : s4;
-            if (s > 0.f) fast_codes(lds_chunk<true>(srow, c), s, seg8 ? inv8 : inv4, seg8 ? exact8 : exact4, t);
+            Chunk<true> ch;
+            if constexpr (M == 16) {
+                const int a = c >> 1, q = 2 * (c & 1);
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const uint4 u = *reinterpret_cast<const uint4*>(hrow + quarter_at(a, q + h));
+                    ch.w[4 * h] = u.x; ch.w[4 * h + 1] = u.y; ch.w[4 * h + 2] = u.z; ch.w[4 * h + 3] = u.w;
+                }
+            } else {
+                ch = lds_chunk<true>(srow, c);
+            }
+            if (s > 0.f) fast_codes(ch, s, seg8 ? inv8 : inv4, seg8 ? exact8 : exact4, t);
             else {
 #pragma unroll
                 for (int k = 0; k < 8; ++k) t[k] = 0;
@@ -829,22 +942,21 @@ cudaError_t launch_hadamard_quantize(const void* X, size_t rows, int K, int r, i
         // Once per device: the shared-memory limit of the kernels.
         for (auto k : {hadamard_quantize_kernel<1, kThreads>, hadamard_quantize_kernel<12, kThreads>,
                        hadamard_quantize_kernel<28, kThreads>, hadamard_quantize_kernel<12, kThreads, false>,
-                       hadamard_quantize_kernel<28, kThreads, false>, hadamard_quantize_kernel<1, kWideThreads>,
+                       hadamard_quantize_kernel<28, kThreads, false>, hadamard_quantize_kernel<16, kThreads>,
                        hadamard_quantize_kernel<12, kWideThreads>, hadamard_quantize_kernel<28, kWideThreads>})
             if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024)) != cudaSuccess)
                 return e;
         ready[dev] = true;
     }
+    // 1024 threads per row only when rows do not outnumber the SMs: at 28672-wide rows (two 256-thread CTAs per SM)
+    // the wide form measured slower for many rows (0.89 against 0.72 ms at 8192 rows).
+    const bool wide = rows <= kWideMaxRows && m != 1;
+    if (m == 1 && K >= kSixteensWidth) kbits -= 4;  // the group's own bits
     const float inv_sqrt_k = static_cast<float>(1.0 / sqrt(static_cast<double>(K)));
     const unsigned grid = static_cast<unsigned>(rows < 148u * 16u ? rows : 148u * 16u);
     const __nv_bfloat16* x = static_cast<const __nv_bfloat16*>(X);
-    // 1024 threads per row only when rows do not outnumber the SMs: at 28672-wide rows (two 256-thread CTAs per SM)
-    // the wide form measured slower for many rows (0.89 against 0.72 ms at 8192 rows).
-    const bool wide = rows <= kWideMaxRows;
-    auto kern = wide ? (m == 1    ? hadamard_quantize_kernel<1, kWideThreads>
-                        : m == 12 ? hadamard_quantize_kernel<12, kWideThreads>
-                                  : hadamard_quantize_kernel<28, kWideThreads>)
-                : m == 1         ? hadamard_quantize_kernel<1, kThreads>
+    auto kern = wide ? (m == 12 ? hadamard_quantize_kernel<12, kWideThreads> : hadamard_quantize_kernel<28, kWideThreads>)
+                : m == 1         ? (K < kSixteensWidth ? hadamard_quantize_kernel<1, kThreads> : hadamard_quantize_kernel<16, kThreads>)
                 : K < kPairWidth ? (m == 12 ? hadamard_quantize_kernel<12, kThreads, false> : hadamard_quantize_kernel<28, kThreads, false>)
                                  : (m == 12 ? hadamard_quantize_kernel<12, kThreads> : hadamard_quantize_kernel<28, kThreads>);
     count_launch();
