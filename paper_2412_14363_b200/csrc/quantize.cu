@@ -4,6 +4,7 @@
 // keeps up to kMaxChunks of them in registers so the row is read from memory once, reduces the two
 // per-segment absmax values with warp shuffles + one shared-memory step, then emits int8 codes
 // (8-byte stores) and packed int4 codes (4-byte stores).
+#include <algorithm>
 #include <cmath>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -439,6 +440,10 @@ struct Conference {
 
 constexpr int kWideThreads = 1024;  // threads per row when there are at most kWideMaxRows rows (one CTA per SM)
 constexpr int kWideMaxRows = 148;
+// Place of group a of M coefficients in the row buffer: one group is left free behind every 2^run, a run being what a thread of the first
+// pass walks through.  The threads of a warp take neighbouring runs there, which all begin at the same bank otherwise (2^run * M words, 2 ways).
+__device__ __forceinline__ int slot_of(int a, int run) { return a + (a >> run); }
+__device__ __forceinline__ int slot_stride(int s, int run) { return (1 << s) + (s >= run ? 1 << (s - run) : 0); }  // of index bit s
 // One pass of the Sylvester butterflies: index bits [s, s + NB) of a, 2^NB values per thread in registers.  The last
 // pass also scales by 1 / sqrt(K) and collects the two absmax values (elements below r belong to the INT8 segment).
 template <int M, int NT, int NB>
@@ -481,15 +486,15 @@ __device__ __forceinline__ void butterfly_pass(float* hrow, int K, int s, int ti
 
 // The same for M even, a thread taking coefficients b and b + 1 of its 2^NB groups as pairs: half the instructions.
 template <int M, int NT, int NB>
-__device__ __forceinline__ void butterfly_pairs(float* hrow, int K, int s, int tid, bool last, float inv_sqrt_k, int r, float& a8,
+__device__ __forceinline__ void butterfly_pairs(float* hrow, int K, int s, int run, int tid, bool last, float inv_sqrt_k, int r, float& a8,
                                                 float& a4) {
     constexpr int N = 1 << NB;
     const int count = K >> (NB + 1);
-    const int stride = M << s;
+    const int estride = M << s, stride = slot_stride(s, run) * M;  // of the coefficients, of their places
     for (int i = tid; i < count; i += NT) {
         const int arest = i / (M / 2), b = 2 * (i - arest * (M / 2));
         const int a0 = ((arest >> s) << (s + NB)) | (arest & ((1 << s) - 1));
-        f2* base = reinterpret_cast<f2*>(hrow + a0 * M + b);
+        f2* base = reinterpret_cast<f2*>(hrow + slot_of(a0, run) * M + b);
         f2 v[N];
 #pragma unroll
         for (int j = 0; j < N; ++j) v[j] = base[j * (stride / 2)];
@@ -519,7 +524,7 @@ __device__ __forceinline__ void butterfly_pairs(float* hrow, int K, int s, int t
 #pragma unroll
                 for (int j = 0; j < N; ++j) {
                     const float2 x = unpack2(v[j]);
-                    float& m = e0 + j * stride < r ? a8 : a4;
+                    float& m = e0 + j * estride < r ? a8 : a4;
                     m = fmaxf(m, fmaxf(fabsf(x.x), fabsf(x.y)));
                 }
             }
@@ -531,21 +536,21 @@ __device__ __forceinline__ void butterfly_pairs(float* hrow, int K, int s, int t
 
 // Rows of 2^k with PAIRS: the first four index bits are the "small factor", groups of M = 16 coefficients.  Group a's 16-byte quarters sit
 // in the order q ^ (a >> 1 & 3), so that eight groups' quarters, which eight threads write together, cover all banks (in order: 4 ways).
-__device__ __forceinline__ int quarter_at(int a, int q) { return 16 * a + 4 * (q ^ ((a >> 1) & 3)); }
+__device__ __forceinline__ int quarter_at(int a, int q, int run) { return 16 * slot_of(a, run) + 4 * (q ^ ((a >> 1) & 3)); }
 
 // butterfly_pairs over these groups.  FIRST: s = 0, and the threads' groups are whole runs of 2^NB, NB >= 3, so the order of quarters
 // follows from j; later passes have s >= 3, and it is the same for all j.
 template <int NT, int NB, bool FIRST>
-__device__ __forceinline__ void butterfly_sixteens(float* hrow, int K, int s, int tid, bool last, float inv_sqrt_k, int r, float& a8, float& a4) {
+__device__ __forceinline__ void butterfly_sixteens(float* hrow, int K, int s, int run, int tid, bool last, float inv_sqrt_k, int r, float& a8, float& a4) {
     constexpr int N = 1 << NB;
     const int count = K >> (NB + 1);
     for (int i = tid; i < count; i += NT) {
         const int arest = i >> 3, b = 2 * (i & 7);
         const int a0 = FIRST ? arest << NB : ((arest >> s) << (s + NB)) | (arest & ((1 << s) - 1));
-        const int stride = FIRST ? 16 : 16 << s;
+        const int estride = FIRST ? 16 : 16 << s, stride = FIRST ? 16 : 16 * slot_stride(s, run);
         float* at[4];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) at[c] = hrow + quarter_at(a0, (b >> 2) ^ (FIRST ? c : 0)) + (b & 2);
+        for (int c = 0; c < 4; ++c) at[c] = hrow + quarter_at(a0, (b >> 2) ^ (FIRST ? c : 0), run) + (b & 2);
         auto place = [&](int j) { return reinterpret_cast<f2*>(at[FIRST ? (j >> 1) & 3 : 0] + j * stride); };
         f2 v[N];
 #pragma unroll
@@ -576,7 +581,7 @@ __device__ __forceinline__ void butterfly_sixteens(float* hrow, int K, int s, in
 #pragma unroll
                 for (int j = 0; j < N; ++j) {
                     const float2 x = unpack2(v[j]);
-                    float& m = e0 + j * stride < r ? a8 : a4;
+                    float& m = e0 + j * estride < r ? a8 : a4;
                     m = fmaxf(m, fmaxf(fabsf(x.x), fabsf(x.y)));
                 }
             }
@@ -598,7 +603,7 @@ constexpr int kPairWidth = 1792;
 constexpr int kSixteensWidth = 1024;
 template <int M, int NT, bool PAIRS = (M > 1 && NT == kThreads)>
 __global__ void __launch_bounds__(NT, NT == kThreads ? (M > 1 ? 3 : 5) : 1)
-hadamard_quantize_kernel(const __nv_bfloat16* X, size_t rows, int K, int kbits, int r, float inv_sqrt_k,
+hadamard_quantize_kernel(const __nv_bfloat16* X, size_t rows, int K, int kbits, int run, int r, float inv_sqrt_k,
                          int8_t* __restrict__ q8, uint8_t* __restrict__ q4, float* __restrict__ s8_out,
                          float* __restrict__ s4_out, int8_t* __restrict__ q4e) {
     extern __shared__ __align__(16) float hrow[];  // [K]
@@ -649,7 +654,7 @@ hadamard_quantize_kernel(const __nv_bfloat16* X, size_t rows, int K, int kbits, 
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
                     const float2 lo = unpack2(v[2 * q]), hi = unpack2(v[2 * q + 1]);
-                    *reinterpret_cast<float4*>(hrow + quarter_at(a, q)) = make_float4(lo.x, lo.y, hi.x, hi.y);
+                    *reinterpret_cast<float4*>(hrow + quarter_at(a, q, run)) = make_float4(lo.x, lo.y, hi.x, hi.y);
                 }
             }
             __syncthreads();
@@ -658,7 +663,7 @@ hadamard_quantize_kernel(const __nv_bfloat16* X, size_t rows, int K, int kbits, 
             constexpr int H2 = M / 2;
             for (int a = tid; a < (K / M); a += NT) {
                 // M * 4 bytes is a multiple of 16: the group moves as float4s (conflict-free at this stride)
-                float4* gp = reinterpret_cast<float4*>(hrow + a * M);
+                float4* gp = reinterpret_cast<float4*>(hrow + (PAIRS ? slot_of(a, run) : a) * M);
                 const uint2* xg = reinterpret_cast<const uint2*>(X + row * static_cast<size_t>(K) + static_cast<size_t>(a) * M);
                 float y[M];
                 f2 pm[H2];  // (x_2i + x_2i+1, x_2i - x_2i+1)
@@ -717,7 +722,7 @@ hadamard_quantize_kernel(const __nv_bfloat16* X, size_t rows, int K, int kbits, 
             const bool last = s + nb >= kbits;
             if constexpr (M == 16) {
                 auto pass = [&](auto bits, auto first) {
-                    butterfly_sixteens<NT, decltype(bits)::value, decltype(first)::value>(hrow, K, s, tid, last, inv_sqrt_k, r, a8, a4);
+                    butterfly_sixteens<NT, decltype(bits)::value, decltype(first)::value>(hrow, K, s, run, tid, last, inv_sqrt_k, r, a8, a4);
                 };
                 using std::integral_constant;
                 if (s == 0) {
@@ -728,11 +733,11 @@ hadamard_quantize_kernel(const __nv_bfloat16* X, size_t rows, int K, int kbits, 
                 else if (nb == 4) pass(integral_constant<int, 4>(), std::false_type());
                 else pass(integral_constant<int, 5>(), std::false_type());
             } else if constexpr (PAIRS) {  // 1024 threads have no registers for 32 pairs; M = 1 has odd neighbours in the first pass
-                if (nb == 1) butterfly_pairs<M, NT, 1>(hrow, K, s, tid, last, inv_sqrt_k, r, a8, a4);
-                else if (nb == 2) butterfly_pairs<M, NT, 2>(hrow, K, s, tid, last, inv_sqrt_k, r, a8, a4);
-                else if (nb == 3) butterfly_pairs<M, NT, 3>(hrow, K, s, tid, last, inv_sqrt_k, r, a8, a4);
-                else if (nb == 4) butterfly_pairs<M, NT, 4>(hrow, K, s, tid, last, inv_sqrt_k, r, a8, a4);
-                else butterfly_pairs<M, NT, 5>(hrow, K, s, tid, last, inv_sqrt_k, r, a8, a4);
+                if (nb == 1) butterfly_pairs<M, NT, 1>(hrow, K, s, run, tid, last, inv_sqrt_k, r, a8, a4);
+                else if (nb == 2) butterfly_pairs<M, NT, 2>(hrow, K, s, run, tid, last, inv_sqrt_k, r, a8, a4);
+                else if (nb == 3) butterfly_pairs<M, NT, 3>(hrow, K, s, run, tid, last, inv_sqrt_k, r, a8, a4);
+                else if (nb == 4) butterfly_pairs<M, NT, 4>(hrow, K, s, run, tid, last, inv_sqrt_k, r, a8, a4);
+                else butterfly_pairs<M, NT, 5>(hrow, K, s, run, tid, last, inv_sqrt_k, r, a8, a4);
             } else if (nb == 1) butterfly_pass<M, NT, 1>(hrow, K, s, tid, last, inv_sqrt_k, r, a8, a4);
             else if (nb == 2) butterfly_pass<M, NT, 2>(hrow, K, s, tid, last, inv_sqrt_k, r, a8, a4);
             else if (nb == 3) butterfly_pass<M, NT, 3>(hrow, K, s, tid, last, inv_sqrt_k, r, a8, a4);
@@ -791,11 +796,14 @@ hadamard_quantize_kernel(const __nv_bfloat16* X, size_t rows, int K, int kbits, 
                 const int a = c >> 1, q = 2 * (c & 1);
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
-                    const uint4 u = *reinterpret_cast<const uint4*>(hrow + quarter_at(a, q + h));
+                    const uint4 u = *reinterpret_cast<const uint4*>(hrow + quarter_at(a, q + h, run));
                     ch.w[4 * h] = u.x; ch.w[4 * h + 1] = u.y; ch.w[4 * h + 2] = u.z; ch.w[4 * h + 3] = u.w;
                 }
-            } else {
-                ch = lds_chunk<true>(srow, c);
+            } else {  // no run ends within a chunk
+                const uint4* p = reinterpret_cast<const uint4*>(srow) + 2 * c + (PAIRS ? M / 4 * ((8 * c / M) >> run) : 0);
+                const uint4 u = p[0], v = p[1];
+                ch.w[0] = u.x; ch.w[1] = u.y; ch.w[2] = u.z; ch.w[3] = u.w;
+                ch.w[4] = v.x; ch.w[5] = v.y; ch.w[6] = v.z; ch.w[7] = v.w;
             }
             if (s > 0.f) fast_codes(ch, s, seg8 ? inv8 : inv4, seg8 ? exact8 : exact4, t);
             else {
@@ -932,8 +940,9 @@ cudaError_t launch_hadamard_quantize(const void* X, size_t rows, int K, int r, i
     if (rows == 0) return cudaSuccess;
     int kbits = 0, m = 0;
     if (!hadamard_factor(K, &kbits, &m)) return cudaErrorNotSupported;
-    const size_t smem = static_cast<size_t>(K) * 4;
-    if (smem > 200u * 1024u) return cudaErrorNotSupported;
+    constexpr size_t kMaxSmem = 200 * 1024;
+    size_t smem = static_cast<size_t>(K) * 4;
+    if (smem > kMaxSmem) return cudaErrorNotSupported;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
@@ -944,23 +953,37 @@ cudaError_t launch_hadamard_quantize(const void* X, size_t rows, int K, int r, i
                        hadamard_quantize_kernel<28, kThreads>, hadamard_quantize_kernel<12, kThreads, false>,
                        hadamard_quantize_kernel<28, kThreads, false>, hadamard_quantize_kernel<16, kThreads>,
                        hadamard_quantize_kernel<12, kWideThreads>, hadamard_quantize_kernel<28, kWideThreads>})
-            if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024)) != cudaSuccess)
+            if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem)) != cudaSuccess)
                 return e;
         ready[dev] = true;
     }
     // 1024 threads per row only when rows do not outnumber the SMs: at 28672-wide rows (two 256-thread CTAs per SM)
     // the wide form measured slower for many rows (0.89 against 0.72 ms at 8192 rows).
     const bool wide = rows <= kWideMaxRows && m != 1;
-    if (m == 1 && K >= kSixteensWidth) kbits -= 4;  // the group's own bits
+    if (m == 1 && K >= kSixteensWidth) { m = 16; kbits -= 4; }  // the group's own bits
+    const bool pairs = !wide && m > 1 && (m == 16 || K >= kPairWidth);
+    // A place left free behind every run of the first pass (slot_of), unless fewer CTAs then fit an SM (rows of 28672: two).  1537 rows, us, without
+    // / with: 6144 22.4 / 19.4, 8192 23.9 / 22.1, 14336 39.2 / 37.1, 24576 103 / 87; in the other forms it cost 3 to 8 % (28672, 1024 threads a row).
+    int run = 31;
+    if (pairs && kbits > 5) {
+        const int first = kbits > 10 ? 5 : (kbits + 1) / 2;
+        const size_t spaced = smem + static_cast<size_t>((K / m) >> first) * m * 4;
+        auto ctas = [](size_t bytes) { return std::min<size_t>(3, 228 * 1024 / (bytes + 1280)); };
+        if (spaced <= kMaxSmem && ctas(spaced) == ctas(smem)) {
+            run = first;
+            smem = spaced;
+        }
+    }
     const float inv_sqrt_k = static_cast<float>(1.0 / sqrt(static_cast<double>(K)));
     const unsigned grid = static_cast<unsigned>(rows < 148u * 16u ? rows : 148u * 16u);
     const __nv_bfloat16* x = static_cast<const __nv_bfloat16*>(X);
     auto kern = wide ? (m == 12 ? hadamard_quantize_kernel<12, kWideThreads> : hadamard_quantize_kernel<28, kWideThreads>)
-                : m == 1         ? (K < kSixteensWidth ? hadamard_quantize_kernel<1, kThreads> : hadamard_quantize_kernel<16, kThreads>)
-                : K < kPairWidth ? (m == 12 ? hadamard_quantize_kernel<12, kThreads, false> : hadamard_quantize_kernel<28, kThreads, false>)
-                                 : (m == 12 ? hadamard_quantize_kernel<12, kThreads> : hadamard_quantize_kernel<28, kThreads>);
+                : m == 1  ? hadamard_quantize_kernel<1, kThreads>
+                : m == 16 ? hadamard_quantize_kernel<16, kThreads>
+                : !pairs  ? (m == 12 ? hadamard_quantize_kernel<12, kThreads, false> : hadamard_quantize_kernel<28, kThreads, false>)
+                          : (m == 12 ? hadamard_quantize_kernel<12, kThreads> : hadamard_quantize_kernel<28, kThreads>);
     count_launch();
-    return launch_programmatic(kern, grid, wide ? kWideThreads : kThreads, smem, st, x, rows, K, kbits, r, inv_sqrt_k, q8, q4,
+    return launch_programmatic(kern, grid, wide ? kWideThreads : kThreads, smem, st, x, rows, K, kbits, run, r, inv_sqrt_k, q8, q4,
                                s8, s4, q4_i8);
 }
 
