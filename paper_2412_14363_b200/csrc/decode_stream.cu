@@ -853,13 +853,16 @@ Plan make_plan(int T, int N, int K, int r, int sms) {
     if (pl.units >= (1 << 24)) return pl;  // the kernel's 32-bit unit arithmetic
     pl.TT = T <= 8 ? 1 : 2;
     pl.TR = T % 8 == 0 ? T : T + 1;  // a zero row for the token columns beyond T
-    // Configurations in order of preference: split staging of the INT4 activations before packed for T <= 8 and the
-    // reverse above, the larger chunk (5 steps) before the smaller (3 steps); the first that leaves every warp four
-    // stages wins, else the last one tried that leaves two.
+    // Configurations in order of preference: split staging of the INT4 activations before packed for T <= 8, and above while the split codes
+    // take no more than 40 KB from the ring (beyond 2560 wide only where every SM has a unit), else the reverse; the larger chunk (5 steps)
+    // before the smaller (3 steps); the first that leaves every warp four stages wins, else the last one tried that leaves two.
+    // Time packed / split of 9, 12 and 16 tokens over five widths N from 1024 to 28672, both forms of codes: K = 256 to 1024 1.07-1.21, 2048 1.02-1.16,
+    // 2560 1.01-1.14; 3072 1.03-1.12 (N = 1024 0.96-1.06); 4096 at 9 tokens 1.02-1.10 (N = 1024 0.97), at 12 and 16 0.90-1.02.
+    const bool split_first = pl.TT == 1 || (pl.TR * K <= 40 * 1024 && (K <= 2560 || pl.units > sms));
     for (int pass = 0; pass < 2 && !pl.ok; ++pass) {
         const int need = pass == 0 ? 4 : kMinStages;
         for (int k = 0; k < 2 && !pl.ok; ++k) {
-            const int sp = pl.TT == 1 ? 1 - k : k;  // measured: split staging pays for T <= 8 only
+            const int sp = split_first ? 1 - k : k;
             for (int c : {5, 3}) {
                 const int chunk = 64 * c;
                 pl.c8 = (r + chunk - 1) / chunk;

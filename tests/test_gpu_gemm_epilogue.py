@@ -1,5 +1,5 @@
-"""The last step of the mixed products beyond 16 tokens: exact sums of every split of the reduction, then the scaled values, at the edges of the
-token groups and channel tiles, with and without the sums written out."""
+"""The mixed products, exact sums first, then the scaled values, with and without the sums written out: beyond 16 tokens every split of the
+reduction at the edges of the token groups and channel tiles; from 9 to 16 tokens both forms of staged activations."""
 import pytest
 import torch
 
@@ -18,12 +18,15 @@ def _unpack(w4, K4):
 @pytest.mark.parametrize("T,K,r,N,splits", [
     (17, 512, 64, 200, 1), (33, 256, 32, 264, 1), (300, 1024, 96, 520, 1), (40, 256, 224, 8, 1), (1537, 14336, 0, 4096, 1),
     (17, 8192, 1024, 8192, 2), (250, 14336, 0, 2184, 2), (23, 6144, 6112, 256, 3), (61, 14336, 1792, 1032, 3), (257, 14336, 32, 2048, 3),
-    (1700, 256, 32, 3000, 0), (2049, 512, 480, 2056, 0), (1793, 384, 0, 4104, 0), (2100, 256, 128, 2064, 0)])  # 0: 256 x 256 tiles
+    (1700, 256, 32, 3000, 0), (2049, 512, 480, 2056, 0), (1793, 384, 0, 4104, 0), (2100, 256, 128, 2064, 0),
+    (9, 256, 32, 1024, None), (16, 2560, 320, 136, None), (16, 2592, 320, 136, None), (9, 4096, 512, 1192, None), (9, 4096, 512, 1176, None),
+    (12, 3136, 0, 2000, None), (13, 2944, 2912, 2400, None), (15, 2048, 256, 3072, None)])  # None: weights streamed; 0: 256 x 256 tiles
 def test_sums_and_scales(T, K, r, N, splits, asym):
     import paper_2412_14363_b200 as resq
 
-    pl = plans.mid(T, K, N, r)
-    assert (pl.splits if pl.use else 0) == splits
+    if splits is not None:
+        pl = plans.mid(T, K, N, r)
+        assert (pl.splits if pl.use else 0) == splits
     g = torch.Generator(device="cuda").manual_seed(T + K)
     K4 = K - r
     desc = resq.layer_desc(K, N, r, resq.SCALE_FP16 if T % 2 else resq.SCALE_FP32)
