@@ -49,6 +49,7 @@ struct Params {
     // per tile) and summed in slice order by project_reduce_kernel.  0: no split.
     int full_items, split_tiles, splits, kb_slice, prows;
     float* partial;
+    int wide;  // C and the partial tiles start on 32 bytes
 };
 
 struct Item {
@@ -405,10 +406,18 @@ project_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_c
                 const int nb = it.n0 + c * 32;
                 if (!it.bounded || it.m0 + lrow < p.T) {
                     float* cp = it.dst + static_cast<size_t>(lrow) * it.ld + c * 32;
+                    // A store of 32 bytes is a whole sector, of 16 half of one: 4096 tokens 2048 x 2048 32.5 -> 30.2 us, 4096 x 4096 102 -> 97.6; 500 tokens
+                    // 14336 x 14336 191 -> 184.  K is a multiple of 8, so only C itself may lie otherwise.
+                    if (p.wide) {
 #pragma unroll
-                    for (int g = 0; g < 8; ++g)
-                        if (!it.bounded || nb + g * 4 < p.K)
-                            reinterpret_cast<uint4*>(cp)[g] = make_uint4(v[4 * g], v[4 * g + 1], v[4 * g + 2], v[4 * g + 3]);
+                        for (int g = 0; g < 4; ++g)
+                            if (!it.bounded || nb + g * 8 < p.K) st_global_8(cp + 8 * g, v + 8 * g);
+                    } else {
+#pragma unroll
+                        for (int g = 0; g < 8; ++g)
+                            if (!it.bounded || nb + g * 4 < p.K)
+                                reinterpret_cast<uint4*>(cp)[g] = make_uint4(v[4 * g], v[4 * g + 1], v[4 * g + 2], v[4 * g + 3]);
+                    }
                 }
             }
             tc_fence_before();
@@ -663,6 +672,7 @@ cudaError_t launch_project_few(const void* X, const void* P, int T, int K, float
     p.C = C;
     p.status = device_status_ptr();
     p.partial = static_cast<float*>(scratch);
+    p.wide = 0;  // of the tile kernel
     int sms = 148;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int tiles = p.n_tiles, all_pairs = sms / 2;
@@ -742,6 +752,7 @@ cudaError_t launch_project_gemm(const void* X, const void* P, int T, int K, floa
     if (tiles < pairs) pairs = tiles;
     // A last round that fills less than half of the grid is cut along K so that it takes a fraction of a round:
     // each of its tiles becomes `splits` work items whose partial tiles a second kernel adds up in slice order.
+    p.wide = (reinterpret_cast<uintptr_t>(C) | reinterpret_cast<uintptr_t>(scratch) | static_cast<uintptr_t>(K) * 4) % 32 == 0;
     p.full_items = tiles;
     p.split_tiles = p.splits = p.kb_slice = p.prows = 0;
     p.partial = static_cast<float*>(scratch);

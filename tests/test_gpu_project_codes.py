@@ -47,3 +47,27 @@ def test_codes_of_projected_rows(T, K, r, asym):
         assert torch.equal(q.float(), want)
     lohi = q4e.to(torch.int16) & 15
     assert torch.equal(q4.to(torch.int16), lohi[:, ::2] | lohi[:, 1::2] << 4)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("T,K", [(65, 264), (300, 1024), (1300, 4096), (257, 2056)])
+def test_projected_rows_anywhere(T, K):
+    """The same coefficients on 32 bytes (stores of 32) and 16 behind (stores of 16), and nothing behind the last row."""
+    import paper_2412_14363_b200 as resq
+
+    g = torch.Generator(device="cuda").manual_seed(T + K)
+    X = torch.randn(T, K, device="cuda", generator=g).to(torch.bfloat16)
+    P = (torch.randn(K, K, device="cuda", generator=g) / K ** 0.5).to(torch.bfloat16)
+    ws = torch.empty(int(resq.lib.resq_project_workspace_bytes()), dtype=torch.uint8, device="cuda")
+    outs = []
+    for skip in (0, 4):
+        buf = torch.full((skip + (T + 1) * K,), 9.0, device="cuda")
+        C = buf[skip:].view(T + 1, K)
+        resq.resq_project(X, P, C[:T], ws)
+        assert resq.resq_device_status() == resq.OK
+        assert (C[T] == 9).all() and (buf[:skip] == 9).all()
+        outs.append(C[:T])
+    assert torch.equal(*outs)
+    want = X.double() @ P.double()
+    size = X.double().abs() @ P.double().abs()
+    assert ((outs[0].double() - want).abs() <= K * 2.0 ** -23 * size).all()  # fp32 sums of exact products
