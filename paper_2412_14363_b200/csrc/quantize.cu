@@ -857,11 +857,12 @@ cudaError_t launch_fast(const void* in, size_t rows, int K, int r, int8_t* q8, u
     // Two stages when they are cheap (several CTAs per SM still fit) and a CTA has more than one group to do.  Asymmetric rows
     // take more arithmetic per byte and gain from more warps per SM instead: a CTA per group, one stage (8192 rows of 2048 /
     // 4096 / 14336: 19.0 / 34.6 / 100.4 us against 21.7 / 37.0 / 105.5 with two stages).
+    // With one stage a CTA per group, too, for wide symmetric rows: the next CTA's copy starts as soon as one has left (fp32 rows, us, a walk of as many
+    // CTAs as fit / this: 4096 of 14336 59.8 / 57.0, of 16384 64.5 / 61.1, 2048 of 28672 61.1 / 59.7, 1024 of 14336
+    // 17.5 / 16.5; bf16 rows 4096 of 20480 77 / 61.6, of 28672 91.2 / 87, 1000 of 28672 29.2 / 27).
     int nstages = 1;
-    size_t grid = 148 * ctas_per_sm(group_bytes);
-    if (ASYM) {
-        grid = groups;
-    } else if (groups > grid && 2 * group_bytes <= 64u * 1024u) {
+    size_t grid = groups;
+    if (!ASYM && groups > 148 * ctas_per_sm(group_bytes) && 2 * group_bytes <= 64u * 1024u) {
         nstages = 2;
         grid = 148 * ctas_per_sm(2 * group_bytes);
     }

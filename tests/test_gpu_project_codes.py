@@ -71,3 +71,26 @@ def test_projected_rows_anywhere(T, K):
     want = X.double() @ P.double()
     size = X.double().abs() @ P.double().abs()
     assert ((outs[0].double() - want).abs() <= K * 2.0 ** -23 * size).all()  # fp32 sums of exact products
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("T,K,r", [(1000, 16416, 2048), (700, 28672, 0)])
+def test_many_wide_rows(T, K, r):
+    """Rows too wide for two stages, more of them than CTAs fit: the codes of the same rows a hundred at a time."""
+    import paper_2412_14363_b200 as resq
+
+    g = torch.Generator(device="cuda").manual_seed(K)
+    X = torch.randn(T, K, device="cuda", generator=g).to(torch.bfloat16)
+
+    def run(X):
+        n = X.shape[0]
+        z = lambda shape, dt: torch.full(shape, 77, dtype=dt, device="cuda")
+        o = [z((n, r), torch.int8) if r else None, z((n, (K - r) // 2), torch.uint8), z((n,), torch.float32), z((n,), torch.float32),
+             z((n, K - r), torch.int8)]
+        resq.resq_project_quantize(X, None, r, *o)
+        assert resq.resq_device_status() == resq.OK
+        return [t for t in o if t is not None]
+
+    parts = [run(X[i:i + 100]) for i in range(0, T, 100)]
+    for i, got in enumerate(run(X)):
+        assert torch.equal(got, torch.cat([p[i] for p in parts]))
