@@ -273,8 +273,10 @@ int resq_project_quantize_static(const void* X, const void* P, int T, int K, int
  *  RESQ_OPT_DECODE_EARLY_WEIGHTS (default 0): when 1, the few-token kernel (T <= 16) is launched so
  *    that it may begin while the preceding kernel of the stream is still running; it then streams its
  *    packed weights into shared memory at once and only waits for that kernel before it reads the
- *    activation codes and scales.  (Inside resq_linear / resq_linear_asym that kernel is the library's quantizer,
- *    which starts its dependents only once everything before it is complete, so there it is always done.)  Generation is memory-bound (paper, Introduction), and this hides
+ *    activation codes and scales.  (Inside resq_linear / resq_linear_asym it follows the library's own quantizer, which
+ *    starts its dependents only once everything before it is complete, so there it is always done.  Calls of up to eight tokens that
+ *    quantize inside the product have no such kernel: they take their first weights behind the wait, whatever the
+ *    option says, and may directly follow the packing of their layer.)  Generation is memory-bound (paper, Introduction), and this hides
  *    the ramp of each short kernel behind the tail of the previous one.  The caller promises that the
  *    kernel enqueued just before writes none of the packed weights and scales (true for weights packed at load
  *    time; false if resq_pack_weights is that kernel): what was enqueued before the call that enqueued that one is

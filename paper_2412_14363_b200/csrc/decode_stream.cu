@@ -41,6 +41,7 @@
 // QUANT: the rows come as bf16 and every CTA quantizes all of them itself while its first weights are on their way, instead of reading the
 // codes that a kernel before this one wrote.  That kernel costs a launch on the host (2.4 us) and 2 to 3 us on the device, against
 // T K / 256 values per thread here.  A call of one token, 2048 x 3072: 6.6 -> 5.4 us on the device, 8.5 -> 5.8 on the host; where the rule lies: plans.h.
+// The kernel before this form is the caller's and may have packed the weights: it waits before its first copy.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -924,7 +925,7 @@ cudaError_t launch_mixed_gemm_stream(int T, int N, int K, int r, const int8_t* x
     p.c8 = pl.c8; p.c4 = pl.c4; p.pitch8 = pl.pitch8; p.pitch4 = pl.pitch4;
     p.nstages = pl.nstages;
     p.ring_ofs = static_cast<int>(pl.fixed);
-    p.early_weights = g_early_weights ? g_early_weights : after_quantizer ? kAfterQuantizer : 0;
+    p.early_weights = X ? 0 : g_early_weights ? g_early_weights : after_quantizer ? kAfterQuantizer : 0;
     p.x8 = x8; p.x4 = x4; p.s_x8 = s_x8; p.s_x4 = s_x4; p.s_w8 = s_w8; p.s_w4 = s_w4;
     p.w_fp16 = w_scale_fp16 ? 1 : 0;
     p.z_x8 = z_x8; p.z_x4 = z_x4; p.wsum8 = wsum8; p.wsum4 = wsum4;

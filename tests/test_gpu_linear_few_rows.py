@@ -59,3 +59,48 @@ def test_linear_of_few_rows(T, K, r, N, asym):
             assert resq.resq_device_status() == resq.OK
             same = (Y == want) | (Y.isnan() & want.isnan())
             assert same.all(), (X is forms[2], dt, (~same).sum().item())
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("asym", [False, True])
+@pytest.mark.parametrize("T,K,r,N", [(1, 4096, 512, 6144), (4, 2048, 256, 2048), (8, 1024, 128, 4096)])
+def test_weights_packed_just_before(T, K, r, N, asym):
+    """The call may directly follow the packing of its layer, also with the option that lets products of few tokens stream weights early."""
+    import ctypes
+
+    import paper_2412_14363_b200 as resq
+
+    g = torch.Generator(device="cuda").manual_seed(K)
+    desc = resq.layer_desc(K, N, r)
+    raw = [torch.randn(N, K, device="cuda", generator=g) for _ in range(2)]
+    W = resq.resq_pack_weights(desc, raw[0])
+    ws = (resq.alloc_workspace_asym if asym else resq.alloc_workspace)(desc, T, False, True)
+    X, Y = _rows(T, K, g), torch.empty((T, N), device="cuda")
+
+    def pack(i):
+        assert resq.lib.resq_pack_weights(ctypes.byref(desc), raw[i].data_ptr(), *(t.data_ptr() for t in (W.w8, W.w4, W.s_w8, W.s_w4, W.w4_i8)),
+                                          torch.cuda.current_stream().cuda_stream) == resq.OK
+
+    def linear(sums):
+        if asym:
+            resq.resq_linear_asym(W, *sums, X, None, Y, ws)
+        else:
+            resq.resq_linear(W, X, None, Y, ws)
+
+    sums, want = [], []
+    for i in range(2):
+        pack(i)
+        sums.append(resq.resq_weight_row_sums(W))
+        torch.cuda.synchronize()
+        linear(sums[i])
+        want.append(Y.clone())
+    resq.resq_set_option(resq.OPT_DECODE_EARLY_WEIGHTS, 1)
+    try:
+        for k in range(40):
+            torch.cuda._sleep(200000)  # the calls below are enqueued before the first of them runs
+            pack(k & 1)
+            linear(sums[k & 1])
+            assert torch.equal(Y, want[k & 1]), k
+    finally:
+        resq.resq_set_option(resq.OPT_DECODE_EARLY_WEIGHTS, 0)
+    assert resq.resq_device_status() == resq.OK

@@ -59,6 +59,15 @@ def test_what_another_grid_may_still_write_is_not_read_as_read_only(name):
             assert not re.search(r"const\s+\w+\s*\*\s*__restrict__", head), head
 
 
+def test_a_product_that_quantizes_its_rows_reads_no_weight_before_its_wait():
+    """The kernel before it is the caller's (resq_pack_weights, say), not a quantizer of the same call, and the option that a caller sets
+    for resq_mixed_gemm promises nothing about it."""
+    text = _code("decode_stream.cu")
+    assert re.findall(r"\bp\.early_weights = ([^;]*)", text) == ["X ? 0 : g_early_weights ? g_early_weights : after_quantizer ? kAfterQuantizer : 0"]
+    kernel = next(body for head, body in _kernels(text) if "mixed_gemm_stream_kernel" in head)
+    assert kernel.index("if (!p.early_weights) griddep_wait();") < kernel.index("issue(0)")
+
+
 TMEM_ACCESS = r"(?<!__forceinline__ void )\btmem_(?:ld|st)\d\w*\("
 TMEM_ACCESSES = {"kv_prefill.cu": 7, "mixed_gemm.cu": 2, "mixed_gemm_mid.cu": 3, "project.cu": 2}
 
