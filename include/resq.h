@@ -197,7 +197,9 @@ int resq_mixed_gemm(const resq_layer_desc_t* desc, int T, const int8_t* x8, cons
 
 /*
  * The whole layer: resq_project_quantize followed by resq_mixed_gemm, with the quantized
- * activations held in the workspace.  X bf16 [T][K]; P bf16 [K][K] or NULL; Y [T][n_out].
+ * activations held in the workspace.  X bf16 [T][K]; P bf16 [K][K] or NULL; Y [T][n_out].  Y may lie over X.
+ * Up to eight tokens without P are quantized inside the product, with the same codes, where that is the shorter way and Y does not
+ * meet X; the workspace, still required, then stays as it is.
  */
 int resq_linear(const resq_layer_desc_t* desc, int T, const void* X, const void* P,
                 const resq_weights_t* W, void* Y, int y_dtype, void* workspace, size_t workspace_bytes,

@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include "internal.h"
+#include "plans.h"
 #include "ptx.cuh"
 
 namespace resq {
@@ -104,6 +105,11 @@ Workspace carve(int K, int n_out, int r, int T, bool has_P, bool has_w4_i8) {
     w.panel = o;  o += has_P ? align_up(static_cast<size_t>(T < kPanelRows ? T : kPanelRows) * K * 4) + align_up(project_split_scratch_bytes()) : 0;
     w.total = o;
     return w;
+}
+
+// Whether Y of a layer may be written while X is still read.
+bool y_apart_from_x(const resq_layer_desc_t* d, int T, const void* X, const void* Y, int y_dtype) {
+    return !ranges_meet(X, static_cast<size_t>(T) * d->K * 2, Y, static_cast<size_t>(T) * d->n_out * (y_dtype == RESQ_Y_BF16 ? 2 : 4));
 }
 
 cudaError_t g_last_cuda_error = cudaSuccess;  // what the latest RESQ_ERR_CUDA stood for
@@ -349,7 +355,7 @@ int resq_linear(const resq_layer_desc_t* d, int T, const void* X, const void* P,
     float* s_x8 = reinterpret_cast<float*>(ws + map.sx8);
     float* s_x4 = reinterpret_cast<float*>(ws + map.sx4);
     const bool tiles = T > kDecodeMaxT;
-    if (!P && !tiles) {  // few rows: quantized by the product itself where that is the shorter way
+    if (!P && !tiles && y_apart_from_x(d, T, X, Y, y_dtype)) {  // few rows: quantized by the product itself where that is the shorter way
         const cudaError_t e = launch_mixed_gemm_stream(T, d->n_out, d->K, d->r, nullptr, nullptr, nullptr, nullptr, W->w8, W->w4, W->s_w8, W->s_w4,
                                                        d->w_scale_dtype == RESQ_SCALE_FP16, Y, y_dtype, nullptr, nullptr,
                                                        static_cast<cudaStream_t>(stream), false, nullptr, nullptr, nullptr, nullptr, X);
@@ -518,7 +524,7 @@ int resq_linear_asym(const resq_layer_desc_t* d, int T, const void* X, const voi
     float* s_x4 = reinterpret_cast<float*>(ws + map.sx4);
     float* z_x8 = reinterpret_cast<float*>(ws + map.zx8);
     float* z_x4 = reinterpret_cast<float*>(ws + map.zx4);
-    if (!P && T <= kDecodeMaxT) {  // few rows: quantized by the product itself where that is the shorter way
+    if (!P && T <= kDecodeMaxT && y_apart_from_x(d, T, X, Y, y_dtype)) {  // few rows: quantized by the product itself where that is the shorter way
         const cudaError_t e = launch_mixed_gemm_stream(T, d->n_out, d->K, d->r, nullptr, nullptr, nullptr, nullptr, W->w8, W->w4, W->s_w8, W->s_w4,
                                                        d->w_scale_dtype == RESQ_SCALE_FP16, Y, y_dtype, nullptr, nullptr,
                                                        static_cast<cudaStream_t>(stream), false, nullptr, nullptr, wsum8, wsum4, X);

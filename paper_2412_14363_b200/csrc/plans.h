@@ -58,6 +58,12 @@ inline bool quantizes_rows(int T, int K) {
     return T <= 8 && K <= (T > 2 ? 32 : 64) * threads;
 }
 
+// Not where Y lies over some of X: every CTA reads all rows, while others store already.  A quantizer of its own has read X by then.
+inline bool ranges_meet(const void* a, size_t a_bytes, const void* b, size_t b_bytes) {
+    const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+    return x < y ? y - x < a_bytes : x - y < b_bytes;
+}
+
 // ---- GPTQ packing (gptq.cu): rows per CTA, one CTA per SM.  As many as fit its shared memory (8 bytes per weight), then no
 // more than spread the rows evenly over the rounds this takes.
 constexpr int kGptqMaxRows = 8;                 // one rounding warp each

@@ -15,6 +15,7 @@ extern "C" {
 void mid(int T, int N, int kbt, int* o) { MidPlan p = mid_plan(T, N, kbt); o[0] = p.use; o[1] = p.ntok; o[2] = p.tok_tiles; o[3] = p.splits; }
 int together(int d, int kv_tiles, int tiles) { return append_tiles_together(d, kv_tiles, tiles); }
 int few(int T, int K) { return quantizes_rows(T, K); }
+int meet(size_t a, size_t an, size_t b, size_t bn) { return ranges_meet((const void*)a, an, (const void*)b, bn); }
 int gptq(int N, int K) { return gptq_rows_per_cta(N, K); }
 void prefill(int pos0, int T, int g, int Hkv, int d, int* o) {
     PrefillPlan p = prefill_plan(pos0, T, g, Hkv, d); o[0] = p.tiles_per_cta; o[1] = p.splits; o[2] = (int)p.row_groups; o[3] = p.pair; }
@@ -58,6 +59,10 @@ def gptq_rows(N, K):
 
 def quantizes_rows(T, K):
     return _lib().few(T, K)
+
+
+def ranges_meet(a, a_bytes, b, b_bytes):
+    return bool(_lib().meet(*(ctypes.c_size_t(v) for v in (a, a_bytes, b, b_bytes))))
 
 
 def append_together(d, T, Hq, Hkv):

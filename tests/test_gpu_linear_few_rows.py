@@ -12,6 +12,14 @@ def test_rule_for_quantizing_rows():
     assert not plans.quantizes_rows(9, 64)
 
 
+def test_ranges_that_meet():
+    base = 0x7F0000000000
+    for a, an, b, bn in ((0, 64, 64, 16), (64, 16, 0, 64), (0, 4096, 8192, 16), (0, 16, 16, 1 << 40)):
+        assert not plans.ranges_meet(base + a, an, base + b, bn)
+    for a, an, b, bn in ((0, 64, 0, 64), (0, 64, 48, 64), (48, 64, 0, 64), (0, 1 << 40, 1 << 39, 16), (16, 16, 0, 1 << 40), (0, 65, 64, 16)):
+        assert plans.ranges_meet(base + a, an, base + b, bn)
+
+
 def _rows(T, K, g):
     x = torch.randn(T, K, device="cuda", generator=g) * torch.exp2(torch.randint(-6, 7, (T, 1), device="cuda", generator=g))
     x[:, :: 97] *= 20
@@ -103,4 +111,46 @@ def test_weights_packed_just_before(T, K, r, N, asym):
             assert torch.equal(Y, want[k & 1]), k
     finally:
         resq.resq_set_option(resq.OPT_DECODE_EARLY_WEIGHTS, 0)
+    assert resq.resq_device_status() == resq.OK
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("asym", [False, True])
+@pytest.mark.parametrize("T,K,N,dt,at", [
+    (1, 2048, 2048, torch.bfloat16, 0), (4, 2048, 2048, torch.bfloat16, 0), (8, 1024, 1024, torch.bfloat16, 0), (9, 1024, 1024, torch.bfloat16, 0),
+    (17, 1024, 1024, torch.bfloat16, 0), (2, 4096, 2048, torch.float32, 0), (8, 1024, 512, torch.float32, 32), (3, 1024, 4096, torch.bfloat16, 4096),
+    (1, 16384, 16384, torch.bfloat16, 32752)])
+def test_y_over_x(T, K, N, dt, at, asym):
+    """Y on X, or on a part of it from byte `at` on: the bits of a call with buffers apart, many times over; right behind X it is one launch."""
+    import paper_2412_14363_b200 as resq
+
+    g = torch.Generator(device="cuda").manual_seed(K + T)
+    r = K // 8
+    desc = resq.layer_desc(K, N, r)
+    W = resq.resq_pack_weights(desc, torch.randn(N, K, device="cuda", generator=g))
+    sums = resq.resq_weight_row_sums(W) if asym else None
+    ws = (resq.alloc_workspace_asym if asym else resq.alloc_workspace)(desc, T, False, True)
+    x_bytes, y_bytes = T * K * 2, T * N * dt.itemsize
+    buf = torch.zeros(x_bytes + y_bytes, dtype=torch.uint8, device="cuda")
+    view = lambda start, n, t, cols: buf[start:start + n].view(t).view(T, cols)
+    X0 = _rows(T, K, g)
+
+    def linear(Y):
+        X = view(0, x_bytes, torch.bfloat16, K)
+        X.copy_(X0)
+        before = resq.resq_launch_count()
+        if asym:
+            resq.resq_linear_asym(W, *sums, X, None, Y, ws)
+        else:
+            resq.resq_linear(W, X, None, Y, ws)
+        return resq.resq_launch_count() - before
+
+    want = torch.empty((T, N), dtype=dt, device="cuda")
+    apart = linear(want)
+    assert linear(view(x_bytes, y_bytes, dt, N)) == apart == (1 if plans.quantizes_rows(T, K) else 2)
+    assert torch.equal(view(x_bytes, y_bytes, dt, N), want)
+    Y = view(at, y_bytes, dt, N)
+    for _ in range(25):
+        assert linear(Y) == 2
+        assert torch.equal(Y, want)
     assert resq.resq_device_status() == resq.OK
