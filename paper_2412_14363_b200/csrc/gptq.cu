@@ -229,14 +229,14 @@ __global__ void __launch_bounds__(kCtaThreads, 1) gptq_rows_kernel(const Params 
     const int rows = min(R, p.N - n0);
     const int K = p.K, r = p.r;
     const float* U = p.U;
+    // Blocks are kBlock wide but for the first, which takes what is left: a narrow last one would keep threads idle through all columns.
+    const int first_width = (K - 1) % kBlock + 1, first_groups = first_width >> 5;
     if (tid == 0) {
-        mbar_init(&ready, kWarps);
+        mbar_init(&ready, kWarps + max(kWarps - first_groups, 0));  // and the rounding warps without a group in the first block
         for (int g = 0; g < kGroups; ++g) mbar_init(&done[g], 1);
         abort_flag = 0;
         fence_mbar_init();
     }
-    // Blocks are kBlock wide but for the first, which takes what is left: a narrow last one would keep threads idle through all columns.
-    const int first_width = (K - 1) % kBlock + 1, first_groups = first_width >> 5;
     // parity of group g's phase in block b (groups beyond the first block's start a block later)
     auto done_parity = [&](int g, int b) { return static_cast<uint32_t>(b + (g >= first_groups ? 1 : 0)) & 1u; };
 
@@ -365,9 +365,18 @@ __global__ void __launch_bounds__(kCtaThreads, 1) gptq_rows_kernel(const Params 
         const int rr = active ? row : R - 1;
         const double s8 = static_cast<double>(scale[0][min(rr, rows - 1)]), s4 = static_cast<double>(scale[1][min(rr, rows - 1)]);
         const double s8_inv = s8 > 0.0 ? __ddiv_rn(1.0, s8) : 0.0, s4_inv = s4 > 0.0 ? __ddiv_rn(1.0, s4) : 0.0;
+        // A warp without a group in the first block has no say in its phase of `ready`, and two could complete while it sleeps in its wait.
+        // So it arrives too: at its start, then for the next phase when it has seen this one.
+        const bool onlooker = warp - kWarps >= first_groups;
+        if (onlooker && lane == 0) mbar_arrive(&ready);
+        auto block_ready = [&](int b) {
+            if (!warp_wait(&ready, b & 1, &abort_flag)) return false;
+            if (onlooker && lane == 0) mbar_arrive(&ready);
+            return true;
+        };
         for (int b = 0, c0 = 0; c0 < K; c0 += b == 0 ? first_width : kBlock, ++b) {
             const int groups = b == 0 ? first_groups : kGroups;
-            if (warp - kWarps >= groups && !warp_wait(&ready, b & 1, &abort_flag)) goto failed;  // every phase is waited for
+            if (warp - kWarps >= groups && !block_ready(b)) goto failed;
             // Diagonal blocks, two by turns: behind the errors where that fits, else in slots of two rows that wait for nothing now: the next
             // block's, which is handed over when this one is rounded, or behind the last block the second one's, whose errors nobody reads any more.
             double* diag = p.diag_pitch ? err + static_cast<size_t>(c0 + kBlock < K ? c0 + (b == 0 ? first_width : kBlock) : first_width)
@@ -387,7 +396,7 @@ __global__ void __launch_bounds__(kCtaThreads, 1) gptq_rows_kernel(const Params 
                 double* tri_ud = diag + (g & 1) * static_cast<size_t>(diag_pitch);
                 double2 y;
                 bool vouched = reciprocal_pair(d_own, y.x, y.y);
-                if (g < kWarps && !warp_wait(&ready, b & 1, &abort_flag)) goto failed;
+                if (g < kWarps && !block_ready(b)) goto failed;
                 auto keep_diagonal = [&] {  // once the group before the last has left its place
 #pragma unroll
                     for (int i = 0; i < 31; ++i)
