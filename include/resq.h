@@ -286,7 +286,8 @@ int resq_project_quantize_static(const void* X, const void* P, int T, int K, int
  *  RESQ_OPT_WAIT_LIMIT_US (default 2 000 000): wall-clock limit, in microseconds, of a single wait inside a
  *    kernel (for a copy to land, for a pipeline stage to be released).  Stored on the CURRENT device with a
  *    blocking copy; kernels enqueued afterwards on that device use it.  value >= 1; the kernels look at the
- *    limit only once a wait has lasted 100 us, so smaller values act as 100.
+ *    limit only once a wait has lasted 100 us, so smaller values act as 100 (in resq_pack_weights_gptq, whose warps wait for a
+ *    whole block of columns, values below a second act as a second).
  * Returns RESQ_ERR_SHAPE for an unknown option or value.
  */
 enum { RESQ_OPT_DECODE_EARLY_WEIGHTS = 1, RESQ_OPT_WAIT_LIMIT_US = 2 };
@@ -301,8 +302,8 @@ int resq_unpack_int4(const uint8_t* packed, int8_t* out, size_t rows, size_t col
 int resq_device_status(void* stream);
 
 /* Self-test of the failure path (no counterpart in the paper).  Every wait inside the kernels of this library is
- * bounded (Conventions above).  This call enqueues one small kernel whose only CTA waits for a barrier phase
- * that nothing completes: the wait runs out after the limit of RESQ_OPT_WAIT_LIMIT_US, the kernel records the
+ * bounded (Conventions above).  This call enqueues one small kernel whose only CTA waits, in each of the two forms of wait that
+ * the kernels use, for a barrier phase that nothing completes: the waits run out after the limit of RESQ_OPT_WAIT_LIMIT_US, the kernel records the
  * condition and returns by itself -- nothing traps, the context stays usable -- and the next resq_device_status
  * returns RESQ_ERR_TIMEOUT (and RESQ_OK again after that).  Set a short limit first (say 1000 us) and restore it
  * afterwards; with the default limit the kernel runs for two seconds. */

@@ -17,20 +17,23 @@ struct __align__(16) DeviceState {
 };
 __device__ DeviceState g_state = {0, 0, 2000000000ull};
 
-// A CTA that waits for a barrier phase nothing will ever complete: the bounded wait runs out, the kernel records
-// the condition and returns by itself.  Exercises the path every other kernel takes when a copy never lands.
+// A CTA whose two warps wait for a barrier phase nothing will ever complete, one in each form of a bounded wait: both run out, the
+// kernel records the condition and returns by itself.  Exercises the path every other kernel takes when a copy never lands.
 __global__ void wait_runs_out_kernel(int* status) {
     __shared__ uint64_t bar;
-    __shared__ int abort_flag;
+    __shared__ int abort_flag[2], ran_out;
     if (threadIdx.x == 0) {
         mbar_init(&bar, 1);
         fence_mbar_init();
-        abort_flag = 0;
+        abort_flag[0] = abort_flag[1] = ran_out = 0;
     }
     __syncthreads();
-    const bool done = mbar_wait(&bar, 0, &abort_flag, status);  // every thread polls; the first to time out tells the rest
+    const int form = threadIdx.x >> 5;
+    // polling: every thread for itself, and the first to time out tells the rest
+    const bool done = form == 0 ? mbar_wait(&bar, 0, &abort_flag[0], status) : mbar_wait_asleep(&bar, 0, &abort_flag[1], status, 0);
+    if (!done && (threadIdx.x & 31) == 0) atomicAdd(&ran_out, 1);
     __syncthreads();
-    if (threadIdx.x == 0 && (!done || abort_flag)) atomicOr(status, kStatusBitTimeout);
+    if (threadIdx.x == 0 && ran_out == 2) atomicOr(status, kStatusBitTimeout);
 }
 
 int* device_status_ptr() {

@@ -183,34 +183,9 @@ __device__ __forceinline__ void feed_back(double (&acc)[C][R], const float (&u)[
 }
 
 __device__ __forceinline__ void prefetch_l2(const float* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
-// Whole warp: waits for the phase of that parity; false when it does not come.  The warp sleeps in the wait, up to a millisecond at a time:
-// polling warps take issue slots from the updating ones (3 %).  The limit is the kernel's own, in wall-clock time (a sweep takes
-// tens of milliseconds at most): the library's limit of a wait may be set below what an updating warp takes for a block.
-__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
-    auto sleep_wait = [&] {
-        uint32_t ok;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(ok)
-            : "r"(smem_u32(bar)), "r"(parity), "r"(1000000u)
-            : "memory");
-        return ok != 0;
-    };
-    bool ok = sleep_wait();
-    if (!ok) {
-        const uint64_t t0 = global_timer_ns();
-        while (!(ok = sleep_wait())) {
-            if (*abort_flag) break;
-            if (global_timer_ns() - t0 > 10000000000ull) {
-                *abort_flag = 1;
-                break;
-            }
-        }
-    }
-    return __all_sync(0xffffffffu, ok);
-}
+// A block takes a millisecond at most (K = 14336: 0.3), so the caller's limit counts from a second on.  Polling instead of sleeping
+// takes issue slots from the updating warps (3 %).
+constexpr uint64_t kBlockNs = 1000000000;
 
 template <int R>
 __global__ void __launch_bounds__(kCtaThreads, 1) gptq_rows_kernel(const Params p) {
@@ -237,6 +212,7 @@ __global__ void __launch_bounds__(kCtaThreads, 1) gptq_rows_kernel(const Params 
         abort_flag = 0;
         fence_mbar_init();
     }
+    auto warp_wait = [&](uint64_t* bar, uint32_t parity) { return mbar_wait_asleep(bar, parity, &abort_flag, p.status, kBlockNs); };
     // parity of group g's phase in block b (groups beyond the first block's start a block later)
     auto done_parity = [&](int g, int b) { return static_cast<uint32_t>(b + (g >= first_groups ? 1 : 0)) & 1u; };
 
@@ -345,7 +321,7 @@ __global__ void __launch_bounds__(kCtaThreads, 1) gptq_rows_kernel(const Params 
             };
             for (int j = 0; j < prev0; j += 32) feed_32(j);
             for (int j = prev0; j < c0; j += 32) {  // the block before, group by group as it is rounded
-                if (!warp_wait(&done[(j - prev0) >> 5], done_parity((j - prev0) >> 5, b - 1), &abort_flag)) goto failed;
+                if (!warp_wait(&done[(j - prev0) >> 5], done_parity((j - prev0) >> 5, b - 1))) goto failed;
                 feed_32(j);
             }
             if (live) {  // handed over where its errors will go
@@ -370,7 +346,7 @@ __global__ void __launch_bounds__(kCtaThreads, 1) gptq_rows_kernel(const Params 
         const bool onlooker = warp - kWarps >= first_groups;
         if (onlooker && lane == 0) mbar_arrive(&ready);
         auto block_ready = [&](int b) {
-            if (!warp_wait(&ready, b & 1, &abort_flag)) return false;
+            if (!warp_wait(&ready, b & 1)) return false;
             if (onlooker && lane == 0) mbar_arrive(&ready);
             return true;
         };
@@ -410,7 +386,7 @@ __global__ void __launch_bounds__(kCtaThreads, 1) gptq_rows_kernel(const Params 
 #pragma unroll
                     for (int k = 0; k < R; ++k) acc[0][k] = err[static_cast<size_t>(k) * K + j0 + lane];
                     for (int before = 0; before < g; ++before) {
-                        if (!warp_wait(&done[before], done_parity(before, b), &abort_flag)) goto failed;
+                        if (!warp_wait(&done[before], done_parity(before, b))) goto failed;
 #pragma unroll
                         for (int part = 0; part < 2; ++part) {
                             float u_now[1][16];

@@ -91,6 +91,35 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
     return true;
 }
 
+// The same for a whole warp, asleep in the wait up to a millisecond at a time: for long waits beside warps whose issue slots polling would
+// take.  `at_least_ns`: what the wait may take when all is well, where the caller's limit may be set below that.
+__device__ __forceinline__ bool mbar_wait_asleep(uint64_t* bar, uint32_t parity, volatile int* abort_flag, const int* status, uint64_t at_least_ns) {
+    auto sleep_wait = [&] {
+        uint32_t ok;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok)
+            : "r"(smem_u32(bar)), "r"(parity), "r"(1000000u)
+            : "memory");
+        return ok != 0;
+    };
+    bool ok = sleep_wait();
+    if (!ok) {
+        const uint64_t t0 = global_timer_ns();
+        while (!(ok = sleep_wait())) {
+            if (*abort_flag) break;
+            const uint64_t limit = *reinterpret_cast<const volatile unsigned long long*>(status + 2);
+            if (global_timer_ns() - t0 > (limit > at_least_ns ? limit : at_least_ns)) {
+                *abort_flag = 1;
+                break;
+            }
+        }
+    }
+    return __all_sync(0xffffffffu, ok);
+}
+
 // ---------------------------------------------------------------- TMA
 __device__ __forceinline__ void tma_prefetch_desc(const void* tmap) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(tmap)) : "memory");

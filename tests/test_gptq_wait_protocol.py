@@ -84,6 +84,6 @@ def test_the_kernel_waits_as_the_model_does():
     assert "const bool onlooker = warp - kWarps >= first_groups;" in rounding
     assert rounding.count("if (onlooker && lane == 0) mbar_arrive(&ready);") == rounding.count("mbar_arrive(&ready)") == 2
     assert rounding.count("warp_wait(&ready") == 1 and "done_parity(before, b)" in rounding
-    assert re.search(r"if \(!warp_wait\(&ready, b & 1, &abort_flag\)\) return false;\s*if \(onlooker && lane == 0\) mbar_arrive\(&ready\);\s*return true;", rounding)
+    assert re.search(r"if \(!warp_wait\(&ready, b & 1\)\) return false;\s*if \(onlooker && lane == 0\) mbar_arrive\(&ready\);\s*return true;", rounding)
     assert len(re.findall(r"!block_ready\(b\)\) goto failed;", rounding)) == 2
     assert "return static_cast<uint32_t>(b + (g >= first_groups ? 1 : 0)) & 1u;" in text

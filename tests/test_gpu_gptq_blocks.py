@@ -45,3 +45,25 @@ def test_pack_weights_gptq_blocks(N, K, r, R, fp16):
     assert (host(W.w4)[rows] == pw.w4_packed).all()
     assert (host(W.s_w8.float())[rows].view(np.uint32) == pw.s8.view(np.uint32)).all()
     assert (host(W.s_w4.float())[rows].view(np.uint32) == pw.s4.view(np.uint32)).all()
+
+
+def test_a_short_wait_limit_leaves_a_sweep_alone():
+    """Warps wait for whole blocks of columns (0.2 ms here), longer than a limit that serves the waits of other kernels."""
+    import torch
+
+    import paper_2412_14363_b200 as resq
+
+    K, N = 8192, 296
+    g = torch.Generator(device="cuda").manual_seed(K)
+    Wp = torch.randn(N, K, device="cuda", generator=g) / K ** 0.5
+    U = torch.triu(torch.randn(K, K, device="cuda", generator=g) / K ** 0.5)
+    U.diagonal().copy_(torch.rand(K, device="cuda", generator=g) + 0.5)
+    desc = resq.layer_desc(K, N, 1024)
+    want = resq.resq_pack_weights_gptq(desc, Wp, U)
+    resq.resq_set_option(resq.OPT_WAIT_LIMIT_US, 100)
+    try:
+        got = resq.resq_pack_weights_gptq(desc, Wp, U)
+        assert resq.resq_device_status() == resq.OK
+    finally:
+        resq.resq_set_option(resq.OPT_WAIT_LIMIT_US, 2_000_000)
+    assert torch.equal(got.w8, want.w8) and torch.equal(got.w4_i8, want.w4_i8)

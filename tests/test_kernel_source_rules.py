@@ -68,6 +68,22 @@ def test_a_product_that_quantizes_its_rows_reads_no_weight_before_its_wait():
     assert kernel.index("if (!p.early_weights) griddep_wait();") < kernel.index("issue(0)")
 
 
+def test_waits_are_bounded_by_the_library_s_limit():
+    """Both forms of a bounded wait compare the clock with the limit that the caller may set.  Elsewhere it bounds only what a kernel does after a
+    wait has run out: up to a tenth of a second for copies still in flight."""
+    for name in SOURCES:
+        if name != "ptx.cuh":
+            text = _code(name)
+            drains = re.findall(r"global_timer_ns\(\) - \w+ < (\d+)ull\) \{\}", text)
+            assert text.count("global_timer_ns") == text.count("= global_timer_ns();") + len(drains), name
+            assert all(int(ns) <= 100_000_000 for ns in drains), name
+    text = _code("ptx.cuh")
+    forms = [_block(text, m.start()) for m in re.finditer(r"\bbool mbar_wait\w*\(", text)]
+    assert len(forms) == 2 and text.count("global_timer_ns") == 1 + sum(f.count("global_timer_ns") for f in forms)
+    for f in forms:
+        assert "const volatile unsigned long long*>(status + 2)" in f
+
+
 TMEM_ACCESS = r"(?<!__forceinline__ void )\btmem_(?:ld|st)\d\w*\("
 TMEM_ACCESSES = {"kv_prefill.cu": 7, "mixed_gemm.cu": 2, "mixed_gemm_mid.cu": 3, "project.cu": 2}
 
