@@ -510,21 +510,37 @@ __global__ void __launch_bounds__(kWarps * 32, 1) attention_decode_kernel(const 
     }
 }
 
+__device__ __forceinline__ void cp_async_16(void* smem, const float* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(smem)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
 // Merges the partial records of one (sequence, query head): out = sum_i 2^(m_i - M) o_i / sum_i 2^(m_i - M) l_i.
 // The warps that hold a record of this (sequence, KV head) are those whose runs meet its range of the block
 // list.  The CTA has 128 x G threads, an output coefficient each: group g adds records CHUNK g .. CHUNK (g + 1) - 1, then those
-// G * CHUNK on, and the groups' sums meet in shared memory.  G = 4 when few (sequence, head) pairs share the grid's warps (long contexts:
+// G * CHUNK on, and the groups' sums meet in shared memory.  G = 2 or 4 when few (sequence, head) pairs share the grid's warps (long contexts:
 // hundreds of records each), else 1.  What bounds it is latency: a thread asks for coefficient, reference and sum of a whole chunk of
 // records at once, a single trip to memory (with the references first, a vote on their maximum and then the records: 5.1 us from the
-// end of the wait to the last output, now 3.6; references by lanes and shuffles: slower).  CHUNK is what a pair has by the sizes: a chunk of 16
-// takes 103 registers, and with four CTAs per SM 8192 merges of two or three records take 5 us longer (74 us of a call) than with chunks of four.
+// end of the wait to the last output, now 3.6; references by lanes and shuffles: slower).  CHUNK is what a pair has by the sizes, if all sequences are
+// equally long: a chunk of 16 takes 103 registers, and with four CTAs per SM 8192 merges of two or three records take 5 us longer (74 us of
+// a call) than with chunks of four.
+// One long sequence among many short ones has hundreds of records all the same.  Four at a trip they set the call's time, so from kMany + 1
+// on the four warps take four of every sixteen each through shared memory (the aligned 16-byte pieces that hold the head's 130 floats), the
+// next four on their way.  80 sequences of 8 heads (32 query heads), one of 32768 positions beside 32 73.7 -> 55.6 us, of 8192 beside 200
+// 32.5 -> 28.3; all of 400: within 1 %.  All 128 threads in step over sixteen records: 63.8 and 32.0.
 // Launched so that it may start while the attention kernel drains: everything before griddepcontrol.wait reads only the sequence lengths, which are
 // complete (the attention kernel lets its dependents start after its own wait).
-constexpr int kMaxGroups = 4;
+constexpr int kMaxGroups = 4, kMany = 16, kRecVecs = (kD + 2 + 2) / 4;
+static_assert(kRecFloats % 4 == 0 && kMany == 4 * (kD / 32), "aligned pieces, those of a record's last head end with it; four to a warp");
 template <int CHUNK>
 __global__ void __launch_bounds__(kD * kMaxGroups, CHUNK == 4 ? 3 : 1) attention_combine_kernel(const AttnParams p) {
     __shared__ long long red[2][kD * kMaxGroups / 32];
     __shared__ float part_s[kMaxGroups][kD], ml_s[kMaxGroups][2];  // of the groups
+    __shared__ float4 many_s[CHUNK == 4 ? kD / 32 : 1][2][CHUNK == 4 ? CHUNK : 1][kRecVecs];
     const int n_q_heads = p.n_kv_heads * p.group;
     const int b = blockIdx.x / n_q_heads, hq = blockIdx.x - b * n_q_heads;
     const int hk = hq / p.group, hg = hq - hk * p.group;
@@ -577,47 +593,100 @@ __global__ void __launch_bounds__(kD * kMaxGroups, CHUNK == 4 ? 3 : 1) attention
     }
     if (w_first == w_last) return;  // one warp saw the whole (sequence, head) and wrote the output itself
     const long long s = static_cast<long long>(b) * p.n_kv_heads + hk;
-    float M = -INFINITY, num = 0.f, den = 0.f;  // this group's share
-    for (int w0 = w_first + CHUNK * grp; w0 <= w_last;) {
-        const float* rec = p.partial + (w0 + s) * kRecFloats + hg * (kD + 2);
-        float2 ml[CHUNK];
-        float v[CHUNK];
-#pragma unroll
-        for (int k = 0; k < CHUNK; ++k) {
-            ml[k] = make_float2(-INFINITY, 0.f);
-            v[k] = 0.f;
-            if (mask >> k & 1u) {
-                ml[k] = __ldcg(reinterpret_cast<const float2*>(rec + k * kRecFloats));
-                v[k] = __ldcg(rec + k * kRecFloats + 2 + d);
+    int sums = groups;
+    if (CHUNK == 4 && w_last - w_first >= kMany) {
+        const int skip = hg & 1 ? 2 : 0;  // records of odd heads start 8 bytes behind 16
+        float M = -INFINITY, den = 0.f, num[4] = {0.f, 0.f, 0.f, 0.f};  // this warp's share, coefficients 4 lane to 4 lane + 3
+        auto ask = [&](int w0, int buf) {
+            const unsigned have = records(w0);
+            const float* rec = p.partial + (w0 + s) * kRecFloats + hg * (kD + 2) - skip;
+            for (int i = lane; i < CHUNK * kRecVecs; i += 32) {
+                const int k = i / kRecVecs, j = i - k * kRecVecs;
+                if (have >> k & 1u) cp_async_16(&many_s[warp][buf][k][j], rec + k * kRecFloats + 4 * j);
             }
-        }
-        float Mn = M;
+            cp_async_commit();
+            return have;
+        };
+        int w0 = w_first + CHUNK * warp, buf = 0;
+        unsigned next = ask(w0, 0), behind = ask(w0 + kMany, 1);
+        for (; w0 <= w_last; w0 += kMany, buf ^= 1) {
+            cp_async_wait<1>();
+            __syncwarp();
+            const float* r = reinterpret_cast<const float*>(many_s[warp][buf]) + skip;
+            float2 ml[CHUNK];
+            float Mn = M;
 #pragma unroll
-        for (int k = 0; k < CHUNK; ++k) Mn = fmaxf(Mn, ml[k].x);
-        const float resc = M == -INFINITY ? 0.f : ex2(M - Mn);
-        num *= resc;
-        den *= resc;
-        M = Mn;
+            for (int k = 0; k < CHUNK; ++k) {
+                ml[k] = *reinterpret_cast<const float2*>(r + 4 * kRecVecs * k);
+                if (!(next >> k & 1u)) ml[k] = make_float2(-INFINITY, 0.f);
+                Mn = fmaxf(Mn, ml[k].x);
+            }
+            const float resc = M == -INFINITY ? 0.f : ex2(M - Mn);
+            M = Mn;
+            den *= resc;
 #pragma unroll
-        for (int k = 0; k < CHUNK; ++k) {
-            const float f = mask >> k & 1u ? ex2(ml[k].x - Mn) : 0.f;
-            num = fmaf(f, v[k], num);
-            den = fmaf(f, ml[k].y, den);
+            for (int j = 0; j < 4; ++j) num[j] *= resc;
+#pragma unroll
+            for (int k = 0; k < CHUNK; ++k) {
+                if (!(next >> k & 1u)) continue;
+                const float f = ex2(ml[k].x - Mn);
+                const float2 a = *reinterpret_cast<const float2*>(r + 4 * kRecVecs * k + 2 + 4 * lane);
+                const float2 b = *reinterpret_cast<const float2*>(r + 4 * kRecVecs * k + 4 + 4 * lane);
+                den = fmaf(f, ml[k].y, den);
+                num[0] = fmaf(f, a.x, num[0]); num[1] = fmaf(f, a.y, num[1]);
+                num[2] = fmaf(f, b.x, num[2]); num[3] = fmaf(f, b.y, num[3]);
+            }
+            __syncwarp();  // before the next ones come in
+            next = behind;
+            behind = ask(w0 + 2 * kMany, buf);
         }
-        w0 += CHUNK * groups;
-        if (w0 <= w_last) mask = records(w0);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) part_s[warp][4 * lane + j] = num[j];
+        if (lane == 0) { ml_s[warp][0] = M; ml_s[warp][1] = den; }
+        sums = kD / 32;
+    } else {
+        float M = -INFINITY, num = 0.f, den = 0.f;  // this group's share
+        for (int w0 = w_first + CHUNK * grp; w0 <= w_last;) {
+            const float* rec = p.partial + (w0 + s) * kRecFloats + hg * (kD + 2);
+            float2 ml[CHUNK];
+            float v[CHUNK];
+    #pragma unroll
+            for (int k = 0; k < CHUNK; ++k) {
+                ml[k] = make_float2(-INFINITY, 0.f);
+                v[k] = 0.f;
+                if (mask >> k & 1u) {
+                    ml[k] = __ldcg(reinterpret_cast<const float2*>(rec + k * kRecFloats));
+                    v[k] = __ldcg(rec + k * kRecFloats + 2 + d);
+                }
+            }
+            float Mn = M;
+    #pragma unroll
+            for (int k = 0; k < CHUNK; ++k) Mn = fmaxf(Mn, ml[k].x);
+            const float resc = M == -INFINITY ? 0.f : ex2(M - Mn);
+            num *= resc;
+            den *= resc;
+            M = Mn;
+    #pragma unroll
+            for (int k = 0; k < CHUNK; ++k) {
+                const float f = mask >> k & 1u ? ex2(ml[k].x - Mn) : 0.f;
+                num = fmaf(f, v[k], num);
+                den = fmaf(f, ml[k].y, den);
+            }
+            w0 += CHUNK * groups;
+            if (w0 <= w_last) mask = records(w0);
+        }
+        if (groups == 1) {
+            out[d] = num / den;
+            return;
+        }
+        part_s[grp][d] = num;
+        if (d == 0) { ml_s[grp][0] = M; ml_s[grp][1] = den; }
     }
-    if (groups == 1) {
-        out[d] = num / den;
-        return;
-    }
-    part_s[grp][d] = num;
-    if (d == 0) { ml_s[grp][0] = M; ml_s[grp][1] = den; }
     __syncthreads();
     if (grp == 0) {
-        float Mn = M, nsum = 0.f, dsum = 0.f;
-        for (int g = 1; g < groups; ++g) Mn = fmaxf(Mn, ml_s[g][0]);
-        for (int g = 0; g < groups; ++g) {
+        float Mn = ml_s[0][0], nsum = 0.f, dsum = 0.f;
+        for (int g = 1; g < sums; ++g) Mn = fmaxf(Mn, ml_s[g][0]);
+        for (int g = 0; g < sums; ++g) {
             const float f = ml_s[g][0] == -INFINITY ? 0.f : ex2(ml_s[g][0] - Mn);  // -INF: no record
             nsum = fmaf(f, part_s[g][d], nsum);
             dsum = fmaf(f, ml_s[g][1], dsum);

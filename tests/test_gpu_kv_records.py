@@ -1,6 +1,6 @@
 """Attention of single rows at d_head = 128 where its block list and its merge have edges: more sequences than a warp scans at once,
-runs of no block, records of one (sequence, head) in more than one chunk of sixteen and in all four groups of threads, every group size of
-heads; against softmax in 64 bits over the dequantized cache."""
+runs of no block, records of one (sequence, head) in more than one chunk of sixteen and in all four groups of threads, in chunks of eight, and
+many of one sequence beside few of the others (edges of the sixteen that four warps share); against softmax in 64 bits over the dequantized cache."""
 import math
 
 import pytest
@@ -32,6 +32,9 @@ def _dequantize(cache, b, n, which):
     (3, 2, [17 + 29 * i for i in range(33)]),         # a second scan of one sequence
     (8, 4, [(37 * i) % 600 for i in range(100)]),     # four scans, lengths of 0 among them
     (8, 7, [6000 - 371 * i for i in range(16)]),      # records in one chunk of sixteen
+    (2, 3, [100 + 31 * i for i in range(150)]),       # in one chunk of eight
+    (8, 4, [512, 513, 545, 1056, 1088] + [20] * 75),  # 16, 17, 18, 33 and 34 records of single blocks, some runs of none
+    (4, 7, [9000, 3000] + [50 + i for i in range(160)]),  # about 200 and 65 records
 ])
 def test_attention_records(Hkv, group, lens):
     import paper_2412_14363_b200 as resq
