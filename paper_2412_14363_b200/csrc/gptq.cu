@@ -23,7 +23,7 @@
 // 512 columns of U take in the updating warps alone, R = 7 (112 in the fp64 pipe): 165 with one column per thread, 135 with two
 // (half the broadcasts and loads), 131 with four or eight rows of U asked for again where they were used instead of copied.
 // K = N = 4096: 65.1 ms right-looking, 11.5 ms left-looking with all warps waiting for the chain (two CTAs per
-// SM), 7.2 ms with a rounding warp per row, 6.2 with blocks of 256 and one column per thread, 5.4 ms as it stands (3.7 ms if the fp64 pipe
+// SM), 7.2 ms with a rounding warp per row, 6.2 with blocks of 256 and one column per thread, 5.5 ms as it stands (3.7 ms if the fp64 pipe
 // were always busy).  Of its 10300 cycles alone a group of 32 columns spent 8500 in the chain, 270 a step; now 4200 of 6100
 // (512 columns, 256 rows: 105 -> 78 us).  U comes from DRAM where it
 // does not stay in L2 (the first call on it, K above 4096), later than the loads a thread has on their way: the updating warps ask L2
@@ -183,7 +183,7 @@ __device__ __forceinline__ void feed_back(double (&acc)[C][R], const float (&u)[
 }
 
 __device__ __forceinline__ void prefetch_l2(const float* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
-// A block takes a millisecond at most (K = 14336: 0.3), so the caller's limit counts from a second on.  Polling instead of sleeping
+// A block takes a millisecond at most (K = 14336: 0.5), so the caller's limit counts from a second on.  Polling instead of sleeping
 // takes issue slots from the updating warps (3 %).
 constexpr uint64_t kBlockNs = 1000000000;
 

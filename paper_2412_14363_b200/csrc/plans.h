@@ -19,9 +19,9 @@ struct MidPlan {
 //   tile kernel  rounds * (k-blocks * 295 + 4100) + 5800, a round being 74 tiles of 256 x 256 (within a tenth of 1214 times
 //                over 22 layer shapes, 1024 x 2048 to 28672 x 8192, and 17 to 4096 tokens, weights in L2 and not).
 // Where several waves follow one another the first line is short by 12 % and 1500 ns a wave, for the ends that the persistent
-// kernel overlaps.  Over those 1214 calls the choice is 0.1 % slower than the better kernel of each, at most 4 %; with
-// the tile kernel taken at rounds * (294 k-blocks + 5000) + 10600, as measured before its products were issued by a
-// converged warp, and 5 % for several waves, it was 2.1 % (4096 x 4096 at 3500 tokens 71 us instead of 51).
+// kernel overlaps.  All of this was measured with the epilogues that both kernels had before the present ones: over those 1214 calls
+// the choice was 0.1 % slower than the better kernel of each, at most 4 %.  With the present epilogues (both kernels over 240
+// shapes, 917 runs) it is 0.4 %, a new fit of the same form 0.15 %.
 inline MidPlan mid_plan(int T, int N, int kbt) {
     constexpr int kTile = 256;  // tokens and channels of a large tile
     const long ch = (N + kTile - 1) / kTile;
@@ -52,7 +52,8 @@ inline MidPlan mid_plan(int T, int N, int kbt) {
 // its values in registers: up to 64 each, where all or half of the threads share a row, else 32.  us on the device, a quantizer before / in the
 // product (K x N, symmetric): one row 1024 x 1024 6.8 / 4.8, 2048 x 3072 6.6 / 5.4, 4096 x 28672 14.1 / 13.2, 14336 x 4096 12.1 / 10.7; two rows
 // 2048 x 3072 6.9 / 6.0, 8192 x 8192 12.2 / 11.9; four rows 2048 x 3072 7.3 / 6.7, but 4096 x 6144 9.0 / 9.8; six rows 1024 x 1024 6.6 / 6.4, but
-// 2048 x 3072 7.4 / 8.2.
+// 2048 x 3072 7.4 / 8.2.  Weights from memory, 130 calls within the rule, both forms of codes: 0.73 to 1.00 of the time, but two rows of
+// 6144 x 6144 and 8192 x 8192 and three of 2048 x 16384 1.03 to 1.04, one of 12288 x 4096 1.02 (the host's 2.4 us less beside it).
 inline bool quantizes_rows(int T, int K) {
     const int threads = T > 4 ? 32 : T > 2 ? 64 : T > 1 ? 128 : 256;  // of a row
     return T <= 8 && K <= (T > 2 ? 32 : 64) * threads;
@@ -100,7 +101,8 @@ struct PrefillPlan {
 // to 1184 tokens behind 0 to 8 times as many, within 3 % but for one round more), ns: in turn 1330 a step and 13500, together 2080
 // a step of two tiles and 10000; CTAs beyond 148 are a part of the last row group and follow another part of it.  1024 tokens, us in
 // turn / together: at 0 36 / 44, behind 512 57 / 60, 1024 79 / 77, 4096 205 / 176, 8192 376 / 310.  Beyond two rounds
-// together: 2048 tokens 114 / 82, behind 4096 447 / 349.
+// together: 2048 tokens 114 / 82, behind 4096 447 / 349.  Measured while all scores of a pair came behind its output product; now a
+// step of it takes 2030, which would take one of those 35 shapes to the other form (1184 tokens behind 592).
 inline bool prefill_together(int pos0, int T, int g, int Hkv, long long single) {
     auto steps = [=](long long tile) -> long long {  // of 64 positions, up to the last one that the tile's rows see
         const long long last = (tile * 128 + 127) / g;

@@ -606,7 +606,7 @@ __global__ void __launch_bounds__(NT, NT == kThreads ? (M > 1 ? 3 : 5) : 1)
 hadamard_quantize_kernel(const __nv_bfloat16* X, size_t rows, int K, int kbits, int run, int r, float inv_sqrt_k,
                          int8_t* __restrict__ q8, uint8_t* __restrict__ q4, float* __restrict__ s8_out,
                          float* __restrict__ s4_out, int8_t* __restrict__ q4e) {
-    extern __shared__ __align__(16) float hrow[];  // [K]
+    extern __shared__ __align__(16) float hrow[];  // [K], and the places left free behind runs (slot_of)
     __shared__ float red[2][NT / 32];
     const int tid = threadIdx.x;
     const int nchunks = K >> 3, rchunks = r >> 3;

@@ -1,5 +1,5 @@
-"""GPTQ packing where its blocks of 512 columns have edges: a narrow first block, one to eight blocks, and rows so long that U's diagonal
-blocks lie in the errors' slots.  Rows do not interact, so the oracle's fp64 sweep takes some of them: those of the first and the last
+"""GPTQ packing where its blocks of 512 columns have edges: a narrow first block, alone or before others, one to 28 blocks, and rows so long that
+U's diagonal blocks lie in the errors' slots.  Rows do not interact, so the oracle's fp64 sweep takes some of them: those of the first and the last
 CTA and a few between.  Bit for bit."""
 import numpy as np
 import pytest
@@ -13,6 +13,8 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("N,K,r,R,fp16", [
+    (24, 96, 32, 1, True),        # a block of three groups: rounding warps without one
+    (592, 512, 64, 4, False),     # one whole block
     (16, 544, 32, 1, False),      # a first block of one group
     (304, 1056, 64, 3, True),     # the same before two whole ones
     (904, 992, 96, 7, False),     # a first block of 15 groups
